@@ -117,9 +117,8 @@ enum {
   V3DG_OPT_CAP_NODES = 3,    /* current render-list capacity in clusters (>= 64); grows on demand */
   V3DG_OPT_CAP_PAIRS = 4,    /* current (tile, Gaussian) pair capacity (>= 4096); grows on demand */
   V3DG_OPT_COUNT_WORK = 5,   /* 1: the blend also counts its evaluations (v3dg_stats.blend_*) */
-  V3DG_OPT_SPLIT_PAIRS = 6,  /* tiles with at least this many pairs are blended as four 8x8
-                                quadrants by separate blocks (default 2^32 - 1: no split; the
-                                image does not depend on it) */
+  V3DG_OPT_SPLIT_PAIRS = 6,  /* 1 .. 2^32 - 1: accepted and without effect (blend variant 0 always
+                                spreads a tile over eight warps, variant 1 never splits one) */
   V3DG_OPT_ATTR_FP16 = 7,    /* 1: assets loaded from now on keep opacity and SH in float16 (rounded
                                 to nearest even); means, scales and rotations stay float32 and all
                                 arithmetic stays float32 */
@@ -130,16 +129,15 @@ enum {
                                 to its parent, Sec. 3.4), in the same order.  0: the flat test of
                                 every (instance, node).  2 (default): top-down when that would be
                                 more than 8M tests, else flat. */
-  V3DG_OPT_BLEND_BATCH = 9,    /* records the blend stages per batch in shared memory: 128, 256
-                                or 512 (default); the image does not depend on it */
+  V3DG_OPT_BLEND_BATCH = 9,    /* records that blend variant 1 stages per batch in shared memory: 128,
+                                256 or 512 (default); the image does not depend on it */
   V3DG_OPT_BLEND_MODE = 11,    /* blend kernel variant, the same image bit for bit: 0 (default)
-                                two phases per batch, a record-parallel alpha test into per-pixel
-                                masks, then pixel-parallel compositing; 1: each batch staged into
+                                every warp walks its tile's list for 8x4 pixels on its own; 1: one
+                                block per tile, each batch staged into
                                 shared memory by bulk copies (cp.async.bulk, one per 48-byte record,
                                 completing on an mbarrier with a bounded wait), then composited by
                                 warps that each own two pixel rows and walk only the records whose
-                                box spans them.  Variant 1 always blends whole tiles
-                                (V3DG_OPT_SPLIT_PAIRS is ignored). */
+                                box spans them. */
   V3DG_OPT_SERVE_MERGE = 12,   /* server (read at v3dg_server_start): a slot that takes a request
                                 also takes up to this many - 1 queued requests with the same image
                                 size, intrinsics and near plane whose memory estimates fit the
@@ -212,12 +210,11 @@ v3dg_status v3dg_select_views(v3dg_ctx* ctx, const v3dg_camera* cams, uint32_t n
  * (V3DG_ENOTFOUND otherwise). */
 v3dg_status v3dg_render(v3dg_ctx* ctx, float* rgb_out, float* T_out);
 
-/* Autotuner of the blend's kernel variant, batch size and work split.  Re-runs the blend stage of
- * the last rendered frame (its sorted pairs and records are still on the device) with every
- * combination of variant (V3DG_OPT_BLEND_MODE 0, 1), records per batch (128, 256, 512) and, for
- * variant 0, long-tile split threshold (4096, 16384, 65536 pairs, or none), times each with CUDA
- * events (best of 3 after one warm-up run) and keeps the fastest as V3DG_OPT_BLEND_MODE,
- * V3DG_OPT_BLEND_BATCH and V3DG_OPT_SPLIT_PAIRS for the frames that follow.  None changes the
+/* Autotuner of the blend's kernel variant and batch size.  Re-runs the blend stage of the last
+ * rendered frame (its sorted pairs and records are still on the device) with variant 0
+ * (V3DG_OPT_BLEND_MODE) and with variant 1 at 128, 256 and 512 records per batch, times each with
+ * CUDA events (best of 3 after one warm-up run) and keeps the fastest as V3DG_OPT_BLEND_MODE and
+ * V3DG_OPT_BLEND_BATCH for the frames that follow; *split_pairs is 2^32 - 1.  None changes the
  * image.  Synchronous; the caller's image is not touched.  V3DG_ENOTFOUND without a rendered
  * frame, V3DG_EOVERFLOW if that frame was not valid.  mode, batch, split_pairs, best_ms: the choice
  * and its time, each may be NULL.  The paper has no counterpart (its rasterizer is fixed). */

@@ -1,21 +1,28 @@
 // Per-tile front-to-back alpha blending (Sec. 2.1): C = sum_i c_i a_i prod_{j<i} (1 - a_j).
 //
-// One 256-thread block per 16x16 tile, or per 8x8 quadrant of a tile with a long list
-// (persistent blocks take work items heaviest-first: tiles differ in cost by orders of magnitude).
-// The tile's depth-ordered records are taken in batches (128, 256 or 512 records); each batch runs
-// in two phases:
-//  - record-parallel test: each thread stages its own records and evaluates each at the pixels of
-//    its alpha >= 1/255 box that are still accumulating; a pixel where the skip rule passes gets
-//    the record's bit in its mask (one bit per record of the batch);
-//  - pixel-parallel blend: each thread walks its pixel's mask in record (= depth) order and
-//    blends exactly those records: a = min(0.999, 2^(na dx^2 + nb dx dy + nc dy^2 + log2 o)),
-//    stopping before T (1 - a) < 1e-4.
-// So sequential work is spent only where a Gaussian contributes, and small Gaussians (a few
-// pixels each) no longer occupy whole warps.  Records are staged through shared memory; a batch
-// is filled only with records whose box holds a pixel that is still accumulating, found by
-// scanning ahead in the sorted pair keys, which carry each Gaussian's box within the tile (so
-// skipped records cost one coalesced 4-byte read).  Each record's mean is stored relative to the
-// pixel origin of its first tile, so dx, dy are differences of small numbers.
+// k_blend (variant 0): the work item is one warp's 8x4 pixels of a 16x16 tile, and no warp ever waits
+// for another one.  A warp walks its tile's depth-ordered list of pairs by the keys alone (they
+// carry each Gaussian's box within the tile), collects the records whose box meets the bounding
+// rectangle of its unfinished pixels, gathers 32 of them at a time (one per lane), stages them in
+// two lists, one for each 4x4 half of its pixels, and composites those in order, each half-warp its
+// own list: a = min(0.999, 2^(na dx^2 + nb dx dy + nc dy^2 + log2 o)), stopping before
+// T (1 - a) < 1e-4.  Key loads, slot loads, record loads and compositing belong to successive
+// batches, so the three dependent global latencies overlap with the compositing.
+//
+// Why warps and 8x4: the blend is bound by the serial chain of the longest lists (a tile whose pixels
+// never all finish walks its whole list: 125k pairs in the 1080p crowd) and, on full frames, by
+// issue and shared-memory reads.  A block per tile with a barrier around each batch (the two-phase
+// kernel before this one) had one block on each long list, its warps idle at the barriers.  Blend
+// stage on a GB300, before -> now: 96x80 thumbnail 158 -> 35 us, 256x256 viewer 266 -> 61 us, 200
+// instances at 640x360 655 -> 289 us, one asset filling 1080p 1671 -> 309 us, the same 50 units
+// away 768 -> 254 us, crowd at 1080p 2.75 -> 1.29 ms, 16 crowd views 31.9 -> 11.2 ms.  The same
+// kernel with 8x8 pixels a warp (two per lane, four lists): 57 us, 510 us, 293 us and 1.74 ms on the
+// thumbnail, the 200 instances, the near asset and the crowd; 8x4 with one list: 72, 414, 307 us and
+// 1.41 ms; 4 or 8 records ahead and 5 to 8 blocks per SM: within 10% of each other.
+// Each record's mean is stored relative to the pixel origin of its first tile, so dx, dy are
+// differences of small numbers.
+//
+// k_blend_px (variant 1): one block per tile, batches staged by bulk copies (see below).
 #include <algorithm>
 
 #include "dev_common.cuh"
@@ -23,8 +30,10 @@
 namespace v3dg {
 namespace {
 
-constexpr int kBlendThreads = 256;
-constexpr int kBlendWarps = kBlendThreads / 32;
+constexpr int kBlendThreads = 128;   // four independent warps (the block is only a launch unit)
+constexpr int kBlendBlocks = 6;      // resident blocks per SM: 24 warps of at most 80 registers
+constexpr int kPxThreads = 256;
+constexpr int kPxWarps = kPxThreads / 32;
 constexpr float kLog2MinAlpha = -7.9943534f;  // log2(1/255)
 
 // log2(alpha) of a staged record at tile-local pixel centre (fx, fy); one definition for both phases
@@ -54,6 +63,253 @@ __device__ __forceinline__ bool composite_step(float l2a, float r, float g, floa
   return true;
 }
 
+// ---------------------------------------------------------------- variant 0: a warp per 8x4 pixels
+
+constexpr int kSubTiles = 8;      // 8x4 pixel blocks of a tile: two across, four down
+constexpr int kScanKeys = 4;      // keys per lane and scan step
+constexpr int kRing = 256;        // list positions waiting to be gathered: < 32 + 32 * kScanKeys
+constexpr uint32_t kNoKey = (15u << 20) | (3u << 28);   // an empty box: meets no rectangle of a sub-tile
+
+constexpr int kAhead = 4;         // records whose alphas are computed ahead of the transmittance chain
+
+// The staged records, one list for each 4x4 half of the sub-tile: the two half-warps composite
+// different records at once, so that a small Gaussian occupies 16 lanes and not 32.
+struct BlendWarp {
+  float4 g[2][32];     // (u, v, na, nb) in the tile's pixel frame
+  float4 c[2][32];     // (nc, log2 o, mask of the warp's pixels in the record's box, b)
+  float2 rg[2][32];    // (r, g)
+  uint32_t ring[kRing];
+};
+
+__device__ __forceinline__ float ex2_approx(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+// (r, g, b) += w (cr, cg, cb) where `on`, by predicated instructions: a branch per record costs more
+// than the three of them (a colour may be infinite, so that w = 0 would not do).
+__device__ __forceinline__ void add_if(bool on, float w, float cr, float cg, float cb, float& r, float& g, float& b) {
+  asm("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %7, 0;\n\t@p fma.rn.f32 %0, %3, %4, %0;\n\t@p fma.rn.f32 %1, %3, %5, %1;\n\t"
+      "@p fma.rn.f32 %2, %3, %6, %2;\n\t}"
+      : "+f"(r), "+f"(g), "+f"(b)
+      : "f"(w), "f"(cr), "f"(cg), "f"(cb), "r"(uint32_t(on)));
+}
+
+// The bounding rectangle of a warp's unfinished pixels, as the constants of key_hits: rows r0..r1
+// and column quads c0..c1 of the tile.
+struct KeyTest {
+  uint32_t lo, hi;
+};
+
+// live: the unfinished pixels of the sub-tile, bit 16 (x / 4) + 4 y + x % 4, not zero.
+__device__ __forceinline__ KeyTest key_test(uint32_t live, uint32_t sub) {
+  const uint32_t any = (live | (live >> 16)) & 0xFFFFu;
+  const uint32_t r0 = 4u * (sub >> 1) + (uint32_t(__ffs(any) - 1) >> 2);
+  const uint32_t r1 = 4u * (sub >> 1) + (uint32_t(31 - __clz(any)) >> 2);
+  const uint32_t c0 = 2u * (sub & 1u) + ((live & 0xFFFFu) ? 0u : 1u);
+  const uint32_t c1 = 2u * (sub & 1u) + ((live >> 16) ? 1u : 0u);
+  return {((15u - r1) << 20) | ((3u - c1) << 28), ((16u - r0) << 20) | ((4u - c0) << 26)};
+}
+
+// Whether the box that a pair key carries (rows y0..y1, column quads q0..q1, see kPairTileMask)
+// meets the rectangle.  Four comparisons in two additions: y0 > r1 carries into bit 24 and q0 > c1
+// into bit 30 of the first sum, y1 >= r0 into bit 24 and q1 >= c0 into bit 28 of the second.
+__device__ __forceinline__ bool key_hits(uint32_t key, KeyTest t) {
+  const uint32_t a = (key & 0x30F00000u) + t.lo;
+  const uint32_t b = ((key >> 4) & 0x0CF00000u) + t.hi;
+  return ((a & 0x41000000u) | (~b & 0x11000000u)) == 0u;
+}
+
+// kCount: also count the evaluations and contributions into work[0], work[1].
+template <bool kCount>
+__global__ void __launch_bounds__(kBlendThreads, kBlendBlocks)
+k_blend(const uint2* __restrict__ ranges, const uint32_t* __restrict__ items, uint32_t n_tiles,
+        uint32_t* __restrict__ tile_counter, const uint32_t* __restrict__ tk, const uint32_t* __restrict__ pv,
+        const float4* __restrict__ rec, uint32_t cap_slots, int width, int height, int tiles_x, int tiles_per_view,
+        float* __restrict__ rgb, float* __restrict__ t_out, unsigned long long* __restrict__ work,
+        uint32_t* __restrict__ frame, uint32_t* __restrict__ sticky) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    if (frame[kOverflow]) atomicOr(sticky, 1u);
+    if (frame[kTimeout]) atomicOr(sticky + 1, 1u);
+  }
+  __shared__ BlendWarp s_warp[kBlendThreads / 32];
+  const uint32_t lane = threadIdx.x & 31u;
+  BlendWarp& S = s_warp[threadIdx.x >> 5];
+  uint32_t n_eval = 0, n_contrib = 0;
+  for (;;) {
+    uint32_t it = 0;
+    if (lane == 0) it = atomicAdd(tile_counter, 1u);
+    it = __shfl_sync(0xffffffffu, it, 0);
+    if (it >= n_tiles * uint32_t(kSubTiles)) break;
+    const int tile = int(items[it / kSubTiles]);   // (view, tile) id
+    const uint32_t sub = it % kSubTiles;
+    const int view = tile / tiles_per_view, vt = tile - view * tiles_per_view;
+    const int tx = vt % tiles_x, ty = vt / tiles_x;
+    const int sx = 8 * int(sub & 1u), sy = 4 * int(sub >> 1);   // the sub-tile's first pixel in the tile
+    const int lx = sx + int(4u * (lane >> 4) + (lane & 3u)), ly = sy + int((lane >> 2) & 3u);
+    const int px = tx * 16 + lx, py = ty * 16 + ly;
+    const float fx = float(lx) + 0.5f, fy = float(ly) + 0.5f;
+    const bool inside = px < width && py < height;
+    float T = 1.f, cr = 0.f, cg = 0.f, cb = 0.f;
+    uint32_t mybit = inside ? 1u << lane : 0u;   // 0 once the pixel has stopped
+    uint32_t live = __ballot_sync(0xffffffffu, inside);
+    const uint2 range = ranges[tile];
+    uint32_t sp = range.x;                  // next list position to scan
+    const uint32_t end = live ? range.y : range.x;
+    if (sp < end) {
+      KeyTest kt = key_test(live, sub);
+      uint32_t head = 0, tail = 0;          // the ring's waiting positions
+      uint32_t key[kScanKeys];
+#pragma unroll
+      for (int k = 0; k < kScanKeys; ++k) {
+        const uint32_t pos = sp + 32u * k + lane;
+        key[k] = pos < end ? tk[pos] : kNoKey;
+      }
+      // the next at most 32 hits of the list, their slots one per lane; returns their number
+      auto next_slots = [&](uint32_t& slot) -> uint32_t {
+        while (tail - head < 32u && sp < end) {
+#pragma unroll
+          for (int k = 0; k < kScanKeys; ++k) {
+            const bool hit = key_hits(key[k], kt);
+            const uint32_t b = __ballot_sync(0xffffffffu, hit);
+            if (hit) S.ring[(tail + __popc(b & lanemask_lt())) % kRing] = sp + 32u * k + lane;
+            tail += __popc(b);
+          }
+          sp += 32u * kScanKeys;
+#pragma unroll
+          for (int k = 0; k < kScanKeys; ++k) {   // the next step's keys, on their way during the compositing
+            const uint32_t pos = sp + 32u * k + lane;
+            key[k] = pos < end ? tk[pos] : kNoKey;
+          }
+        }
+        __syncwarp();
+        const uint32_t n = min(tail - head, 32u);
+        slot = lane < n ? pv[S.ring[(head + lane) % kRing]] : 0xFFFFFFFFu;
+        head += n;
+        return n;
+      };
+      float4 r0, r1, r2;
+      bool valid = false;
+      auto load_record = [&](uint32_t slot) {
+        valid = slot < cap_slots;   // (a slot beyond the buffers never occurs in a valid frame)
+        if (valid) {
+          const float4* r = rec + 3 * size_t(slot);
+          r0 = r[0];
+          r1 = r[1];
+          r2 = r[2];
+        }
+      };
+      uint32_t slot;
+      uint32_t n_rec = next_slots(slot);
+      load_record(slot);
+      uint32_t n_slot = next_slots(slot);
+      while (n_rec) {
+        // stage the records whose box holds an unfinished pixel of this warp, in order
+        uint32_t m = 0;
+        if (valid) {
+          const uint32_t bx = __float_as_uint(r2.z), by = __float_as_uint(r2.w);
+          const int ox = tx * 16 + sx, oy = ty * 16 + sy;
+          const int x0 = max(int(bx & 0xFFFFu) - ox, 0), x1 = min(int(bx >> 16) - ox, 7);
+          const int y0 = max(int(by & 0xFFFFu) - oy, 0), y1 = min(int(by >> 16) - oy, 3);
+          if (x0 <= x1 && y0 <= y1) {
+            const uint32_t cols = (0xFFu >> (7 - x1)) & (0xFFu << x0), rows = (0xFFFFu << (4 * y0)) & (0xFFFFu >> (12 - 4 * y1));
+            m = ((((cols & 15u) * 0x1111u) & rows) | ((((cols >> 4) & 15u) * 0x1111u & rows) << 16)) & live;
+          }
+        }
+        const uint32_t ml = m & 0xFFFFu, mr = m >> 16;   // the left and right 4x4 pixels
+        const uint32_t bl = __ballot_sync(0xffffffffu, ml != 0u), br = __ballot_sync(0xffffffffu, mr != 0u);
+        const int nl = __popc(bl), nr = __popc(br);
+        const int n = (max(nl, nr) + kAhead - 1) / kAhead * kAhead;
+        if (m) {
+          const uint32_t org = __float_as_uint(r2.y);
+          const float ox = float(16 * (tx - int(org & 0xFFFFu))), oy = float(16 * (ty - int(org >> 16)));
+          const float4 g = make_float4(r0.x - ox, r0.y - oy, r0.z, r0.w);
+          const float4 c = make_float4(r1.x, r1.y, __uint_as_float(m), r2.x);
+          const float2 rg = make_float2(r1.z, r1.w);
+          if (ml) {
+            const int i = __popc(bl & lanemask_lt());
+            S.g[0][i] = g;
+            S.c[0][i] = c;
+            S.rg[0][i] = rg;
+          }
+          if (mr) {
+            const int i = __popc(br & lanemask_lt());
+            S.g[1][i] = g;
+            S.c[1][i] = c;
+            S.rg[1][i] = rg;
+          }
+        }
+        // the shorter list, and both up to a multiple of kAhead, end in records without pixels
+        if (int(lane) >= nl && int(lane) < n) S.c[0][lane].z = 0.f;
+        if (int(lane) >= nr && int(lane) < n) S.c[1][lane].z = 0.f;
+        n_rec = n_slot;
+        load_record(slot);
+        n_slot = n_rec ? next_slots(slot) : 0u;   // (n_slot == 0: the loop ends after this batch)
+        __syncwarp();
+        const float4* sg = S.g[lane >> 4];
+        const float4* sc = S.c[lane >> 4];
+        const float2* srg = S.rg[lane >> 4];
+        for (int i = 0; i < n; i += kAhead) {
+          // the alphas of kAhead records (0: does not contribute to this pixel), independent of T.  As
+          // composite_step: alpha = min(0.999, 2^l2a), skipped below 1/255 (and for a NaN)
+          float a[kAhead], blue[kAhead];
+#pragma unroll
+          for (int q = 0; q < kAhead; ++q) {
+            const float4 c = sc[i + q];
+            blue[q] = c.w;
+            const float l2a = log2_alpha(sg[i + q], c, fx, fy);
+            const float al = fminf(0.999f, ex2_approx(l2a));
+            const bool in = (__float_as_uint(c.z) & mybit) != 0u;
+            if (kCount) n_eval += in ? 1u : 0u;
+            a[q] = in && l2a >= kLog2MinAlpha && al >= 1.f / 255.f ? al : 0.f;
+          }
+          // T after each of them: a record that does not contribute multiplies by exactly 1, and past
+          // the one that would take T below 1e-4 every T is below it, so nothing else contributes
+          float t[kAhead + 1];
+          t[0] = T;
+#pragma unroll
+          for (int q = 0; q < kAhead; ++q) {
+            t[q + 1] = t[q] * (1.f - a[q]);
+            const float2 rg = srg[i + q];
+            const bool on = a[q] > 0.f && t[q + 1] >= 1e-4f;
+            add_if(on, a[q] * t[q], rg.x, rg.y, blue[q], cr, cg, cb);
+            if (kCount) n_contrib += on ? 1u : 0u;
+          }
+          // (where the pixel stops, T stays as the last contributing record left it)
+#pragma unroll
+          for (int q = 1; q <= kAhead; ++q) T = t[q] >= 1e-4f ? t[q] : T;
+          if (t[kAhead] < 1e-4f) mybit = 0u;
+        }
+        live = __ballot_sync(0xffffffffu, mybit != 0u);
+        if (live == 0u) break;
+        __syncwarp();   // the batch is consumed before the next one is staged
+        kt = key_test(live, sub);
+      }
+      __syncwarp();   // the warp's staged records and ring are free for the next item
+    }
+    if (inside) {
+      const size_t p = (size_t(view) * height + py) * width + px;
+      rgb[3 * p + 0] = cr;
+      rgb[3 * p + 1] = cg;
+      rgb[3 * p + 2] = cb;
+      if (t_out) t_out[p] = T;
+    }
+  }  // next item
+  if (kCount) {
+    unsigned long long e = n_eval, cnt = n_contrib;
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+      e += __shfl_xor_sync(0xffffffffu, e, d);
+      cnt += __shfl_xor_sync(0xffffffffu, cnt, d);
+    }
+    if (lane == 0) {
+      atomicAdd(work, e);
+      atomicAdd(work + 1, cnt);
+    }
+  }
+}
+
 // True when the box that a pair key carries (see kPairTileMask: rows y0..y1, column quads
 // q0..q1) holds a pixel whose bit is set in `live` (one word per row pair: row 2w in bits
 // 0..15, row 2w + 1 in 16..31).
@@ -63,15 +319,6 @@ __device__ __forceinline__ bool box_live(uint32_t key, const uint32_t* live) {
   for (uint32_t y = y0; y <= y1; ++y)
     if ((live[y >> 1] >> ((y & 1u) * 16u)) & cols) return true;
   return false;
-}
-
-// A record's pixel box (from its third float4) clipped to tile (tx, ty), tile-local.
-__device__ __forceinline__ void box_in_tile(const float4 r2, int tx, int ty, int* x0, int* x1, int* y0, int* y1) {
-  const uint32_t bx = __float_as_uint(r2.z), by = __float_as_uint(r2.w);
-  *x0 = max(int(bx & 0xFFFFu) - 16 * tx, 0);
-  *x1 = min(int(bx >> 16) - 16 * tx, 15);
-  *y0 = max(int(by & 0xFFFFu) - 16 * ty, 0);
-  *y1 = min(int(by >> 16) - 16 * ty, 15);
 }
 
 // The next batch of a work item: the records from list position *sp on whose box (carried by the
@@ -91,14 +338,14 @@ __device__ __forceinline__ uint32_t fill_batch(const uint32_t* __restrict__ tk, 
     uint32_t key[kScan], ball[kScan], hits = 0;
 #pragma unroll
     for (int k = 0; k < kScan; ++k) {
-      const uint32_t pos = sp + k * kBlendThreads + threadIdx.x;
+      const uint32_t pos = sp + k * kPxThreads + threadIdx.x;
       key[k] = 0;
       if (pos < end) {
         key[k] = tk[pos];
         if (box_live(key[k], s_live)) hits |= 1u << k;
       }
       ball[k] = __ballot_sync(0xffffffffu, (hits >> k) & 1u);
-      if (lane == 0) s_cnt[k * kBlendWarps + warp] = __popc(ball[k]);
+      if (lane == 0) s_cnt[k * kPxWarps + warp] = __popc(ball[k]);
     }
     __syncthreads();
     if (warp == 0) {   // exclusive scan over (step, warp) = list order
@@ -116,8 +363,8 @@ __device__ __forceinline__ uint32_t fill_batch(const uint32_t* __restrict__ tk, 
 #pragma unroll
     for (int k = 0; k < kScan; ++k) {
       if ((hits >> k) & 1u) {
-        const uint32_t pos = sp + k * kBlendThreads + threadIdx.x;
-        const uint32_t idx = q + s_cnt[k * kBlendWarps + warp] + __popc(ball[k] & lanemask_lt());
+        const uint32_t pos = sp + k * kPxThreads + threadIdx.x;
+        const uint32_t idx = q + s_cnt[k * kPxWarps + warp] + __popc(ball[k] & lanemask_lt());
         if (idx < uint32_t(kBatch)) {
           const uint32_t slot = pv[pos];
           s_qslot[idx] = slot;
@@ -136,176 +383,13 @@ __device__ __forceinline__ uint32_t fill_batch(const uint32_t* __restrict__ tk, 
       sp = *s_resume;
       q = kBatch;
     } else {
-      sp = min(sp + uint32_t(kBlendThreads * kScan), end);
+      sp = min(sp + uint32_t(kPxThreads * kScan), end);
       q += total;
     }
-    static_assert(kScan * kBlendWarps == 32, "one scan lane per (step, warp)");
+    static_assert(kScan * kPxWarps == 32, "one scan lane per (step, warp)");
   }
   *sp_io = sp;
   return q;
-}
-
-// Resident blocks per SM: batches of 128 records keep shared memory (10 KB) and registers (40)
-// small enough for 6 blocks, the larger ones run 4.
-constexpr int blend_blocks_per_sm(int batch) { return batch == 128 ? 6 : 4; }
-
-// kBatch: records staged per batch (128, 256 or 512; the image does not depend on it).
-template <bool kCount, int kBatch>
-__global__ void __launch_bounds__(kBlendThreads, blend_blocks_per_sm(kBatch))
-k_blend(const uint2* __restrict__ ranges, const uint32_t* __restrict__ items, const uint32_t* __restrict__ n_items,
-        uint32_t* __restrict__ tile_counter, const uint32_t* __restrict__ tk, const uint32_t* __restrict__ pv,
-        const float4* __restrict__ rec, uint32_t cap_slots, int width,
-        int height, int tiles_x, int tiles_per_view, float* __restrict__ rgb, float* __restrict__ t_out,
-        unsigned long long* __restrict__ work, uint32_t* __restrict__ frame, uint32_t* __restrict__ sticky) {
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    if (frame[kOverflow]) atomicOr(sticky, 1u);
-    if (frame[kTimeout]) atomicOr(sticky + 1, 1u);
-  }
-  constexpr int kPer = kBatch >= kBlendThreads ? kBatch / kBlendThreads : 1;   // records staged per thread
-  constexpr int kMaskWords = kBatch / 32;                                       // per-pixel mask words
-  static_assert(kBatch % 32 == 0 && (kBatch <= kBlendThreads || kBatch % kBlendThreads == 0), "batch size");
-  __shared__ float4 s_g[kBatch];                    // (u, v, na, nb) in this tile's pixel frame
-  __shared__ float4 s_c[kBatch];                    // (nc, log2 o, r, g)
-  __shared__ float s_b[kBatch];                     // b
-  __shared__ uint32_t s_mask[kBlendThreads][kMaskWords];  // [pixel][record word]: contributing records
-  __shared__ uint32_t s_live[kBlendWarps];          // unfinished pixels of the item, one word per row pair
-  __shared__ uint32_t s_qslot[kBatch];              // the batch: slots of its records, in list order
-  __shared__ uint32_t s_cnt[32];
-  __shared__ uint32_t s_next, s_resume, s_total;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int lx = threadIdx.x & 15, ly = threadIdx.x >> 4;   // this thread's pixel in the tile
-  const float fx = float(lx) + 0.5f, fy = float(ly) + 0.5f;
-  uint32_t n_eval = 0, n_contrib = 0;
-#pragma unroll
-  for (int k = 0; k < kMaskWords; ++k) s_mask[threadIdx.x][k] = 0u;
-  for (;;) {
-    if (threadIdx.x == 0) s_next = atomicAdd(tile_counter, 1u);
-    __syncthreads();
-    const uint32_t next = s_next;
-    __syncthreads();
-    if (next >= *n_items) break;
-    const uint32_t item = items[next];
-    const int tile = int(item & 0xFFFFFFu), region = int(item >> 24);   // (view, tile) id
-    const int view = tile / tiles_per_view, vt = tile - view * tiles_per_view;
-    const int tx = vt % tiles_x, ty = vt / tiles_x;
-    // the item's pixel rectangle within the tile: the whole tile or one 8x8 quadrant
-    const int qx0 = region ? 8 * ((region - 1) & 1) : 0, qy0 = region ? 8 * ((region - 1) >> 1) : 0;
-    const int qx1 = region ? qx0 + 7 : 15, qy1 = region ? qy0 + 7 : 15;
-    const int px = tx * 16 + lx, py = ty * 16 + ly;
-    const bool mine = lx >= qx0 && lx <= qx1 && ly >= qy0 && ly <= qy1;
-    const bool inside = px < width && py < height && mine;
-    const uint2 range = ranges[tile];
-    float T = 1.f, cr = 0.f, cg = 0.f, cb = 0.f;
-    bool done = !inside;
-    uint32_t sp = range.x;   // next list position to look at (uniform across the block)
-    for (;;) {
-      // the item's unfinished pixels, one word per row pair (row 2w: bits 0..15, row 2w + 1: 16..31)
-      const uint32_t dword = __ballot_sync(0xffffffffu, done);
-      if (lane == 0) s_live[warp] = ~dword;
-      __syncthreads();
-      uint32_t any_live = 0;
-#pragma unroll
-      for (int w = 0; w < kBlendWarps; ++w) any_live |= s_live[w];
-      if (any_live == 0 || sp >= range.y) break;
-      // the batch: the next records of the list whose box (carried by the pair key) holds an
-      // unfinished pixel, in list order; kScan * 256 consecutive keys per step
-      const uint32_t q = fill_batch<kBatch>(tk, pv, range.y, cap_slots, s_live, s_qslot, nullptr, s_cnt, &s_resume, &s_total, &sp);
-      if (q == 0) break;
-      // stage the batch (kPer consecutive records per thread) for the compositing phase, and test
-      // each of this thread's records at the pixels of its box that are still accumulating: a
-      // pixel where alpha >= 1/255 gets the record's bit in its mask
-#pragma unroll
-      for (int k = 0; k < kPer; ++k) {
-        const uint32_t i = threadIdx.x * kPer + k;
-        if (i >= q) continue;
-        const uint32_t slot = s_qslot[i];
-        if (slot >= cap_slots) continue;
-        const float4* r = rec + 3 * size_t(slot);
-        const float4 r0 = r[0], r1 = r[1], r2 = r[2];
-        const uint32_t org = __float_as_uint(r2.y);
-        const float ox = float(16 * (tx - int(org & 0xFFFFu))), oy = float(16 * (ty - int(org >> 16)));
-        const float4 g = make_float4(r0.x - ox, r0.y - oy, r0.z, r0.w);
-        s_g[i] = g;
-        s_c[i] = r1;
-        s_b[i] = r2.x;
-        int x0, x1, y0, y1;
-        box_in_tile(r2, tx, ty, &x0, &x1, &y0, &y1);
-        x0 = max(x0, qx0); x1 = min(x1, qx1); y0 = max(y0, qy0); y1 = min(y1, qy1);
-        if (x0 > x1) continue;
-        const uint32_t cols = (0xFFFFu >> (15 - x1)) & (0xFFFFu << x0);
-        const uint32_t bit = 1u << (i & 31);
-        for (int yy = y0; yy <= y1; ++yy) {
-          uint32_t m = (s_live[yy >> 1] >> ((yy & 1) * 16)) & cols;
-          while (m) {
-            const int xx = __ffs(m) - 1;
-            m &= m - 1;
-            const float l2a = log2_alpha(g, r1, float(xx) + 0.5f, float(yy) + 0.5f);
-            if (kCount) ++n_eval;
-            // alpha = min(0.999, 2^l2a) >= 1/255; well above the threshold it holds without exp2
-            if (l2a >= kLog2MinAlpha + 1e-5f ||
-                (l2a >= kLog2MinAlpha && fminf(0.999f, exp2f(l2a)) >= 1.f / 255.f))
-              atomicOr(&s_mask[yy * 16 + xx][i >> 5], bit);
-          }
-        }
-      }
-      __syncthreads();
-      // pixel-parallel blend of the contributing records, in depth order
-#pragma unroll
-      for (int wd = 0; wd < kMaskWords; ++wd) {
-        uint32_t bits = s_mask[threadIdx.x][wd];
-        if (!bits) continue;
-        s_mask[threadIdx.x][wd] = 0u;
-        while (bits && !done) {
-          // two records at a time: their alphas are independent, only T is a chain
-          constexpr int kAhead = 2;
-          int jj[kAhead], n = 0;
-#pragma unroll
-          for (int q = 0; q < kAhead; ++q) {
-            jj[q] = wd * 32 + __ffs(bits) - 1;   // bits == 0: a valid index, not used
-            if (bits) {
-              bits &= bits - 1;
-              n = q + 1;
-            }
-          }
-          float l2a[kAhead], r[kAhead], g[kAhead], b[kAhead];
-#pragma unroll
-          for (int q = 0; q < kAhead; ++q) {
-            const int j = max(jj[q], wd * 32);
-            const float4 c = s_c[j];
-            l2a[q] = log2_alpha(s_g[j], c, fx, fy);
-            r[q] = c.z;
-            g[q] = c.w;
-            b[q] = s_b[j];
-          }
-#pragma unroll
-          for (int q = 0; q < kAhead; ++q) {
-            if (q >= n || done) break;
-            if (composite_step(l2a[q], r[q], g[q], b[q], T, cr, cg, cb, done) && kCount) ++n_contrib;
-          }
-        }
-      }
-      __syncthreads();
-    }
-    if (inside) {   // this item's pixels only
-      const size_t p = (size_t(view) * height + py) * width + px;
-      rgb[3 * p + 0] = cr;
-      rgb[3 * p + 1] = cg;
-      rgb[3 * p + 2] = cb;
-      if (t_out) t_out[p] = T;
-    }
-  }  // next tile
-  if (kCount) {
-    unsigned long long e = n_eval, cnt = n_contrib;
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) {
-      e += __shfl_xor_sync(0xffffffffu, e, d);
-      cnt += __shfl_xor_sync(0xffffffffu, cnt, d);
-    }
-    if (lane == 0) {
-      atomicAdd(work, e);
-      atomicAdd(work + 1, cnt);
-    }
-  }
 }
 
 // ---------------------------------------------------------------- bulk-copy staging
@@ -368,13 +452,11 @@ constexpr int blend_px_blocks_per_sm(int batch) { return batch == 512 ? 4 : 5; }
 // (lane = pixel) and walks, in list (= depth) order, only the batch records whose box spans one of
 // its rows (known from the pair key at fill time), so a warp never visits a record that cannot
 // reach it; each lane evaluates the record where its pixel lies in the record's box and is still
-// accumulating, and composites at once (composite_step, the same arithmetic as the two-phase
-// kernel, so the image is the same bit for bit).  A warp whose 32 pixels are all done skips the
-// rest of the batch.  Quadrant work items are handled (the other rows' warps idle), though the
-// launch keeps whole tiles for this variant.
+// accumulating, and composites at once (composite_step, the same arithmetic as k_blend, so the image is the same bit for bit).  A warp whose 32 pixels are all done skips the
+// rest of the batch.
 template <bool kCount, int kBatch>
-__global__ void __launch_bounds__(kBlendThreads, blend_px_blocks_per_sm(kBatch))
-k_blend_px(const uint2* __restrict__ ranges, const uint32_t* __restrict__ items, const uint32_t* __restrict__ n_items,
+__global__ void __launch_bounds__(kPxThreads, blend_px_blocks_per_sm(kBatch))
+k_blend_px(const uint2* __restrict__ ranges, const uint32_t* __restrict__ items, uint32_t n_items,
            uint32_t* __restrict__ tile_counter, const uint32_t* __restrict__ tk, const uint32_t* __restrict__ pv,
            const float4* __restrict__ rec, uint32_t cap_slots, int width, int height, int tiles_x, int tiles_per_view,
            float* __restrict__ rgb, float* __restrict__ t_out, unsigned long long* __restrict__ work,
@@ -383,14 +465,14 @@ k_blend_px(const uint2* __restrict__ ranges, const uint32_t* __restrict__ items,
     if (frame[kOverflow]) atomicOr(sticky, 1u);
     if (frame[kTimeout]) atomicOr(sticky + 1, 1u);
   }
-  constexpr int kPer = kBatch >= kBlendThreads ? kBatch / kBlendThreads : 1;
+  constexpr int kPer = kBatch >= kPxThreads ? kBatch / kPxThreads : 1;
   constexpr int kWords = kBatch / 32;
-  static_assert(kBatch % 32 == 0 && kWords <= 32 && (kBatch <= kBlendThreads || kBatch % kBlendThreads == 0),
+  static_assert(kBatch % 32 == 0 && kWords <= 32 && (kBatch <= kPxThreads || kBatch % kPxThreads == 0),
                 "batch size");
   __shared__ __align__(16) float4 s_rec[3 * kBatch];   // the batch's records, as stored by the projection
   __shared__ uint32_t s_qslot[kBatch];
   __shared__ uint8_t s_rows[kBatch];                   // bit w: the record's box spans rows 2w or 2w + 1
-  __shared__ uint32_t s_live[kBlendWarps];
+  __shared__ uint32_t s_live[kPxWarps];
   __shared__ uint32_t s_cnt[32];
   __shared__ uint32_t s_next, s_resume, s_total;
   __shared__ __align__(8) uint64_t s_bar;
@@ -406,15 +488,12 @@ k_blend_px(const uint2* __restrict__ ranges, const uint32_t* __restrict__ items,
     __syncthreads();
     const uint32_t next = s_next;
     __syncthreads();
-    if (next >= *n_items) break;
-    const uint32_t item = items[next];
-    const int tile = int(item & 0xFFFFFFu), region = int(item >> 24);
+    if (next >= n_items) break;
+    const int tile = int(items[next]);   // (view, tile) id
     const int view = tile / tiles_per_view, vt = tile - view * tiles_per_view;
     const int tx = vt % tiles_x, ty = vt / tiles_x;
-    const int qx0 = region ? 8 * ((region - 1) & 1) : 0, qy0 = region ? 8 * ((region - 1) >> 1) : 0;
-    const int qx1 = region ? qx0 + 7 : 15, qy1 = region ? qy0 + 7 : 15;
     const int px = tx * 16 + lx, py = ty * 16 + ly;
-    const bool inside = px < width && py < height && lx >= qx0 && lx <= qx1 && ly >= qy0 && ly <= qy1;
+    const bool inside = px < width && py < height;
     const uint2 range = ranges[tile];
     float T = 1.f, cr = 0.f, cg = 0.f, cb = 0.f;
     bool done = !inside;
@@ -425,7 +504,7 @@ k_blend_px(const uint2* __restrict__ ranges, const uint32_t* __restrict__ items,
       __syncthreads();
       uint32_t any_live = 0;
 #pragma unroll
-      for (int w = 0; w < kBlendWarps; ++w) any_live |= s_live[w];
+      for (int w = 0; w < kPxWarps; ++w) any_live |= s_live[w];
       if (any_live == 0 || sp >= range.y) break;
       const uint32_t q = fill_batch<kBatch>(tk, pv, range.y, cap_slots, s_live, s_qslot, s_rows, s_cnt, &s_resume, &s_total, &sp);
       if (q == 0) break;
@@ -434,7 +513,7 @@ k_blend_px(const uint2* __restrict__ ranges, const uint32_t* __restrict__ items,
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 #pragma unroll
       for (int k = 0; k < kPer; ++k) {
-        const uint32_t i = threadIdx.x + k * kBlendThreads;
+        const uint32_t i = threadIdx.x + k * kPxThreads;
         if (i >= q) continue;
         uint32_t slot = s_qslot[i];
         if (slot >= cap_slots) slot = 0;   // never for a valid frame; no warp reads the record (rows 0)
@@ -507,20 +586,16 @@ out:
   }
 }
 
-// Work items, heaviest first.  A tile with at least split_pairs pairs becomes four items, one
-// per 8x8 quadrant (each scans the tile's list by boxes but stages and evaluates only the
-// records that reach its quadrant, so a long list is spread over four blocks); other tiles are
-// one item.  Item = tile | region << 24 (region 0: whole tile, 1 + q: quadrant q).  One block
-// buckets the items by floor(log2(pairs + 1)), descending.
+// The tiles, those with the longest lists first (bucketed by floor(log2(pairs + 1)), descending), so
+// that the work items that take longest start first.  One block.
 __global__ void __launch_bounds__(1024) k_blend_items(const uint2* __restrict__ ranges, int n_tiles,
-                                                      uint32_t split_pairs, uint32_t* __restrict__ items,
-                                                      uint32_t* __restrict__ n_items) {
+                                                      uint32_t* __restrict__ items) {
   __shared__ uint32_t s_hist[32];
   if (threadIdx.x < 32) s_hist[threadIdx.x] = 0;
   __syncthreads();
   for (int t = threadIdx.x; t < n_tiles; t += blockDim.x) {
     const uint32_t len = ranges[t].y - ranges[t].x;
-    atomicAdd(&s_hist[__clz(len + 1u)], len >= split_pairs ? 4u : 1u);   // clz: 0 for the heaviest
+    atomicAdd(&s_hist[__clz(len + 1u)], 1u);   // clz: 0 for the heaviest
   }
   __syncthreads();
   if (threadIdx.x < 32) {
@@ -532,17 +607,11 @@ __global__ void __launch_bounds__(1024) k_blend_items(const uint2* __restrict__ 
       if (threadIdx.x >= d) incl += t;
     }
     s_hist[threadIdx.x] = incl - v;   // cursor: first position of the bucket
-    if (threadIdx.x == 31) *n_items = incl;
   }
   __syncthreads();
   for (int t = threadIdx.x; t < n_tiles; t += blockDim.x) {
     const uint32_t len = ranges[t].y - ranges[t].x;
-    if (len >= split_pairs) {
-      const uint32_t pos = atomicAdd(&s_hist[__clz(len + 1u)], 4u);
-      for (uint32_t q = 0; q < 4; ++q) items[pos + q] = uint32_t(t) | ((q + 1u) << 24);
-    } else {
-      items[atomicAdd(&s_hist[__clz(len + 1u)], 1u)] = uint32_t(t);
-    }
+    items[atomicAdd(&s_hist[__clz(len + 1u)], 1u)] = uint32_t(t);
   }
 }
 
@@ -550,58 +619,21 @@ __global__ void __launch_bounds__(1024) k_blend_items(const uint2* __restrict__ 
 
 namespace {
 
-template <int kMode, bool kCount, int kBatch>
-void blend_launch_one(int grid, cudaStream_t st, const uint2* ranges, const uint32_t* items, const uint32_t* n_items,
-                      uint32_t* tile_counter, const uint32_t* tk, const uint32_t* pv, const float4* rec,
-                      uint32_t cap_slots, const CamConst& cam, float* rgb, float* t_out, unsigned long long* work,
-                      uint32_t* frame, uint32_t* sticky) {
-  if (kMode == 0)
-    k_blend<kCount, kBatch><<<grid, kBlendThreads, 0, st>>>(ranges, items, n_items, tile_counter, tk, pv, rec, cap_slots,
-                                                            cam.width, cam.height, cam.tiles_x,
-                                                            cam.tiles_x * cam.tiles_y, rgb, t_out, work, frame, sticky);
-  else
-    k_blend_px<kCount, kBatch><<<grid, kBlendThreads, 0, st>>>(ranges, items, n_items, tile_counter, tk, pv, rec,
-                                                               cap_slots, cam.width, cam.height, cam.tiles_x,
-                                                               cam.tiles_x * cam.tiles_y, rgb, t_out, work, frame,
-                                                               sticky);
-}
-
-template <int kMode, int kBatch>
-void blend_launch(int grid, cudaStream_t st, const uint2* ranges, const uint32_t* items, const uint32_t* n_items,
-                  uint32_t* tile_counter, const uint32_t* tk, const uint32_t* pv, const float4* rec, uint32_t cap_slots,
-                  const CamConst& cam, float* rgb, float* t_out, unsigned long long* work, uint32_t* frame,
-                  uint32_t* sticky) {
-  if (work)
-    blend_launch_one<kMode, true, kBatch>(grid, st, ranges, items, n_items, tile_counter, tk, pv, rec, cap_slots, cam,
-                                          rgb, t_out, work, frame, sticky);
-  else
-    blend_launch_one<kMode, false, kBatch>(grid, st, ranges, items, n_items, tile_counter, tk, pv, rec, cap_slots, cam,
-                                           rgb, t_out, nullptr, frame, sticky);
-}
-
-template <int kMode>
-void blend_launch_batch(int batch, int grid, cudaStream_t st, const uint2* ranges, const uint32_t* items,
-                        const uint32_t* n_items, uint32_t* tile_counter, const uint32_t* tk, const uint32_t* pv,
-                        const float4* rec, uint32_t cap_slots, const CamConst& cam, float* rgb, float* t_out,
-                        unsigned long long* work, uint32_t* frame, uint32_t* sticky) {
-  if (batch == 128)
-    blend_launch<kMode, 128>(grid, st, ranges, items, n_items, tile_counter, tk, pv, rec, cap_slots, cam, rgb, t_out,
-                             work, frame, sticky);
-  else if (batch == 256)
-    blend_launch<kMode, 256>(grid, st, ranges, items, n_items, tile_counter, tk, pv, rec, cap_slots, cam, rgb, t_out,
-                             work, frame, sticky);
-  else
-    blend_launch<kMode, 512>(grid, st, ranges, items, n_items, tile_counter, tk, pv, rec, cap_slots, cam, rgb, t_out,
-                             work, frame, sticky);
+template <bool kCount, int kBatch>
+void blend_px_launch(int grid, cudaStream_t st, const uint2* ranges, const uint32_t* items, uint32_t n_tiles,
+                     uint32_t* tile_counter, const uint32_t* tk, const uint32_t* pv, const float4* rec,
+                     uint32_t cap_slots, const CamConst& cam, float* rgb, float* t_out, unsigned long long* work,
+                     uint32_t* frame, uint32_t* sticky) {
+  k_blend_px<kCount, kBatch><<<grid, kPxThreads, 0, st>>>(ranges, items, n_tiles, tile_counter, tk, pv, rec, cap_slots,
+                                                          cam.width, cam.height, cam.tiles_x,
+                                                          cam.tiles_x * cam.tiles_y, rgb, t_out, work, frame, sticky);
 }
 
 }  // namespace
 
 cudaError_t blend_set_attributes() {
-  // several resident blocks of 11-43 KB shared memory per SM want the largest carveout
-  const void* fns[] = {(const void*)k_blend<true, 128>,     (const void*)k_blend<false, 128>,
-                       (const void*)k_blend<true, 256>,     (const void*)k_blend<false, 256>,
-                       (const void*)k_blend<true, 512>,     (const void*)k_blend<false, 512>,
+  // several resident blocks of 10-28 KB shared memory per SM want the largest carveout
+  const void* fns[] = {(const void*)k_blend<true>,          (const void*)k_blend<false>,
                        (const void*)k_blend_px<true, 128>,  (const void*)k_blend_px<false, 128>,
                        (const void*)k_blend_px<true, 256>,  (const void*)k_blend_px<false, 256>,
                        (const void*)k_blend_px<true, 512>,  (const void*)k_blend_px<false, 512>};
@@ -615,23 +647,34 @@ cudaError_t blend_set_attributes() {
 
 cudaError_t launch_blend(const uint2* ranges, uint32_t* items, uint32_t* tile_counter, const uint32_t* tk,
                          const uint32_t* pv, const float4* rec, uint32_t cap_slots, const CamConst& cam, float* rgb,
-                         float* t_out, unsigned long long* work, uint32_t* frame, uint32_t* sticky,
-                         uint32_t split_pairs, int batch, int mode, int n_views, int sm_count, cudaStream_t st) {
+                         float* t_out, unsigned long long* work, uint32_t* frame, uint32_t* sticky, int batch, int mode,
+                         int n_views, int sm_count, cudaStream_t st) {
   const int n_tiles = cam.tiles_x * cam.tiles_y * n_views;
   if (n_tiles == 0) return cudaSuccess;
   if (batch != 128 && batch != 256 && batch != 512) return cudaErrorInvalidValue;
   if (mode != 0 && mode != 1) return cudaErrorInvalidValue;
-  uint32_t* n_items = items + 4 * size_t(n_tiles);
-  // the pixel-loop variant keeps whole tiles (a quadrant item would leave six of its warps idle)
-  k_blend_items<<<1, 1024, 0, st>>>(ranges, n_tiles, mode == 1 ? 0xFFFFFFFFu : split_pairs, items, n_items);
-  const int per_sm = mode == 1 ? blend_px_blocks_per_sm(batch) : blend_blocks_per_sm(batch);
-  const int grid = std::min(4 * n_tiles, sm_count * per_sm);   // persistent: the resident blocks
-  if (mode == 0)
-    blend_launch_batch<0>(batch, grid, st, ranges, items, n_items, tile_counter, tk, pv, rec, cap_slots, cam, rgb, t_out,
-                          work, frame, sticky);
-  else
-    blend_launch_batch<1>(batch, grid, st, ranges, items, n_items, tile_counter, tk, pv, rec, cap_slots, cam, rgb, t_out,
-                          work, frame, sticky);
+  k_blend_items<<<1, 1024, 0, st>>>(ranges, n_tiles, items);
+  // persistent grids: the resident blocks
+  if (mode == 0) {
+    const int per_block = kBlendThreads / 32;
+    const int grid = std::min((kSubTiles * n_tiles + per_block - 1) / per_block, sm_count * kBlendBlocks);
+    const int tiles_per_view = cam.tiles_x * cam.tiles_y;
+    if (work)
+      k_blend<true><<<grid, kBlendThreads, 0, st>>>(ranges, items, uint32_t(n_tiles), tile_counter, tk, pv, rec, cap_slots,
+                                                    cam.width, cam.height, cam.tiles_x, tiles_per_view, rgb, t_out, work,
+                                                    frame, sticky);
+    else
+      k_blend<false><<<grid, kBlendThreads, 0, st>>>(ranges, items, uint32_t(n_tiles), tile_counter, tk, pv, rec, cap_slots,
+                                                     cam.width, cam.height, cam.tiles_x, tiles_per_view, rgb, t_out,
+                                                     nullptr, frame, sticky);
+    return cudaGetLastError();
+  }
+  const int grid = std::min(n_tiles, sm_count * blend_px_blocks_per_sm(batch));
+  const auto launch = batch == 128   ? (work ? blend_px_launch<true, 128> : blend_px_launch<false, 128>)
+                      : batch == 256 ? (work ? blend_px_launch<true, 256> : blend_px_launch<false, 256>)
+                                     : (work ? blend_px_launch<true, 512> : blend_px_launch<false, 512>);
+  launch(grid, st, ranges, items, uint32_t(n_tiles), tile_counter, tk, pv, rec, cap_slots, cam, rgb, t_out, work, frame,
+         sticky);
   return cudaGetLastError();
 }
 

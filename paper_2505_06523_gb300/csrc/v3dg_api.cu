@@ -117,7 +117,7 @@ struct v3dg_ctx {
   DevBuf d_assets;
   std::atomic<uint64_t> launches{0};
   bool sync_check = true, stage_timing = false, count_work = false;
-  uint32_t split_pairs = 0xFFFFFFFFu;   // long-tile split threshold (none by default)
+  uint32_t split_pairs = 0xFFFFFFFFu;   // long-tile split threshold: accepted, no blend variant splits tiles
   bool attr_fp16 = false;   // store opacity and SH of the next loaded assets as float16
   int topdown = 2;          // 0 flat, 1 level by level from the roots (same cut), 2 top-down for large scenes
   int blend_batch = 512;    // records staged per blend batch: 128, 256 or 512
@@ -574,7 +574,7 @@ v3dg_status enqueue_render(Pipe* c, float* rgb, float* t_out) {
 
   stage_event(c, kStageRanges);
   ST(ensure(c, c->d_ranges, sizeof(uint2) * size_t(n_tiles)));
-  ST(ensure(c, c->d_order, sizeof(uint32_t) * (4 * size_t(n_tiles) + 1)));
+  ST(ensure(c, c->d_order, sizeof(uint32_t) * size_t(n_tiles)));
   CU(launch_ranges(tk, c->cap_pairs, frame, P<uint2>(c->d_ranges), n_tiles, sm, c->stream));
   c->ctx->launches += 1;
 
@@ -584,8 +584,7 @@ v3dg_status enqueue_render(Pipe* c, float* rgb, float* t_out) {
   if (work) CU(cudaMemsetAsync(work, 0, 2 * sizeof(unsigned long long), c->stream));
   // d_misc[12], [13]: sticky overflow / timeout flags of all frames since the last v3dg_frame_stats
   CU(launch_blend(P<uint2>(c->d_ranges), P<uint32_t>(c->d_order), frame + kTileCounters + 10, tk, tv, P<float4>(c->d_rec),
-                  c->cap_slots, k, rgb, t_out, work, frame, P<uint32_t>(c->d_misc) + 12, c->ctx->split_pairs,
-                  c->ctx->blend_batch, c->ctx->blend_mode, int(c->n_views), sm, c->stream));
+                  c->cap_slots, k, rgb, t_out, work, frame, P<uint32_t>(c->d_misc) + 12, c->ctx->blend_batch, c->ctx->blend_mode, int(c->n_views), sm, c->stream));
   c->ctx->launches += 2;
   if (work)
     CU(cudaMemcpyAsync(c->h_tmp + kFrameWords, work, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, c->stream));
@@ -645,7 +644,6 @@ std::vector<uint64_t> graph_key(Pipe* c, float* rgb, float* t_out) {
                              c->cap_slots, c->status_words, uint64_t(uintptr_t(rgb)), uint64_t(uintptr_t(t_out)),
                              uint64_t(use_topdown(c)), uint64_t(use_project_order(c)), uint64_t(ctx->blend_batch),
                              uint64_t(ctx->blend_mode),
-                             ctx->split_pairs,
                              uint64_t(ctx->count_work), uint64_t(c->color_formats), ctx->assets.size(),
                              uint64_t(uintptr_t(ctx->d_assets.p))};
   const DevBuf* bufs[] = {&c->d_inst, &c->d_frame, &c->d_misc, &c->d_list, &c->d_ref, &c->d_keys0, &c->d_keys1,
@@ -666,7 +664,7 @@ v3dg_status run_graph_frame(Pipe* c, float* rgb, float* t_out, bool sync) {
   ST(ensure_work(c));
   const int n_tiles = c->cc.tiles_x * c->cc.tiles_y * int(c->n_views);
   ST(ensure(c, c->d_ranges, sizeof(uint2) * size_t(n_tiles)));
-  ST(ensure(c, c->d_order, sizeof(uint32_t) * (4 * size_t(n_tiles) + 1)));
+  ST(ensure(c, c->d_order, sizeof(uint32_t) * size_t(n_tiles)));
   if (use_topdown(c)) {
     TopDown td{};
     ST(topdown_buffers(c, &td));
@@ -1704,15 +1702,12 @@ v3dg_status v3dg_autotune_blend(v3dg_ctx* ctx, uint32_t* mode_out, uint32_t* bat
     return fail(c, V3DG_ECUDA, "cudaEventCreate failed");
   }
   const int batches[] = {128, 256, 512};
-  const uint32_t splits[] = {4096u, 16384u, 65536u, 0xFFFFFFFFu};
   float best = INFINITY;
   int best_b = ctx->blend_batch, best_m = ctx->blend_mode;
-  uint32_t best_s = ctx->split_pairs;
   cudaError_t e = cudaSuccess;
   for (int mode = 0; mode < 2; ++mode)
-  for (int b : batches) {
-    for (uint32_t sp : splits) {
-      if (mode == 1 && sp != 0xFFFFFFFFu) continue;   // that variant always blends whole tiles
+    for (int b : batches) {
+      if (mode == 0 && b != 512) continue;   // variant 0 has no batch size (512 is the option's default)
       float t_min = INFINITY;
       for (int rep = 0; rep < 4 && e == cudaSuccess; ++rep) {   // the first run warms up
         e = cudaMemsetAsync(frame + kTileCounters + 10, 0, sizeof(uint32_t), c->stream);
@@ -1720,7 +1715,7 @@ v3dg_status v3dg_autotune_blend(v3dg_ctx* ctx, uint32_t* mode_out, uint32_t* bat
         if (e == cudaSuccess)
           e = launch_blend(P<uint2>(c->d_ranges), P<uint32_t>(c->d_order), frame + kTileCounters + 10, tk, tv,
                            P<float4>(c->d_rec), c->cap_slots, k, P<float>(c->d_img), nullptr, nullptr, frame,
-                           P<uint32_t>(c->d_misc) + 12, sp, b, mode, int(c->n_views), ctx->sm_count, c->stream);
+                           P<uint32_t>(c->d_misc) + 12, b, mode, int(c->n_views), ctx->sm_count, c->stream);
         if (e == cudaSuccess) e = cudaEventRecord(e1, c->stream);
         if (e == cudaSuccess) e = cudaEventSynchronize(e1);
         float ms = 0.f;
@@ -1731,20 +1726,17 @@ v3dg_status v3dg_autotune_blend(v3dg_ctx* ctx, uint32_t* mode_out, uint32_t* bat
       if (t_min < best) {
         best = t_min;
         best_b = b;
-        best_s = sp;
         best_m = mode;
       }
     }
-  }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (e != cudaSuccess) return fail(c, V3DG_ECUDA, "CUDA error %s", cudaGetErrorString(e));
   ctx->blend_batch = best_b;
-  ctx->split_pairs = best_s;
   ctx->blend_mode = best_m;
   if (mode_out) *mode_out = uint32_t(best_m);
   if (batch_out) *batch_out = uint32_t(best_b);
-  if (split_out) *split_out = best_s;
+  if (split_out) *split_out = 0xFFFFFFFFu;
   if (ms_out) *ms_out = best;
   c->err.clear();
   return V3DG_OK;

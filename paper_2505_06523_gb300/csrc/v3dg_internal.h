@@ -194,16 +194,14 @@ cudaError_t launch_ranges(const uint32_t* tile_keys, uint32_t cap_pairs, const u
 // work != nullptr: also count (evaluations, contributions) into work[0], work[1].
 // sticky[0] |= frame[kOverflow], sticky[1] |= frame[kTimeout] (the flags of every frame since the
 // host last cleared them).
-// items: 4 * n_tiles + 1 words of scratch (the heaviest-first work items and their count);
-// tile_counter: a zeroed word.  batch: records staged per batch, 128, 256 or 512.  n_views
+// items: n_tiles words of scratch (the tiles, longest lists first); tile_counter: a zeroed word.
+// batch: records that variant 1 stages per batch, 128, 256 or 512.  n_views
 // images of cam's size, one after the other in rgb (and t_out); tile ids are (view, tile).
 // tk, pair_vals: the sorted pair keys (tile id and in-tile box, see kPairTileMask) and values.
-// mode 0: two-phase blend (record-parallel alpha test into per-pixel masks, then pixel-parallel
-// compositing); mode 1: batches staged by bulk copies and composited by warps over row pairs.  The
-// image is the same bit for bit.
+// mode 0: every warp composites 8x4 pixels on its own; mode 1: batches staged by bulk copies and
+// composited by warps over row pairs.  The image is the same bit for bit.
 cudaError_t launch_blend(const uint2* ranges, uint32_t* items, uint32_t* tile_counter, const uint32_t* tk,
                          const uint32_t* pair_vals, const float4* rec, uint32_t cap_slots, const CamConst& cam, float* rgb, float* t_out,
-                         unsigned long long* work, uint32_t* frame, uint32_t* sticky, uint32_t split_pairs,
-                         int batch, int mode, int n_views, int sm_count, cudaStream_t st);
+                         unsigned long long* work, uint32_t* frame, uint32_t* sticky, int batch, int mode, int n_views, int sm_count, cudaStream_t st);
 
 }  // namespace v3dg
