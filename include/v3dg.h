@@ -227,7 +227,9 @@ v3dg_status v3dg_render_host(v3dg_ctx* ctx, float* rgb_host, float* T_host);
 /* Synchronise the stream and report the last frame's counters. */
 v3dg_status v3dg_frame_stats(v3dg_ctx* ctx, v3dg_stats* out);
 
-/* Parity read-back (synchronising, host outputs).
+/* Parity read-back (synchronising, host outputs).  Large frames are sorted and blended in several
+ * depth slabs, which leave out what the front ones hide; for such a frame the first of these calls
+ * makes the sorted lists of the whole frame again, so they return the same for every frame.
  * v3dg_get_cut: the cut of the last v3dg_select before the visibility cull, as (instance, node)
  *   pairs in ascending (instance, node) order; 2 * cap uint32 slots; *n receives the size.
  * v3dg_get_projected: every visible Gaussian of the last render in global-id order; per entry

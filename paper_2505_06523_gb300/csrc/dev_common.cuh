@@ -79,35 +79,47 @@ __device__ __forceinline__ uint32_t chain_lookback(uint64_t* status, uint32_t st
   return excl;
 }
 
-// The look-back of one chain by a whole warp (all 32 lanes call it, converged): lane i reads the
-// word of tile j - i, so each round covers 32 tiles; the nearest inclusive prefix or unwritten
-// word ends the round.  Returns the exclusive prefix in every lane; lane 0 publishes.
+// The look-back of one chain by a whole warp (all 32 lanes call it, converged): a round reads the
+// words of the 128 tiles before j (four independent loads a lane) and consumes them 32 at a time; the
+// nearest inclusive prefix or unwritten word ends it.  About a thousand tiles of a persistent grid
+// are in flight at once, and a walk passes every one of them that has only its aggregate: with 32
+// words a round that took most of the expansion's time.  Returns the exclusive prefix in every lane;
+// lane 0 publishes.
 __device__ __forceinline__ uint32_t chained_exclusive_warp(uint64_t* status, uint32_t tile, uint32_t agg,
                                                            uint32_t epoch, uint32_t* err,
                                                            uint32_t spin_limit = kSpinLimit) {
+  constexpr int kWords = 4;
   const uint32_t lane = threadIdx.x & 31u;
   if (lane == 0) chain_publish(status, 1, tile, agg, epoch);
   if (tile == 0) return 0;
   uint32_t excl = 0, spins = 0;
   int64_t j = int64_t(tile) - 1;
-  for (;;) {
-    const int64_t q = j - int64_t(lane);
-    // before tile 0 (never reached: tile 0 publishes an inclusive prefix) reads as a zero prefix
-    const uint64_t s = q >= 0 ? ld_status(status + q) : pack_status(epoch, kFlagPrefix, 0);
-    const uint32_t flag = uint32_t(s >> 32) & 3u;
-    const bool ready = uint32_t(s >> 34) == epoch && flag != 0;
-    const uint32_t not_ready = __ballot_sync(0xffffffffu, !ready);
-    const uint32_t prefix = __ballot_sync(0xffffffffu, ready && flag == kFlagPrefix);
-    const uint32_t first_wait = not_ready ? uint32_t(__ffs(not_ready) - 1) : 32u;
-    const uint32_t first_prefix = prefix ? uint32_t(__ffs(prefix) - 1) : 32u;
-    const uint32_t take = first_prefix < first_wait ? first_prefix + 1 : first_wait;
-    uint32_t v = lane < take ? uint32_t(s) : 0u;
+  bool done = false;
+  while (!done) {
+    uint64_t s[kWords];
 #pragma unroll
-    for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
-    excl += v;
-    if (first_prefix < first_wait) break;
-    j -= take;
-    if (take == 0) {
+    for (int w = 0; w < kWords; ++w) {
+      const int64_t q = j - 32 * w - int64_t(lane);
+      // before tile 0 (never reached: tile 0 publishes an inclusive prefix) reads as a zero prefix
+      s[w] = q >= 0 ? ld_status(status + q) : pack_status(epoch, kFlagPrefix, 0);
+    }
+    bool wait = false;
+#pragma unroll
+    for (int w = 0; w < kWords; ++w) {
+      if (done || wait) continue;   // (uniform)
+      const uint32_t flag = uint32_t(s[w] >> 32) & 3u;
+      const bool ready = uint32_t(s[w] >> 34) == epoch && flag != 0;
+      const uint32_t not_ready = __ballot_sync(0xffffffffu, !ready);
+      const uint32_t prefix = __ballot_sync(0xffffffffu, ready && flag == kFlagPrefix);
+      const uint32_t first_wait = not_ready ? uint32_t(__ffs(not_ready) - 1) : 32u;
+      const uint32_t first_prefix = prefix ? uint32_t(__ffs(prefix) - 1) : 32u;
+      done = first_prefix < first_wait;
+      wait = !done && first_wait < 32u;
+      const uint32_t take = done ? first_prefix + 1 : first_wait;
+      excl += __reduce_add_sync(0xffffffffu, lane < take ? uint32_t(s[w]) : 0u);
+      j -= take;
+    }
+    if (wait) {
       if (++spins > spin_limit) {
         if (lane == 0) atomicOr(err, 1u);
         break;
@@ -124,6 +136,26 @@ __device__ __forceinline__ uint32_t chained_exclusive(uint64_t* status, uint32_t
                                                       uint32_t agg, uint32_t epoch, uint32_t* err) {
   chain_publish(status, stride, tile, agg, epoch);
   return chain_lookback(status, stride, tile, agg, epoch, err);
+}
+
+// Passes that a sort of `bits` key bits takes (the result is in the second buffers when odd).
+__device__ __forceinline__ uint32_t sort_passes(uint32_t bits) { return (bits + 7u) / 8u; }
+
+// The tiles of a pixel box (x0 | x1 << 16, y0 | y1 << 16, inclusive pixels).
+struct TileRect {
+  uint32_t x, y, w, h;
+};
+
+__device__ __forceinline__ TileRect tile_rect(const uint2 b) {
+  const uint32_t x = (b.x & 0xFFFFu) >> 4, y = (b.y & 0xFFFFu) >> 4;
+  return {x, y, ((b.x >> 16) >> 4) - x + 1u, ((b.y >> 16) >> 4) - y + 1u};
+}
+
+// Live bits of w <= 32 tiles from column x on; row: the first word of their row in TileLive::bits
+// (the spare word after each row makes the second load valid).
+__device__ __forceinline__ uint32_t live_row(const uint32_t* __restrict__ row, uint32_t x, uint32_t w) {
+  const uint32_t v = __funnelshift_r(row[x >> 5], row[(x >> 5) + 1], x & 31u);
+  return w < 32u ? v & ((1u << w) - 1u) : v;
 }
 
 __device__ __forceinline__ uint32_t lanemask_lt() {

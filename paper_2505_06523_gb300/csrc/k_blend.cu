@@ -66,11 +66,11 @@ __device__ __forceinline__ bool composite_step(float l2a, float r, float g, floa
 // ---------------------------------------------------------------- variant 0: a warp per 8x4 pixels
 
 constexpr int kSubTiles = 8;      // 8x4 pixel blocks of a tile: two across, four down
-constexpr int kScanKeys = 4;      // keys per lane and scan step
-constexpr int kRing = 256;        // list positions waiting to be gathered: < 32 + 32 * kScanKeys
+constexpr int kScanKeys = 8;      // keys per lane and scan step
+constexpr int kRing = 512;        // list positions waiting to be gathered: < 32 + 32 * kScanKeys
 constexpr uint32_t kNoKey = (15u << 20) | (3u << 28);   // an empty box: meets no rectangle of a sub-tile
 
-constexpr int kAhead = 4;         // records whose alphas are computed ahead of the transmittance chain
+constexpr int kAhead = 8;         // records whose alphas are computed ahead of the transmittance chain
 
 // The staged records, one list for each 4x4 half of the sub-tile: the two half-warps composite
 // different records at once, so that a small Gaussian occupies 16 lanes and not 32.
@@ -87,13 +87,28 @@ __device__ __forceinline__ float ex2_approx(float x) {
   return y;
 }
 
-// (r, g, b) += w (cr, cg, cb) where `on`, by predicated instructions: a branch per record costs more
-// than the three of them (a colour may be infinite, so that w = 0 would not do).
-__device__ __forceinline__ void add_if(bool on, float w, float cr, float cg, float cb, float& r, float& g, float& b) {
-  asm("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %7, 0;\n\t@p fma.rn.f32 %0, %3, %4, %0;\n\t@p fma.rn.f32 %1, %3, %5, %1;\n\t"
-      "@p fma.rn.f32 %2, %3, %6, %2;\n\t}"
-      : "+f"(r), "+f"(g), "+f"(b)
-      : "f"(w), "f"(cr), "f"(cg), "f"(cb), "r"(uint32_t(on)));
+// One front-to-back step at a pixel, as composite_step, by predicated instructions (a branch per record
+// costs more than all of them).  in: not zero where the pixel is unfinished and in the record's box;
+// l2a: its log2 alpha; al: min(0.999, 2^l2a).  A record below 1/255 (or not a number) does nothing.
+// t carries the transmittance along: past the record that takes it below 1e-4 it stays below, so
+// nothing else contributes; T stays as the last contributing record left it.
+__device__ __forceinline__ void blend_step(uint32_t in, float l2a, float al, float cr, float cg, float cb, float& t,
+                                           float& T, float& r, float& g, float& b) {
+  asm("{\n\t.reg .pred p, q;\n\t.reg .f32 om, tn, w;\n\t"
+      "setp.ne.u32 p, %5, 0;\n\t"
+      "setp.ge.and.f32 p, %6, %11, p;\n\t"
+      "setp.ge.and.f32 p, %7, %12, p;\n\t"
+      "sub.rn.f32 om, 0f3F800000, %7;\n\t"
+      "mul.rn.f32 w, %7, %0;\n\t"
+      "mul.rn.f32 tn, %0, om;\n\t"
+      "setp.ge.and.f32 q, tn, %13, p;\n\t"
+      "@p mov.f32 %0, tn;\n\t"
+      "@q mov.f32 %1, tn;\n\t"
+      "@q fma.rn.f32 %2, w, %8, %2;\n\t"
+      "@q fma.rn.f32 %3, w, %9, %3;\n\t"
+      "@q fma.rn.f32 %4, w, %10, %4;\n\t}"
+      : "+f"(t), "+f"(T), "+f"(r), "+f"(g), "+f"(b)
+      : "r"(in), "f"(l2a), "f"(al), "f"(cr), "f"(cg), "f"(cb), "f"(kLog2MinAlpha), "f"(1.f / 255.f), "f"(1e-4f));
 }
 
 // The bounding rectangle of a warp's unfinished pixels, as the constants of key_hits: rows r0..r1
@@ -121,28 +136,55 @@ __device__ __forceinline__ bool key_hits(uint32_t key, KeyTest t) {
   return ((a & 0x41000000u) | (~b & 0x11000000u)) == 0u;
 }
 
+// The tile at position i of the classes' regions, one after the other (see k_blend_items; cls_incl:
+// in lane c, the tiles of classes 0 .. c).  All lanes call it.
+__device__ __forceinline__ uint32_t item_tile(const uint32_t* __restrict__ items, uint32_t n_tiles, uint32_t cls_incl, uint32_t i) {
+  const uint32_t cls = __popc(__ballot_sync(0xffffffffu, cls_incl <= i));   // lanes beyond the classes hold 2^32 - 1
+  const uint32_t before = __shfl_sync(0xffffffffu, cls_incl, cls ? cls - 1u : 0u);
+  return items[size_t(cls) * n_tiles + (i - (cls ? before : 0u))];
+}
+
+// In lane c, the tiles of classes 0 .. c.
+__device__ __forceinline__ uint32_t item_classes(const uint32_t* __restrict__ class_count) {
+  const uint32_t lane = threadIdx.x & 31u;
+  uint32_t incl = lane < uint32_t(kItemClasses) ? class_count[lane] : 0u;
+#pragma unroll
+  for (int d = 1; d < kItemClasses; d <<= 1) {
+    const uint32_t t = __shfl_up_sync(0xffffffffu, incl, d);
+    if (lane >= uint32_t(d)) incl += t;
+  }
+  return lane < uint32_t(kItemClasses) ? incl : 0xFFFFFFFFu;
+}
+
 // kCount: also count the evaluations and contributions into work[0], work[1].
-template <bool kCount>
+// kSlabbed: one of the frame's depth slabs (the first one covers every tile, later ones those with
+// pairs): the pixels' T goes through live.state (negative once the pixel has stopped) and their
+// colour through the image, and the 4x4 blocks whose last pixel stops are cleared in live.
+template <bool kCount, bool kSlabbed>
 __global__ void __launch_bounds__(kBlendThreads, kBlendBlocks)
 k_blend(const uint2* __restrict__ ranges, const uint32_t* __restrict__ items, uint32_t n_tiles,
-        uint32_t* __restrict__ tile_counter, const uint32_t* __restrict__ tk, const uint32_t* __restrict__ pv,
-        const float4* __restrict__ rec, uint32_t cap_slots, int width, int height, int tiles_x, int tiles_per_view,
-        float* __restrict__ rgb, float* __restrict__ t_out, unsigned long long* __restrict__ work,
-        uint32_t* __restrict__ frame, uint32_t* __restrict__ sticky) {
+        const uint32_t* __restrict__ class_count, uint32_t* __restrict__ slab, bool first, TileLive live_tiles, const uint32_t* __restrict__ tk,
+        const uint32_t* __restrict__ pv, const float4* __restrict__ rec, uint32_t cap_slots, int width, int height,
+        int tiles_x, int tiles_per_view, float* __restrict__ rgb, float* __restrict__ t_out,
+        unsigned long long* __restrict__ work, uint32_t* __restrict__ frame, uint32_t* __restrict__ sticky) {
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     if (frame[kOverflow]) atomicOr(sticky, 1u);
     if (frame[kTimeout]) atomicOr(sticky + 1, 1u);
   }
+  const uint32_t cls_incl = item_classes(class_count);
+  // (a later slab leaves out the tiles without pairs)
+  const uint32_t n_items =
+      (kSlabbed && !first ? __shfl_sync(0xffffffffu, cls_incl, kItemClasses - 2) : n_tiles) * uint32_t(kSubTiles);
   __shared__ BlendWarp s_warp[kBlendThreads / 32];
   const uint32_t lane = threadIdx.x & 31u;
   BlendWarp& S = s_warp[threadIdx.x >> 5];
   uint32_t n_eval = 0, n_contrib = 0;
   for (;;) {
     uint32_t it = 0;
-    if (lane == 0) it = atomicAdd(tile_counter, 1u);
+    if (lane == 0) it = atomicAdd(slab + kSlabBlendItem, 1u);
     it = __shfl_sync(0xffffffffu, it, 0);
-    if (it >= n_tiles * uint32_t(kSubTiles)) break;
-    const int tile = int(items[it / kSubTiles]);   // (view, tile) id
+    if (it >= n_items) break;
+    const int tile = int(item_tile(items, n_tiles, cls_incl, it / kSubTiles));   // (view, tile) id
     const uint32_t sub = it % kSubTiles;
     const int view = tile / tiles_per_view, vt = tile - view * tiles_per_view;
     const int tx = vt % tiles_x, ty = vt / tiles_x;
@@ -153,7 +195,23 @@ k_blend(const uint2* __restrict__ ranges, const uint32_t* __restrict__ items, ui
     const bool inside = px < width && py < height;
     float T = 1.f, cr = 0.f, cg = 0.f, cb = 0.f;
     uint32_t mybit = inside ? 1u << lane : 0u;   // 0 once the pixel has stopped
-    uint32_t live = __ballot_sync(0xffffffffu, inside);
+    const size_t p = (size_t(view) * height + py) * width + px;   // (inside: the pixel's place)
+    if (kSlabbed && !first && inside) {
+      T = live_tiles.state[p];
+      if (T < 0.f) {
+        mybit = 0u;
+        T = -T;
+      }
+    }
+    uint32_t live = __ballot_sync(0xffffffffu, mybit != 0u);
+    if (kSlabbed && !first) {
+      if (live == 0u) continue;   // (finished in an earlier slab)
+      if (inside) {
+        cr = rgb[3 * p + 0];
+        cg = rgb[3 * p + 1];
+        cb = rgb[3 * p + 2];
+      }
+    }
     const uint2 range = ranges[tile];
     uint32_t sp = range.x;                  // next list position to scan
     const uint32_t end = live ? range.y : range.x;
@@ -250,36 +308,29 @@ k_blend(const uint2* __restrict__ ranges, const uint32_t* __restrict__ items, ui
         const float4* sg = S.g[lane >> 4];
         const float4* sc = S.c[lane >> 4];
         const float2* srg = S.rg[lane >> 4];
+        // kAhead records at a time: their alphas are independent, only t is a chain
+        float t = T;
         for (int i = 0; i < n; i += kAhead) {
-          // the alphas of kAhead records (0: does not contribute to this pixel), independent of T.  As
-          // composite_step: alpha = min(0.999, 2^l2a), skipped below 1/255 (and for a NaN)
-          float a[kAhead], blue[kAhead];
+          float l2a[kAhead], al[kAhead], blue[kAhead];
+          uint32_t in[kAhead];
 #pragma unroll
           for (int q = 0; q < kAhead; ++q) {
             const float4 c = sc[i + q];
+            l2a[q] = log2_alpha(sg[i + q], c, fx, fy);
+            al[q] = fminf(0.999f, ex2_approx(l2a[q]));
+            in[q] = __float_as_uint(c.z) & mybit;
             blue[q] = c.w;
-            const float l2a = log2_alpha(sg[i + q], c, fx, fy);
-            const float al = fminf(0.999f, ex2_approx(l2a));
-            const bool in = (__float_as_uint(c.z) & mybit) != 0u;
-            if (kCount) n_eval += in ? 1u : 0u;
-            a[q] = in && l2a >= kLog2MinAlpha && al >= 1.f / 255.f ? al : 0.f;
           }
-          // T after each of them: a record that does not contribute multiplies by exactly 1, and past
-          // the one that would take T below 1e-4 every T is below it, so nothing else contributes
-          float t[kAhead + 1];
-          t[0] = T;
 #pragma unroll
           for (int q = 0; q < kAhead; ++q) {
-            t[q + 1] = t[q] * (1.f - a[q]);
+            if (kCount) {
+              n_eval += in[q] ? 1u : 0u;
+              n_contrib += in[q] && l2a[q] >= kLog2MinAlpha && al[q] >= 1.f / 255.f && t * (1.f - al[q]) >= 1e-4f ? 1u : 0u;
+            }
             const float2 rg = srg[i + q];
-            const bool on = a[q] > 0.f && t[q + 1] >= 1e-4f;
-            add_if(on, a[q] * t[q], rg.x, rg.y, blue[q], cr, cg, cb);
-            if (kCount) n_contrib += on ? 1u : 0u;
+            blend_step(in[q], l2a[q], al[q], rg.x, rg.y, blue[q], t, T, cr, cg, cb);
           }
-          // (where the pixel stops, T stays as the last contributing record left it)
-#pragma unroll
-          for (int q = 1; q <= kAhead; ++q) T = t[q] >= 1e-4f ? t[q] : T;
-          if (t[kAhead] < 1e-4f) mybit = 0u;
+          if (t < 1e-4f) mybit = 0u;   // the pixel has stopped
         }
         live = __ballot_sync(0xffffffffu, mybit != 0u);
         if (live == 0u) break;
@@ -289,11 +340,24 @@ k_blend(const uint2* __restrict__ ranges, const uint32_t* __restrict__ items, ui
       __syncwarp();   // the warp's staged records and ring are free for the next item
     }
     if (inside) {
-      const size_t p = (size_t(view) * height + py) * width + px;
       rgb[3 * p + 0] = cr;
       rgb[3 * p + 1] = cg;
       rgb[3 * p + 2] = cb;
       if (t_out) t_out[p] = T;
+      if (kSlabbed) live_tiles.state[p] = mybit ? T : -T;
+    }
+    if (kSlabbed && lane == 0 && (!(live & 0xFFFFu) || !(live >> 16))) {
+      // 4x4 blocks without an unfinished pixel (again, where an earlier slab finished them)
+      const uint32_t left = 1u << (4u * (sub >> 1) + 2u * (sub & 1u));
+      const uint32_t gone = (live & 0xFFFFu ? 0u : left) | (live >> 16 ? 0u : left << 1);
+      const uint32_t old = atomicAnd(live_tiles.blocks + tile, ~gone);
+      if (old != 0u && (old & ~gone) == 0u) {   // the tile's last
+        const TileLive& L = live_tiles;
+        atomicAnd(L.bits + size_t(view * L.tiles_y + ty) * L.words + (tx >> 5), ~(1u << (tx & 31)));
+        const uint32_t gx = uint32_t(tx) >> 3, row = view * L.groups_y + (uint32_t(ty) >> 3);
+        if (atomicSub(L.coarse_tiles + size_t(row) * L.groups_x + gx, 1u) == 1u)   // and the group's last
+          atomicAnd(L.coarse + size_t(row) * L.coarse_words + (gx >> 5), ~(1u << (gx & 31u)));
+      }
     }
   }  // next item
   if (kCount) {
@@ -457,7 +521,8 @@ constexpr int blend_px_blocks_per_sm(int batch) { return batch == 512 ? 4 : 5; }
 template <bool kCount, int kBatch>
 __global__ void __launch_bounds__(kPxThreads, blend_px_blocks_per_sm(kBatch))
 k_blend_px(const uint2* __restrict__ ranges, const uint32_t* __restrict__ items, uint32_t n_items,
-           uint32_t* __restrict__ tile_counter, const uint32_t* __restrict__ tk, const uint32_t* __restrict__ pv,
+           const uint32_t* __restrict__ class_count, uint32_t* __restrict__ tile_counter,
+           const uint32_t* __restrict__ tk, const uint32_t* __restrict__ pv,
            const float4* __restrict__ rec, uint32_t cap_slots, int width, int height, int tiles_x, int tiles_per_view,
            float* __restrict__ rgb, float* __restrict__ t_out, unsigned long long* __restrict__ work,
            uint32_t* __restrict__ frame, uint32_t* __restrict__ sticky) {
@@ -481,6 +546,7 @@ k_blend_px(const uint2* __restrict__ ranges, const uint32_t* __restrict__ items,
   const float fx = float(lx) + 0.5f, fy = float(ly) + 0.5f;
   uint32_t n_eval = 0, n_contrib = 0, phase = 0;
   bool failed = false;
+  const uint32_t cls_incl = item_classes(class_count);
   if (threadIdx.x == 0) mbar_init(&s_bar, 1);
   __syncthreads();
   for (;;) {
@@ -489,7 +555,7 @@ k_blend_px(const uint2* __restrict__ ranges, const uint32_t* __restrict__ items,
     const uint32_t next = s_next;
     __syncthreads();
     if (next >= n_items) break;
-    const int tile = int(items[next]);   // (view, tile) id
+    const int tile = int(item_tile(items, n_items, cls_incl, next));   // (view, tile) id
     const int view = tile / tiles_per_view, vt = tile - view * tiles_per_view;
     const int tx = vt % tiles_x, ty = vt / tiles_x;
     const int px = tx * 16 + lx, py = ty * 16 + ly;
@@ -586,33 +652,27 @@ out:
   }
 }
 
-// The tiles, those with the longest lists first (bucketed by floor(log2(pairs + 1)), descending), so
-// that the work items that take longest start first.  One block.
-__global__ void __launch_bounds__(1024) k_blend_items(const uint2* __restrict__ ranges, int n_tiles,
-                                                      uint32_t* __restrict__ items) {
-  __shared__ uint32_t s_hist[32];
-  if (threadIdx.x < 32) s_hist[threadIdx.x] = 0;
-  __syncthreads();
-  for (int t = threadIdx.x; t < n_tiles; t += blockDim.x) {
-    const uint32_t len = ranges[t].y - ranges[t].x;
-    atomicAdd(&s_hist[__clz(len + 1u)], 1u);   // clz: 0 for the heaviest
-  }
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    const uint32_t v = s_hist[threadIdx.x];
-    uint32_t incl = v;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const uint32_t t = __shfl_up_sync(0xffffffffu, incl, d);
-      if (threadIdx.x >= d) incl += t;
-    }
-    s_hist[threadIdx.x] = incl - v;   // cursor: first position of the bucket
-  }
-  __syncthreads();
-  for (int t = threadIdx.x; t < n_tiles; t += blockDim.x) {
-    const uint32_t len = ranges[t].y - ranges[t].x;
-    items[atomicAdd(&s_hist[__clz(len + 1u)], 1u)] = uint32_t(t);
-  }
+// The tiles by the length of their lists, in kItemClasses regions of n_tiles entries (class 0: 2^16
+// pairs or more, then an octave each, the last but one: 1 to 7 pairs, the last: none), so that the
+// work items that take longest start first.
+constexpr int kLastClass = kItemClasses - 1;
+__device__ __forceinline__ uint32_t item_class(uint32_t len) {
+  return len ? uint32_t(min(max(int(__clz(len)) - 15, 0), kLastClass - 1)) : uint32_t(kLastClass);
+}
+
+__global__ void __launch_bounds__(256) k_blend_items(const uint2* __restrict__ ranges, uint32_t n_tiles,
+                                                     uint32_t* __restrict__ items, uint32_t* __restrict__ class_count) {
+  const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
+  const uint32_t mask = __ballot_sync(0xffffffffu, t < n_tiles);
+  if (t >= n_tiles) return;
+  const uint2 r = ranges[t];
+  const uint32_t cls = item_class(r.y - r.x);
+  const uint32_t peers = __match_any_sync(mask, cls);
+  const int leader = __ffs(peers) - 1;
+  uint32_t base = 0;
+  if (int(threadIdx.x & 31u) == leader) base = atomicAdd(class_count + cls, __popc(peers));
+  base = __shfl_sync(peers, base, leader);
+  items[size_t(cls) * n_tiles + base + __popc(peers & lanemask_lt())] = t;
 }
 
 }  // namespace
@@ -621,11 +681,11 @@ namespace {
 
 template <bool kCount, int kBatch>
 void blend_px_launch(int grid, cudaStream_t st, const uint2* ranges, const uint32_t* items, uint32_t n_tiles,
-                     uint32_t* tile_counter, const uint32_t* tk, const uint32_t* pv, const float4* rec,
-                     uint32_t cap_slots, const CamConst& cam, float* rgb, float* t_out, unsigned long long* work,
+                     const uint32_t* class_count, uint32_t* tile_counter, const uint32_t* tk, const uint32_t* pv,
+                     const float4* rec, uint32_t cap_slots, const CamConst& cam, float* rgb, float* t_out, unsigned long long* work,
                      uint32_t* frame, uint32_t* sticky) {
-  k_blend_px<kCount, kBatch><<<grid, kPxThreads, 0, st>>>(ranges, items, n_tiles, tile_counter, tk, pv, rec, cap_slots,
-                                                          cam.width, cam.height, cam.tiles_x,
+  k_blend_px<kCount, kBatch><<<grid, kPxThreads, 0, st>>>(ranges, items, n_tiles, class_count, tile_counter, tk, pv, rec,
+                                                          cap_slots, cam.width, cam.height, cam.tiles_x,
                                                           cam.tiles_x * cam.tiles_y, rgb, t_out, work, frame, sticky);
 }
 
@@ -633,7 +693,8 @@ void blend_px_launch(int grid, cudaStream_t st, const uint2* ranges, const uint3
 
 cudaError_t blend_set_attributes() {
   // several resident blocks of 10-28 KB shared memory per SM want the largest carveout
-  const void* fns[] = {(const void*)k_blend<true>,          (const void*)k_blend<false>,
+  const void* fns[] = {(const void*)k_blend<true, false>,   (const void*)k_blend<false, false>,
+                       (const void*)k_blend<true, true>,    (const void*)k_blend<false, true>,
                        (const void*)k_blend_px<true, 128>,  (const void*)k_blend_px<false, 128>,
                        (const void*)k_blend_px<true, 256>,  (const void*)k_blend_px<false, 256>,
                        (const void*)k_blend_px<true, 512>,  (const void*)k_blend_px<false, 512>};
@@ -645,36 +706,33 @@ cudaError_t blend_set_attributes() {
   return cudaSuccess;
 }
 
-cudaError_t launch_blend(const uint2* ranges, uint32_t* items, uint32_t* tile_counter, const uint32_t* tk,
-                         const uint32_t* pv, const float4* rec, uint32_t cap_slots, const CamConst& cam, float* rgb,
-                         float* t_out, unsigned long long* work, uint32_t* frame, uint32_t* sticky, int batch, int mode,
-                         int n_views, int sm_count, cudaStream_t st) {
+cudaError_t launch_blend(const uint2* ranges, uint32_t* items, uint32_t* class_count, const uint32_t* tk,
+                         const uint32_t* pv, const float4* rec, uint32_t cap_slots, const CamConst& cam, float* rgb, float* t_out,
+                         unsigned long long* work, uint32_t* frame, uint32_t* sticky, int slab, const TileLive& live,
+                         int batch, int mode, int n_views, int sm_count, cudaStream_t st) {
   const int n_tiles = cam.tiles_x * cam.tiles_y * n_views;
   if (n_tiles == 0) return cudaSuccess;
   if (batch != 128 && batch != 256 && batch != 512) return cudaErrorInvalidValue;
-  if (mode != 0 && mode != 1) return cudaErrorInvalidValue;
-  k_blend_items<<<1, 1024, 0, st>>>(ranges, n_tiles, items);
+  if ((mode != 0 && mode != 1) || (mode == 1 && live.bits)) return cudaErrorInvalidValue;
+  uint32_t* words = frame + kSlabBase + slab * kSlabWords;
+  k_blend_items<<<(n_tiles + 255) / 256, 256, 0, st>>>(ranges, uint32_t(n_tiles), items, class_count);
   // persistent grids: the resident blocks
   if (mode == 0) {
     const int per_block = kBlendThreads / 32;
     const int grid = std::min((kSubTiles * n_tiles + per_block - 1) / per_block, sm_count * kBlendBlocks);
-    const int tiles_per_view = cam.tiles_x * cam.tiles_y;
-    if (work)
-      k_blend<true><<<grid, kBlendThreads, 0, st>>>(ranges, items, uint32_t(n_tiles), tile_counter, tk, pv, rec, cap_slots,
-                                                    cam.width, cam.height, cam.tiles_x, tiles_per_view, rgb, t_out, work,
-                                                    frame, sticky);
-    else
-      k_blend<false><<<grid, kBlendThreads, 0, st>>>(ranges, items, uint32_t(n_tiles), tile_counter, tk, pv, rec, cap_slots,
-                                                     cam.width, cam.height, cam.tiles_x, tiles_per_view, rgb, t_out,
-                                                     nullptr, frame, sticky);
+    const auto kernel = live.bits ? (work ? k_blend<true, true> : k_blend<false, true>)
+                                  : (work ? k_blend<true, false> : k_blend<false, false>);
+    kernel<<<grid, kBlendThreads, 0, st>>>(ranges, items, uint32_t(n_tiles), class_count, words, slab == 0, live, tk, pv, rec, cap_slots,
+                                           cam.width, cam.height, cam.tiles_x, cam.tiles_x * cam.tiles_y, rgb, t_out, work,
+                                           frame, sticky);
     return cudaGetLastError();
   }
   const int grid = std::min(n_tiles, sm_count * blend_px_blocks_per_sm(batch));
   const auto launch = batch == 128   ? (work ? blend_px_launch<true, 128> : blend_px_launch<false, 128>)
                       : batch == 256 ? (work ? blend_px_launch<true, 256> : blend_px_launch<false, 256>)
                                      : (work ? blend_px_launch<true, 512> : blend_px_launch<false, 512>);
-  launch(grid, st, ranges, items, uint32_t(n_tiles), tile_counter, tk, pv, rec, cap_slots, cam, rgb, t_out, work, frame,
-         sticky);
+  launch(grid, st, ranges, items, uint32_t(n_tiles), class_count, words + kSlabBlendItem, tk, pv, rec, cap_slots, cam, rgb, t_out, work,
+         frame, sticky);
   return cudaGetLastError();
 }
 

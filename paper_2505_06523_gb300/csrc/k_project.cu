@@ -123,11 +123,13 @@ static_assert(offsetof(InstFrame, m) % 16 == 0 && offsetof(InstFrame, cam_a) % 1
               offsetof(InstFrame, s) == offsetof(InstFrame, cam_a) + 12, "InstFrame float4 views");
 
 // Projects a Gaussian of a cluster (its pre-computed values G) for one entry (its constants E)
-// into slot `slot`; returns whether it is visible.  bc: the cluster's bound centre (asset frame).
-__device__ __forceinline__ bool project_one(const GaussPre& G, size_t slot, const EntryConst& E,
+// into slot `slot`; returns the number of tiles its pixel box covers (0: not visible) and its depth
+// key.  bc: the cluster's bound centre (asset frame).
+__device__ __forceinline__ uint32_t project_one(const GaussPre& G, size_t slot, const EntryConst& E,
                                             const CamConst& cam, const float4 bc, int nsh,
                                             float4* __restrict__ rec, uint2* __restrict__ rect,
-                                            uint32_t* __restrict__ keys, uint32_t* __restrict__ frame) {
+                                            uint32_t* __restrict__ keys, uint32_t* __restrict__ frame,
+                                            uint32_t* key_out) {
   const float4 M0 = E.m0, M1 = E.m1, M2 = E.m2, CA = E.cam, r0 = E.r0, r1 = E.r1;
   const struct { float m[12]; float cam_a[3]; } I = {{M0.x, M0.y, M0.z, M0.w, M1.x, M1.y, M1.z, M1.w, M2.x, M2.y, M2.z, M2.w},
                                                     {CA.x, CA.y, CA.z}};
@@ -210,7 +212,7 @@ __device__ __forceinline__ bool project_one(const GaussPre& G, size_t slot, cons
   vis = vis && (x0 <= x1) && (y0 <= y1) && isfinite(u) && isfinite(v);
   if (!vis) {
     keys[slot] = 0xFFFFFFFFu;
-    return false;
+    return 0u;
   }
   const int tx0 = int(x0) >> 4, ty0 = int(y0) >> 4;
   // mean relative to the first tile's pixel origin (exact subtraction of the integer part)
@@ -252,8 +254,22 @@ __device__ __forceinline__ bool project_one(const GaussPre& G, size_t slot, cons
   rp[2] = make_float4(rgb[2], __uint_as_float(origin), __uint_as_float(uint32_t(x0) | (uint32_t(x1) << 16)),
                       __uint_as_float(uint32_t(y0) | (uint32_t(y1) << 16)));
   rect[slot] = make_uint2(uint32_t(x0) | (uint32_t(x1) << 16), uint32_t(y0) | (uint32_t(y1) << 16));
-  keys[slot] = __float_as_uint(z32);
-  return true;
+  *key_out = __float_as_uint(z32);
+  keys[slot] = *key_out;
+  return uint32_t((int(x1) >> 4) - tx0 + 1) * uint32_t((int(y1) >> 4) - ty0 + 1);
+}
+
+// What a lane adds up over the Gaussians it projects.
+struct ProjTotals {
+  uint32_t visible = 0, key_min = 0xFFFFFFFFu, key_max = 0;
+  unsigned long long pairs = 0;
+};
+
+// The depth histogram's bin of a cluster at depth z (its centre: a bin of most of its Gaussians; the
+// slabs' limits need no more).
+__device__ __forceinline__ uint32_t depth_bin(float z) {
+  const int b = z > 0.f ? int(__float_as_uint(z) >> kDepthShift) - kDepthBase : 0;
+  return uint32_t(min(max(b, 0), kDepthBins - 1));
 }
 
 // One run of render-list entries that draw the same cluster (entries e = a .. b - 1 of the warp's
@@ -261,12 +277,12 @@ __device__ __forceinline__ bool project_one(const GaussPre& G, size_t slot, cons
 // lane and lane + 32 of the cluster, loads their attributes and computes their
 // instance-independent values once, and projects them for every entry of the run.
 template <typename TC>
-__device__ __forceinline__ uint32_t project_run(int lane, int a, int b, uint32_t ci, uint32_t cnt,
+__device__ __forceinline__ void project_run(int lane, int a, int b, uint32_t ci, uint32_t cnt,
                                                 const EntryConst* ent, const CamConst& cam, const float4 bc, int nsh,
                                                 const float* __restrict__ at, const TC* __restrict__ col,
                                                 float4* __restrict__ rec, uint2* __restrict__ rect,
-                                                uint32_t* __restrict__ keys, uint32_t* __restrict__ frame) {
-  uint32_t nvis = 0;
+                                                uint32_t* __restrict__ keys, uint32_t* __restrict__ frame,
+                                                ProjTotals& tot, uint32_t* s_hist) {
 #pragma unroll 1
   for (int h = 0; h < 2; ++h) {
     const uint32_t j = lane + 32 * h;
@@ -276,14 +292,25 @@ __device__ __forceinline__ uint32_t project_run(int lane, int a, int b, uint32_t
     for (int e = a; e < b; ++e) {
       const uint32_t ce = __shfl_sync(0xffffffffu, ci, e);
       const size_t slot = size_t(ce) * kSlots + j;
+      uint32_t area = 0;
       if (j >= cnt) {
         keys[slot] = 0xFFFFFFFFu;
-        continue;
+      } else {
+        uint32_t key = 0;
+        area = project_one(G, slot, ent[e], cam, bc, nsh, rec, rect, keys, frame, &key);
+        if (area) {
+          ++tot.visible;
+          tot.pairs += area;
+          tot.key_min = min(tot.key_min, key);
+          tot.key_max = max(tot.key_max, key);
+        }
       }
-      nvis += project_one(G, slot, ent[e], cam, bc, nsh, rec, rect, keys, frame) ? 1u : 0u;
+      if (s_hist) {   // (uniform)
+        const uint32_t sum = __reduce_add_sync(0xffffffffu, area);
+        if (lane == 0 && sum) atomicAdd(&s_hist[depth_bin(ent[e].r1.z)], sum);
+      }
     }
   }
-  return nvis;
 }
 
 // kFormats: bit 0 = float32 colour planes occur, bit 1 = float16 ones occur.  Each warp takes
@@ -300,14 +327,23 @@ k_project(const uint2* __restrict__ list, uint32_t cap_nodes, const InstFrame* _
           const AssetDev* __restrict__ assets, CamConst cam, const float4* __restrict__ ref,
           float4* __restrict__ rec, uint2* __restrict__ rect, uint32_t* __restrict__ keys,
           uint32_t* __restrict__ frame, const uint32_t* __restrict__ order,
-          const uint32_t* __restrict__ sorted_keys, int chunk) {
-  __shared__ uint32_t s_vis[kProjThreads / 32], s_dist[kProjThreads / 32];
+          const uint32_t* __restrict__ sorted_keys, uint32_t* __restrict__ depth_hist,
+          float2* __restrict__ depth_range, int chunk) {
+  __shared__ uint32_t s_vis[kProjThreads / 32], s_dist[kProjThreads / 32], s_min[kProjThreads / 32], s_max[kProjThreads / 32];
+  __shared__ unsigned long long s_pairs[kProjThreads / 32];
+  __shared__ uint32_t s_hist[kDepthBins];
   __shared__ EntryConst s_ent[kProjThreads / 32][kMaxChunk];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t n_nodes = min(frame[kRenderNodes], cap_nodes);
   const uint32_t n_chunks = (n_nodes + chunk - 1) / chunk;
   EntryConst* ent = s_ent[warp];
-  uint32_t nvis = 0, ndist = 0;
+  if (depth_hist) {
+    for (int i = threadIdx.x; i < kDepthBins; i += kProjThreads) s_hist[i] = 0;
+    __syncthreads();
+  }
+  uint32_t* hist = depth_hist ? s_hist : nullptr;
+  ProjTotals tot;
+  uint32_t ndist = 0;
   for (;;) {   // persistent warps take the chunks in turn from a frame counter
     uint32_t ch = 0;
     if (lane == 0) ch = atomicAdd(frame + kTileCounters + kProjChunkCounter, 1u);
@@ -331,6 +367,12 @@ k_project(const uint2* __restrict__ list, uint32_t cap_nodes, const InstFrame* _
       E.cam = *reinterpret_cast<const float4*>(I.cam_a);
       E.r0 = ref[2 * ci];
       E.r1 = ref[2 * ci + 1];
+      if (depth_hist) {   // the node's depths: its centre's +- its radius, with a slack above the keys' rounding
+        const float4 b = assets[asset].bound[node];
+        const float reach = E.cam.w * b.w;
+        const float slack = 4e-6f * (fabsf(E.m2.x * b.x) + fabsf(E.m2.y * b.y) + fabsf(E.m2.z * b.z) + fabsf(E.m2.w) + 4.f * reach) + 1e-30f;
+        depth_range[ci] = make_float2(E.r1.z - reach - slack, E.r1.z + reach + slack);
+      }
       if (sorted_keys && (p == 0 || sorted_keys[p] != sorted_keys[p - 1])) ++ndist;
     }
     __syncwarp();
@@ -350,32 +392,51 @@ k_project(const uint2* __restrict__ list, uint32_t cap_nodes, const InstFrame* _
       const float* at = reinterpret_cast<const float*>(blk);    // geometry planes
       const unsigned char* col = blk + size_t(kGeoPlanes) * kSlots * 4;   // colour planes
       if (kFormats == 2 || (kFormats == 3 && A.half_color))
-        nvis += project_run<__half>(lane, a, b, ci, cnt, ent, cam, bc, int(A.sh_coeffs), at,
-                                    reinterpret_cast<const __half*>(col), rec, rect, keys, frame);
+        project_run<__half>(lane, a, b, ci, cnt, ent, cam, bc, int(A.sh_coeffs), at,
+                            reinterpret_cast<const __half*>(col), rec, rect, keys, frame, tot, hist);
       else
-        nvis += project_run<float>(lane, a, b, ci, cnt, ent, cam, bc, int(A.sh_coeffs), at,
-                                   reinterpret_cast<const float*>(col), rec, rect, keys, frame);
+        project_run<float>(lane, a, b, ci, cnt, ent, cam, bc, int(A.sh_coeffs), at,
+                           reinterpret_cast<const float*>(col), rec, rect, keys, frame, tot, hist);
     }
   }
-  // one atomic per block for the visible count (and the distinct clusters)
+  // one atomic per block for each total
+  uint32_t nvis = tot.visible;
 #pragma unroll
   for (int d = 16; d > 0; d >>= 1) {
     nvis += __shfl_xor_sync(0xffffffffu, nvis, d);
     ndist += __shfl_xor_sync(0xffffffffu, ndist, d);
+    tot.pairs += __shfl_xor_sync(0xffffffffu, tot.pairs, d);
   }
+  const uint32_t kmin = __reduce_min_sync(0xffffffffu, tot.key_min), kmax = __reduce_max_sync(0xffffffffu, tot.key_max);
   if (lane == 0) {
-    s_vis[threadIdx.x >> 5] = nvis;
-    s_dist[threadIdx.x >> 5] = ndist;
+    s_vis[warp] = nvis;
+    s_dist[warp] = ndist;
+    s_pairs[warp] = tot.pairs;
+    s_min[warp] = kmin;
+    s_max[warp] = kmax;
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    uint32_t t = 0, u = 0;
+    uint32_t t = 0, u = 0, mn = 0xFFFFFFFFu, mx = 0;
+    unsigned long long np = 0;
     for (int w = 0; w < kProjThreads / 32; ++w) {
       t += s_vis[w];
       u += s_dist[w];
+      np += s_pairs[w];
+      mn = min(mn, s_min[w]);
+      mx = max(mx, s_max[w]);
     }
-    if (t) atomicAdd(frame + kVisible, t);
+    if (t) {
+      atomicAdd(frame + kVisible, t);
+      atomicAdd(reinterpret_cast<unsigned long long*>(frame + kPairs64), np);
+      atomicMax(frame + kKeyMinInv, ~mn);
+      atomicMax(frame + kKeyMax, mx);
+    }
     if (u) atomicAdd(frame + kRenderClusters, u);
+  }
+  if (depth_hist) {
+    for (int i = threadIdx.x; i < kDepthBins; i += kProjThreads)
+      if (s_hist[i]) atomicAdd(depth_hist + i, s_hist[i]);
   }
 }
 
@@ -405,17 +466,15 @@ cudaError_t launch_noderef(const uint2* list, uint32_t cap, const InstFrame* ins
 cudaError_t launch_project(const uint2* list, uint32_t cap_nodes, const InstFrame* inst, const AssetDev* assets,
                            const CamConst& cam, const float4* ref, float4* rec, uint2* rect, uint32_t* keys,
                            uint32_t* frame, const uint32_t* order, const uint32_t* sorted_keys,
-                           int color_formats, int sm_count, cudaStream_t st) {
+                           int color_formats, uint32_t* depth_hist, float2* depth_range, int sm_count,
+                           cudaStream_t st) {
   // persistent grid: the resident blocks of the specialisation
   const int f = color_formats == 2 ? 2 : color_formats == 3 ? 3 : 1;
   const int grid = sm_count * std::max(g_project_blocks_per_sm[f], 1);
   const int chunk = order ? kProjChunkGrouped : kProjChunkList;
-  if (color_formats == 2)
-    k_project<2><<<grid, kProjThreads, 0, st>>>(list, cap_nodes, inst, assets, cam, ref, rec, rect, keys, frame, order, sorted_keys, chunk);
-  else if (color_formats == 3)
-    k_project<3><<<grid, kProjThreads, 0, st>>>(list, cap_nodes, inst, assets, cam, ref, rec, rect, keys, frame, order, sorted_keys, chunk);
-  else
-    k_project<1><<<grid, kProjThreads, 0, st>>>(list, cap_nodes, inst, assets, cam, ref, rec, rect, keys, frame, order, sorted_keys, chunk);
+  const auto kernel = f == 2 ? k_project<2> : f == 3 ? k_project<3> : k_project<1>;
+  kernel<<<grid, kProjThreads, 0, st>>>(list, cap_nodes, inst, assets, cam, ref, rec, rect, keys, frame, order,
+                                        sorted_keys, depth_hist, depth_range, chunk);
   return cudaGetLastError();
 }
 

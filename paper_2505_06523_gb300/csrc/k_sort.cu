@@ -2,23 +2,24 @@
 //
 // One histogram kernel reads the keys once and counts all digit passes (as many passes as 8-bit
 // digits need, the key's bits then spread evenly over them: 13 tile bits as 7 + 6); then each
-// pass is a single kernel: a block takes the next 4096-key tile (virtual id from an atomic counter),
+// pass is a single kernel: a block scans the pass's digit counts, then takes the next 4096-key tile (virtual id from an atomic counter),
 // ranks its keys per digit within each warp (stable: item-major then lane order within a warp,
 // warps in order), publishes its per-digit counts (the sums of the warps' counts), reorders the
 // tile by digit in shared memory (so that the global writes come out in runs), and looks back
 // across earlier tiles per digit (one thread per digit, 4 status words per round, bounded waits)
 // to find its global offsets.
 #include <algorithm>
+#include <utility>
 
 #include "dev_common.cuh"
 
 namespace v3dg {
 namespace {
 
-constexpr int kBins = 256;
+constexpr int kBins = kSortBins;
 constexpr int kLookback = 4;   // status words read per look-back round
 constexpr int kWarps = kSortThreads / 32;
-static_assert(kSortThreads >= kBins, "one thread per digit");
+static_assert(kSortThreads == kBins, "one thread per digit");
 
 // Digit counts of every pass in one read of the keys (one shared histogram per pass and block).
 // A thread counts a run of kHistRun consecutive keys and adds each pass's digit to the shared
@@ -27,19 +28,37 @@ static_assert(kSortThreads >= kBins, "one thread per digit");
 // atomics on the few hot bins of the high digits from serialising.
 constexpr int kHistRun = 16;
 
+// The digits of a sort: pass p covers `width` bits from begin + p * width (the last one what is left
+// of them).  On the device, bits_dev replaces the host's bit range.
+struct SortDigits {
+  int begin, end, passes, width;
+};
+
+__host__ __device__ __forceinline__ SortDigits sort_digits(int begin, int end) {
+  const int passes = (end - begin + 7) / 8;
+  return {begin, end, passes, passes > 0 ? (end - begin + passes - 1) / passes : 8};
+}
+
+__device__ __forceinline__ SortDigits sort_digits(SortDigits d, const uint32_t* bits_dev) {
+  return bits_dev ? sort_digits(0, int(*bits_dev)) : d;
+}
+
 __global__ void __launch_bounds__(256)
-k_hist(const uint32_t* __restrict__ keys, const uint32_t* __restrict__ n_dev, uint32_t cap, int begin_bit,
-       int end_bit, int passes, int width, uint32_t* __restrict__ hist) {
+k_hist(const uint32_t* __restrict__ keys, const uint32_t* __restrict__ n_dev, uint32_t cap, SortDigits dg,
+       const uint32_t* __restrict__ bits_dev, uint32_t* __restrict__ hist) {
   __shared__ uint32_t sh[4][kBins];
+  const uint32_t n = min(*n_dev, cap);
+  if (uint64_t(blockIdx.x) * blockDim.x * kHistRun >= n) return;   // no run for this block
+  dg = sort_digits(dg, bits_dev);
+  const int passes = dg.passes;
   for (int i = threadIdx.x; i < 4 * kBins; i += blockDim.x) sh[i / kBins][i % kBins] = 0;
   __syncthreads();
-  const uint32_t n = min(*n_dev, cap);
   int sh_[4];
   uint32_t m[4];
 #pragma unroll
   for (int p = 0; p < 4; ++p) {
-    sh_[p] = begin_bit + width * p;
-    m[p] = (1u << min(max(end_bit - sh_[p], 0), width)) - 1u;
+    sh_[p] = dg.begin + dg.width * p;
+    m[p] = (1u << min(max(dg.end - sh_[p], 0), dg.width)) - 1u;
   }
   const uint32_t runs = (n + kHistRun - 1) / kHistRun;
   const bool aligned = (reinterpret_cast<uintptr_t>(keys) & 15u) == 0;
@@ -98,23 +117,12 @@ k_hist(const uint32_t* __restrict__ keys, const uint32_t* __restrict__ n_dev, ui
   }
 }
 
-// Exclusive scan over digits of each pass's global histogram: the first output position of each
-// digit (one block, one thread per digit).
-__global__ void __launch_bounds__(kBins) k_hist_scan(const uint32_t* __restrict__ hist, int passes,
-                                                     uint32_t* __restrict__ excl) {
-  __shared__ uint32_t s_scan[kBins / 32 + 1];
-  for (int p = 0; p < passes; ++p) {
-    uint32_t total;
-    excl[p * kBins + threadIdx.x] = block_exclusive_scan<kBins / 32>(hist[p * kBins + threadIdx.x], s_scan, &total);
-  }
-}
-
 template <bool kImplicit>
 __global__ void __launch_bounds__(kSortThreads, 4)
 k_onesweep(const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin, uint32_t* __restrict__ kout,
-           uint32_t* __restrict__ vout, const uint32_t* __restrict__ n_dev, uint32_t cap, int shift, uint32_t dmask,
-           const uint32_t* __restrict__ gexcl, uint64_t* __restrict__ status, uint32_t* __restrict__ tile_counter,
-           uint32_t epoch, uint32_t* __restrict__ err) {
+           uint32_t* __restrict__ vout, const uint32_t* __restrict__ n_dev, uint32_t cap, SortDigits dg, int pass,
+           const uint32_t* __restrict__ bits_dev, const uint32_t* __restrict__ hist, uint64_t* __restrict__ status,
+           uint32_t* __restrict__ tile_counter, uint32_t epoch, uint32_t* __restrict__ err) {
   __shared__ uint32_t s_keys[kSortTile];
   __shared__ uint32_t s_vals[kSortTile];
   __shared__ uint16_t s_wh[kWarps][kBins];   // per-warp digit counts, then per-warp exclusive offsets
@@ -128,6 +136,13 @@ k_onesweep(const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin, u
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t n = min(*n_dev, cap);
   const uint32_t ntiles = (n + kSortTile - 1) / kSortTile;
+  dg = sort_digits(dg, bits_dev);
+  if (pass >= dg.passes || blockIdx.x >= ntiles) return;
+  const int shift = dg.begin + dg.width * pass;
+  const uint32_t dmask = (1u << min(dg.end - shift, dg.width)) - 1u;
+  // the first output position of this thread's digit: exclusive scan of the pass's digit counts
+  uint32_t all;
+  const uint32_t gexcl = block_exclusive_scan<kWarps>(hist[tid], s_scan, &all);
   for (int i = tid; i < kWarps * kBins; i += kSortThreads) (&s_match[0][0])[i] = 0u;
   // persistent blocks: tiles in the order of an atomic counter, so every tile a look-back waits
   // for is held by a running block
@@ -212,7 +227,7 @@ k_onesweep(const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin, u
   }
   if (tid <= dmask) {   // (the digit's count and start reloaded: no registers held over the reorder)
     const uint32_t excl = chain_lookback<kLookback>(status + tid, kBins, tile, s_cnt[tid], epoch, err);
-    s_goff[tid] = gexcl[tid] + excl - s_start[tid];   // wraps; dst = s_goff + p is exact below 2^32
+    s_goff[tid] = gexcl + excl - s_start[tid];   // wraps; dst = s_goff + p is exact below 2^32
   }
   __syncthreads();
   const uint32_t valid = min(uint32_t(kSortTile), n - tile * kSortTile);
@@ -265,42 +280,35 @@ cudaError_t sort_set_attributes() {
 cudaError_t launch_sort(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1, const uint32_t* n_dev,
                         uint32_t cap, int begin_bit, int end_bit, bool implicit_vals, const SortScratch& sc,
                         uint32_t* err_flag, uint32_t& epoch, int sm_count, cudaStream_t st, bool* result_in_1,
-                        int* launches) {
-  const int passes = (end_bit - begin_bit + 7) / 8;
-  const int width = passes > 0 ? (end_bit - begin_bit + passes - 1) / passes : 8;   // balanced digits
+                        int* launches, const uint32_t* bits_dev) {
+  const SortDigits dg = sort_digits(begin_bit, end_bit);
   *result_in_1 = false;
-  if (passes <= 0 || cap == 0) return cudaSuccess;
-  if (passes > 4) return cudaErrorInvalidValue;
+  if (dg.passes <= 0 || cap == 0) return cudaSuccess;
+  if (dg.passes > kSortPasses) return cudaErrorInvalidValue;
   const uint32_t max_tiles = (cap + kSortTile - 1) / kSortTile;
   if (max_tiles > sc.max_tiles) return cudaErrorInvalidValue;
   // persistent grid: the resident blocks, whatever the capacity (surplus blocks cost launches)
   const uint32_t grid = std::min<uint32_t>(max_tiles, uint32_t(sm_count) * uint32_t(g_sort_blocks_per_sm));
-  cudaError_t e = cudaMemsetAsync(sc.hist, 0, sizeof(uint32_t) * kBins * passes, st);
+  cudaError_t e = cudaSuccess;
+  if (!sc.hist_zeroed) e = cudaMemsetAsync(sc.hist, 0, sizeof(uint32_t) * kBins * dg.passes, st);
   if (e != cudaSuccess) return e;
-  k_hist<<<sm_count * 4, 256, 0, st>>>(k0, n_dev, cap, begin_bit, end_bit, passes, width, sc.hist);
-  k_hist_scan<<<1, kBins, 0, st>>>(sc.hist, passes, sc.hist + 4 * kBins);
-  *launches += 2;
+  k_hist<<<sm_count * 4, 256, 0, st>>>(k0, n_dev, cap, dg, bits_dev, sc.hist);
+  ++*launches;
   uint32_t *ki = k0, *vi = v0, *ko = k1, *vo = v1;
-  for (int p = 0; p < passes; ++p) {
-    const int shift = begin_bit + width * p;
-    const uint32_t dmask = (1u << std::min(end_bit - shift, width)) - 1u;
+  for (int p = 0; p < dg.passes; ++p) {
     epoch = (epoch + 1) & 0x3FFFFFFFu;
     if (epoch == 0) epoch = 1;
     const uint32_t ep = epoch;
-    if (p == 0 && implicit_vals)
-      k_onesweep<true><<<grid, kSortThreads, 0, st>>>(ki, vi, ko, vo, n_dev, cap, shift, dmask, sc.hist + 4 * kBins + kBins * p,
-                                                           sc.status, sc.tile_counters + p, ep, err_flag);
-    else
-      k_onesweep<false><<<grid, kSortThreads, 0, st>>>(ki, vi, ko, vo, n_dev, cap, shift, dmask, sc.hist + 4 * kBins + kBins * p,
-                                                            sc.status, sc.tile_counters + p, ep, err_flag);
+    const auto kernel = p == 0 && implicit_vals ? k_onesweep<true> : k_onesweep<false>;
+    kernel<<<grid, kSortThreads, 0, st>>>(ki, vi, ko, vo, n_dev, cap, dg, p, bits_dev, sc.hist + kBins * p, sc.status,
+                                          sc.tile_counters + p, ep, err_flag);
     ++*launches;
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    uint32_t* t;
-    t = ki; ki = ko; ko = t;
-    t = vi; vi = vo; vo = t;
+    std::swap(ki, ko);
+    std::swap(vi, vo);
   }
-  *result_in_1 = (passes & 1) != 0;
+  *result_in_1 = (dg.passes & 1) != 0;
   return cudaSuccess;
 }
 

@@ -53,6 +53,7 @@ constexpr uint32_t kInitNodes = 1u << 14;
 constexpr uint32_t kInitPairs = 1u << 22;
 constexpr uint32_t kMaxNodes = 1u << 25;               // render-list clusters: at most 2^31 slots
 constexpr uint32_t kMaxPairs = 0xFFFFFFFFu - 4096u;    // pair indices are 32-bit (a sort tile of headroom)
+constexpr uint32_t kManyPairs = 1u << 24;              // pairs of the previous frame from which one is taken in slabs
 enum { kStageSelect = 0, kStageProject, kStageDepthSort, kStageBin, kStageTileSort, kStageRanges, kStageBlend, kStages };
 
 }  // namespace
@@ -92,13 +93,23 @@ struct Pipe {
   uint32_t* h_tmp = nullptr;     // pinned scratch: [0, 48) frame words of read-backs, [48, 52) blend work
 
   uint32_t cap_nodes = 0, cap_slots = 0, cap_pairs = 0, status_words = 0, cap_cut = 0;
-  DevBuf d_list, d_ref, d_keys0, d_keys1, d_vals0, d_vals1, d_rec, d_rect;
+  // d_keys0: the projection's depth keys per slot; (d_keys1, d_vals1) and (d_keys2, d_vals0): the
+  // depth sort's buffers
+  DevBuf d_list, d_ref, d_keys0, d_keys1, d_keys2, d_vals0, d_vals1, d_rec, d_rect;
   DevBuf d_pk0, d_pk1, d_pv0, d_pv1, d_ranges, d_status, d_hist, d_cut;
   DevBuf d_img, d_timg, d_sort_k, d_sort_v, d_order;
   DevBuf d_front0, d_front1, d_tdcount, d_bitmap;   // top-down selection
-  bool depth_in1 = false, tiles_in1 = false;
+  // several slabs: the tiles' liveness and the pixels' T between them; per node the depth range and
+  // the marked slots, and their counts
+  DevBuf d_tlive, d_state, d_marks;
+  bool tiles_in1 = false;
+  uint32_t pairs_hint = 0;   // pairs of the previous frame (of one still running: of the one before)
+  int slabs = 1;             // depth slabs of the last rendered frame
+  bool full_lists = false;   // the sorted Gaussians and pairs of the whole frame are on the device
   uint32_t epoch = 1;
-  cudaEvent_t ev[kStages + 1] = {};
+  // stage events: [0] select, [1] project, then six per slab (depth sort, bin, tile sort, ranges,
+  // blend, its end)
+  cudaEvent_t ev[2 + 6 * kMaxSlabs] = {};
   // CUDA-graph frames (V3DG_OPT_GRAPHS): the selection is enqueued with the render, and both are
   // captured once per configuration (gkey) on cap_stream, then replayed on `stream`
   bool select_pending = false;
@@ -224,6 +235,54 @@ v3dg_status ensure_status(Pipe* c, uint64_t words) {
   return V3DG_OK;
 }
 
+// d_hist: the classes of the blend's work items in each slab, the digit counts of a frame's sorts
+// (cluster order or the standalone sort, then depth and tile sort of each slab), the depth histogram.
+constexpr int kFrameSorts = 1 + 2 * kMaxSlabs;
+constexpr uint32_t kSortHist = kMaxSlabs * kItemClasses, kDepthHist = kSortHist + kFrameSorts * kSortPasses * kSortBins,
+                   kHistWords = kDepthHist + kDepthBins;
+
+// Depth slabs of the next frame (see k_slab.cu): several when the pipe's previous frame had at least
+// kManyPairs pairs, one otherwise and for blend variant 1, which keeps no state between slabs.  The
+// image does not depend on it.  Several slabs of a small frame cost up to 0.3 ms of launches and of
+// tails (measured on the asset 50 units away, 0.5M pairs: 0.53 -> 0.85 ms); frames of 30M pairs and
+// more take 0.4 to 0.8 times as long (see k_slab.cu).  The frame's own pair count is not known when its
+// launches are made, and consecutive frames of a viewer or a batch are alike.
+int slab_count(const Pipe* c) { return c->pairs_hint >= kManyPairs && c->ctx->blend_mode == 0 ? kMaxSlabs : 1; }
+
+TileLive tile_live(Pipe* c, int slabs) {
+  TileLive l{};
+  l.tiles_x = uint32_t(c->cc.tiles_x);
+  l.tiles_y = uint32_t(c->cc.tiles_y);
+  l.groups_x = (l.tiles_x + 7) / 8;
+  l.groups_y = (l.tiles_y + 7) / 8;
+  l.words = (l.tiles_x + 31) / 32 + 1;
+  l.coarse_words = (l.groups_x + 31) / 32 + 1;
+  if (slabs == 1 || !c->d_tlive.p) return l;
+  l.bits = P<uint32_t>(c->d_tlive);
+  l.blocks = l.bits + size_t(l.words) * l.tiles_y * c->n_views;
+  l.coarse = l.blocks + size_t(l.tiles_x) * l.tiles_y * c->n_views;
+  l.coarse_tiles = l.coarse + size_t(l.coarse_words) * l.groups_y * c->n_views;
+  l.state = P<float>(c->d_state);
+  return l;
+}
+
+// The buffers that a render adds for its image size: tile ranges of every slab, work items and, for
+// several slabs, the tiles' liveness and the pixels' state.
+v3dg_status ensure_image_work(Pipe* c) {
+  const int slabs = slab_count(c);
+  const size_t n_tiles = size_t(c->cc.tiles_x) * size_t(c->cc.tiles_y) * c->n_views;
+  ST(ensure(c, c->d_ranges, sizeof(uint2) * n_tiles * size_t(slabs)));
+  ST(ensure(c, c->d_order, sizeof(uint32_t) * n_tiles * kItemClasses));
+  if (slabs > 1) {
+    ST(ensure(c, c->d_marks, (sizeof(uint2) + sizeof(float2)) * size_t(c->cap_nodes) + sizeof(uint32_t) * (size_t(c->cap_nodes) / 256 + 1)));
+    const TileLive l = tile_live(c, slabs);
+    ST(ensure(c, c->d_tlive, sizeof(uint32_t) * (n_tiles + (size_t(l.tiles_y) * l.words + size_t(l.groups_y) *
+                                                            (l.coarse_words + l.groups_x)) * c->n_views)));
+    ST(ensure(c, c->d_state, sizeof(float) * size_t(c->cc.width) * size_t(c->cc.height) * c->n_views));
+  }
+  return V3DG_OK;
+}
+
 // Work buffers sized by the current capacities.
 v3dg_status ensure_work(Pipe* c) {
   if (c->cap_nodes == 0) c->cap_nodes = kInitNodes;
@@ -234,6 +293,7 @@ v3dg_status ensure_work(Pipe* c) {
   ST(ensure(c, c->d_ref, sizeof(float4) * 2 * c->cap_nodes));
   ST(ensure(c, c->d_keys0, 4 * S));
   ST(ensure(c, c->d_keys1, 4 * S));
+  ST(ensure(c, c->d_keys2, 4 * S));
   ST(ensure(c, c->d_vals0, 4 * S));
   ST(ensure(c, c->d_vals1, 4 * S));
   ST(ensure(c, c->d_rec, sizeof(float4) * 3 * S));
@@ -247,13 +307,16 @@ v3dg_status ensure_work(Pipe* c) {
   words = std::max<uint64_t>(words, uint64_t(c->n_inst_frame) * uint64_t(std::max(c->node_blocks, 1)));
   words = std::max<uint64_t>(words, (uint64_t(S) + 1023) / 1024);
   ST(ensure_status(c, words));
-  ST(ensure(c, c->d_hist, 2 * 4 * 256 * 4));  // counts + exclusive offsets of up to 4 passes
+  ST(ensure(c, c->d_hist, sizeof(uint32_t) * kHistWords));
   return V3DG_OK;
 }
 
-SortScratch sort_scratch(Pipe* c, uint32_t* tile_counters) {
+// Scratch of the pipe's sort number `which` (each has its own digit counts; zeroed: cleared by the
+// frame's start).
+SortScratch sort_scratch(Pipe* c, int which, bool zeroed, uint32_t* tile_counters) {
   SortScratch sc;
-  sc.hist = P<uint32_t>(c->d_hist);
+  sc.hist = P<uint32_t>(c->d_hist) + kSortHist + which * kSortPasses * kSortBins;
+  sc.hist_zeroed = zeroed;
   sc.status = P<uint64_t>(c->d_status);
   sc.max_tiles = c->status_words / 256;
   sc.tile_counters = tile_counters;
@@ -307,6 +370,7 @@ v3dg_status setup_views(Pipe* c, const ViewSpec* views, uint32_t n_views) {
     nf64 += views[v].n;
   }
   const v3dg_camera* cam = views[0].cam;
+  if (c->rendered) c->pairs_hint = *const_cast<const volatile uint32_t*>(c->h_frame + kPairs);
   if (c->ctx->assets.empty()) return fail(c, V3DG_ENOTFOUND, "no hierarchy loaded");
   const uint64_t tiles = uint64_t((cam->width + kTile - 1) / kTile) * uint64_t((cam->height + kTile - 1) / kTile);
   if (tiles * n_views > uint64_t(kMaxTiles))
@@ -474,7 +538,7 @@ v3dg_status launch_selection(Pipe* c, int mode, uint2* out, uint32_t cap, uint32
 v3dg_status enqueue_select(Pipe* c) {
   ST(ensure_work(c));
   CU(cudaMemsetAsync(c->d_frame.p, 0, sizeof(uint32_t) * kFrameWords, c->stream));
-  stage_event(c, kStageSelect);
+  stage_event(c, 0);
   ST(launch_selection(c, 0, P<uint2>(c->d_list), c->cap_nodes, P<uint32_t>(c->d_frame)));
   return V3DG_OK;
 }
@@ -489,26 +553,68 @@ bool use_project_order(const Pipe* c) {
   return c->n_inst_frame >= 2 * uint64_t(std::max<uint32_t>(c->distinct_assets, 1)) && c->n_inst_frame >= 4;
 }
 
-// Start of a render: zero the render stages' counters (select's words stay, so that a render
-// list overflow still invalidates the frame) and count the slots the depth sort covers.
-__global__ void k_render_reset(uint32_t* frame, uint32_t cap_nodes) {
-  const int i = threadIdx.x;
-  if (i == kVisible || i == kPairs || i == kPairsEff || i == kConicFp64 || i == kRenderClusters || i == kPairs64 ||
-      i == kPairs64 + 1 ||
-      (i > kTileCounters && i < kFrameWords))
-    frame[i] = 0;
-  if (i == kSlotCount) frame[kSlotCount] = min(frame[kRenderNodes], cap_nodes) * uint32_t(kSlots);
-}
-
 __global__ void k_set_word(uint32_t* p, uint32_t v) { *p = v; }
+
+// One depth slab's Gaussians, depth-sorted, expanded into pairs, tile-sorted, with their tile ranges.
+v3dg_status enqueue_slab_lists(Pipe* c, int slab, bool filter, const TileLive& live) {
+  const CamConst& k = c->cc;
+  uint32_t* frame = P<uint32_t>(c->d_frame);
+  uint32_t* words = frame + kSlabBase + slab * kSlabWords;
+  const int sm = c->ctx->sm_count;
+  const InstFrame* inst_views = c->n_views > 1 ? P<InstFrame>(c->d_inst) : nullptr;
+  const int tiles_view = k.tiles_x * k.tiles_y, n_tiles = tiles_view * int(c->n_views);   // (view, tile) ids
+  stage_event(c, 2 + 6 * slab);
+  if (live.bits) {
+    float2* depth_range = P<float2>(c->d_marks);
+    uint2* marks = reinterpret_cast<uint2*>(depth_range + c->cap_nodes);
+    CU(launch_pick_slab(P<uint32_t>(c->d_keys0), P<uint2>(c->d_rect), c->cap_nodes, P<uint2>(c->d_list), inst_views, live,
+                        filter, depth_range, marks, reinterpret_cast<uint32_t*>(marks + c->cap_nodes),
+                        P<uint32_t>(c->d_keys1), P<uint32_t>(c->d_vals1), frame, slab, sm, c->stream));
+    c->ctx->launches += 2;
+  } else {
+    CU(launch_pick(P<uint32_t>(c->d_keys0), c->cap_nodes, P<uint32_t>(c->d_keys1), P<uint32_t>(c->d_vals1), frame, slab,
+                   P<uint64_t>(c->d_status), next_epoch(c), sm, c->stream));
+  }
+  bool unused = false;
+  int nl = 0;
+  CU(launch_sort(P<uint32_t>(c->d_keys1), P<uint32_t>(c->d_vals1), P<uint32_t>(c->d_keys2), P<uint32_t>(c->d_vals0),
+                 words + kSlabCount, c->cap_slots, 0, 32, false, sort_scratch(c, 1 + 2 * slab, true, words + kSlabDepthTiles),
+                 frame + kTimeout, c->epoch, sm, c->stream, &unused, &nl, words + kSlabBits));
+  next_epoch(c);
+  stage_event(c, 2 + 6 * slab + 1);
+  CU(launch_expand(P<uint32_t>(c->d_vals1), P<uint32_t>(c->d_vals0), P<uint2>(c->d_rect), c->cap_slots, c->cap_pairs,
+                   k.tiles_x, P<uint2>(c->d_list), inst_views, uint32_t(tiles_view), live, filter,
+                   P<uint32_t>(c->d_keys1), P<uint32_t>(c->d_keys2), P<uint32_t>(c->d_pk0), P<uint32_t>(c->d_pv0), frame,
+                   slab, P<uint64_t>(c->d_status), next_epoch(c), sm, c->stream));
+  stage_event(c, 2 + 6 * slab + 2);
+  int tile_bits = 1;
+  while ((1 << tile_bits) < n_tiles) ++tile_bits;
+  CU(launch_sort(P<uint32_t>(c->d_pk0), P<uint32_t>(c->d_pv0), P<uint32_t>(c->d_pk1), P<uint32_t>(c->d_pv1),
+                 words + kSlabPairs, c->cap_pairs, 0, tile_bits, false,
+                 sort_scratch(c, 2 + 2 * slab, true, words + kSlabPairTiles), frame + kTimeout, c->epoch, sm, c->stream,
+                 &c->tiles_in1, &nl));
+  next_epoch(c);
+  stage_event(c, 2 + 6 * slab + 3);
+  CU(launch_ranges(P<uint32_t>(c->tiles_in1 ? c->d_pk1 : c->d_pk0), c->cap_pairs, frame, slab,
+                   P<uint2>(c->d_ranges) + size_t(slab) * size_t(n_tiles), n_tiles, sm, c->stream));
+  c->ctx->launches += uint64_t(nl) + 4;
+  return V3DG_OK;
+}
 
 v3dg_status enqueue_render(Pipe* c, float* rgb, float* t_out) {
   const CamConst& k = c->cc;
   uint32_t* frame = P<uint32_t>(c->d_frame);
   const int sm = c->ctx->sm_count;
-  stage_event(c, kStageProject);
-  k_render_reset<<<1, kFrameWords, 0, c->stream>>>(frame, c->cap_nodes);
-  CU(cudaGetLastError());
+  const int slabs = slab_count(c);
+  const int n_tiles = k.tiles_x * k.tiles_y * int(c->n_views);   // (view, tile) ids
+  ST(ensure_image_work(c));
+  const TileLive live = tile_live(c, slabs);
+  uint32_t* depth_hist = slabs > 1 ? P<uint32_t>(c->d_hist) + kDepthHist : nullptr;
+  stage_event(c, 1);
+  CU(launch_frame_init(frame, P<uint32_t>(c->d_hist), kSortHist + uint32_t(1 + 2 * slabs) * kSortPasses * kSortBins,
+                       depth_hist,
+                       P<uint2>(c->d_ranges), uint32_t(n_tiles) * uint32_t(slabs), live, uint32_t(n_tiles), int(c->n_views),
+                       sm, c->stream));
   // projection order: grouped by cluster (the render list's global cluster ids, sorted on at most
   // 24 bits, keeping the high ones) when several instances draw the same assets.  The keys and
   // the order use d_keys1 (4 x cap_nodes words of its 4 x 64 x cap_nodes), which the depth sort
@@ -527,8 +633,8 @@ v3dg_status enqueue_render(Pipe* c, float* rgb, float* t_out) {
     bool oin1 = false;
     int nl = 0;
     CU(launch_sort(okeys, okeys + cn, okeys + 2 * cn, okeys + 3 * cn, frame + kRenderNodes, c->cap_nodes, 0,
-                   key_bits - key_shift, true, sort_scratch(c, frame + kTileCounters + 11), frame + kTimeout, c->epoch,
-                   sm, c->stream, &oin1, &nl));
+                   key_bits - key_shift, true, sort_scratch(c, 0, true, frame + kTileCounters + 11), frame + kTimeout,
+                   c->epoch, sm, c->stream, &oin1, &nl));
     next_epoch(c);
     c->ctx->launches += nl;
     order = oin1 ? okeys + 3 * cn : okeys + cn;
@@ -536,61 +642,57 @@ v3dg_status enqueue_render(Pipe* c, float* rgb, float* t_out) {
   }
   CU(launch_project(P<uint2>(c->d_list), c->cap_nodes, P<InstFrame>(c->d_inst), P<AssetDev>(c->ctx->d_assets), k,
                     P<float4>(c->d_ref), P<float4>(c->d_rec), P<uint2>(c->d_rect), P<uint32_t>(c->d_keys0), frame,
-                    order, sorted_keys, c->color_formats, sm, c->stream));
-  c->ctx->launches += 1;
-
-  stage_event(c, kStageDepthSort);
-  bool in1 = false;
-  int nl = 0;
-  CU(launch_sort(P<uint32_t>(c->d_keys0), P<uint32_t>(c->d_vals0), P<uint32_t>(c->d_keys1), P<uint32_t>(c->d_vals1),
-                 frame + kSlotCount, c->cap_slots, 0, 32, true, sort_scratch(c, frame + kTileCounters + 2),
-                 frame + kTimeout, c->epoch, sm, c->stream, &in1, &nl));
-  next_epoch(c);
-  c->ctx->launches += nl;
-  c->depth_in1 = in1;
-  const uint32_t* dslots = in1 ? P<uint32_t>(c->d_vals1) : P<uint32_t>(c->d_vals0);
-
-  stage_event(c, kStageBin);
-  const int tiles_view = k.tiles_x * k.tiles_y;
-  CU(launch_expand(dslots, P<uint2>(c->d_rect), c->cap_slots, c->cap_pairs, k.tiles_x, P<uint2>(c->d_list),
-                   c->n_views > 1 ? P<InstFrame>(c->d_inst) : nullptr, uint32_t(tiles_view), P<uint32_t>(c->d_pk0),
-                   P<uint32_t>(c->d_pv0), frame, 1, P<uint64_t>(c->d_status), next_epoch(c), sm, c->stream));
+                    order, sorted_keys, c->color_formats, depth_hist, slabs > 1 ? P<float2>(c->d_marks) : nullptr, sm,
+                    c->stream));
+  CU(launch_slab_limits(frame, depth_hist, slabs, c->cap_pairs, c->stream));
   c->ctx->launches += 2;
 
-  stage_event(c, kStageTileSort);
-  const int n_tiles = tiles_view * int(c->n_views);   // (view, tile) ids
-  int tile_bits = 1;
-  while ((1 << tile_bits) < n_tiles) ++tile_bits;
-  bool tin1 = false;
-  nl = 0;
-  CU(launch_sort(P<uint32_t>(c->d_pk0), P<uint32_t>(c->d_pv0), P<uint32_t>(c->d_pk1), P<uint32_t>(c->d_pv1),
-                 frame + kPairsEff, c->cap_pairs, 0, tile_bits, false, sort_scratch(c, frame + kTileCounters + 6),
-                 frame + kTimeout, c->epoch, sm, c->stream, &tin1, &nl));
-  next_epoch(c);
-  c->ctx->launches += nl;
-  c->tiles_in1 = tin1;
-  const uint32_t* tk = tin1 ? P<uint32_t>(c->d_pk1) : P<uint32_t>(c->d_pk0);
-  const uint32_t* tv = tin1 ? P<uint32_t>(c->d_pv1) : P<uint32_t>(c->d_pv0);
-
-  stage_event(c, kStageRanges);
-  ST(ensure(c, c->d_ranges, sizeof(uint2) * size_t(n_tiles)));
-  ST(ensure(c, c->d_order, sizeof(uint32_t) * size_t(n_tiles)));
-  CU(launch_ranges(tk, c->cap_pairs, frame, P<uint2>(c->d_ranges), n_tiles, sm, c->stream));
-  c->ctx->launches += 1;
-
-  stage_event(c, kStageBlend);
   // d_misc: [0..7] the standalone sort's words, [8..11] two 64-bit blend work counters
   unsigned long long* work = c->ctx->count_work ? reinterpret_cast<unsigned long long*>(P<uint32_t>(c->d_misc) + 8) : nullptr;
   if (work) CU(cudaMemsetAsync(work, 0, 2 * sizeof(unsigned long long), c->stream));
-  // d_misc[12], [13]: sticky overflow / timeout flags of all frames since the last v3dg_frame_stats
-  CU(launch_blend(P<uint2>(c->d_ranges), P<uint32_t>(c->d_order), frame + kTileCounters + 10, tk, tv, P<float4>(c->d_rec),
-                  c->cap_slots, k, rgb, t_out, work, frame, P<uint32_t>(c->d_misc) + 12, c->ctx->blend_batch, c->ctx->blend_mode, int(c->n_views), sm, c->stream));
-  c->ctx->launches += 2;
+  for (int slab = 0; slab < slabs; ++slab) {
+    ST(enqueue_slab_lists(c, slab, slab > 0, live));
+    stage_event(c, 2 + 6 * slab + 4);
+    const uint32_t* tk = P<uint32_t>(c->tiles_in1 ? c->d_pk1 : c->d_pk0);
+    const uint32_t* tv = P<uint32_t>(c->tiles_in1 ? c->d_pv1 : c->d_pv0);
+    // d_misc[12], [13]: sticky overflow / timeout flags of all frames since the last v3dg_frame_stats
+    CU(launch_blend(P<uint2>(c->d_ranges) + size_t(slab) * size_t(n_tiles), P<uint32_t>(c->d_order),
+                    P<uint32_t>(c->d_hist) + slab * kItemClasses, tk, tv, P<float4>(c->d_rec), c->cap_slots, k, rgb, t_out,
+                    work, frame, P<uint32_t>(c->d_misc) + 12, slab, live, c->ctx->blend_batch, c->ctx->blend_mode, int(c->n_views), sm, c->stream));
+    c->ctx->launches += 2;
+    stage_event(c, 2 + 6 * slab + 5);
+  }
   if (work)
     CU(cudaMemcpyAsync(c->h_tmp + kFrameWords, work, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, c->stream));
-  stage_event(c, kStages);
   CU(cudaMemcpyAsync(c->h_frame, c->d_frame.p, sizeof(uint32_t) * kFrameWords, cudaMemcpyDeviceToHost, c->stream));
+  c->slabs = slabs;
+  c->full_lists = slabs == 1;
   c->rendered = true;
+  return V3DG_OK;
+}
+
+// The whole frame's sorted Gaussians, pairs and tile ranges (the parity read-backs and the blend
+// autotuner read them): a frame rendered in several slabs has only the last one's, so its lists are
+// made again in one slab without the filter, from the keys, boxes and records that are still there.
+v3dg_status ensure_full_lists(Pipe* c) {
+  if (c->full_lists) return V3DG_OK;
+  const int n_tiles = c->cc.tiles_x * c->cc.tiles_y * int(c->n_views);
+  uint32_t* frame = P<uint32_t>(c->d_frame);
+  CU(cudaMemsetAsync(frame + kSlabBase, 0, sizeof(uint32_t) * kSlabWords, c->stream));
+  CU(cudaMemsetAsync(P<uint32_t>(c->d_hist) + kSortHist + kSortPasses * kSortBins, 0,
+                     sizeof(uint32_t) * 2 * kSortPasses * kSortBins, c->stream));
+  CU(cudaMemsetAsync(c->d_ranges.p, 0, sizeof(uint2) * size_t(n_tiles), c->stream));
+  CU(launch_slab_limits(frame, nullptr, 1, c->cap_pairs, c->stream));
+  ++c->ctx->launches;
+  const bool timing = c->ctx->stage_timing;   // (the frame's own stage events stay)
+  c->ctx->stage_timing = false;
+  const v3dg_status st = enqueue_slab_lists(c, 0, false, tile_live(c, 1));
+  c->ctx->stage_timing = timing;
+  ST(st);
+  CU(cudaMemcpyAsync(c->h_frame, c->d_frame.p, sizeof(uint32_t) * kFrameWords, cudaMemcpyDeviceToHost, c->stream));
+  CU(cudaStreamSynchronize(c->stream));
+  if (c->h_frame[kTimeout]) return fail(c, V3DG_ETIMEOUT, "a bounded device-side wait gave up");
+  c->full_lists = true;
   return V3DG_OK;
 }
 
@@ -600,6 +702,7 @@ v3dg_status enqueue_render(Pipe* c, float* rgb, float* t_out) {
 v3dg_status grow_and_reselect(Pipe* c) {
   const uint32_t* f = c->h_frame;
   bool grew = false;
+  c->pairs_hint = f[kPairs];
   if (f[kRenderNodes] > c->cap_nodes) {
     if (f[kRenderNodes] > kMaxNodes)
       return fail(c, V3DG_EOVERFLOW, "render list of %u nodes exceeds the limit", f[kRenderNodes]);
@@ -642,14 +745,16 @@ std::vector<uint64_t> graph_key(Pipe* c, float* rgb, float* t_out) {
   const v3dg_ctx* ctx = c->ctx;
   std::vector<uint64_t> k = {c->n_inst_frame, c->n_views, uint64_t(c->node_blocks), c->cap_nodes, c->cap_pairs,
                              c->cap_slots, c->status_words, uint64_t(uintptr_t(rgb)), uint64_t(uintptr_t(t_out)),
-                             uint64_t(use_topdown(c)), uint64_t(use_project_order(c)), uint64_t(ctx->blend_batch),
+                             uint64_t(use_topdown(c)), uint64_t(use_project_order(c)), uint64_t(slab_count(c)),
+                             uint64_t(ctx->blend_batch),
                              uint64_t(ctx->blend_mode),
                              uint64_t(ctx->count_work), uint64_t(c->color_formats), ctx->assets.size(),
                              uint64_t(uintptr_t(ctx->d_assets.p))};
   const DevBuf* bufs[] = {&c->d_inst, &c->d_frame, &c->d_misc, &c->d_list, &c->d_ref, &c->d_keys0, &c->d_keys1,
                           &c->d_vals0, &c->d_vals1, &c->d_rec, &c->d_rect, &c->d_pk0, &c->d_pk1, &c->d_pv0,
                           &c->d_pv1, &c->d_ranges, &c->d_status, &c->d_hist, &c->d_order, &c->d_front0,
-                          &c->d_front1, &c->d_tdcount, &c->d_bitmap};
+                          &c->d_front1, &c->d_tdcount, &c->d_bitmap, &c->d_keys2, &c->d_tlive, &c->d_state,
+                          &c->d_marks};
   for (const DevBuf* b : bufs) k.push_back(uint64_t(uintptr_t(b->p)));
   uint64_t w[sizeof(CamConst) / 8 + 1] = {};
   std::memcpy(w, &c->cc, sizeof(CamConst));
@@ -662,9 +767,7 @@ std::vector<uint64_t> graph_key(Pipe* c, float* rgb, float* t_out) {
 // itself, because a replay reuses the epochs that were baked in at capture.
 v3dg_status run_graph_frame(Pipe* c, float* rgb, float* t_out, bool sync) {
   ST(ensure_work(c));
-  const int n_tiles = c->cc.tiles_x * c->cc.tiles_y * int(c->n_views);
-  ST(ensure(c, c->d_ranges, sizeof(uint2) * size_t(n_tiles)));
-  ST(ensure(c, c->d_order, sizeof(uint32_t) * size_t(n_tiles)));
+  ST(ensure_image_work(c));
   if (use_topdown(c)) {
     TopDown td{};
     ST(topdown_buffers(c, &td));
@@ -701,6 +804,8 @@ v3dg_status run_graph_frame(Pipe* c, float* rgb, float* t_out, bool sync) {
   }
   CU(cudaGraphLaunch(c->gexec, c->stream));
   c->ctx->launches += c->glaunches;
+  c->slabs = slab_count(c);
+  c->full_lists = c->slabs == 1;
   c->rendered = true;
   if (!sync) return V3DG_OK;
   CU(cudaStreamSynchronize(c->stream));
@@ -738,6 +843,12 @@ v3dg_status sync_frame(Pipe* c) {
   CU(cudaStreamSynchronize(c->stream));
   if (!c->rendered) CU(cudaMemcpy(c->h_frame, c->d_frame.p, sizeof(uint32_t) * kFrameWords, cudaMemcpyDeviceToHost));
   return V3DG_OK;
+}
+
+// The slots of the whole frame's visible Gaussians in depth order (ensure_full_lists).
+const uint32_t* sorted_slots(Pipe* c) {
+  const bool in1 = ((c->h_frame[kSlabBase + kSlabBits] + 7u) / 8u) & 1u;
+  return P<uint32_t>(in1 ? c->d_vals0 : c->d_vals1);
 }
 
 // The cut itself (mode 1), into d_cut; returns its size.
@@ -821,7 +932,8 @@ void pipe_free(Pipe* c) {
                   &c->d_keys1, &c->d_vals0, &c->d_vals1, &c->d_rec, &c->d_rect, &c->d_pk0, &c->d_pk1,
                   &c->d_pv0, &c->d_pv1, &c->d_ranges, &c->d_status, &c->d_hist, &c->d_cut, &c->d_img,
                   &c->d_timg, &c->d_sort_k, &c->d_sort_v, &c->d_order, &c->d_front0, &c->d_front1,
-                  &c->d_tdcount, &c->d_bitmap};
+                  &c->d_tdcount, &c->d_bitmap, &c->d_keys2, &c->d_tlive, &c->d_state,
+                          &c->d_marks};
   for (DevBuf* b : bs) dfree(c, *b);
   if (c->h_inst) cudaFreeHost(c->h_inst);
   if (c->h_frame) cudaFreeHost(c->h_frame);
@@ -837,11 +949,13 @@ void pipe_free(Pipe* c) {
 
 // The frame buffers a pipe holds (they grow with the largest frame it has rendered).
 DevBuf* const* frame_buffers(Pipe* c, size_t* n) {
-  static thread_local DevBuf* bs[24];
+  static thread_local DevBuf* bs[32];
   DevBuf* list[] = {&c->d_list, &c->d_ref, &c->d_keys0, &c->d_keys1, &c->d_vals0, &c->d_vals1, &c->d_rec,
                     &c->d_rect, &c->d_pk0, &c->d_pk1, &c->d_pv0, &c->d_pv1, &c->d_ranges, &c->d_status,
                     &c->d_cut, &c->d_img, &c->d_timg, &c->d_sort_k, &c->d_sort_v, &c->d_order, &c->d_front0,
-                    &c->d_front1, &c->d_bitmap};
+                    &c->d_front1, &c->d_bitmap, &c->d_keys2, &c->d_tlive, &c->d_state,
+                          &c->d_marks};
+  static_assert(sizeof(list) <= sizeof(bs), "room for every buffer");
   *n = sizeof(list) / sizeof(list[0]);
   for (size_t i = 0; i < *n; ++i) bs[i] = list[i];
   return bs;
@@ -1559,19 +1673,20 @@ v3dg_status v3dg_get_projected(v3dg_ctx* ctx, uint64_t cap, uint64_t* n, uint32_
   if (!c || !n) return V3DG_EINVAL;
   if (!c->rendered) return fail(c, V3DG_ENOTFOUND, "no frame rendered");
   ST(sync_frame(c));
+  ST(ensure_full_lists(c));
   const uint32_t nr = std::min(c->h_frame[kRenderNodes], c->cap_nodes);
-  const uint32_t nv = c->h_frame[kVisible];
+  const uint32_t nv = c->h_frame[kSlabBase + kSlabCount];
   const size_t S = size_t(nr) * kSlots;
   std::vector<uint2> list(nr);
-  std::vector<uint32_t> keys(nv), slots(nv);
+  std::vector<uint32_t> keys(S), slots(nv);
   std::vector<float4> rec(3 * S);
   std::vector<uint2> rc(S);
   if (nr) CU(cudaMemcpy(list.data(), c->d_list.p, sizeof(uint2) * nr, cudaMemcpyDeviceToHost));
   if (nv) {
-    CU(cudaMemcpy(keys.data(), (c->depth_in1 ? c->d_keys1 : c->d_keys0).p, 4 * size_t(nv), cudaMemcpyDeviceToHost));
-    CU(cudaMemcpy(slots.data(), (c->depth_in1 ? c->d_vals1 : c->d_vals0).p, 4 * size_t(nv), cudaMemcpyDeviceToHost));
+    CU(cudaMemcpy(slots.data(), sorted_slots(c), 4 * size_t(nv), cudaMemcpyDeviceToHost));
   }
   if (S) {
+    CU(cudaMemcpy(keys.data(), c->d_keys0.p, 4 * S, cudaMemcpyDeviceToHost));
     CU(cudaMemcpy(rec.data(), c->d_rec.p, sizeof(float4) * 3 * S, cudaMemcpyDeviceToHost));
     CU(cudaMemcpy(rc.data(), c->d_rect.p, sizeof(uint2) * S, cudaMemcpyDeviceToHost));
   }
@@ -1607,7 +1722,7 @@ v3dg_status v3dg_get_projected(v3dg_ctx* ctx, uint64_t cap, uint64_t* n, uint32_
       rgb[3 * q + 1] = r1.w;
       rgb[3 * q + 2] = r2.x;
     }
-    if (depth_key) depth_key[q] = keys[k];
+    if (depth_key) depth_key[q] = keys[slot];
     if (rect) {
       rect[4 * q] = int32_t((rr.x & 0xFFFFu) >> 4);   // the pixel box's tiles
       rect[4 * q + 1] = int32_t((rr.x >> 16) >> 4);
@@ -1625,24 +1740,20 @@ v3dg_status v3dg_get_pairs(v3dg_ctx* ctx, uint64_t cap, uint64_t* n, uint32_t* t
   if (!c || !n) return V3DG_EINVAL;
   if (!c->rendered) return fail(c, V3DG_ENOTFOUND, "no frame rendered");
   ST(sync_frame(c));
+  ST(ensure_full_lists(c));
   const uint32_t np = std::min(c->h_frame[kPairsEff], c->cap_pairs);
   const uint32_t nr = std::min(c->h_frame[kRenderNodes], c->cap_nodes);
-  const uint32_t nv = c->h_frame[kVisible];
   *n = np;
   const uint64_t m = std::min<uint64_t>(cap, np);
   if (m == 0) return V3DG_OK;
-  std::vector<uint32_t> tk(m), tv(m), keys(nv), slots(nv);
+  std::vector<uint32_t> tk(m), tv(m), key_of(size_t(nr) * kSlots);
   std::vector<uint2> list(nr);
   CU(cudaMemcpy(tk.data(), (c->tiles_in1 ? c->d_pk1 : c->d_pk0).p, 4 * m, cudaMemcpyDeviceToHost));
   CU(cudaMemcpy(tv.data(), (c->tiles_in1 ? c->d_pv1 : c->d_pv0).p, 4 * m, cudaMemcpyDeviceToHost));
-  if (nv) {
-    CU(cudaMemcpy(keys.data(), (c->depth_in1 ? c->d_keys1 : c->d_keys0).p, 4 * size_t(nv), cudaMemcpyDeviceToHost));
-    CU(cudaMemcpy(slots.data(), (c->depth_in1 ? c->d_vals1 : c->d_vals0).p, 4 * size_t(nv), cudaMemcpyDeviceToHost));
+  if (nr) {
+    CU(cudaMemcpy(list.data(), c->d_list.p, sizeof(uint2) * nr, cudaMemcpyDeviceToHost));
+    CU(cudaMemcpy(key_of.data(), c->d_keys0.p, 4 * key_of.size(), cudaMemcpyDeviceToHost));
   }
-  if (nr) CU(cudaMemcpy(list.data(), c->d_list.p, sizeof(uint2) * nr, cudaMemcpyDeviceToHost));
-  std::vector<uint32_t> key_of(size_t(nr) * kSlots, 0xFFFFFFFFu);
-  for (uint32_t k = 0; k < nv; ++k)
-    if (slots[k] < key_of.size()) key_of[slots[k]] = keys[k];
   for (uint64_t q = 0; q < m; ++q) {
     const uint32_t slot = tv[q];
     if (tile) tile[q] = tk[q] & kPairTileMask;
@@ -1662,6 +1773,7 @@ v3dg_status v3dg_get_tile_ranges(v3dg_ctx* ctx, uint32_t* range, uint64_t cap, u
   if (!c || !n_tiles) return V3DG_EINVAL;
   if (!c->rendered) return fail(c, V3DG_ENOTFOUND, "no frame rendered");
   ST(sync_frame(c));
+  ST(ensure_full_lists(c));
   const uint64_t nt = uint64_t(c->cc.tiles_x) * uint64_t(c->cc.tiles_y) * c->n_views;
   *n_tiles = nt;
   if (range && cap) CU(cudaMemcpy(range, c->d_ranges.p, sizeof(uint2) * std::min(cap, nt), cudaMemcpyDeviceToHost));
@@ -1676,7 +1788,18 @@ v3dg_status v3dg_stage_times(v3dg_ctx* ctx, float* ms, int n, uint64_t* launches
   if (ms && n > 0) {
     if (!ctx->stage_timing || !c->rendered) return fail(c, V3DG_ENOTFOUND, "stage timing is off or no frame rendered");
     CU(cudaStreamSynchronize(c->stream));
-    for (int i = 0; i < n && i < kStages; ++i) CU(cudaEventElapsedTime(ms + i, c->ev[i], c->ev[i + 1]));
+    for (int i = 0; i < n && i < kStages; ++i) {
+      ms[i] = 0.f;
+      if (i < 2) {   // selection, projection
+        CU(cudaEventElapsedTime(ms + i, c->ev[i], c->ev[i + 1]));
+        continue;
+      }
+      for (int slab = 0; slab < c->slabs; ++slab) {   // the other stages, over the frame's slabs
+        float t = 0.f;
+        CU(cudaEventElapsedTime(&t, c->ev[6 * slab + i], c->ev[6 * slab + i + 1]));
+        ms[i] += t;
+      }
+    }
   }
   c->err.clear();
   return V3DG_OK;
@@ -1689,6 +1812,7 @@ v3dg_status v3dg_autotune_blend(v3dg_ctx* ctx, uint32_t* mode_out, uint32_t* bat
   if (!c->rendered) return fail(c, V3DG_ENOTFOUND, "no frame rendered");
   ST(sync_frame(c));
   if (c->h_frame[kOverflow] || c->h_frame[kTimeout]) return fail(c, V3DG_EOVERFLOW, "the last frame was not valid");
+  ST(ensure_full_lists(c));
   const CamConst& k = c->cc;
   const size_t px = size_t(k.width) * size_t(k.height) * c->n_views;
   ST(ensure(c, c->d_img, sizeof(float) * 3 * std::max<size_t>(px, 1)));
@@ -1710,12 +1834,13 @@ v3dg_status v3dg_autotune_blend(v3dg_ctx* ctx, uint32_t* mode_out, uint32_t* bat
       if (mode == 0 && b != 512) continue;   // variant 0 has no batch size (512 is the option's default)
       float t_min = INFINITY;
       for (int rep = 0; rep < 4 && e == cudaSuccess; ++rep) {   // the first run warms up
-        e = cudaMemsetAsync(frame + kTileCounters + 10, 0, sizeof(uint32_t), c->stream);
+        e = cudaMemsetAsync(frame + kSlabBase + kSlabBlendItem, 0, sizeof(uint32_t), c->stream);
+        if (e == cudaSuccess) e = cudaMemsetAsync(c->d_hist.p, 0, sizeof(uint32_t) * kItemClasses, c->stream);
         if (e == cudaSuccess) e = cudaEventRecord(e0, c->stream);
         if (e == cudaSuccess)
-          e = launch_blend(P<uint2>(c->d_ranges), P<uint32_t>(c->d_order), frame + kTileCounters + 10, tk, tv,
-                           P<float4>(c->d_rec), c->cap_slots, k, P<float>(c->d_img), nullptr, nullptr, frame,
-                           P<uint32_t>(c->d_misc) + 12, b, mode, int(c->n_views), ctx->sm_count, c->stream);
+          e = launch_blend(P<uint2>(c->d_ranges), P<uint32_t>(c->d_order), P<uint32_t>(c->d_hist), tk, tv,
+                           P<float4>(c->d_rec), c->cap_slots, k, P<float>(c->d_img), nullptr, nullptr, frame, P<uint32_t>(c->d_misc) + 12, 0, TileLive{}, b,
+                           mode, int(c->n_views), ctx->sm_count, c->stream);
         if (e == cudaSuccess) e = cudaEventRecord(e1, c->stream);
         if (e == cudaSuccess) e = cudaEventSynchronize(e1);
         float ms = 0.f;
@@ -1753,7 +1878,7 @@ v3dg_status v3dg_sort_pairs(v3dg_ctx* ctx, uint32_t* keys, uint32_t* vals, uint6
   ST(ensure(c, c->d_sort_k, 4 * n));
   ST(ensure(c, c->d_sort_v, 4 * n));
   ST(ensure_status(c, ((n + kSortTile - 1) / kSortTile) * 256));
-  ST(ensure(c, c->d_hist, 2 * 4 * 256 * 4));  // counts + exclusive offsets of up to 4 passes
+  ST(ensure(c, c->d_hist, sizeof(uint32_t) * kHistWords));
   uint32_t* misc = P<uint32_t>(c->d_misc);  // [0] n, [1..4] tile counters, [5] timeout flag
   CU(cudaMemsetAsync(misc, 0, sizeof(uint32_t) * 8, c->stream));
   k_set_word<<<1, 1, 0, c->stream>>>(misc, uint32_t(n));
@@ -1761,7 +1886,7 @@ v3dg_status v3dg_sort_pairs(v3dg_ctx* ctx, uint32_t* keys, uint32_t* vals, uint6
   bool in1 = false;
   int nl = 0;
   CU(launch_sort(keys, vals, P<uint32_t>(c->d_sort_k), P<uint32_t>(c->d_sort_v), misc, uint32_t(n), begin_bit, end_bit,
-                 false, sort_scratch(c, misc + 1), misc + 5, c->epoch, ctx->sm_count, c->stream, &in1, &nl));
+                 false, sort_scratch(c, 0, false, misc + 1), misc + 5, c->epoch, ctx->sm_count, c->stream, &in1, &nl));
   next_epoch(c);
   ctx->launches += nl + 1;
   if (in1) {

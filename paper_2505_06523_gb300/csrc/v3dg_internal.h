@@ -75,15 +75,51 @@ struct CamConst {
 // Frame counters (device, uint32 each).
 enum Counter : int {
   kCutNodes = 0, kCutGauss, kRenderNodes, kVisible, kPairs, kOverflow, kTimeout,
-  kSlotCount = 7,          // render nodes (clamped) * 64: the slots the depth sort covers
-  kPairsEff = 8,           // pairs the tile sort / blend use: kPairs, or 0 when the frame overflowed
+  kPairsEff = 8,           // pairs of the frame, or 0 when it overflowed
   kTdReached = 9,          // top-down selection: (instance, node) entries it tested
   kConicFp64 = 10,         // Gaussians whose 2D covariance had det < 1e-12 and was inverted in FP64
   kRenderClusters = 11,    // distinct clusters of the render list (projection grouped by cluster)
   kPairs64 = 12,           // [12, 14): the pair total as a 64-bit sum (detects totals beyond 2^32)
-  kNumCounters = 16,
-  kTileCounters = 16,      // [16, 48): atomic tile counters of the chained-scan kernels
-  kFrameWords = 48,
+  kKeyMinInv = 14,         // ~(smallest depth key of a visible Gaussian)
+  kKeyMax = 15,            // largest depth key of a visible Gaussian
+  kTileCounters = 16,      // [16, 32): atomic tile counters: [16] selection, [27, 31) cluster order, [31] projection
+  kSlabBase = 32,          // kSlabWords words for each depth slab
+};
+
+// A frame is binned, sorted and blended in one or more depth slabs, front to back: slab k holds the
+// visible Gaussians with depth keys in [lo, hi).  From the second slab on, Gaussians and pairs that
+// only meet tiles whose pixels have all stopped are left out (they cannot change a pixel).
+constexpr int kMaxSlabs = 4, kSlabWords = 24, kFrameWords = kSlabBase + kMaxSlabs * kSlabWords;
+enum SlabWord : int {
+  kSlabCount = 0,          // Gaussians picked
+  kSlabPairs,              // their pairs
+  kSlabPickTile,           // tile counters of the kernels
+  kSlabDepthTiles,         // 4 words
+  kSlabExpandTile = kSlabDepthTiles + 4,
+  kSlabPairTiles,          // 4 words
+  kSlabBlendItem = kSlabPairTiles + 4,
+  kSlabLo, kSlabHi,        // depth keys [lo, hi)
+  kSlabBits,               // key bits of the slab's depth sort: keys are stored as key - lo
+  kSlabLarge,              // Gaussians left to the large-box expansion
+};
+static_assert(kSlabLarge < kSlabWords, "slab words");
+constexpr int kItemClasses = 16;   // classes of the blend's work items
+
+// Depth histogram of the pairs (weights: tiles covered), for the slabs' limits: 16 bins per octave
+// of the float32 depth from 2^-7 up (the first and last bin take what lies beyond).
+constexpr int kDepthBins = 2048, kDepthShift = 19, kDepthBase = 1920;
+
+// Which tiles still have an unfinished pixel (several slabs): one bit per tile, rows of `words`
+// 32-bit words (one of them spare, zero), row view * tiles_y + ty; and per tile a bit for each of its
+// 4x4 pixel blocks (4 row + column) that has one.  NULL bits: a frame of one slab.
+struct TileLive {
+  uint32_t* bits;
+  uint32_t* blocks;
+  uint32_t* coarse;        // the same bits of groups of 8x8 tiles, and per group its live tiles
+  uint32_t* coarse_tiles;
+  float* state;            // per pixel: T, negative once the pixel has stopped
+  uint32_t words, coarse_words;
+  uint32_t tiles_x, tiles_y, groups_x, groups_y;
 };
 
 // Status words of the chained (decoupled look-back) scans: epoch << 34 | flag << 32 | value.
@@ -147,17 +183,45 @@ cudaError_t launch_noderef(const uint2* render_list, uint32_t cap_nodes, const I
 // cluster, the instances that draw one cluster read its attributes one after the other, and all
 // but the first find them in L2.  sorted_keys (may be NULL): the global cluster id of each
 // position of `order`; the distinct ones are counted into frame[kRenderClusters].
+// Also adds up frame[kVisible], the pairs (tiles covered) into frame[kPairs64], the smallest and
+// largest key, and -- unless depth_hist is NULL -- the depth histogram of the pairs and a conservative
+// depth range of every render-list node.
 cudaError_t launch_project(const uint2* render_list, uint32_t cap_nodes, const InstFrame* inst,
                            const AssetDev* assets, const CamConst& cam, const float4* ref, float4* rec,
                            uint2* rect, uint32_t* keys, uint32_t* frame, const uint32_t* order,
-                           const uint32_t* sorted_keys, int color_formats, int sm_count, cudaStream_t st);
+                           const uint32_t* sorted_keys, int color_formats, uint32_t* depth_hist,
+                           float2* depth_range, int sm_count, cudaStream_t st);
+
+// Start of a render: the render's counters (the selection's words stay, so that a render list
+// overflow still invalidates the frame), the sorts' digit counts, the depth histogram, the tile
+// ranges of every slab and the tiles' liveness.
+cudaError_t launch_frame_init(uint32_t* frame, uint32_t* hist, uint32_t hist_words, uint32_t* depth_hist, uint2* ranges,
+                              uint32_t n_ranges, const TileLive& live, uint32_t n_tiles, int n_views, int sm_count,
+                              cudaStream_t st);
+// After the projection: the frame's pair count and overflow, and the limits of its `slabs` slabs.
+cudaError_t launch_slab_limits(uint32_t* frame, const uint32_t* depth_hist, int slabs, uint32_t cap_pairs,
+                               cudaStream_t st);
+// A one-slab frame's visible Gaussians, in slot order: (key - lo, slot).
+cudaError_t launch_pick(const uint32_t* keys, uint32_t cap_nodes, uint32_t* kout, uint32_t* vout, uint32_t* frame,
+                        int slab, uint64_t* status, uint32_t epoch, int sm_count, cudaStream_t st);
+// The same of one of several slabs: keys in [lo, hi) and, with filter, boxes that meet a live tile.
+// depth_range: a conservative depth range per render-list node.  marks, counts: scratch of cap_nodes
+// and ceil(cap_nodes / 256) entries.
+cudaError_t launch_pick_slab(const uint32_t* keys, const uint2* rect, uint32_t cap_nodes, const uint2* list,
+                             const InstFrame* inst_views, const TileLive& live, bool filter, const float2* depth_range,
+                             uint2* marks, uint32_t* counts, uint32_t* kout, uint32_t* vout, uint32_t* frame, int slab,
+                             int sm_count, cudaStream_t st);
 
 // Radix sort of (key, value) pairs, n read from *n_dev (clamped to cap).  Ping-pongs between
 // (k0, v0) and (k1, v1); the result lands in (k0, v0) when the pass count is even, else in
 // (k1, v1) -- *result_in_1 tells which.  implicit_vals: the values of the first pass are the
-// element indices (v0 is not read).
+// element indices (v0 is not read).  bits_dev (may be NULL): the sort covers key bits
+// [0, *bits_dev) instead, in as few passes as 8-bit digits need (the launches beyond return at
+// once); the result is in (k1, v1) when that number is odd.
+constexpr int kSortPasses = 4, kSortBins = 256;
 struct SortScratch {
-  uint32_t* hist;          // 4 passes * 256 counts, then 4 passes * 256 exclusive offsets
+  uint32_t* hist;          // kSortPasses * kSortBins digit counts
+  bool hist_zeroed;        // already zero (else launch_sort clears them)
   uint64_t* status;        // max_tiles * 256
   uint32_t max_tiles;
   uint32_t* tile_counters; // one per pass (zeroed by the caller's frame memset)
@@ -166,7 +230,7 @@ constexpr int kSortThreads = 256, kSortItems = 16, kSortTile = kSortThreads * kS
 cudaError_t launch_sort(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1, const uint32_t* n_dev,
                         uint32_t cap, int begin_bit, int end_bit, bool implicit_vals,
                         const SortScratch& sc, uint32_t* err_flag, uint32_t& epoch, int sm_count,
-                        cudaStream_t st, bool* result_in_1, int* launches);
+                        cudaStream_t st, bool* result_in_1, int* launches, const uint32_t* bits_dev = nullptr);
 
 // Pair keys: tile id in bits 0..19 (at most 2^20 tiles), then the Gaussian's pixel box clipped
 // to the tile, tile-local and inclusive: rows y0 in bits 20..23 and y1 in 24..27, columns rounded
@@ -180,28 +244,36 @@ cudaError_t sort_set_attributes();
 cudaError_t blend_set_attributes();
 cudaError_t project_set_attributes();
 
-// Expansion of the depth-sorted visible Gaussians into (tile, slot) pairs in depth order; writes
-// frame[kPairs] (the total) and frame[kPairsEff] (0 if the frame overflowed).  rect: per slot,
-// the pixel box (x0 | x1 << 16, y0 | y1 << 16) of the alpha >= 1/255 ellipse, inclusive.
+// Expansion of a slab's depth-sorted Gaussians into (tile, slot) pairs in depth order (filter: only of
+// tiles that are still live); writes the slab's pair count.  slots0 / slots1: the two places where
+// the depth sort may have left the slots (see launch_sort, bits_dev).  rect: per slot, the pixel box
+// (x0 | x1 << 16, y0 | y1 << 16) of the alpha >= 1/255 ellipse, inclusive.
 // Several views: the tile id of a pair is view * tiles_per_view + tile, with the view of the
 // Gaussian's instance frame (inst_views[list[slot / 64].x].view; inst_views NULL: one view).
-cudaError_t launch_expand(const uint32_t* sorted_slots, const uint2* rect, uint32_t cap_slots, uint32_t cap_pairs,
-                          int tiles_x, const uint2* list, const InstFrame* inst_views, uint32_t tiles_per_view,
-                          uint32_t* pair_keys, uint32_t* pair_vals, uint32_t* frame, uint32_t tile_counter_slot,
+// large_slot, large_pos: cap_slots words each, scratch (the Gaussians with large boxes).
+cudaError_t launch_expand(const uint32_t* slots0, const uint32_t* slots1, const uint2* rect, uint32_t cap_slots,
+                          uint32_t cap_pairs, int tiles_x, const uint2* list, const InstFrame* inst_views,
+                          uint32_t tiles_per_view, const TileLive& live, bool filter, uint32_t* large_slot,
+                          uint32_t* large_pos, uint32_t* pair_keys, uint32_t* pair_vals, uint32_t* frame, int slab,
                           uint64_t* status, uint32_t epoch, int sm_count, cudaStream_t st);
-cudaError_t launch_ranges(const uint32_t* tile_keys, uint32_t cap_pairs, const uint32_t* frame,
+// ranges: n_tiles zeroed entries.
+cudaError_t launch_ranges(const uint32_t* tile_keys, uint32_t cap_pairs, const uint32_t* frame, int slab,
                           uint2* ranges, int n_tiles, int sm_count, cudaStream_t st);
 // work != nullptr: also count (evaluations, contributions) into work[0], work[1].
 // sticky[0] |= frame[kOverflow], sticky[1] |= frame[kTimeout] (the flags of every frame since the
 // host last cleared them).
-// items: n_tiles words of scratch (the tiles, longest lists first); tile_counter: a zeroed word.
+// items, class_count: kItemClasses * n_tiles words of scratch and kItemClasses zeroed words (the tiles
+// by the length of their lists); the slab's word kSlabBlendItem is zero.  live.bits != NULL: one of
+// several slabs, first to last from 0 -- the pixels' state is kept in live.state and the image
+// between them (mode 0 only).
 // batch: records that variant 1 stages per batch, 128, 256 or 512.  n_views
 // images of cam's size, one after the other in rgb (and t_out); tile ids are (view, tile).
 // tk, pair_vals: the sorted pair keys (tile id and in-tile box, see kPairTileMask) and values.
 // mode 0: every warp composites 8x4 pixels on its own; mode 1: batches staged by bulk copies and
 // composited by warps over row pairs.  The image is the same bit for bit.
-cudaError_t launch_blend(const uint2* ranges, uint32_t* items, uint32_t* tile_counter, const uint32_t* tk,
+cudaError_t launch_blend(const uint2* ranges, uint32_t* items, uint32_t* class_count, const uint32_t* tk,
                          const uint32_t* pair_vals, const float4* rec, uint32_t cap_slots, const CamConst& cam, float* rgb, float* t_out,
-                         unsigned long long* work, uint32_t* frame, uint32_t* sticky, int batch, int mode, int n_views, int sm_count, cudaStream_t st);
+                         unsigned long long* work, uint32_t* frame, uint32_t* sticky, int slab, const TileLive& live,
+                         int batch, int mode, int n_views, int sm_count, cudaStream_t st);
 
 }  // namespace v3dg

@@ -36,7 +36,7 @@ constexpr size_t kOffKeys = 0;
 constexpr size_t kOffVals = kOffKeys + 4 * kMaxPairs;
 constexpr size_t kOffStatus = kOffVals + 4 * kMaxPairs;
 constexpr size_t kOffHist = kOffStatus + 8 * size_t(kTiles) * 256;
-constexpr size_t kOffMisc = kOffHist + 2 * 4 * 256 * 4;   // [0] n, [1..4] tile counters, [5] timeout flag
+constexpr size_t kOffMisc = kOffHist + 4 * size_t(kSortPasses) * kSortBins;   // [0] n, [1..4] tile counters, [5] timeout flag
 constexpr size_t kBytes = kOffMisc + 256;
 constexpr int kMaxDevices = 64;
 
@@ -79,6 +79,7 @@ extern "C" v3dg_status v3dg_sort_pairs_noalloc(uint32_t* keys, uint32_t* vals, u
   k_store_n<<<1, 1, 0, st>>>(misc, uint32_t(n));
   SortScratch sc;
   sc.hist = reinterpret_cast<uint32_t*>(b + kOffHist);
+  sc.hist_zeroed = false;
   sc.status = reinterpret_cast<uint64_t*>(b + kOffStatus);
   sc.max_tiles = kTiles;
   sc.tile_counters = misc + 1;

@@ -1,0 +1,78 @@
+"""Frames taken in depth slabs (at least 2^24 pairs) against the same frames taken in one."""
+import dataclasses
+
+import numpy as np
+import pytest
+
+from synth import scenes
+
+pytestmark = pytest.mark.gpu
+
+
+def _scene(n, spread):
+    """n copies of asset 0, turned and scaled differently, around the origin."""
+    rng = np.random.Generator(np.random.PCG64(n))
+    return scenes.Instances(np.zeros(n, np.uint32), scenes.random_rotations(rng, n), rng.uniform(-spread, spread, (n, 3)),
+                            rng.uniform(0.7, 1.4, n))
+
+
+@pytest.mark.parametrize("n,spread,width,height,views,graphs", [
+    (12, 0.5, 1920, 1080, 1, 0),    # a pile next to the camera: large boxes, early stops
+    (40, 6.0, 1001, 563, 3, 0),     # ragged images, several views
+    (40, 6.0, 1001, 563, 3, 1),     # the same, captured
+])
+def test_slabs_change_nothing(tiny_asset, n, spread, width, height, views, graphs):
+    """Blend variant 1 keeps its frames in one slab and gives the same image bit for bit; the sorted lists that the
+    read-backs return are those of the whole frame either way."""
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2505_06523_gb300 import Context
+    from paper_2505_06523_gb300._native import V3DG_OPT_BLEND_MODE, V3DG_OPT_GRAPHS
+    inst = _scene(n, spread)
+    cams = [scenes.look_at((0.3 * v, -2.0 - spread, 0.5), (0.0, 0.0, 0.0), width, height, 70.0) for v in range(views)]
+    got = []
+    with Context(0) as ctx:
+        ctx.set_option(V3DG_OPT_GRAPHS, graphs)
+        ctx.load_hierarchy(tiny_asset)
+        ctx.set_instances(inst)
+        for mode in (1, 0):
+            ctx.set_option(V3DG_OPT_BLEND_MODE, mode)
+            for _ in range(2):   # (the second frame knows the first one's size)
+                ctx.select_views(cams, 0.25)
+                rgb, T = ctx.render(want_T=True)
+            got.append({"rgb": rgb.cpu().numpy(), "T": T.cpu().numpy(),
+                        **{"proj_" + k: v for k, v in ctx.get_projected().items()}, "ranges": ctx.tile_ranges(),
+                        **{"pair_" + k: v for k, v in ctx.get_pairs().items()}, "stats": ctx.frame_stats()})
+            again = ctx.render(want_T=True)   # the lists were made again in between
+            assert (again[0].cpu().numpy() == got[-1]["rgb"]).all()
+    one, slabs = got
+    assert one["stats"]["pairs"] >= 1 << 24, "too few pairs for slabs"
+    assert one["stats"] == {**slabs["stats"]}
+    assert float(np.abs(one["rgb"]).sum()) > 0 and (one["T"] < 1e-3).any()
+    for k in one:
+        if k != "stats":
+            assert one[k].shape == slabs[k].shape and (one[k] == slabs[k]).all(), k
+
+
+def test_slabs_with_depths_in_one_bin(tiny_asset):
+    """Every Gaussian in a narrow depth range (fewer histogram bins than slabs): the empty slabs change nothing."""
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2505_06523_gb300 import Context
+    from paper_2505_06523_gb300._native import V3DG_OPT_BLEND_MODE
+    flat = dataclasses.replace(tiny_asset, means=(tiny_asset.means * np.array([1.0, 1e-3, 1.0], np.float32)))
+    n = 24
+    inst = scenes.Instances(np.zeros(n, np.uint32), np.repeat(np.eye(3)[None], n, 0), np.zeros((n, 3)), np.ones(n))
+    cam = scenes.look_at((0.0, -1.31, 0.0), (0.0, 0.0, 0.0), 1600, 900, 80.0)
+    imgs = []
+    with Context(0) as ctx:
+        ctx.load_hierarchy(flat)
+        ctx.set_instances(inst)
+        for mode in (1, 0):
+            ctx.set_option(V3DG_OPT_BLEND_MODE, mode)
+            for _ in range(2):
+                ctx.select(cam, 0.25)
+                rgb, T = ctx.render(want_T=True)
+            imgs.append((rgb.cpu().numpy(), T.cpu().numpy()))
+        assert ctx.frame_stats()["pairs"] >= 1 << 24
+    assert (imgs[0][0] == imgs[1][0]).all() and (imgs[0][1] == imgs[1][1]).all()
