@@ -1,20 +1,26 @@
 // Projection of the selected Gaussians (Sec. 2.1; Sec. 5.1: EWA splatting without 2D dilation).
 //
-// k_noderef: one thread per render-list node computes, in FP64, the view-space position of the
-//   node's mean centre and its pixel position, so that every Gaussian of the node can be placed
-//   relative to it with small float32 offsets (the screen mean stays accurate to ~1e-7 of the
-//   node's extent instead of 1 ulp of the whole view distance).
-// k_project: a warp takes a chunk of consecutive render-list entries at a time (16 in list
-//   order; 32 when, for scenes of many instances of few assets, the entries come grouped by
-//   cluster through a radix sort of their global cluster ids), stages the chunk's per-entry
-//   constants (instance matrix, camera centre, FP64 reference) in shared memory, and projects
+// k_order_keys: the render list's global cluster ids, whose radix sort groups the list by cluster.
+// k_project: a warp takes a chunk of consecutive render-list entries at a time (up to 16 in list
+//   order; up to 32 when, for scenes of many instances of few assets, the entries come grouped by
+//   cluster), stages the chunk's per-entry constants (instance matrix, camera centre, and an FP64
+//   reference: the view-space position of the entry's mean centre and its pixel position, from which
+//   every Gaussian is placed by small float32 offsets, so that the screen mean stays accurate to
+//   ~1e-7 of the node's extent instead of 1 ulp of the view distance) in shared memory, one entry
+//   per lane, and projects
 //   each run of entries that draw the same cluster together, 2 Gaussians per lane: a Gaussian's
 //   attributes -- mean, opacity, normalised quaternion, scales and all SH coefficients -- are
 //   loaded into registers once per run and used for every entry of it, so a cluster drawn by k
 //   instances is read once, not k times.  Loads are attribute-major (each cluster's attributes
 //   are one contiguous block of planes of 64 values, so every warp load is one 128-byte line).
 //   Writes a 48-byte blend record, the pixel box and the float32 depth key per Gaussian;
-//   culled slots get the key 0xFFFFFFFF so that the depth sort moves them behind all visible ones.
+//   culled slots get the key 0xFFFFFFFF, which no slab picks.
+//   The FP64 references were a kernel of their own (FP64 issue: 118 us of a 1080p crowd frame, 7 us of
+//   a thumbnail); here the other warps' float32 work hides them.  Projection stage on a GB300 with the
+//   references and small chunks, before -> now: 96x80 thumbnail 67 -> 26 us, 300k-leaf asset at
+//   1001x563 116 -> 42 us, 200 instances at 640x360 159 -> 118 us, crowd at 1080p 1.66 -> 1.61 ms,
+//   5000 instances at 4K 11.1 -> 10.5 ms.  It stays bound by registers (128: a Gaussian's 59
+//   attributes; 16 warps per SM) and by its 60 bytes written per Gaussian.
 #include <algorithm>
 
 #include <cuda_fp16.h>
@@ -42,35 +48,36 @@ constexpr float kY3d = 0.3731763325901154f;   // 1/4 sqrt(7/pi)
 constexpr float kY3e = 1.445305721320277f;    // 1/4 sqrt(105/pi)
 
 __global__ void __launch_bounds__(256)
-k_noderef(const uint2* __restrict__ list, uint32_t cap, const InstFrame* __restrict__ inst,
-          const AssetDev* __restrict__ assets, CamConst cam, float4* __restrict__ ref,
-          const uint32_t* __restrict__ frame, uint32_t* __restrict__ order_keys, int key_shift) {
+k_order_keys(const uint2* __restrict__ list, uint32_t cap, const InstFrame* __restrict__ inst,
+             const AssetDev* __restrict__ assets, const uint32_t* __restrict__ frame, uint32_t* __restrict__ order_keys,
+             int key_shift) {
   const uint32_t n = min(frame[kRenderNodes], cap);
   for (uint32_t ci = blockIdx.x * blockDim.x + threadIdx.x; ci < n; ci += gridDim.x * blockDim.x) {
     const uint2 e = list[ci];
-    const InstFrame& I = inst[e.x];
-    const AssetDev& A = assets[I.asset];
-    if (order_keys) order_keys[ci] = (A.node_base + e.y) >> key_shift;
-    const float4 b = A.bound[e.y];
-    const double bx = b.x, by = b.y, bz = b.z;
-    const double X = ((I.m64[0] * bx + I.m64[1] * by) + I.m64[2] * bz) + I.m64[3];
-    const double Y = ((I.m64[4] * bx + I.m64[5] * by) + I.m64[6] * bz) + I.m64[7];
-    const double Z = ((I.m64[8] * bx + I.m64[9] * by) + I.m64[10] * bz) + I.m64[11];
-    const double rho = I.s64 * double(b.w);
-    float4 r0, r1;
-    if (Z > 4.0 * rho && Z > 1e-6 && fabs(X) <= 4.0 * Z && fabs(Y) <= 4.0 * Z) {
-      const double rx = X / Z, ry = Y / Z;
-      const double U = double(cam.fx) * rx + double(cam.cx);
-      const double V = double(cam.fy) * ry + double(cam.cy);
-      const float uh = float(U), vh = float(V);
-      r0 = make_float4(uh, float(U - double(uh)), vh, float(V - double(vh)));
-      r1 = make_float4(float(rx), float(ry), float(Z), 1.f);
-    } else {
-      r0 = make_float4(cam.cx, 0.f, cam.cy, 0.f);
-      r1 = make_float4(float(X), float(Y), float(Z), 0.f);
-    }
-    ref[2 * ci] = r0;
-    ref[2 * ci + 1] = r1;
+    order_keys[ci] = (assets[inst[e.x].asset].node_base + e.y) >> key_shift;
+  }
+}
+
+// The FP64 reference of an entry whose mean centre (asset frame) is b and its radius b.w:
+//   r0 = (U0 hi, U0 lo, V0 hi, V0 lo): pixel position of the centre as float pairs,
+//   r1 = (rho_x, rho_y, Pz, mode): X/Z, Y/Z and Z of the centre in view space; mode 1 = compensated
+//   (centre well in front), 0 = direct (rho_x, rho_y then hold X, Y).
+__device__ __forceinline__ void entry_reference(const InstFrame& I, const float4 b, const CamConst& cam, float4* r0, float4* r1) {
+  const double bx = b.x, by = b.y, bz = b.z;
+  const double X = ((I.m64[0] * bx + I.m64[1] * by) + I.m64[2] * bz) + I.m64[3];
+  const double Y = ((I.m64[4] * bx + I.m64[5] * by) + I.m64[6] * bz) + I.m64[7];
+  const double Z = ((I.m64[8] * bx + I.m64[9] * by) + I.m64[10] * bz) + I.m64[11];
+  const double rho = I.s64 * double(b.w);
+  if (Z > 4.0 * rho && Z > 1e-6 && fabs(X) <= 4.0 * Z && fabs(Y) <= 4.0 * Z) {
+    const double rx = X / Z, ry = Y / Z;
+    const double U = double(cam.fx) * rx + double(cam.cx);
+    const double V = double(cam.fy) * ry + double(cam.cy);
+    const float uh = float(U), vh = float(V);
+    *r0 = make_float4(uh, float(U - double(uh)), vh, float(V - double(vh)));
+    *r1 = make_float4(float(rx), float(ry), float(Z), 1.f);
+  } else {
+    *r0 = make_float4(cam.cx, 0.f, cam.cy, 0.f);
+    *r1 = make_float4(float(X), float(Y), float(Z), 0.f);
   }
 }
 
@@ -113,7 +120,7 @@ __device__ __forceinline__ GaussPre gauss_pre(uint32_t j, int nsh, const float* 
 
 // Per-entry constants of a warp's chunk, staged in shared memory: the rows of the instance
 // frame's float32 M, its camera centre in the asset frame (and scale), and the entry's FP64
-// reference from k_noderef.
+// reference.
 struct EntryConst {
   float4 m0, m1, m2;   // M[0..3], M[4..7], M[8..11]
   float4 cam;          // cam_a[0..2], s
@@ -129,7 +136,7 @@ __device__ __forceinline__ uint32_t project_one(const GaussPre& G, size_t slot, 
                                             const CamConst& cam, const float4 bc, int nsh,
                                             float4* __restrict__ rec, uint2* __restrict__ rect,
                                             uint32_t* __restrict__ keys, uint32_t* __restrict__ frame,
-                                            uint32_t* key_out) {
+                                            uint32_t* key) {
   const float4 M0 = E.m0, M1 = E.m1, M2 = E.m2, CA = E.cam, r0 = E.r0, r1 = E.r1;
   const struct { float m[12]; float cam_a[3]; } I = {{M0.x, M0.y, M0.z, M0.w, M1.x, M1.y, M1.z, M1.w, M2.x, M2.y, M2.z, M2.w},
                                                     {CA.x, CA.y, CA.z}};
@@ -254,15 +261,19 @@ __device__ __forceinline__ uint32_t project_one(const GaussPre& G, size_t slot, 
   rp[2] = make_float4(rgb[2], __uint_as_float(origin), __uint_as_float(uint32_t(x0) | (uint32_t(x1) << 16)),
                       __uint_as_float(uint32_t(y0) | (uint32_t(y1) << 16)));
   rect[slot] = make_uint2(uint32_t(x0) | (uint32_t(x1) << 16), uint32_t(y0) | (uint32_t(y1) << 16));
-  *key_out = __float_as_uint(z32);
-  keys[slot] = *key_out;
+  *key = __float_as_uint(z32);
+  keys[slot] = *key;
   return uint32_t((int(x1) >> 4) - tx0 + 1) * uint32_t((int(y1) >> 4) - ty0 + 1);
 }
 
-// What a lane adds up over the Gaussians it projects.
+// What a lane adds up over a chunk (at most 64 Gaussians of at most 2^20 tiles).
 struct ProjTotals {
-  uint32_t visible = 0, key_min = 0xFFFFFFFFu, key_max = 0;
-  unsigned long long pairs = 0;
+  uint32_t visible, pairs;
+};
+// What a warp adds up over its chunks (in shared memory: the projection has no register to spare).
+struct WarpTotals {
+  unsigned long long pairs;
+  uint32_t visible, key_min, key_max;
 };
 
 // The depth histogram's bin of a cluster at depth z (its centre: a bin of most of its Gaussians; the
@@ -274,17 +285,17 @@ __device__ __forceinline__ uint32_t depth_bin(float z) {
 
 // One run of render-list entries that draw the same cluster (entries e = a .. b - 1 of the warp's
 // chunk; their indices ci are in lanes e, their constants in ent[e]): each lane takes Gaussians
-// lane and lane + 32 of the cluster, loads their attributes and computes their
+// lane and lane + 32 of the cluster (or one of them: halves h0 .. h1 - 1), loads their attributes and computes their
 // instance-independent values once, and projects them for every entry of the run.
-template <typename TC>
-__device__ __forceinline__ void project_run(int lane, int a, int b, uint32_t ci, uint32_t cnt,
+template <typename TC, bool kSlabs>
+__device__ __forceinline__ void project_run(int lane, int a, int b, int h0, int h1, uint32_t ci, uint32_t cnt,
                                                 const EntryConst* ent, const CamConst& cam, const float4 bc, int nsh,
                                                 const float* __restrict__ at, const TC* __restrict__ col,
                                                 float4* __restrict__ rec, uint2* __restrict__ rect,
                                                 uint32_t* __restrict__ keys, uint32_t* __restrict__ frame,
-                                                ProjTotals& tot, uint32_t* s_hist) {
+                                                ProjTotals& tot, uint32_t* s_hist, WarpTotals* s_tot) {
 #pragma unroll 1
-  for (int h = 0; h < 2; ++h) {
+  for (int h = h0; h < h1; ++h) {
     const uint32_t j = lane + 32 * h;
     GaussPre G;
     if (j < cnt) G = gauss_pre<TC>(j, nsh, at, col);
@@ -292,66 +303,76 @@ __device__ __forceinline__ void project_run(int lane, int a, int b, uint32_t ci,
     for (int e = a; e < b; ++e) {
       const uint32_t ce = __shfl_sync(0xffffffffu, ci, e);
       const size_t slot = size_t(ce) * kSlots + j;
-      uint32_t area = 0;
+      uint32_t area = 0, key = 0;
       if (j >= cnt) {
         keys[slot] = 0xFFFFFFFFu;
       } else {
-        uint32_t key = 0;
         area = project_one(G, slot, ent[e], cam, bc, nsh, rec, rect, keys, frame, &key);
-        if (area) {
-          ++tot.visible;
-          tot.pairs += area;
-          tot.key_min = min(tot.key_min, key);
-          tot.key_max = max(tot.key_max, key);
-        }
+        tot.visible += area ? 1u : 0u;
+        tot.pairs += area;
       }
-      if (s_hist) {   // (uniform)
+      if (kSlabs) {
         const uint32_t sum = __reduce_add_sync(0xffffffffu, area);
         if (lane == 0 && sum) atomicAdd(&s_hist[depth_bin(ent[e].r1.z)], sum);
+      } else {
+        const uint32_t kmin = __reduce_min_sync(0xffffffffu, area ? key : 0xFFFFFFFFu);
+        const uint32_t kmax = __reduce_max_sync(0xffffffffu, area ? key : 0u);
+        if (lane == 0) {
+          s_tot->key_min = min(s_tot->key_min, kmin);
+          s_tot->key_max = max(s_tot->key_max, kmax);
+        }
       }
     }
   }
 }
 
 // kFormats: bit 0 = float32 colour planes occur, bit 1 = float16 ones occur.  Each warp takes
-// chunks of `chunk` (1..32) consecutive positions of the order (list order when `order` is NULL),
+// chunks of at most max_chunk (1..32) consecutive positions of the order (list order when `order` is NULL),
 // stages their constants in shared memory and splits the chunk into runs of entries that draw the
 // same (asset, cluster).
 constexpr int kMaxChunk = 32;
 // chunk sizes (measured on the crowd: 8 to 32 within 1% grouped; 16 best in list order)
 constexpr int kProjChunkGrouped = 32, kProjChunkList = 16;
 constexpr int kProjChunkCounter = 15;   // the frame's tile-counter word of the chunk queue
-template <int kFormats>
+// kSlabs: a frame of several slabs (the depth histogram and the entries' depth ranges; else the
+// smallest and largest key).
+template <int kFormats, bool kSlabs>
 __global__ void __launch_bounds__(kProjThreads, 2)
 k_project(const uint2* __restrict__ list, uint32_t cap_nodes, const InstFrame* __restrict__ inst,
-          const AssetDev* __restrict__ assets, CamConst cam, const float4* __restrict__ ref,
+          const AssetDev* __restrict__ assets, CamConst cam,
           float4* __restrict__ rec, uint2* __restrict__ rect, uint32_t* __restrict__ keys,
           uint32_t* __restrict__ frame, const uint32_t* __restrict__ order,
           const uint32_t* __restrict__ sorted_keys, uint32_t* __restrict__ depth_hist,
-          float2* __restrict__ depth_range, int chunk) {
-  __shared__ uint32_t s_vis[kProjThreads / 32], s_dist[kProjThreads / 32], s_min[kProjThreads / 32], s_max[kProjThreads / 32];
-  __shared__ unsigned long long s_pairs[kProjThreads / 32];
-  __shared__ uint32_t s_hist[kDepthBins];
+          float2* __restrict__ depth_range, int max_chunk) {
+  __shared__ WarpTotals s_tot[kProjThreads / 32];
+  __shared__ uint32_t s_dist[kProjThreads / 32];
+  __shared__ uint32_t s_hist[kSlabs ? kDepthBins : 1];
   __shared__ EntryConst s_ent[kProjThreads / 32][kMaxChunk];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t n_nodes = min(frame[kRenderNodes], cap_nodes);
-  const uint32_t n_chunks = (n_nodes + chunk - 1) / chunk;
+  // small frames: chunks just large enough that every warp gets one, then half entries, so that the
+  // few entries there are do not queue up in a few warps (96x80 thumbnail, 313 entries in chunks of 16:
+  // 59 us; halves: 17 us)
+  const uint32_t warps = gridDim.x * (kProjThreads / 32);
+  const bool halves = 2u * n_nodes <= warps;
+  const int chunk = halves ? 1 : int(min((n_nodes + warps - 1u) / warps, uint32_t(max_chunk)));
+  const uint32_t n_chunks = halves ? 2u * n_nodes : chunk ? (n_nodes + chunk - 1) / chunk : 0u;
   EntryConst* ent = s_ent[warp];
-  if (depth_hist) {
+  if (kSlabs) {
     for (int i = threadIdx.x; i < kDepthBins; i += kProjThreads) s_hist[i] = 0;
     __syncthreads();
   }
-  uint32_t* hist = depth_hist ? s_hist : nullptr;
-  ProjTotals tot;
+  if (lane == 0) s_tot[warp] = {0ull, 0u, 0xFFFFFFFFu, 0u};
   uint32_t ndist = 0;
   for (;;) {   // persistent warps take the chunks in turn from a frame counter
     uint32_t ch = 0;
     if (lane == 0) ch = atomicAdd(frame + kTileCounters + kProjChunkCounter, 1u);
     ch = __shfl_sync(0xffffffffu, ch, 0);
     if (ch >= n_chunks) break;
-    const uint32_t p = ch * chunk + lane;
+    const int h0 = halves ? int(ch & 1u) : 0, h1 = halves ? h0 + 1 : 2;
+    const uint32_t p = (halves ? ch >> 1 : ch * chunk) + lane;
     const bool okp = lane < chunk && p < n_nodes;
-    uint32_t ci = 0, node = 0, asset = 0xFFFFFFFFu;
+    uint32_t ci = 0, node = 0, asset = 0xFFFFFFFFu, key0 = 0xFFFFFFFFu, key1 = 0;
     __syncwarp();   // the previous chunk's constants are consumed
     if (okp) {
       ci = order ? order[p] : p;   // a permutation of [0, n_nodes)
@@ -365,17 +386,32 @@ k_project(const uint2* __restrict__ list, uint32_t cap_nodes, const InstFrame* _
       E.m1 = mi[1];
       E.m2 = mi[2];
       E.cam = *reinterpret_cast<const float4*>(I.cam_a);
-      E.r0 = ref[2 * ci];
-      E.r1 = ref[2 * ci + 1];
-      if (depth_hist) {   // the node's depths: its centre's +- its radius, with a slack above the keys' rounding
-        const float4 b = assets[asset].bound[node];
+      const float4 b = assets[asset].bound[node];
+      entry_reference(I, b, cam, &E.r0, &E.r1);
+      if (kSlabs) {
+        // the entry's depths are its centre's +- its radius, with a slack above the
+        // keys' rounding; visible keys lie in [key0, key1] (all of them when that is not a number)
         const float reach = E.cam.w * b.w;
         const float slack = 4e-6f * (fabsf(E.m2.x * b.x) + fabsf(E.m2.y * b.y) + fabsf(E.m2.z * b.z) + fabsf(E.m2.w) + 4.f * reach) + 1e-30f;
-        depth_range[ci] = make_float2(E.r1.z - reach - slack, E.r1.z + reach + slack);
+        const float z0 = E.r1.z - reach - slack, z1 = E.r1.z + reach + slack;
+        depth_range[ci] = make_float2(z0, z1);
+        if (!(z1 < cam.near_z)) {
+          key0 = __float_as_uint(fmaxf(z0, cam.near_z));
+          key1 = z1 < INFINITY ? __float_as_uint(z1) : 0x7F800000u;
+        }
       }
-      if (sorted_keys && (p == 0 || sorted_keys[p] != sorted_keys[p - 1])) ++ndist;
+      if (sorted_keys && h0 == 0 && (p == 0 || sorted_keys[p] != sorted_keys[p - 1])) ++ndist;
+    }
+    if (kSlabs) {
+      key0 = __reduce_min_sync(0xffffffffu, key0);
+      key1 = __reduce_max_sync(0xffffffffu, key1);
+      if (lane == 0) {
+        s_tot[warp].key_min = min(s_tot[warp].key_min, key0);
+        s_tot[warp].key_max = max(s_tot[warp].key_max, key1);
+      }
     }
     __syncwarp();
+    ProjTotals tot = {0u, 0u};
     // runs: maximal stretches of the chunk with the same (asset, node)
     const uint32_t pa = __shfl_up_sync(0xffffffffu, asset, 1), pn = __shfl_up_sync(0xffffffffu, node, 1);
     const uint32_t valid = __ballot_sync(0xffffffffu, okp);
@@ -392,49 +428,42 @@ k_project(const uint2* __restrict__ list, uint32_t cap_nodes, const InstFrame* _
       const float* at = reinterpret_cast<const float*>(blk);    // geometry planes
       const unsigned char* col = blk + size_t(kGeoPlanes) * kSlots * 4;   // colour planes
       if (kFormats == 2 || (kFormats == 3 && A.half_color))
-        project_run<__half>(lane, a, b, ci, cnt, ent, cam, bc, int(A.sh_coeffs), at,
-                            reinterpret_cast<const __half*>(col), rec, rect, keys, frame, tot, hist);
+        project_run<__half, kSlabs>(lane, a, b, h0, h1, ci, cnt, ent, cam, bc, int(A.sh_coeffs), at,
+                            reinterpret_cast<const __half*>(col), rec, rect, keys, frame, tot, s_hist, s_tot + warp);
       else
-        project_run<float>(lane, a, b, ci, cnt, ent, cam, bc, int(A.sh_coeffs), at,
-                           reinterpret_cast<const float*>(col), rec, rect, keys, frame, tot, hist);
+        project_run<float, kSlabs>(lane, a, b, h0, h1, ci, cnt, ent, cam, bc, int(A.sh_coeffs), at,
+                           reinterpret_cast<const float*>(col), rec, rect, keys, frame, tot, s_hist, s_tot + warp);
+    }
+    const uint32_t nvis = __reduce_add_sync(0xffffffffu, tot.visible), npair = __reduce_add_sync(0xffffffffu, tot.pairs);
+    if (lane == 0) {
+      s_tot[warp].visible += nvis;
+      s_tot[warp].pairs += npair;
     }
   }
   // one atomic per block for each total
-  uint32_t nvis = tot.visible;
 #pragma unroll
-  for (int d = 16; d > 0; d >>= 1) {
-    nvis += __shfl_xor_sync(0xffffffffu, nvis, d);
-    ndist += __shfl_xor_sync(0xffffffffu, ndist, d);
-    tot.pairs += __shfl_xor_sync(0xffffffffu, tot.pairs, d);
-  }
-  const uint32_t kmin = __reduce_min_sync(0xffffffffu, tot.key_min), kmax = __reduce_max_sync(0xffffffffu, tot.key_max);
-  if (lane == 0) {
-    s_vis[warp] = nvis;
-    s_dist[warp] = ndist;
-    s_pairs[warp] = tot.pairs;
-    s_min[warp] = kmin;
-    s_max[warp] = kmax;
-  }
+  for (int d = 16; d > 0; d >>= 1) ndist += __shfl_xor_sync(0xffffffffu, ndist, d);
+  if (lane == 0) s_dist[warp] = ndist;
   __syncthreads();
   if (threadIdx.x == 0) {
-    uint32_t t = 0, u = 0, mn = 0xFFFFFFFFu, mx = 0;
-    unsigned long long np = 0;
-    for (int w = 0; w < kProjThreads / 32; ++w) {
-      t += s_vis[w];
+    WarpTotals t = s_tot[0];
+    uint32_t u = s_dist[0];
+    for (int w = 1; w < kProjThreads / 32; ++w) {
+      t.visible += s_tot[w].visible;
+      t.pairs += s_tot[w].pairs;
+      t.key_min = min(t.key_min, s_tot[w].key_min);
+      t.key_max = max(t.key_max, s_tot[w].key_max);
       u += s_dist[w];
-      np += s_pairs[w];
-      mn = min(mn, s_min[w]);
-      mx = max(mx, s_max[w]);
     }
-    if (t) {
-      atomicAdd(frame + kVisible, t);
-      atomicAdd(reinterpret_cast<unsigned long long*>(frame + kPairs64), np);
-      atomicMax(frame + kKeyMinInv, ~mn);
-      atomicMax(frame + kKeyMax, mx);
+    if (t.visible) {
+      atomicAdd(frame + kVisible, t.visible);
+      atomicAdd(reinterpret_cast<unsigned long long*>(frame + kPairs64), t.pairs);
+      atomicMax(frame + kKeyMinInv, ~t.key_min);
+      atomicMax(frame + kKeyMax, t.key_max);
     }
     if (u) atomicAdd(frame + kRenderClusters, u);
   }
-  if (depth_hist) {
+  if (kSlabs) {
     for (int i = threadIdx.x; i < kDepthBins; i += kProjThreads)
       if (s_hist[i]) atomicAdd(depth_hist + i, s_hist[i]);
   }
@@ -442,38 +471,42 @@ k_project(const uint2* __restrict__ list, uint32_t cap_nodes, const InstFrame* _
 
 }  // namespace
 
-int g_project_blocks_per_sm[4] = {2, 2, 2, 2};   // resident k_project blocks per SM, per colour-format set
+namespace {
+
+using ProjectKernel = decltype(&k_project<1, false>);
+const ProjectKernel kProject[2][4] = {{k_project<1, false>, k_project<1, false>, k_project<2, false>, k_project<3, false>},
+                                      {k_project<1, true>, k_project<1, true>, k_project<2, true>, k_project<3, true>}};
+int g_project_blocks_per_sm[2][4];   // resident blocks per SM of each
+
+}  // namespace
 
 cudaError_t project_set_attributes() {
-  int n1 = 0, n2 = 0, n3 = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n1, k_project<1>, kProjThreads, 0);
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n2, k_project<2>, kProjThreads, 0);
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n3, k_project<3>, kProjThreads, 0);
-  if (e != cudaSuccess) return e;
-  g_project_blocks_per_sm[1] = n1;
-  g_project_blocks_per_sm[2] = n2;
-  g_project_blocks_per_sm[3] = n3;
+  for (int s = 0; s < 2; ++s)
+    for (int f = 0; f < 4; ++f) {
+      int n = 0;
+      const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kProject[s][f], kProjThreads, 0);
+      if (e != cudaSuccess) return e;
+      g_project_blocks_per_sm[s][f] = n;
+    }
   return cudaSuccess;
 }
 
-cudaError_t launch_noderef(const uint2* list, uint32_t cap, const InstFrame* inst, const AssetDev* assets,
-                           const CamConst& cam, float4* ref, const uint32_t* frame, uint32_t* order_keys,
-                           int key_shift, int sm_count, cudaStream_t st) {
-  k_noderef<<<sm_count * 4, 256, 0, st>>>(list, cap, inst, assets, cam, ref, frame, order_keys, key_shift);
+cudaError_t launch_order_keys(const uint2* list, uint32_t cap, const InstFrame* inst, const AssetDev* assets,
+                              const uint32_t* frame, uint32_t* order_keys, int key_shift, int sm_count, cudaStream_t st) {
+  k_order_keys<<<sm_count * 4, 256, 0, st>>>(list, cap, inst, assets, frame, order_keys, key_shift);
   return cudaGetLastError();
 }
 
 cudaError_t launch_project(const uint2* list, uint32_t cap_nodes, const InstFrame* inst, const AssetDev* assets,
-                           const CamConst& cam, const float4* ref, float4* rec, uint2* rect, uint32_t* keys,
-                           uint32_t* frame, const uint32_t* order, const uint32_t* sorted_keys,
+                           const CamConst& cam, float4* rec, uint2* rect, uint32_t* keys, uint32_t* frame, const uint32_t* order, const uint32_t* sorted_keys,
                            int color_formats, uint32_t* depth_hist, float2* depth_range, int sm_count,
                            cudaStream_t st) {
   // persistent grid: the resident blocks of the specialisation
   const int f = color_formats == 2 ? 2 : color_formats == 3 ? 3 : 1;
-  const int grid = sm_count * std::max(g_project_blocks_per_sm[f], 1);
+  const int slabs = depth_hist ? 1 : 0;
+  const int grid = sm_count * std::max(g_project_blocks_per_sm[slabs][f], 1);
   const int chunk = order ? kProjChunkGrouped : kProjChunkList;
-  const auto kernel = f == 2 ? k_project<2> : f == 3 ? k_project<3> : k_project<1>;
-  kernel<<<grid, kProjThreads, 0, st>>>(list, cap_nodes, inst, assets, cam, ref, rec, rect, keys, frame, order,
+  kProject[slabs][f]<<<grid, kProjThreads, 0, st>>>(list, cap_nodes, inst, assets, cam, rec, rect, keys, frame, order,
                                         sorted_keys, depth_hist, depth_range, chunk);
   return cudaGetLastError();
 }

@@ -95,7 +95,7 @@ struct Pipe {
   uint32_t cap_nodes = 0, cap_slots = 0, cap_pairs = 0, status_words = 0, cap_cut = 0;
   // d_keys0: the projection's depth keys per slot; (d_keys1, d_vals1) and (d_keys2, d_vals0): the
   // depth sort's buffers
-  DevBuf d_list, d_ref, d_keys0, d_keys1, d_keys2, d_vals0, d_vals1, d_rec, d_rect;
+  DevBuf d_list, d_keys0, d_keys1, d_keys2, d_vals0, d_vals1, d_rec, d_rect;
   DevBuf d_pk0, d_pk1, d_pv0, d_pv1, d_ranges, d_status, d_hist, d_cut;
   DevBuf d_img, d_timg, d_sort_k, d_sort_v, d_order;
   DevBuf d_front0, d_front1, d_tdcount, d_bitmap;   // top-down selection
@@ -290,7 +290,6 @@ v3dg_status ensure_work(Pipe* c) {
   c->cap_slots = c->cap_nodes * uint32_t(kSlots);
   const size_t S = c->cap_slots, PP = c->cap_pairs;
   ST(ensure(c, c->d_list, sizeof(uint2) * c->cap_nodes));
-  ST(ensure(c, c->d_ref, sizeof(float4) * 2 * c->cap_nodes));
   ST(ensure(c, c->d_keys0, 4 * S));
   ST(ensure(c, c->d_keys1, 4 * S));
   ST(ensure(c, c->d_keys2, 4 * S));
@@ -625,10 +624,11 @@ v3dg_status enqueue_render(Pipe* c, float* rgb, float* t_out) {
   uint32_t* okeys = nullptr;
   const uint32_t *order = nullptr, *sorted_keys = nullptr;
   if (use_project_order(c)) okeys = P<uint32_t>(c->d_keys1);
-  CU(launch_noderef(P<uint2>(c->d_list), c->cap_nodes, P<InstFrame>(c->d_inst), P<AssetDev>(c->ctx->d_assets), k,
-                    P<float4>(c->d_ref), frame, okeys, key_shift, sm, c->stream));
-  c->ctx->launches += 2;
+  ++c->ctx->launches;
   if (okeys) {
+    CU(launch_order_keys(P<uint2>(c->d_list), c->cap_nodes, P<InstFrame>(c->d_inst), P<AssetDev>(c->ctx->d_assets), frame,
+                         okeys, key_shift, sm, c->stream));
+    ++c->ctx->launches;
     const size_t cn = c->cap_nodes;
     bool oin1 = false;
     int nl = 0;
@@ -641,7 +641,7 @@ v3dg_status enqueue_render(Pipe* c, float* rgb, float* t_out) {
     if (key_shift == 0) sorted_keys = oin1 ? okeys + 2 * cn : okeys;   // (exact cluster ids: counted)
   }
   CU(launch_project(P<uint2>(c->d_list), c->cap_nodes, P<InstFrame>(c->d_inst), P<AssetDev>(c->ctx->d_assets), k,
-                    P<float4>(c->d_ref), P<float4>(c->d_rec), P<uint2>(c->d_rect), P<uint32_t>(c->d_keys0), frame,
+                    P<float4>(c->d_rec), P<uint2>(c->d_rect), P<uint32_t>(c->d_keys0), frame,
                     order, sorted_keys, c->color_formats, depth_hist, slabs > 1 ? P<float2>(c->d_marks) : nullptr, sm,
                     c->stream));
   CU(launch_slab_limits(frame, depth_hist, slabs, c->cap_pairs, c->stream));
@@ -750,7 +750,7 @@ std::vector<uint64_t> graph_key(Pipe* c, float* rgb, float* t_out) {
                              uint64_t(ctx->blend_mode),
                              uint64_t(ctx->count_work), uint64_t(c->color_formats), ctx->assets.size(),
                              uint64_t(uintptr_t(ctx->d_assets.p))};
-  const DevBuf* bufs[] = {&c->d_inst, &c->d_frame, &c->d_misc, &c->d_list, &c->d_ref, &c->d_keys0, &c->d_keys1,
+  const DevBuf* bufs[] = {&c->d_inst, &c->d_frame, &c->d_misc, &c->d_list, &c->d_keys0, &c->d_keys1,
                           &c->d_vals0, &c->d_vals1, &c->d_rec, &c->d_rect, &c->d_pk0, &c->d_pk1, &c->d_pv0,
                           &c->d_pv1, &c->d_ranges, &c->d_status, &c->d_hist, &c->d_order, &c->d_front0,
                           &c->d_front1, &c->d_tdcount, &c->d_bitmap, &c->d_keys2, &c->d_tlive, &c->d_state,
@@ -928,7 +928,7 @@ void pipe_free(Pipe* c) {
   drop_graph(c);
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
   c->cap_stream = nullptr;
-  DevBuf* bs[] = {&c->d_inst, &c->d_frame, &c->d_cutframe, &c->d_misc, &c->d_list, &c->d_ref, &c->d_keys0,
+  DevBuf* bs[] = {&c->d_inst, &c->d_frame, &c->d_cutframe, &c->d_misc, &c->d_list, &c->d_keys0,
                   &c->d_keys1, &c->d_vals0, &c->d_vals1, &c->d_rec, &c->d_rect, &c->d_pk0, &c->d_pk1,
                   &c->d_pv0, &c->d_pv1, &c->d_ranges, &c->d_status, &c->d_hist, &c->d_cut, &c->d_img,
                   &c->d_timg, &c->d_sort_k, &c->d_sort_v, &c->d_order, &c->d_front0, &c->d_front1,
@@ -950,7 +950,7 @@ void pipe_free(Pipe* c) {
 // The frame buffers a pipe holds (they grow with the largest frame it has rendered).
 DevBuf* const* frame_buffers(Pipe* c, size_t* n) {
   static thread_local DevBuf* bs[32];
-  DevBuf* list[] = {&c->d_list, &c->d_ref, &c->d_keys0, &c->d_keys1, &c->d_vals0, &c->d_vals1, &c->d_rec,
+  DevBuf* list[] = {&c->d_list, &c->d_keys0, &c->d_keys1, &c->d_vals0, &c->d_vals1, &c->d_rec,
                     &c->d_rect, &c->d_pk0, &c->d_pk1, &c->d_pv0, &c->d_pv1, &c->d_ranges, &c->d_status,
                     &c->d_cut, &c->d_img, &c->d_timg, &c->d_sort_k, &c->d_sort_v, &c->d_order, &c->d_front0,
                     &c->d_front1, &c->d_bitmap, &c->d_keys2, &c->d_tlive, &c->d_state,

@@ -80,8 +80,8 @@ enum Counter : int {
   kConicFp64 = 10,         // Gaussians whose 2D covariance had det < 1e-12 and was inverted in FP64
   kRenderClusters = 11,    // distinct clusters of the render list (projection grouped by cluster)
   kPairs64 = 12,           // [12, 14): the pair total as a 64-bit sum (detects totals beyond 2^32)
-  kKeyMinInv = 14,         // ~(smallest depth key of a visible Gaussian)
-  kKeyMax = 15,            // largest depth key of a visible Gaussian
+  kKeyMinInv = 14,         // ~(lower bound of the visible Gaussians' depth keys); of one slab, the smallest
+  kKeyMax = 15,            // upper bound of them; of one slab, the largest
   kTileCounters = 16,      // [16, 32): atomic tile counters: [16] selection, [27, 31) cluster order, [31] projection
   kSlabBase = 32,          // kSlabWords words for each depth slab
 };
@@ -160,16 +160,10 @@ cudaError_t launch_select_topdown(const InstFrame* inst, int n_inst, const Asset
                                   uint32_t tile_counter_slot, uint64_t* status, uint32_t epoch, int sm_count,
                                   cudaStream_t st, int* launches);
 
-// Per render-list node, FP64 reference for the projection (2 float4 per node):
-//   [0] = (U0 hi, U0 lo, V0 hi, V0 lo): pixel position of the node's mean centre as float pairs
-//   [1] = (rho_x, rho_y, Pz, mode): X/Z, Y/Z and Z of that centre in view space; mode 1 =
-//         compensated (centre well in front), 0 = direct (rho_x, rho_y then hold X, Y).
-// order_keys (may be NULL): also writes, per entry, its cluster's global id (node_base + node)
-// shifted right by key_shift, the key that groups the render list by cluster for the projection.
-cudaError_t launch_noderef(const uint2* render_list, uint32_t cap_nodes, const InstFrame* inst,
-                           const AssetDev* assets, const CamConst& cam, float4* ref,
-                           const uint32_t* frame, uint32_t* order_keys, int key_shift, int sm_count,
-                           cudaStream_t st);
+// Per render-list entry, its cluster's global id (node_base + node) shifted right by key_shift, the key
+// that groups the render list by cluster for the projection.
+cudaError_t launch_order_keys(const uint2* render_list, uint32_t cap_nodes, const InstFrame* inst, const AssetDev* assets,
+                              const uint32_t* frame, uint32_t* order_keys, int key_shift, int sm_count, cudaStream_t st);
 
 // Records (3 float4 per slot, slot = render index * 64 + j):
 //   [0] = (u_rel, v_rel, na, nb), [1] = (nc, log2 o, r, g), [2] = (b, tile origin, x range, y range)
@@ -187,8 +181,8 @@ cudaError_t launch_noderef(const uint2* render_list, uint32_t cap_nodes, const I
 // largest key, and -- unless depth_hist is NULL -- the depth histogram of the pairs and a conservative
 // depth range of every render-list node.
 cudaError_t launch_project(const uint2* render_list, uint32_t cap_nodes, const InstFrame* inst,
-                           const AssetDev* assets, const CamConst& cam, const float4* ref, float4* rec,
-                           uint2* rect, uint32_t* keys, uint32_t* frame, const uint32_t* order,
+                           const AssetDev* assets, const CamConst& cam, float4* rec, uint2* rect,
+                           uint32_t* keys, uint32_t* frame, const uint32_t* order,
                            const uint32_t* sorted_keys, int color_formats, uint32_t* depth_hist,
                            float2* depth_range, int sm_count, cudaStream_t st);
 
