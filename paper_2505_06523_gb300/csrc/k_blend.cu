@@ -9,16 +9,20 @@
 // T (1 - a) < 1e-4.  Key loads, slot loads, record loads and compositing belong to successive
 // batches, so the three dependent global latencies overlap with the compositing.
 //
+// The tiles with the longest lists go first, each sub-tile of them to a whole block (see "long lists").
+//
 // Why warps and 8x4: the blend is bound by the serial chain of the longest lists (a tile whose pixels
 // never all finish walks its whole list: 125k pairs in the 1080p crowd) and, on full frames, by
-// issue and shared-memory reads.  A block per tile with a barrier around each batch (the two-phase
-// kernel before this one) had one block on each long list, its warps idle at the barriers.  Blend
-// stage on a GB300, before -> now: 96x80 thumbnail 158 -> 35 us, 256x256 viewer 266 -> 61 us, 200
-// instances at 640x360 655 -> 289 us, one asset filling 1080p 1671 -> 309 us, the same 50 units
-// away 768 -> 254 us, crowd at 1080p 2.75 -> 1.29 ms, 16 crowd views 31.9 -> 11.2 ms.  The same
-// kernel with 8x8 pixels a warp (two per lane, four lists): 57 us, 510 us, 293 us and 1.74 ms on the
-// thumbnail, the 200 instances, the near asset and the crowd; 8x4 with one list: 72, 414, 307 us and
-// 1.41 ms; 4 or 8 records ahead and 5 to 8 blocks per SM: within 10% of each other.
+// issue and shared-memory reads (near asset: 83% issue-active, 74% of the shared-memory pipe).  A block
+// per tile with a barrier around each batch (the two-phase kernel before this one) had one block on
+// each long list, its warps idle at the barriers.  Blend stage on a GB300, two-phase kernel -> a warp per
+// sub-tile -> and long lists by blocks: 96x80 thumbnail 158 -> 37 -> 29 us, 256x256 viewer 266 -> 62 ->
+// 51 us, 200 instances at 640x360 655 -> 275 -> 174 us, one asset filling 1080p 1671 -> 346 -> 364 us, the
+// same 50 units away 768 -> 230 -> 127 us, crowd at 1080p (four slabs) 2.75 -> 2.03 -> 1.70 ms, 16 crowd
+// views 31.9 -> 11.7 -> 12.0 ms (full frames lose a little: five blocks per SM, not six).  The warp kernel
+// with 8x8 pixels a warp (two per lane, four lists): 57 us, 510 us, 293 us and 1.74 ms on the thumbnail,
+// the 200 instances, the near asset and the crowd; 8x4 with one list: 72, 414, 307 us and 1.41 ms
+// against 35, 289, 309 us and 1.29 ms (one slab).
 // Each record's mean is stored relative to the pixel origin of its first tile, so dx, dy are
 // differences of small numbers.
 //
@@ -30,8 +34,9 @@
 namespace v3dg {
 namespace {
 
-constexpr int kBlendThreads = 128;   // four independent warps (the block is only a launch unit)
-constexpr int kBlendBlocks = 6;      // resident blocks per SM: 24 warps of at most 80 registers
+constexpr int kBlendThreads = 128;   // four warps, independent except on long lists
+constexpr int kBlendBlocks = 5;      // resident blocks per SM: 20 warps of at most 96 registers, 39 KB of shared memory each
+constexpr uint32_t kLongPairs = 256;   // shortest list that a block blends together
 constexpr int kPxThreads = 256;
 constexpr int kPxWarps = kPxThreads / 32;
 constexpr float kLog2MinAlpha = -7.9943534f;  // log2(1/255)
@@ -70,7 +75,7 @@ constexpr int kScanKeys = 8;      // keys per lane and scan step
 constexpr int kRing = 512;        // list positions waiting to be gathered: < 32 + 32 * kScanKeys
 constexpr uint32_t kNoKey = (15u << 20) | (3u << 28);   // an empty box: meets no rectangle of a sub-tile
 
-constexpr int kAhead = 8;         // records whose alphas are computed ahead of the transmittance chain
+constexpr int kAhead = 4;         // records whose alphas are computed ahead of the transmittance chain
 
 // The staged records, one list for each 4x4 half of the sub-tile: the two half-warps composite
 // different records at once, so that a small Gaussian occupies 16 lanes and not 32.
@@ -156,6 +161,226 @@ __device__ __forceinline__ uint32_t item_classes(const uint32_t* __restrict__ cl
   return lane < uint32_t(kItemClasses) ? incl : 0xFFFFFFFFu;
 }
 
+// ---- long lists: a block per sub-tile
+// What bounds a sub-tile with a long list is its chain: 37k keys of a horizon tile took one warp 0.3 ms,
+// a third each for scanning, gathering and compositing, with the chip idle.  So the tiles whose lists
+// are at least a warp's share of the slab's pairs go first, each sub-tile to a whole block: three warps
+// scan, gather and compute the alphas of every pixel, the fourth only composites.  Hit number
+// 96 r + 32 w + j of the list is record j of producer w's batch in round r; in round r the producers make
+// that round's batches while the consumer composites the round before, one block barrier per round.
+constexpr int kProducers = kBlendThreads / 32 - 1;
+constexpr uint32_t kRoundHits = 32 * kProducers;
+constexpr int kLongScan = 4;       // keys per producer lane and scan step
+// Positions waiting for their slots to be loaded: a scan for one round more starts with less than that
+// round's hits missing, all earlier rounds' slots loaded, and ends with at most a step more.
+constexpr uint32_t kLongRing = 512;
+static_assert(kRoundHits + kRoundHits * kLongScan <= kLongRing, "ring");
+
+struct BlendBlock {
+  float4 g[kProducers][2][32];                 // staged records, as in BlendWarp
+  float4 c[kProducers][2][32];
+  float alpha[2][kProducers][32][32];          // [round parity][producer][record][pixel], 0: does not contribute
+  float2 rg[2][kProducers][2][32];             // colours of each half's records
+  float blue[2][kProducers][2][32];
+  uint32_t n[2][kProducers];                   // records of the longer list, a multiple of 4
+  uint32_t ring[kLongRing];
+  uint32_t count[kProducers];
+  uint32_t live[2], hits[2], ended[2], item;
+};
+
+__device__ __forceinline__ void producers_sync() {
+  __syncwarp();
+  asm volatile("bar.sync 1, %0;" ::"n"(32 * kProducers) : "memory");
+}
+
+// blend_step with the alpha ready (0: does nothing).
+__device__ __forceinline__ void blend_alpha(float a, const float2 rg, float blue, float& t, float& T, float& r, float& g, float& b) {
+  asm("{\n\t.reg .pred q;\n\t.reg .f32 om, w;\n\t"
+      "sub.rn.f32 om, 0f3F800000, %5;\n\t"
+      "mul.rn.f32 w, %5, %0;\n\t"
+      "mul.rn.f32 %0, %0, om;\n\t"
+      "setp.gt.f32 q, %5, 0f00000000;\n\t"
+      "setp.ge.and.f32 q, %0, %9, q;\n\t"
+      "@q mov.f32 %1, %0;\n\t"
+      "@q fma.rn.f32 %2, w, %6, %2;\n\t"
+      "@q fma.rn.f32 %3, w, %7, %3;\n\t"
+      "@q fma.rn.f32 %4, w, %8, %4;\n\t}"
+      : "+f"(t), "+f"(T), "+f"(r), "+f"(g), "+f"(b)
+      : "f"(a), "f"(rg.x), "f"(rg.y), "f"(blue), "f"(1e-4f));
+}
+
+// The mask of a record's box (third float4) within the sub-tile whose first pixel is (ox, oy).
+__device__ __forceinline__ uint32_t box_mask(const float4 r2, int ox, int oy) {
+  const uint32_t bx = __float_as_uint(r2.z), by = __float_as_uint(r2.w);
+  const int x0 = max(int(bx & 0xFFFFu) - ox, 0), x1 = min(int(bx >> 16) - ox, 7);
+  const int y0 = max(int(by & 0xFFFFu) - oy, 0), y1 = min(int(by >> 16) - oy, 3);
+  if (x0 > x1 || y0 > y1) return 0u;
+  const uint32_t cols = (0xFFu >> (7 - x1)) & (0xFFu << x0), rows = (0xFFFFu << (4 * y0)) & (0xFFFFu >> (12 - 4 * y1));
+  return (((cols & 15u) * 0x1111u) & rows) | (((((cols >> 4) & 15u) * 0x1111u) & rows) << 16);
+}
+
+// One sub-tile by the whole block: list positions [sp, end) of it, `live` pixels.  The consumer warp's
+// T, colour and mybit are the pixels' state (bit 0 once stopped), as in k_blend; returns the pixels
+// that are left.
+template <bool kCount>
+__device__ __forceinline__ uint32_t blend_long(BlendBlock& S, uint32_t sp, uint32_t end, uint32_t live, uint32_t sub, int tx,
+                                               int ty, float fx, float fy, const uint32_t* __restrict__ tk,
+                                               const uint32_t* __restrict__ pv, const float4* __restrict__ rec,
+                                               uint32_t cap_slots, float& T, float& cr, float& cg, float& cb,
+                                               uint32_t& mybit, uint32_t& n_eval, uint32_t& n_contrib) {
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, half = lane >> 4;
+  const int sx = tx * 16 + 8 * int(sub & 1u), sy = ty * 16 + 4 * int(sub >> 1);
+  const uint32_t lanebit = 1u << lane;
+  const int w = int(warp) - 1;   // producer
+  if (threadIdx.x == 0) S.live[1] = live;
+  __syncthreads();
+  uint32_t tail = 0, key[kLongScan], slot = 0xFFFFFFFFu;
+  float4 r0, r1, r2;
+  bool valid = false;
+  float t = T;
+  const auto load_keys = [&] {
+#pragma unroll
+    for (int k = 0; k < kLongScan; ++k) {
+      const uint32_t pos = sp + uint32_t(w) * (32u * kLongScan) + 32u * k + lane;
+      key[k] = pos < end ? tk[pos] : kNoKey;
+    }
+  };
+  // more hits until hit number `want` is known (or the list has ended)
+  const auto scan = [&](uint32_t want, uint32_t live_now) {
+    if (tail >= want || sp >= end) return;
+    const KeyTest kt = key_test(live_now, sub);
+    do {
+      uint32_t b[kLongScan], cnt = 0;
+#pragma unroll
+      for (int k = 0; k < kLongScan; ++k) {
+        b[k] = __ballot_sync(0xffffffffu, key_hits(key[k], kt));
+        cnt += __popc(b[k]);
+      }
+      if (lane == 0) S.count[w] = cnt;
+      producers_sync();
+      uint32_t at = tail;
+#pragma unroll
+      for (int p = 0; p < kProducers; ++p) {
+        const uint32_t c = S.count[p];
+        if (p < w) at += c;
+        tail += c;
+      }
+#pragma unroll
+      for (int k = 0; k < kLongScan; ++k) {
+        if ((b[k] >> lane) & 1u)
+          S.ring[(at + __popc(b[k] & lanemask_lt())) % kLongRing] = sp + uint32_t(w) * (32u * kLongScan) + 32u * k + lane;
+        at += __popc(b[k]);
+      }
+      sp += kRoundHits * kLongScan;
+      load_keys();
+      producers_sync();   // the counts are read, the ring's new positions visible
+    } while (tail < want && sp < end);
+  };
+  const auto load_slot = [&](uint32_t round) {
+    const uint32_t i = round * kRoundHits + 32u * uint32_t(w) + lane;
+    slot = i < tail ? pv[S.ring[i % kLongRing]] : 0xFFFFFFFFu;
+  };
+  const auto load_record = [&] {
+    valid = slot < cap_slots;
+    if (valid) {
+      const float4* r = rec + 3 * size_t(slot);
+      r0 = r[0];
+      r1 = r[1];
+      r2 = r[2];
+    }
+  };
+  if (w >= 0) {
+    load_keys();
+    scan(kRoundHits, live);
+    load_slot(0);
+    load_record();
+    scan(2u * kRoundHits, live);
+    load_slot(1);
+  }
+  for (uint32_t round = 0;; ++round) {
+    const uint32_t par = round & 1u;
+    if (w >= 0) {
+      const uint32_t live_now = S.live[par ^ 1u];
+      scan((round + 3u) * kRoundHits, live_now);
+      // stage this round's batch
+      const uint32_t m = valid ? box_mask(r2, sx, sy) & live_now : 0u;
+      const uint32_t ml = m & 0xFFFFu, mr = m >> 16;
+      const uint32_t bl = __ballot_sync(0xffffffffu, ml != 0u), br = __ballot_sync(0xffffffffu, mr != 0u);
+      const int nl = __popc(bl), nr = __popc(br), n = (max(nl, nr) + 3) & ~3;
+      if (m) {
+        const uint32_t org = __float_as_uint(r2.y);
+        const float ox = float(16 * (tx - int(org & 0xFFFFu))), oy = float(16 * (ty - int(org >> 16)));
+        const float4 g = make_float4(r0.x - ox, r0.y - oy, r0.z, r0.w);
+        const float4 c = make_float4(r1.x, r1.y, __uint_as_float(m), 0.f);
+        const float2 rg = make_float2(r1.z, r1.w);
+        if (ml) {
+          const int i = __popc(bl & lanemask_lt());
+          S.g[w][0][i] = g;
+          S.c[w][0][i] = c;
+          S.rg[par][w][0][i] = rg;
+          S.blue[par][w][0][i] = r2.x;
+        }
+        if (mr) {
+          const int i = __popc(br & lanemask_lt());
+          S.g[w][1][i] = g;
+          S.c[w][1][i] = c;
+          S.rg[par][w][1][i] = rg;
+          S.blue[par][w][1][i] = r2.x;
+        }
+      }
+      if (int(lane) >= nl && int(lane) < n) S.c[w][0][lane].z = 0.f;   // (records without pixels)
+      if (int(lane) >= nr && int(lane) < n) S.c[w][1][lane].z = 0.f;
+      if (lane == 0) {
+        S.n[par][w] = uint32_t(n);
+        if (w == 0) {
+          S.hits[par] = tail;
+          S.ended[par] = sp >= end ? 1u : 0u;
+        }
+      }
+      load_record();
+      load_slot(round + 2u);
+      __syncwarp();
+      for (int i = 0; i < n; i += 4) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float4 c = S.c[w][half][i + q];
+          const float l2a = log2_alpha(S.g[w][half][i + q], c, fx, fy);
+          const float al = fminf(0.999f, ex2_approx(l2a));
+          const bool in = (__float_as_uint(c.z) & lanebit) != 0u;
+          if (kCount) n_eval += in ? 1u : 0u;
+          S.alpha[par][w][i + q][lane] = in && l2a >= kLog2MinAlpha && al >= 1.f / 255.f ? al : 0.f;
+        }
+      }
+    } else if (round > 0) {
+      const uint32_t prev = par ^ 1u;
+      for (int p = 0; p < kProducers; ++p) {
+        const int n = int(S.n[prev][p]);
+        for (int i = 0; i < n; i += 4) {
+          float a[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) a[q] = S.alpha[prev][p][i + q][lane];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            if (kCount) n_contrib += a[q] > 0.f && t * (1.f - a[q]) >= 1e-4f ? 1u : 0u;
+            blend_alpha(a[q], S.rg[prev][p][half][i + q], S.blue[prev][p][half][i + q], t, T, cr, cg, cb);
+          }
+        }
+      }
+      if (t < 1e-4f) mybit = 0u;
+      live = __ballot_sync(0xffffffffu, mybit != 0u);
+      if (lane == 0) S.live[par] = live;
+    } else if (lane == 0) {
+      S.live[par] = live;
+    }
+    __syncthreads();
+    // the hits below round * kRoundHits are composited
+    if (S.live[par] == 0u || (S.ended[par] && round * kRoundHits >= S.hits[par])) break;
+  }
+  const uint32_t left = S.live[0] & S.live[1];
+  __syncthreads();   // the block's shared words are read
+  return left;
+}
+
 // kCount: also count the evaluations and contributions into work[0], work[1].
 // kSlabbed: one of the frame's depth slabs (the first one covers every tile, later ones those with
 // pairs): the pixels' T goes through live.state (negative once the pixel has stopped) and their
@@ -175,15 +400,33 @@ k_blend(const uint2* __restrict__ ranges, const uint32_t* __restrict__ items, ui
   // (a later slab leaves out the tiles without pairs)
   const uint32_t n_items =
       (kSlabbed && !first ? __shfl_sync(0xffffffffu, cls_incl, kItemClasses - 2) : n_tiles) * uint32_t(kSubTiles);
-  __shared__ BlendWarp s_warp[kBlendThreads / 32];
-  const uint32_t lane = threadIdx.x & 31u;
-  BlendWarp& S = s_warp[threadIdx.x >> 5];
+  extern __shared__ __align__(16) unsigned char s_blend[];   // BlendBlock, then BlendWarp x 4
+  BlendBlock& B = *reinterpret_cast<BlendBlock*>(s_blend);
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  BlendWarp& S = reinterpret_cast<BlendWarp*>(s_blend)[warp];
   uint32_t n_eval = 0, n_contrib = 0;
+  // the classes of long lists: all of them at least a warp's share of the slab's pairs (each key is
+  // scanned by eight warps), below which a warp on its own does not hold the frame up, and the block's
+  // work beyond the stop of a short chain costs more (half the share: 1001x563 143 -> 170 us; twice:
+  // 200 instances 174 -> 256 us), and at least kLongPairs
+  const uint32_t share = max(slab[kSlabPairs] / max(gridDim.x * (kBlendThreads / 32u) / kSubTiles, 1u), kLongPairs);
+  const int long_classes = min(max(16 - int(32 - __clz(share - 1u)), -1), kItemClasses - 3) + 1;   // class c: 2^(16 - c) pairs or more
+  const uint32_t n_long = long_classes ? __shfl_sync(0xffffffffu, cls_incl, long_classes - 1) * uint32_t(kSubTiles) : 0u;
+  bool by_block = n_long > 0u;
   for (;;) {
     uint32_t it = 0;
-    if (lane == 0) it = atomicAdd(slab + kSlabBlendItem, 1u);
-    it = __shfl_sync(0xffffffffu, it, 0);
-    if (it >= n_items) break;
+    if (by_block) {
+      if (threadIdx.x == 0) B.item = atomicAdd(slab + kSlabBlendLong, 1u);
+      __syncthreads();
+      it = B.item;
+      __syncthreads();
+      by_block = it < n_long;
+      if (!by_block) continue;
+    } else {
+      if (lane == 0) it = atomicAdd(slab + kSlabBlendItem, 1u);
+      it = __shfl_sync(0xffffffffu, it, 0) + n_long;
+      if (it >= n_items) break;
+    }
     const int tile = int(item_tile(items, n_tiles, cls_incl, it / kSubTiles));   // (view, tile) id
     const uint32_t sub = it % kSubTiles;
     const int view = tile / tiles_per_view, vt = tile - view * tiles_per_view;
@@ -205,7 +448,7 @@ k_blend(const uint2* __restrict__ ranges, const uint32_t* __restrict__ items, ui
     }
     uint32_t live = __ballot_sync(0xffffffffu, mybit != 0u);
     if (kSlabbed && !first) {
-      if (live == 0u) continue;   // (finished in an earlier slab)
+      if (live == 0u) continue;   // (finished in an earlier slab; the same in all of a block's warps)
       if (inside) {
         cr = rgb[3 * p + 0];
         cg = rgb[3 * p + 1];
@@ -215,7 +458,12 @@ k_blend(const uint2* __restrict__ ranges, const uint32_t* __restrict__ items, ui
     const uint2 range = ranges[tile];
     uint32_t sp = range.x;                  // next list position to scan
     const uint32_t end = live ? range.y : range.x;
-    if (sp < end) {
+    if (by_block) {
+      if (sp < end)
+        live = blend_long<kCount>(B, sp, end, live, sub, tx, ty, fx, fy, tk, pv, rec, cap_slots, T, cr, cg, cb, mybit, n_eval,
+                                  n_contrib);
+      if (warp != 0u) continue;   // (the consumer has the pixels)
+    } else if (sp < end) {
       KeyTest kt = key_test(live, sub);
       uint32_t head = 0, tail = 0;          // the ring's waiting positions
       uint32_t key[kScanKeys];
@@ -264,17 +512,7 @@ k_blend(const uint2* __restrict__ ranges, const uint32_t* __restrict__ items, ui
       uint32_t n_slot = next_slots(slot);
       while (n_rec) {
         // stage the records whose box holds an unfinished pixel of this warp, in order
-        uint32_t m = 0;
-        if (valid) {
-          const uint32_t bx = __float_as_uint(r2.z), by = __float_as_uint(r2.w);
-          const int ox = tx * 16 + sx, oy = ty * 16 + sy;
-          const int x0 = max(int(bx & 0xFFFFu) - ox, 0), x1 = min(int(bx >> 16) - ox, 7);
-          const int y0 = max(int(by & 0xFFFFu) - oy, 0), y1 = min(int(by >> 16) - oy, 3);
-          if (x0 <= x1 && y0 <= y1) {
-            const uint32_t cols = (0xFFu >> (7 - x1)) & (0xFFu << x0), rows = (0xFFFFu << (4 * y0)) & (0xFFFFu >> (12 - 4 * y1));
-            m = ((((cols & 15u) * 0x1111u) & rows) | ((((cols >> 4) & 15u) * 0x1111u & rows) << 16)) & live;
-          }
-        }
+        const uint32_t m = valid ? box_mask(r2, tx * 16 + sx, ty * 16 + sy) & live : 0u;
         const uint32_t ml = m & 0xFFFFu, mr = m >> 16;   // the left and right 4x4 pixels
         const uint32_t bl = __ballot_sync(0xffffffffu, ml != 0u), br = __ballot_sync(0xffffffffu, mr != 0u);
         const int nl = __popc(bl), nr = __popc(br);
@@ -691,6 +929,10 @@ void blend_px_launch(int grid, cudaStream_t st, const uint2* ranges, const uint3
 
 }  // namespace
 
+namespace {
+constexpr int kBlendShared = int(std::max(sizeof(BlendBlock), sizeof(BlendWarp) * (kBlendThreads / 32)));
+}  // namespace
+
 cudaError_t blend_set_attributes() {
   // several resident blocks of 10-28 KB shared memory per SM want the largest carveout
   const void* fns[] = {(const void*)k_blend<true, false>,   (const void*)k_blend<false, false>,
@@ -718,11 +960,10 @@ cudaError_t launch_blend(const uint2* ranges, uint32_t* items, uint32_t* class_c
   k_blend_items<<<(n_tiles + 255) / 256, 256, 0, st>>>(ranges, uint32_t(n_tiles), items, class_count);
   // persistent grids: the resident blocks
   if (mode == 0) {
-    const int per_block = kBlendThreads / 32;
-    const int grid = std::min((kSubTiles * n_tiles + per_block - 1) / per_block, sm_count * kBlendBlocks);
+    const int grid = std::min(kSubTiles * n_tiles, sm_count * kBlendBlocks);
     const auto kernel = live.bits ? (work ? k_blend<true, true> : k_blend<false, true>)
                                   : (work ? k_blend<true, false> : k_blend<false, false>);
-    kernel<<<grid, kBlendThreads, 0, st>>>(ranges, items, uint32_t(n_tiles), class_count, words, slab == 0, live, tk, pv, rec, cap_slots,
+    kernel<<<grid, kBlendThreads, kBlendShared, st>>>(ranges, items, uint32_t(n_tiles), class_count, words, slab == 0, live, tk, pv, rec, cap_slots,
                                            cam.width, cam.height, cam.tiles_x, cam.tiles_x * cam.tiles_y, rgb, t_out, work,
                                            frame, sticky);
     return cudaGetLastError();

@@ -98,6 +98,7 @@ enum SlabWord : int {
   kSlabExpandTile = kSlabDepthTiles + 4,
   kSlabPairTiles,          // 4 words
   kSlabBlendItem = kSlabPairTiles + 4,
+  kSlabBlendLong,          // the same of the items that a block blends together
   kSlabLo, kSlabHi,        // depth keys [lo, hi)
   kSlabBits,               // key bits of the slab's depth sort: keys are stored as key - lo
   kSlabLarge,              // Gaussians left to the large-box expansion

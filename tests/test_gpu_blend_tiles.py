@@ -60,3 +60,54 @@ def test_empty_and_infinite_records(small_asset):
     err = np.abs(imgs[0][0] - imgs[1][0])
     # at most Gaussian 7 itself is missing: one of thousands, of a few pixels
     assert (err.max(-1) > 0).mean() < 0.05
+
+
+@pytest.mark.parametrize("n,aside", [(1, 0), (95, 0), (97, 0), (1000, 0), (4100, 0), (1000, 190), (1500, 234), (2000, 300), (1500, 575)])
+def test_long_lists(n, aside):
+    """One tile with n faint Gaussians on top of each other (only the longest stack stops a pixel): lists below and above the length
+    from which a block blends them together, rounds that end within a batch; against the block-per-tile variant bit
+    for bit, and against the closed form T = (1 - alpha)^k at the centre pixel (n roundings of 2^-24 each).
+    aside: as many more in front, small and in a corner of the same tile, so that the centre's sub-tile meets a sparse
+    stretch of the list before the dense one."""
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2505_06523_gb300 import Context
+    from paper_2505_06523_gb300._native import V3DG_OPT_BLEND_MODE
+    from synth.assets import Asset
+    rng = np.random.default_rng(n)
+    stack, n = n, n + aside
+    nodes = (n + 63) // 64
+    o = np.float32(max(0.005, min(0.5, 2.0 / stack)))
+    means = np.concatenate([rng.uniform(-1e-4, 1e-4, (n, 2)), rng.uniform(-0.01, 0.01, (n, 1))], 1).astype(np.float32)
+    means[:, :2] = 0.0
+    scales = np.full((n, 3), -2.0, np.float32)
+    means[stack:], scales[stack:] = (0.9625, 0.175, -0.5), -4.0   # 11 and 2 px from the centre pixel, 0.2 px wide
+    sh = np.zeros((n, 16, 3), np.float32)
+    sh[:, 0] = rng.uniform(-1, 1, (n, 3))
+    count = np.minimum(64, n - 64 * np.arange(nodes)).astype(np.uint32)
+    first = (64 * np.arange(nodes)).astype(np.uint32)
+    if nodes > 1:   # a root above the leaves: one more Gaussian, never selected
+        means, sh, scales = (np.concatenate([x, x[:1]]) for x in (means, sh, scales))
+        count, first = np.append(count, 1).astype(np.uint32), np.append(first, n).astype(np.uint32)
+    level = np.array([0] * nodes + [1] * (nodes > 1), np.uint8)
+    parent = np.array([nodes if nodes > 1 else -1] * nodes + [-1] * (nodes > 1), np.int32)
+    m = len(means)
+    asset = Asset(means=means, log_scales=scales, quats=np.tile(np.float32([1, 0, 0, 0]), (m, 1)),
+                  opacity=np.full(m, o, np.float32), sh=sh, node_first=first, node_count=count, node_level=level,
+                  node_parent=parent, own_sphere=np.tile(np.float32([0, 0, 0, 1]), (len(count), 1)))
+    inst = scenes.single_instance()
+    cam = scenes.Camera(np.array([[1.0, 0, 0, 0], [0, 1.0, 0, 0], [0, 0, 1.0, 4.0]]), 40.0, 40.0, 20.5, 12.5, 41, 25)
+    out = []
+    with Context(0) as ctx:
+        ctx.load_hierarchy(asset)
+        ctx.set_instances(inst)
+        for mode in (0, 1):
+            ctx.set_option(V3DG_OPT_BLEND_MODE, mode)
+            ctx.select(cam, 0.0)
+            rgb, T = ctx.render(want_T=True)
+            out.append((rgb.cpu().numpy(), T.cpu().numpy()))
+        assert ctx.frame_stats()["visible"] == n
+    assert (out[0][0] == out[1][0]).all() and (out[0][1] == out[1][1]).all()
+    # the centre pixel's alpha is the opacity (2^(log2 o), a few ulp); it stops before T < 1e-4
+    want = (1.0 - float(o)) ** min(stack, int(np.log(1e-4) / np.log(1.0 - float(o))))
+    assert abs(float(out[0][1][12, 20]) / want - 1.0) <= 1e-5 + 4 * n * 2.0 ** -24 * (1 + float(o) / (1 - float(o)))
