@@ -193,15 +193,24 @@ k_mark(const uint32_t* __restrict__ keys, const uint2* __restrict__ rect, uint32
         key[a][0] = a < m ? keys[size_t(node[a]) * kSlots + lane] : 0xFFFFFFFFu;
         key[a][1] = a < m ? keys[size_t(node[a]) * kSlots + 32 + lane] : 0xFFFFFFFFu;
       }
+      // the boxes of the slots in the slab, all on their way before the first is looked at
+      uint2 box[kAhead][2];
+      bool in[kAhead][2];
+#pragma unroll
+      for (int a = 0; a < kAhead; ++a)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          in[a][h] = key[a][h] >= lo && key[a][h] < hi;
+          if (kFilter) box[a][h] = in[a][h] ? rect[size_t(node[a]) * kSlots + 32 * h + lane] : make_uint2(0u, 0u);
+        }
 #pragma unroll
       for (int a = 0; a < kAhead; ++a) {
         if (a >= m) break;   // (uniform)
         uint32_t b[2];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-          bool in = key[a][h] >= lo && key[a][h] < hi;
-          if (kFilter && in) {
-            TileRect r = tile_rect(rect[size_t(node[a]) * kSlots + 32 * h + lane]);
+          if (kFilter && in[a][h]) {
+            TileRect r = tile_rect(box[a][h]);
             const uint32_t view = inst_views ? inst_views[list[node[a]].x].view : 0u;
             const uint32_t* row = live.bits + size_t(view * live.tiles_y + r.y) * live.words;
             uint32_t words = live.words;
@@ -217,9 +226,9 @@ k_mark(const uint32_t* __restrict__ keys, const uint2* __restrict__ rect, uint32
             uint32_t any = 0;
             for (uint32_t y = 0; y < r.h && !any; ++y, row += words)
               for (uint32_t x = 0; x < r.w && !any; x += 32u) any = live_row(row, r.x + x, min(r.w - x, 32u));
-            in = any != 0u;
+            in[a][h] = any != 0u;
           }
-          b[h] = __ballot_sync(0xffffffffu, in);
+          b[h] = __ballot_sync(0xffffffffu, in[a][h]);
           count += __popc(b[h]);
         }
         if (lane == node[a] - node0) mine = make_uint2(b[0], b[1]);
@@ -290,21 +299,30 @@ k_gather(const uint32_t* __restrict__ keys, uint32_t cap_nodes, const uint2* __r
     uint32_t base = counts[blk];
     for (int w = 0; w < int(warp); ++w) base += s_warp[w];
     uint32_t todo = __ballot_sync(0xffffffffu, c != 0u);
-    while (todo) {   // a marked node at a time, its slots by lanes
-      const int l = __ffs(todo) - 1;
-      todo &= todo - 1u;
-      const uint32_t m0 = __shfl_sync(0xffffffffu, mine.x, l), m1 = __shfl_sync(0xffffffffu, mine.y, l);
-      const uint32_t first = base + __shfl_sync(0xffffffffu, incl - c, l);
-      const uint32_t slot = (node0 + uint32_t(l)) * uint32_t(kSlots) + lane;
-      if ((m0 >> lane) & 1u) {
-        const uint32_t p = first + __popc(m0 & lanemask_lt());
-        kout[p] = keys[slot] - lo;
-        vout[p] = slot;
+    while (todo) {   // four marked nodes at a time, their slots by lanes
+      constexpr int kAhead = 4;
+      uint32_t key[kAhead][2], m[kAhead][2], first[kAhead], slot[kAhead];
+#pragma unroll
+      for (int a = 0; a < kAhead; ++a) {
+        const int l = todo ? __ffs(todo) - 1 : 0;
+        m[a][0] = __shfl_sync(0xffffffffu, mine.x, l);
+        m[a][1] = __shfl_sync(0xffffffffu, mine.y, l);
+        if (!todo) m[a][0] = m[a][1] = 0u;
+        todo &= todo - 1u;
+        first[a] = base + __shfl_sync(0xffffffffu, incl - c, l);
+        slot[a] = (node0 + uint32_t(l)) * uint32_t(kSlots) + lane;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) key[a][h] = (m[a][h] >> lane) & 1u ? keys[slot[a] + 32u * h] : 0u;
       }
-      if ((m1 >> lane) & 1u) {
-        const uint32_t p = first + __popc(m0) + __popc(m1 & lanemask_lt());
-        kout[p] = keys[slot + 32u] - lo;
-        vout[p] = slot + 32u;
+#pragma unroll
+      for (int a = 0; a < kAhead; ++a) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+          if ((m[a][h] >> lane) & 1u) {
+            const uint32_t p = first[a] + (h ? __popc(m[a][0]) : 0) + __popc(m[a][h] & lanemask_lt());
+            kout[p] = key[a][h] - lo;
+            vout[p] = slot[a] + 32u * h;
+          }
       }
     }
     __syncthreads();   // s_warp is consumed
