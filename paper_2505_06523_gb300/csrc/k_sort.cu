@@ -19,7 +19,8 @@ namespace {
 constexpr int kBins = kSortBins;
 constexpr int kLookback = 4;   // status words read per look-back round
 constexpr int kWarps = kSortThreads / 32;
-static_assert(kSortThreads == kBins, "one thread per digit");
+constexpr int kSortBlocks = 4;   // resident blocks per SM (64 registers a thread, 52 KB of shared memory)
+static_assert(kSortThreads >= kBins, "one thread per digit");
 
 // Digit counts of every pass in one read of the keys (one shared histogram per pass and block).
 // A thread counts a run of kHistRun consecutive keys and adds each pass's digit to the shared
@@ -117,22 +118,57 @@ k_hist(const uint32_t* __restrict__ keys, const uint32_t* __restrict__ n_dev, ui
   }
 }
 
+// What bounds a pass (20M pairs, ncu): the shared-memory pipe at 72% (38 wavefronts per 32 keys, most of
+// them bank conflicts of the random digits) with 49% of the issue slots, behind it the look-back (9k of
+// a tile's 34k cycles).  Pairs and per-digit words are 8 bytes wide so that ranking takes three shared
+// accesses a key, not five, and reordering one, not two; full tiles test no bounds.  20M pairs, 32 bits:
+// 692 -> 662 us a call, 300k pairs, 13 bits: 84 -> 75 us.  512 threads of 8 keys at 48 warps per SM: 730 us
+// (more warps wait for the same pipe); 8 status words a look-back round: 686 us.
+// Shared memory of a tile.
+struct SortTile {
+  uint2 kv[kSortTile];                // the tile's pairs, reordered by digit
+  uint2 digit[kWarps][kBins];         // per warp and digit: the lanes holding it (zero between items), and its
+                                      // count so far; after the ranking, its first position in the tile
+  uint32_t start[kBins], cnt[kBins];  // each digit's first position in the tile and its count
+  uint32_t goff[kBins];               // global destination offset minus start (mod 2^32)
+  uint32_t scan[kWarps + 1];
+  uint32_t tile;
+};
+
+// Ranks of a warp's items: the number of the warp's earlier keys of the same digit (item-major, then
+// lane order), 16 bits each.  The lanes that share a digit come from a shared-memory OR of lane bits
+// (measured faster than match.any, and than one vote per digit where the warp holds few of them).
+// kFull: every item of the tile is a key.
+template <bool kFull>
+__device__ __forceinline__ void rank_items(const uint32_t (&key)[kSortItems], uint32_t (&rank)[kSortItems / 2], uint2* mine,
+                                           uint32_t base, uint32_t n, int shift, uint32_t dmask) {
+  const uint32_t lane = threadIdx.x & 31u;
+#pragma unroll
+  for (int i = 0; i < kSortItems; ++i) {
+    const uint32_t live = kFull ? 0xffffffffu : __ballot_sync(0xffffffffu, base + i * 32 + lane < n);
+    if (i % 2 == 0) rank[i / 2] = 0;
+    if (kFull || (live >> lane) & 1u) {
+      uint2* const at = mine + ((key[i] >> shift) & dmask);
+      atomicOr(&at->x, 1u << lane);
+      __syncwarp(live);
+      const uint2 v = *at;   // the lanes of this digit, and its earlier keys
+      const uint32_t before = __popc(v.x & lanemask_lt());
+      __syncwarp(live);
+      if (before == 0) *at = make_uint2(0u, v.y + __popc(v.x));   // the digit's first lane
+      __syncwarp(live);
+      rank[i / 2] |= (v.y + before) << (16 * (i % 2));
+    }
+  }
+}
+
 template <bool kImplicit>
-__global__ void __launch_bounds__(kSortThreads, 4)
+__global__ void __launch_bounds__(kSortThreads, kSortBlocks)
 k_onesweep(const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin, uint32_t* __restrict__ kout,
            uint32_t* __restrict__ vout, const uint32_t* __restrict__ n_dev, uint32_t cap, SortDigits dg, int pass,
            const uint32_t* __restrict__ bits_dev, const uint32_t* __restrict__ hist, uint64_t* __restrict__ status,
            uint32_t* __restrict__ tile_counter, uint32_t epoch, uint32_t* __restrict__ err) {
-  __shared__ uint32_t s_keys[kSortTile];
-  __shared__ uint32_t s_vals[kSortTile];
-  __shared__ uint16_t s_wh[kWarps][kBins];   // per-warp digit counts, then per-warp exclusive offsets
-  __shared__ uint32_t s_start[kBins];        // block-local start of each digit
-  __shared__ uint32_t s_goff[kBins];         // global destination offset minus local start (mod 2^32)
-  __shared__ uint32_t s_cnt[kBins];          // the tile's digit counts
-  __shared__ uint32_t s_scan[kWarps + 1];
-  __shared__ uint32_t s_tile;
-  __shared__ uint32_t s_match[kWarps][kBins];   // per warp, the lanes holding each digit (zero between items)
-
+  extern __shared__ __align__(16) unsigned char s_sort[];
+  SortTile& S = *reinterpret_cast<SortTile*>(s_sort);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t n = min(*n_dev, cap);
   const uint32_t ntiles = (n + kSortTile - 1) / kSortTile;
@@ -142,103 +178,88 @@ k_onesweep(const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin, u
   const uint32_t dmask = (1u << min(dg.end - shift, dg.width)) - 1u;
   // the first output position of this thread's digit: exclusive scan of the pass's digit counts
   uint32_t all;
-  const uint32_t gexcl = block_exclusive_scan<kWarps>(hist[tid], s_scan, &all);
-  for (int i = tid; i < kWarps * kBins; i += kSortThreads) (&s_match[0][0])[i] = 0u;
+  const uint32_t gexcl = block_exclusive_scan<kWarps>(tid < kBins ? hist[tid] : 0u, S.scan, &all);
   // persistent blocks: tiles in the order of an atomic counter, so every tile a look-back waits
   // for is held by a running block
   for (;;) {
-  if (tid == 0) s_tile = atomicAdd(tile_counter, 1u);
-  __syncthreads();
-  const uint32_t tile = s_tile;
-  if (tile >= ntiles) return;
-  for (int i = tid; i < kWarps * kBins / 2; i += kSortThreads) reinterpret_cast<uint32_t*>(&s_wh[0][0])[i] = 0;
-  __syncthreads();
-  const uint32_t base = tile * kSortTile + warp * (kSortItems * 32);
-
-  uint32_t key[kSortItems], val[kSortItems], rank[kSortItems];
+    if (tid == 0) S.tile = atomicAdd(tile_counter, 1u);
+    __syncthreads();
+    const uint32_t tile = S.tile;
+    if (tile >= ntiles) return;
+    for (int i = tid; i < kWarps * kBins / 2; i += kSortThreads)
+      reinterpret_cast<uint4*>(&S.digit[0][0])[i] = make_uint4(0u, 0u, 0u, 0u);
+    const uint32_t base = tile * kSortTile + warp * (kSortItems * 32);
+    const bool full = (tile + 1u) * kSortTile <= n;   // (n is below 2^32 - 4096)
+    uint32_t key[kSortItems], val[kSortItems], rank[kSortItems / 2];
 #pragma unroll
-  for (int i = 0; i < kSortItems; ++i) {
-    const uint32_t idx = base + i * 32 + lane;
-    const bool ok = idx < n;
-    key[i] = ok ? kin[idx] : 0xFFFFFFFFu;
-    val[i] = kImplicit ? idx : (ok ? vin[idx] : 0u);
-  }
-  // warp-level stable ranking: item-major, then lane order.  The lanes that share a digit come
-  // from a shared-memory OR of lane bits (measured faster than match.any), or are the whole warp
-  // when every lane has the same digit (common in the high digits of the depth keys, where the
-  // OR would serialise on one word).
+    for (int i = 0; i < kSortItems; ++i) {
+      const uint32_t idx = base + i * 32 + lane;
+      const bool ok = full || idx < n;
+      key[i] = ok ? kin[idx] : 0xFFFFFFFFu;
+      val[i] = kImplicit ? idx : (ok ? vin[idx] : 0u);
+    }
+    __syncthreads();
+    if (full)
+      rank_items<true>(key, rank, S.digit[warp], base, n, shift, dmask);
+    else
+      rank_items<false>(key, rank, S.digit[warp], base, n, shift, dmask);
+    __syncthreads();
+    // per digit (one thread each): the block count and the chain, then every warp's first position
+    uint32_t cw[kWarps], cnt = 0;
+    if (tid < kBins) {
 #pragma unroll
-  for (int i = 0; i < kSortItems; ++i) {
-    const uint32_t idx = base + i * 32 + lane;
-    const bool ok = idx < n;
-    const uint32_t live = __ballot_sync(0xffffffffu, ok);
-    rank[i] = 0;
-    if (ok) {
-      const uint32_t d = (key[i] >> shift) & dmask;
-      const uint32_t d0 = __shfl_sync(live, d, __ffs(live) - 1);
-      const bool same = __all_sync(live, d == d0);   // (uniform over the live lanes)
-      uint32_t peers = live;
-      if (!same) {
-        atomicOr(&s_match[warp][d], 1u << lane);
-        __syncwarp(live);
-        peers = s_match[warp][d];
+      for (int w = 0; w < kWarps; ++w) {
+        cw[w] = S.digit[w][tid].y;
+        cnt += cw[w];
       }
-      const uint32_t before = __popc(peers & lanemask_lt());
-      const uint32_t cur = s_wh[warp][d];
-      __syncwarp(live);
-      if (before == 0) {   // the digit's first lane: advance the warp's count, clear the lane bits
-        s_wh[warp][d] = uint16_t(cur + __popc(peers));
-        if (!same) s_match[warp][d] = 0u;
+    }
+    if (tid <= dmask) chain_publish(status + tid, kBins, tile, cnt, epoch);   // as soon as they are known
+    uint32_t total;
+    const uint32_t start = block_exclusive_scan<kWarps>(cnt, S.scan, &total);
+    if (tid < kBins) {
+      S.start[tid] = start;
+      S.cnt[tid] = cnt;
+      uint32_t at = start;
+#pragma unroll
+      for (int w = 0; w < kWarps; ++w) {
+        S.digit[w][tid].y = at;
+        at += cw[w];
       }
-      __syncwarp(live);
-      rank[i] = cur + before;
     }
-  }
-  __syncthreads();
-  // per digit (threads 0..255): exclusive offsets across warps, the block count, and the chain
-  uint32_t cnt = 0;
-  if (tid < kBins) {
+    __syncthreads();
+    // reorder the tile by digit in shared memory (before the look-back, which needs none of the
+    // tile's registers and gets the earlier tiles more time to publish)
 #pragma unroll
-    for (int w = 0; w < kWarps; ++w) {
-      const uint32_t c = s_wh[w][tid];
-      s_wh[w][tid] = uint16_t(cnt);
-      cnt += c;
+    for (int i = 0; i < kSortItems; ++i) {
+      if (full || base + i * 32 + lane < n) {
+        const uint32_t d = (key[i] >> shift) & dmask;
+        S.kv[S.digit[warp][d].y + ((rank[i / 2] >> (16 * (i % 2))) & 0xFFFFu)] = make_uint2(key[i], val[i]);
+      }
     }
-  }
-  if (tid <= dmask) {   // the tile's digit counts, published as soon as they are known
-    chain_publish(status + tid, kBins, tile, cnt, epoch);
-    s_cnt[tid] = cnt;
-  }
-  uint32_t total;
-  const uint32_t start = block_exclusive_scan<kWarps>(cnt, s_scan, &total);
-  if (tid < kBins) s_start[tid] = start;
-  __syncthreads();
-  // reorder the tile by digit in shared memory (before the look-back, which needs none of the
-  // tile's registers and gets the earlier tiles more time to publish)
-#pragma unroll
-  for (int i = 0; i < kSortItems; ++i) {
-    const uint32_t idx = base + i * 32 + lane;
-    if (idx < n) {
-      const uint32_t dg = (key[i] >> shift) & dmask;
-      const uint32_t pos = s_start[dg] + s_wh[warp][dg] + rank[i];
-      s_keys[pos] = key[i];
-      s_vals[pos] = val[i];
+    if (tid <= dmask) {   // (the digit's count and start reloaded: no registers held over the reorder)
+      const uint32_t excl = chain_lookback<kLookback>(status + tid, kBins, tile, S.cnt[tid], epoch, err);
+      S.goff[tid] = gexcl + excl - S.start[tid];   // wraps; dst = goff + p is exact below 2^32
     }
-  }
-  if (tid <= dmask) {   // (the digit's count and start reloaded: no registers held over the reorder)
-    const uint32_t excl = chain_lookback<kLookback>(status + tid, kBins, tile, s_cnt[tid], epoch, err);
-    s_goff[tid] = gexcl + excl - s_start[tid];   // wraps; dst = s_goff + p is exact below 2^32
-  }
-  __syncthreads();
-  const uint32_t valid = min(uint32_t(kSortTile), n - tile * kSortTile);
-#pragma unroll 4
-  for (uint32_t p = tid; p < valid; p += kSortThreads) {
-    const uint32_t k = s_keys[p];
-    const uint32_t dst = s_goff[(k >> shift) & dmask] + p;
-    kout[dst] = k;
-    vout[dst] = s_vals[p];
-  }
-  __syncthreads();   // the tile's shared data is consumed before the next tile reuses it
+    __syncthreads();
+    if (full) {
+#pragma unroll 8
+      for (uint32_t i = 0; i < kSortItems; ++i) {
+        const uint32_t p = tid + i * kSortThreads;
+        const uint2 kv = S.kv[p];
+        const uint32_t dst = S.goff[(kv.x >> shift) & dmask] + p;
+        kout[dst] = kv.x;
+        vout[dst] = kv.y;
+      }
+    } else {
+      const uint32_t valid = n - tile * kSortTile;
+      for (uint32_t p = tid; p < valid; p += kSortThreads) {
+        const uint2 kv = S.kv[p];
+        const uint32_t dst = S.goff[(kv.x >> shift) & dmask] + p;
+        kout[dst] = kv.x;
+        vout[dst] = kv.y;
+      }
+    }
+    __syncthreads();   // the tile's shared data is consumed before the next tile reuses it
   }  // next tile
 }
 
@@ -265,14 +286,15 @@ __global__ void k_check_wait(uint64_t* __restrict__ status, uint32_t epoch, uint
 int g_sort_blocks_per_sm = 4;   // resident onesweep blocks per SM (set with the attributes)
 
 cudaError_t sort_set_attributes() {
-  cudaError_t e = cudaFuncSetAttribute(k_onesweep<true>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                       cudaSharedmemCarveoutMaxShared);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_onesweep<false>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             cudaSharedmemCarveoutMaxShared);
+  const void* fns[] = {(const void*)k_onesweep<true>, (const void*)k_onesweep<false>};
+  for (const void* f : fns) {
+    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sizeof(SortTile)));
+    if (e != cudaSuccess) return e;
+  }
   int per_sm = 0;
-  if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_onesweep<false>, kSortThreads, 0);
+  const cudaError_t e =
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_onesweep<false>, kSortThreads, sizeof(SortTile));
   if (e == cudaSuccess && per_sm > 0) g_sort_blocks_per_sm = per_sm;
   return e;
 }
@@ -300,7 +322,7 @@ cudaError_t launch_sort(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1, 
     if (epoch == 0) epoch = 1;
     const uint32_t ep = epoch;
     const auto kernel = p == 0 && implicit_vals ? k_onesweep<true> : k_onesweep<false>;
-    kernel<<<grid, kSortThreads, 0, st>>>(ki, vi, ko, vo, n_dev, cap, dg, p, bits_dev, sc.hist + kBins * p, sc.status,
+    kernel<<<grid, kSortThreads, sizeof(SortTile), st>>>(ki, vi, ko, vo, n_dev, cap, dg, p, bits_dev, sc.hist + kBins * p, sc.status,
                                           sc.tile_counters + p, ep, err_flag);
     ++*launches;
     e = cudaGetLastError();

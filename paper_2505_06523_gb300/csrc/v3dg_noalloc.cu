@@ -66,6 +66,7 @@ extern "C" v3dg_status v3dg_sort_pairs_noalloc(uint32_t* keys, uint32_t* vals, u
     if (!g_base[dev]) {
       void* p = nullptr;
       if (cudaGetSymbolAddress(&p, g_scratch) != cudaSuccess || !p) return V3DG_ECUDA;
+      if (sort_set_attributes() != cudaSuccess) return V3DG_ECUDA;   // (no context may have been created)
       g_base[dev] = p;
     }
     base = g_base[dev];
