@@ -2,7 +2,8 @@
 // (Sec. 3.3 Fig. 4, Sec. 3.4), with stable stream compaction of the cut in (instance, node) order.
 //
 // A block covers 2048 consecutive nodes of one instance, 8 per thread (node = base + i * 256 +
-// thread).  Blocks take virtual tile ids from an atomic counter, compact their selected nodes in
+// thread), or 256 of them, one per thread, for scenes of so few nodes that the larger blocks would not
+// fill the GPU (one asset of 20,837 nodes: 22 us with 11 blocks, and 8 us less with 82).  Blocks take virtual tile ids from an atomic counter, compact their selected nodes in
 // (item, warp, lane) order -- which is node order -- and find their output offset with a bounded
 // decoupled look-back, so the cut is written in one pass.
 #include "dev_common.cuh"
@@ -11,7 +12,7 @@ namespace v3dg {
 namespace {
 
 constexpr int kSelThreads = 256;
-constexpr int kSelItems = 8;
+constexpr int kSelMaxItems = 8;
 constexpr int kSelWarps = kSelThreads / 32;
 constexpr float kEps = 5.9604645e-08f;  // 2^-24
 
@@ -86,15 +87,17 @@ __device__ __forceinline__ bool cull_node(const float4 b, float sig, const InstF
   return false;
 }
 
+template <int kSelItems>
 __global__ void __launch_bounds__(kSelThreads)
 k_select(const InstFrame* __restrict__ inst, int n_inst, const AssetDev* __restrict__ assets, int node_blocks,
          CamConst cam, int mode, uint2* __restrict__ out, uint32_t cap, uint32_t* __restrict__ frame,
          uint32_t tc_slot, uint64_t* __restrict__ status, uint32_t epoch) {
   __shared__ uint32_t s_tile, s_excl, s_total;
-  __shared__ uint32_t s_cnt[kSelItems * kSelWarps];   // per (item, warp): selected count, then offset
+  __shared__ uint32_t s_cnt[kSelMaxItems * kSelWarps];   // per (item, warp): selected count, then offset
   __shared__ uint32_t s_gauss[kSelWarps];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (threadIdx.x == 0) s_tile = atomicAdd(frame + kTileCounters + tc_slot, 1u);
+  if (threadIdx.x >= kSelItems * kSelWarps && threadIdx.x < kSelMaxItems * kSelWarps) s_cnt[threadIdx.x] = 0;
   __syncthreads();
   const uint32_t tile = s_tile;
   const uint32_t ntiles = uint32_t(n_inst) * uint32_t(node_blocks);
@@ -307,13 +310,20 @@ cudaError_t launch_select_topdown(const InstFrame* inst, int n_inst, const Asset
   return cudaGetLastError();
 }
 
-cudaError_t launch_select(const InstFrame* inst, int n_inst, const AssetDev* assets, int node_blocks,
+int select_items(uint64_t instances, uint32_t max_nodes, int sm_count) {
+  const uint64_t blocks = instances * ((max_nodes + kSelMaxItems * kSelThreads - 1) / (kSelMaxItems * kSelThreads));
+  return blocks < 2u * uint64_t(sm_count) ? 1 : kSelMaxItems;
+}
+
+cudaError_t launch_select(const InstFrame* inst, int n_inst, const AssetDev* assets, uint32_t max_nodes, int items,
                           const CamConst& cam, int mode, uint2* out, uint32_t cap, uint32_t* frame,
                           uint32_t tile_counter_slot, uint64_t* status, uint32_t epoch, cudaStream_t st) {
+  const int node_blocks = int((max_nodes + items * kSelThreads - 1) / (items * kSelThreads));
   const uint32_t blocks = uint32_t(n_inst) * uint32_t(node_blocks);
   if (blocks == 0) return cudaSuccess;
-  k_select<<<blocks, kSelThreads, 0, st>>>(inst, n_inst, assets, node_blocks, cam, mode, out, cap, frame,
-                                           tile_counter_slot, status, epoch);
+  const auto kernel = items == 1 ? k_select<1> : k_select<kSelMaxItems>;
+  kernel<<<blocks, kSelThreads, 0, st>>>(inst, n_inst, assets, node_blocks, cam, mode, out, cap, frame,
+                                         tile_counter_slot, status, epoch);
   return cudaGetLastError();
 }
 

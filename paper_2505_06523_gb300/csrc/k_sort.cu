@@ -28,6 +28,7 @@ static_assert(kSortThreads >= kBins, "one thread per digit");
 // keys -- depths of one cluster, tiles of one Gaussian -- coincide), which keeps shared-memory
 // atomics on the few hot bins of the high digits from serialising.
 constexpr int kHistRun = 16;
+constexpr uint32_t kHistShort = 1u << 20;   // fewer keys than this: runs of four, so that more threads take part
 
 // The digits of a sort: pass p covers `width` bits from begin + p * width (the last one what is left
 // of them).  On the device, bits_dev replaces the host's bit range.
@@ -49,7 +50,8 @@ k_hist(const uint32_t* __restrict__ keys, const uint32_t* __restrict__ n_dev, ui
        const uint32_t* __restrict__ bits_dev, uint32_t* __restrict__ hist) {
   __shared__ uint32_t sh[4][kBins];
   const uint32_t n = min(*n_dev, cap);
-  if (uint64_t(blockIdx.x) * blockDim.x * kHistRun >= n) return;   // no run for this block
+  const uint32_t run = n < kHistShort ? 4u : uint32_t(kHistRun);
+  if (uint64_t(blockIdx.x) * blockDim.x * run >= n) return;   // no run for this block
   dg = sort_digits(dg, bits_dev);
   const int passes = dg.passes;
   for (int i = threadIdx.x; i < 4 * kBins; i += blockDim.x) sh[i / kBins][i % kBins] = 0;
@@ -61,20 +63,21 @@ k_hist(const uint32_t* __restrict__ keys, const uint32_t* __restrict__ n_dev, ui
     sh_[p] = dg.begin + dg.width * p;
     m[p] = (1u << min(max(dg.end - sh_[p], 0), dg.width)) - 1u;
   }
-  const uint32_t runs = (n + kHistRun - 1) / kHistRun;
+  const uint32_t runs = (n + run - 1) / run;
   const bool aligned = (reinterpret_cast<uintptr_t>(keys) & 15u) == 0;
   for (uint32_t r = blockIdx.x * blockDim.x + threadIdx.x; r < runs; r += gridDim.x * blockDim.x) {
-    const uint32_t i0 = r * kHistRun;
+    const uint32_t i0 = r * run;
     uint32_t cur[4], cnt[4];
 #pragma unroll
     for (int p = 0; p < 4; ++p) {
       cur[p] = 0xFFFFFFFFu;
       cnt[p] = 0;
     }
-    if (aligned && i0 + kHistRun <= n) {   // a full run: four 16-byte loads
+    if (aligned && i0 + run <= n) {   // a full run: 16-byte loads
       const uint4* v = reinterpret_cast<const uint4*>(keys + i0);
 #pragma unroll
       for (int q = 0; q < kHistRun / 4; ++q) {
+        if (4u * q >= run) break;
         const uint4 k4 = v[q];
         const uint32_t kk[4] = {k4.x, k4.y, k4.z, k4.w};
 #pragma unroll
@@ -92,7 +95,7 @@ k_hist(const uint32_t* __restrict__ keys, const uint32_t* __restrict__ n_dev, ui
           }
       }
     } else {
-      for (uint32_t i = i0; i < min(i0 + kHistRun, n); ++i) {
+      for (uint32_t i = i0; i < min(i0 + run, n); ++i) {
         const uint32_t k = keys[i];
 #pragma unroll
         for (int p = 0; p < 4; ++p) {

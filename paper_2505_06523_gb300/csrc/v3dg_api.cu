@@ -82,7 +82,8 @@ struct Pipe {
   uint32_t n_views = 1;        // cameras of the current frame (same intrinsics and image size)
   int color_formats = 1;       // colour storage formats of the current instances' assets (bit 0 FP32, bit 1 FP16)
   uint32_t distinct_assets = 0;   // assets drawn by the current instance frames
-  int node_blocks = 0;
+  uint32_t max_nodes = 0;   // of the loaded assets
+  int select_items = 8;     // nodes per thread of the flat selection
 
   DevBuf d_inst;
   InstFrame* h_inst = nullptr;
@@ -303,7 +304,7 @@ v3dg_status ensure_work(Pipe* c) {
   ST(ensure(c, c->d_pv1, 4 * PP));
   const uint64_t sort_tiles = (std::max<uint64_t>(S, PP) + kSortTile - 1) / kSortTile;
   uint64_t words = sort_tiles * 256;
-  words = std::max<uint64_t>(words, uint64_t(c->n_inst_frame) * uint64_t(std::max(c->node_blocks, 1)));
+  words = std::max<uint64_t>(words, uint64_t(c->n_inst_frame) * (c->max_nodes / (256u * uint32_t(c->select_items)) + 1u));
   words = std::max<uint64_t>(words, (uint64_t(S) + 1023) / 1024);
   ST(ensure_status(c, words));
   ST(ensure(c, c->d_hist, sizeof(uint32_t) * kHistWords));
@@ -397,7 +398,8 @@ v3dg_status setup_views(Pipe* c, const ViewSpec* views, uint32_t n_views) {
 
   uint32_t max_nodes = 0;
   for (auto& a : c->ctx->assets) max_nodes = std::max(max_nodes, a.n_nodes);
-  c->node_blocks = int((max_nodes + 2047) / 2048);   // k_select covers 2048 nodes per block
+  c->max_nodes = max_nodes;
+  c->select_items = select_items(nf, max_nodes, c->ctx->sm_count);
   c->n_inst_frame = nf;
   c->n_views = n_views;
   c->frame_asset.resize(nf);
@@ -527,8 +529,8 @@ v3dg_status launch_selection(Pipe* c, int mode, uint2* out, uint32_t cap, uint32
                              c->stream, &nl));
     c->ctx->launches += nl;
   } else {
-    CU(launch_select(P<InstFrame>(c->d_inst), int(c->n_inst_frame), P<AssetDev>(c->ctx->d_assets), c->node_blocks, c->cc,
-                     mode, out, cap, frame, 0, P<uint64_t>(c->d_status), next_epoch(c), c->stream));
+    CU(launch_select(P<InstFrame>(c->d_inst), int(c->n_inst_frame), P<AssetDev>(c->ctx->d_assets), c->max_nodes,
+                     c->select_items, c->cc, mode, out, cap, frame, 0, P<uint64_t>(c->d_status), next_epoch(c), c->stream));
     ++c->ctx->launches;
   }
   return V3DG_OK;
@@ -743,7 +745,7 @@ void drop_graph(Pipe* c) {
 // each replay): sizes, capacities, buffer addresses, camera constants, options and outputs.
 std::vector<uint64_t> graph_key(Pipe* c, float* rgb, float* t_out) {
   const v3dg_ctx* ctx = c->ctx;
-  std::vector<uint64_t> k = {c->n_inst_frame, c->n_views, uint64_t(c->node_blocks), c->cap_nodes, c->cap_pairs,
+  std::vector<uint64_t> k = {c->n_inst_frame, c->n_views, c->max_nodes, uint64_t(c->select_items), c->cap_nodes, c->cap_pairs,
                              c->cap_slots, c->status_words, uint64_t(uintptr_t(rgb)), uint64_t(uintptr_t(t_out)),
                              uint64_t(use_topdown(c)), uint64_t(use_project_order(c)), uint64_t(slab_count(c)),
                              uint64_t(ctx->blend_batch),

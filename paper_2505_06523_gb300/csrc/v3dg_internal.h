@@ -136,8 +136,10 @@ cudaError_t launch_check_wait(uint64_t* status, uint32_t epoch, uint32_t spin_li
 
 // ---------------------------------------------------------------- launch functions (return cudaError)
 // Selection (Sec. 3.3-3.4).  mode 0: render list (cut minus the visibility cull) + counters;
-// mode 1: the cut itself (parity read-back).
-cudaError_t launch_select(const InstFrame* inst, int n_inst, const AssetDev* assets, int node_blocks,
+// mode 1: the cut itself (parity read-back).  max_nodes: of the assets; items: nodes per thread, as
+// select_items gives them; status: a word per 256 * items nodes of every instance.
+int select_items(uint64_t instances, uint32_t max_nodes, int sm_count);
+cudaError_t launch_select(const InstFrame* inst, int n_inst, const AssetDev* assets, uint32_t max_nodes, int items,
                           const CamConst& cam, int mode, uint2* out, uint32_t cap, uint32_t* frame,
                           uint32_t tile_counter_slot, uint64_t* status, uint32_t epoch, cudaStream_t st);
 
