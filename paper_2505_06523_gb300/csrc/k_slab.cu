@@ -1,4 +1,4 @@
-// Depth slabs: a frame's visible Gaussians are binned, sorted and blended in up to four slabs, front
+// Depth slabs: a frame's visible Gaussians are binned, sorted and blended in up to six slabs, front
 // to back, and a slab leaves out what only meets tiles whose pixels have all stopped.
 //
 // Why: on a composed scene most of what is visible by projection is hidden.  On the 1080p crowd (73M
@@ -7,7 +7,7 @@
 // nearest quarter, 10M of 55M.  Sorting, expanding and sorting again what cannot change a pixel was
 // more than half of those stages.  The image does not change: a pixel that has stopped takes no
 // further record, and a slab's records come in the same order as in the whole list.
-// Measured on a GB300, one slab -> four: depth sort, binning, tile sort and ranges of the 1080p crowd
+// Measured on a GB300, one slab -> several: depth sort, binning, tile sort and ranges of the 1080p crowd
 // 5.2 -> 2.7 ms (its blend 1.3 -> 2.0 ms: each slab waits for its longest tile), of the 5000-instance
 // 4K crowd 51 -> 13.5 ms, of 16 crowd views 50 -> 27 ms; one asset filling 1080p (31M pairs of 225k
 // Gaussians, all tiles finished after 3% of them) 2.4 -> 0.65 ms.
@@ -45,9 +45,16 @@ k_frame_init(uint32_t* __restrict__ frame, uint32_t* __restrict__ hist, uint32_t
   }
 }
 
-// The slabs' limits: at the depths where 1/12, 3/10 and 1/2 of the frame's pairs lie in front (the first slab
-// is small, because everything in it is kept; the last takes what the first three have not hidden).
-// A slab more would leave out a few more pairs and costs about 20 launches.
+// The slabs' limits: at the depths where these thousandths of the frame's pairs lie in front (the first slab
+// is small, because everything in it is kept; the last takes what the others have not hidden).  A slab
+// more leaves out a few more pairs and costs about 20 launches and a tail of the blend, so larger
+// frames take more of them (see slab_count).  Whole frames by number of slabs, 3 / 4 / 6: one asset filling
+// 1080p (31M pairs) 0.93 / 1.03 / 1.29 ms, crowd at 1080p (157M) 6.46 / 6.06 / 6.84 ms, 5000 instances at
+// 4K (1.9G) 29.8 / 27.1 / 25.5 ms, 16 crowd views (1.3G) 53.6 / 47.8 / 45.2 ms.  Limits tried with four:
+// {20, 80, 250}, {30, 120, 350}, {40, 160, 400}, {60, 200, 400}, {70, 250, 450}, {100, 300, 500}: the crowd 7.32,
+// 6.68, 6.87, 6.85, 6.32, 6.15 ms.
+__constant__ const uint32_t kLimits3[2] = {100, 350}, kLimits4[3] = {83, 300, 500}, kLimits6[5] = {50, 140, 280, 430, 600};
+
 __global__ void __launch_bounds__(256)
 k_slab_limits(uint32_t* __restrict__ frame, const uint32_t* __restrict__ depth_hist, int slabs, uint32_t cap_pairs) {
   __shared__ uint32_t s_scan[9], s_edge[kMaxSlabs + 1];
@@ -65,7 +72,12 @@ k_slab_limits(uint32_t* __restrict__ frame, const uint32_t* __restrict__ depth_h
       sum += v[i];
     }
     uint32_t all, excl = block_exclusive_scan<8>(sum, s_scan, &all);
-    const uint32_t target[kMaxSlabs - 1] = {max(all / 12u, 1u), max(uint32_t(uint64_t(all) * 3u / 10u), 1u), max(all / 2u, 1u)};
+    // thousandths of the pairs
+    const uint32_t* const limits = slabs <= 3 ? kLimits3 : slabs == 4 ? kLimits4 : kLimits6;
+    uint32_t target[kMaxSlabs - 1];
+#pragma unroll
+    for (int k = 0; k < kMaxSlabs - 1; ++k)
+      target[k] = k < slabs - 1 ? max(uint32_t(uint64_t(all) * limits[k] / 1000u), 1u) : 0u;
 #pragma unroll
     for (int i = 0; i < kPer; ++i) {
       for (int k = 0; k < slabs - 1; ++k)

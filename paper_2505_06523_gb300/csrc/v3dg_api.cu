@@ -53,7 +53,7 @@ constexpr uint32_t kInitNodes = 1u << 14;
 constexpr uint32_t kInitPairs = 1u << 22;
 constexpr uint32_t kMaxNodes = 1u << 25;               // render-list clusters: at most 2^31 slots
 constexpr uint32_t kMaxPairs = 0xFFFFFFFFu - 4096u;    // pair indices are 32-bit (a sort tile of headroom)
-constexpr uint32_t kManyPairs = 1u << 24;              // pairs of the previous frame from which one is taken in slabs
+constexpr uint64_t kManyPairs = 1u << 26;              // pairs of the previous frame from which one is taken in slabs
 enum { kStageSelect = 0, kStageProject, kStageDepthSort, kStageBin, kStageTileSort, kStageRanges, kStageBlend, kStages };
 
 }  // namespace
@@ -104,7 +104,8 @@ struct Pipe {
   // the marked slots, and their counts
   DevBuf d_tlive, d_state, d_marks;
   bool tiles_in1 = false;
-  uint32_t pairs_hint = 0;   // pairs of the previous frame (of one still running: of the one before)
+  // pairs and visible Gaussians of the previous frame (of one still running: of the one before)
+  uint32_t pairs_hint = 0, visible_hint = 0;
   int slabs = 1;             // depth slabs of the last rendered frame
   bool full_lists = false;   // the sorted Gaussians and pairs of the whole frame are on the device
   uint32_t epoch = 1;
@@ -242,13 +243,19 @@ constexpr int kFrameSorts = 1 + 2 * kMaxSlabs;
 constexpr uint32_t kSortHist = kMaxSlabs * kItemClasses, kDepthHist = kSortHist + kFrameSorts * kSortPasses * kSortBins,
                    kHistWords = kDepthHist + kDepthBins;
 
-// Depth slabs of the next frame (see k_slab.cu): several when the pipe's previous frame had at least
-// kManyPairs pairs, one otherwise and for blend variant 1, which keeps no state between slabs.  The
-// image does not depend on it.  Several slabs of a small frame cost up to 0.3 ms of launches and of
-// tails (measured on the asset 50 units away, 0.5M pairs: 0.53 -> 0.85 ms); frames of 30M pairs and
-// more take 0.4 to 0.8 times as long (see k_slab.cu).  The frame's own pair count is not known when its
-// launches are made, and consecutive frames of a viewer or a batch are alike.
-int slab_count(const Pipe* c) { return c->pairs_hint >= kManyPairs && c->ctx->blend_mode == 0 ? kMaxSlabs : 1; }
+// Depth slabs of the next frame (see k_slab.cu), by the pairs and visible Gaussians of the pipe's
+// previous frame: the frame's own are not known when its launches are made, and consecutive frames of
+// a viewer or a batch are alike.  The image does not depend on it.  One below kManyPairs, and for blend
+// variant 1, which keeps no state between slabs: each slab costs about 20 launches and a tail of the
+// blend (crowds of 30 to 60M pairs, one slab / three: 2.92 / 3.12 and 4.52 / 4.66 ms).  Frames whose
+// Gaussians cover many tiles each (a camera close to an asset) hide theirs early, so they take three
+// from a quarter of that on (one asset at 1.7 and 2 units, 33 and 36M pairs: 1.14 / 1.08 and 1.31 / 1.26 ms).
+int slab_count(const Pipe* c) {
+  const uint64_t pairs = c->pairs_hint;
+  if (c->ctx->blend_mode != 0) return 1;
+  if (pairs < kManyPairs) return pairs >= kManyPairs / 4 && pairs >= 16ull * c->visible_hint ? 3 : 1;
+  return pairs < 2 * kManyPairs ? 3 : pairs < 8 * kManyPairs ? 4 : kMaxSlabs;
+}
 
 TileLive tile_live(Pipe* c, int slabs) {
   TileLive l{};
@@ -370,7 +377,11 @@ v3dg_status setup_views(Pipe* c, const ViewSpec* views, uint32_t n_views) {
     nf64 += views[v].n;
   }
   const v3dg_camera* cam = views[0].cam;
-  if (c->rendered) c->pairs_hint = *const_cast<const volatile uint32_t*>(c->h_frame + kPairs);
+  if (c->rendered) {
+    const volatile uint32_t* f = c->h_frame;
+    c->pairs_hint = f[kPairs];
+    c->visible_hint = f[kVisible];
+  }
   if (c->ctx->assets.empty()) return fail(c, V3DG_ENOTFOUND, "no hierarchy loaded");
   const uint64_t tiles = uint64_t((cam->width + kTile - 1) / kTile) * uint64_t((cam->height + kTile - 1) / kTile);
   if (tiles * n_views > uint64_t(kMaxTiles))
@@ -705,6 +716,7 @@ v3dg_status grow_and_reselect(Pipe* c) {
   const uint32_t* f = c->h_frame;
   bool grew = false;
   c->pairs_hint = f[kPairs];
+  c->visible_hint = f[kVisible];
   if (f[kRenderNodes] > c->cap_nodes) {
     if (f[kRenderNodes] > kMaxNodes)
       return fail(c, V3DG_EOVERFLOW, "render list of %u nodes exceeds the limit", f[kRenderNodes]);

@@ -89,7 +89,7 @@ enum Counter : int {
 // A frame is binned, sorted and blended in one or more depth slabs, front to back: slab k holds the
 // visible Gaussians with depth keys in [lo, hi).  From the second slab on, Gaussians and pairs that
 // only meet tiles whose pixels have all stopped are left out (they cannot change a pixel).
-constexpr int kMaxSlabs = 4, kSlabWords = 24, kFrameWords = kSlabBase + kMaxSlabs * kSlabWords;
+constexpr int kMaxSlabs = 6, kSlabWords = 24, kFrameWords = kSlabBase + kMaxSlabs * kSlabWords;
 enum SlabWord : int {
   kSlabCount = 0,          // Gaussians picked
   kSlabPairs,              // their pairs

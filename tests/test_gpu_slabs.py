@@ -1,4 +1,4 @@
-"""Frames taken in depth slabs (at least 2^24 pairs) against the same frames taken in one."""
+"""Frames taken in depth slabs (2^26 pairs, or 2^24 of large boxes) against the same frames taken in one."""
 import dataclasses
 
 import numpy as np
@@ -16,12 +16,17 @@ def _scene(n, spread):
                             rng.uniform(0.7, 1.4, n))
 
 
-@pytest.mark.parametrize("n,spread,width,height,views,graphs", [
-    (12, 0.5, 1920, 1080, 1, 0),    # a pile next to the camera: large boxes, early stops
-    (40, 6.0, 1001, 563, 3, 0),     # ragged images, several views
-    (40, 6.0, 1001, 563, 3, 1),     # the same, captured
+def _in_slabs(stats, at_least):
+    return stats["pairs"] >= max(at_least, 1 << 24) and (stats["pairs"] >= 1 << 26 or stats["pairs"] >= 16 * stats["visible"])
+
+
+@pytest.mark.parametrize("n,spread,width,height,fov,views,graphs,at_least", [
+    (12, 0.5, 1920, 1080, 70.0, 1, 0, 1 << 24),    # a pile next to the camera: large boxes, early stops: three slabs
+    (12, 0.5, 1001, 563, 40.0, 3, 0, 1 << 24),     # ragged images, several views
+    (12, 0.5, 1001, 563, 40.0, 3, 1, 1 << 24),     # the same, captured
+    (40, 3.0, 1601, 901, 50.0, 8, 0, 1 << 27),     # four slabs
 ])
-def test_slabs_change_nothing(tiny_asset, n, spread, width, height, views, graphs):
+def test_slabs_change_nothing(tiny_asset, n, spread, width, height, fov, views, graphs, at_least):
     """Blend variant 1 keeps its frames in one slab and gives the same image bit for bit; the sorted lists that the
     read-backs return are those of the whole frame either way."""
     import __graft_entry__
@@ -29,7 +34,7 @@ def test_slabs_change_nothing(tiny_asset, n, spread, width, height, views, graph
     from paper_2505_06523_gb300 import Context
     from paper_2505_06523_gb300._native import V3DG_OPT_BLEND_MODE, V3DG_OPT_GRAPHS
     inst = _scene(n, spread)
-    cams = [scenes.look_at((0.3 * v, -2.0 - spread, 0.5), (0.0, 0.0, 0.0), width, height, 70.0) for v in range(views)]
+    cams = [scenes.look_at((0.3 * v, -2.0 - spread, 0.5), (0.0, 0.0, 0.0), width, height, fov) for v in range(views)]
     got = []
     with Context(0) as ctx:
         ctx.set_option(V3DG_OPT_GRAPHS, graphs)
@@ -46,7 +51,7 @@ def test_slabs_change_nothing(tiny_asset, n, spread, width, height, views, graph
             again = ctx.render(want_T=True)   # the lists were made again in between
             assert (again[0].cpu().numpy() == got[-1]["rgb"]).all()
     one, slabs = got
-    assert one["stats"]["pairs"] >= 1 << 24, "too few pairs for slabs"
+    assert _in_slabs(one["stats"], at_least), one["stats"]
     assert one["stats"] == {**slabs["stats"]}
     assert float(np.abs(one["rgb"]).sum()) > 0 and (one["T"] < 1e-3).any()
     for k in one:
@@ -74,5 +79,27 @@ def test_slabs_with_depths_in_one_bin(tiny_asset):
                 ctx.select(cam, 0.25)
                 rgb, T = ctx.render(want_T=True)
             imgs.append((rgb.cpu().numpy(), T.cpu().numpy()))
-        assert ctx.frame_stats()["pairs"] >= 1 << 24
+        assert _in_slabs(ctx.frame_stats(), 1 << 24)
     assert (imgs[0][0] == imgs[1][0]).all() and (imgs[0][1] == imgs[1][1]).all()
+
+
+def test_most_slabs(tiny_asset):
+    """The most slabs (2^29 pairs: sixteen views of a pile): images and transmittances as in one slab, bit for bit."""
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2505_06523_gb300 import Context
+    from paper_2505_06523_gb300._native import V3DG_OPT_BLEND_MODE
+    inst = _scene(30, 0.6)
+    cams = [scenes.look_at((0.2 * v, -2.6, 0.1 * v), (0.0, 0.0, 0.0), 1920, 1080, 70.0) for v in range(16)]
+    imgs = []
+    with Context(0) as ctx:
+        ctx.load_hierarchy(tiny_asset)
+        ctx.set_instances(inst)
+        for mode in (1, 0):
+            ctx.set_option(V3DG_OPT_BLEND_MODE, mode)
+            for _ in range(2):
+                ctx.select_views(cams, 0.25)
+                rgb, T = ctx.render(want_T=True)
+            imgs.append((rgb.clone(), T.clone()))
+        assert _in_slabs(ctx.frame_stats(), 1 << 29), ctx.frame_stats()
+    assert bool((imgs[0][0] == imgs[1][0]).all()) and bool((imgs[0][1] == imgs[1][1]).all())
