@@ -102,69 +102,9 @@ k_slab_limits(uint32_t* __restrict__ frame, const uint32_t* __restrict__ depth_h
   }
 }
 
-constexpr int kPickThreads = 256, kPickItems = 16, kPickTile = kPickThreads * kPickItems;
-constexpr int kPickWarps = kPickThreads / 32;
-
-// One slab: stable compaction of the visible slots.  A block takes 4096 consecutive slots, each warp
-// 512 of them (item-major, so every load is one line), and finds its first output position with a
-// bounded look-back.
-__global__ void __launch_bounds__(kPickThreads)
-k_pick(const uint32_t* __restrict__ keys, uint32_t cap_nodes, uint32_t* __restrict__ kout, uint32_t* __restrict__ vout,
-       uint32_t* __restrict__ frame, uint32_t* __restrict__ slab, uint64_t* __restrict__ status, uint32_t epoch) {
-  __shared__ uint32_t s_tile, s_base;
-  __shared__ uint32_t s_warp[kPickWarps];
-  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-  const uint32_t n = min(frame[kRenderNodes], cap_nodes) * uint32_t(kSlots);
-  const uint32_t ntiles = (n + kPickTile - 1) / kPickTile;
-  const uint32_t lo = slab[kSlabLo], hi = slab[kSlabHi];
-  if (lo >= hi || blockIdx.x >= ntiles) return;
-  for (;;) {   // persistent blocks: tiles in the order of an atomic counter
-    if (threadIdx.x == 0) s_tile = atomicAdd(slab + kSlabPickTile, 1u);
-    __syncthreads();
-    const uint32_t tile = s_tile;
-    if (tile >= ntiles) return;
-    const uint32_t base = tile * kPickTile + warp * (kPickItems * 32) + lane;
-    uint32_t key[kPickItems], count = 0;
-#pragma unroll
-    for (int i = 0; i < kPickItems; ++i) key[i] = base + i * 32 < n ? keys[base + i * 32] : 0xFFFFFFFFu;
-#pragma unroll
-    for (int i = 0; i < kPickItems; ++i) count += __popc(__ballot_sync(0xffffffffu, key[i] >= lo && key[i] < hi));
-    if (lane == 0) s_warp[warp] = count;
-    __syncthreads();
-    uint32_t before = 0, total = 0;
-#pragma unroll
-    for (int w = 0; w < kPickWarps; ++w) {
-      const uint32_t c = s_warp[w];
-      if (w < int(warp)) before += c;
-      total += c;
-    }
-    if (warp == 0) {
-      const uint32_t b = chained_exclusive_warp(status, tile, total, epoch, frame + kTimeout);
-      if (lane == 0) {
-        s_base = b;
-        if (tile == ntiles - 1) slab[kSlabCount] = b + total;
-      }
-    }
-    __syncthreads();
-    uint32_t pos = s_base + before;
-#pragma unroll
-    for (int i = 0; i < kPickItems; ++i) {
-      const bool in = key[i] >= lo && key[i] < hi;
-      const uint32_t b = __ballot_sync(0xffffffffu, in);
-      if (in) {
-        const uint32_t p = pos + __popc(b & lanemask_lt());
-        kout[p] = key[i] - lo;
-        vout[p] = base + i * 32;
-      }
-      pos += __popc(b);
-    }
-    __syncthreads();   // the tile's shared words are consumed
-  }
-}
-
-// Several slabs: the same compaction in three launches without a chain of waits (with the look-back
-// of k_pick, four slabs of the 1080p crowd took 1.5 ms: a thousand tiles in flight wait for one
-// another).  k_mark: a warp takes 32 nodes, drops those whose depth range misses the slab, and writes
+// Several slabs: the stable compaction of a slab's slots in three launches without a chain of waits (with
+// a look-back, four slabs of the 1080p crowd took 1.5 ms: a thousand tiles in flight wait for one
+// another).  (One slab takes none: the depth sort's first pass reads the slots themselves.)  k_mark: a warp takes 32 nodes, drops those whose depth range misses the slab, and writes
 // a bit per slot of the others: in the slab and (kFilter) on a live tile; a block's 256 nodes leave
 // their count.  k_mark_scan: the counts' prefix sums, by one block.  k_gather: the marked slots.
 constexpr int kMarkNodes = 256;   // nodes of a block
@@ -356,16 +296,6 @@ cudaError_t launch_frame_init(uint32_t* frame, uint32_t* hist, uint32_t hist_wor
 cudaError_t launch_slab_limits(uint32_t* frame, const uint32_t* depth_hist, int slabs, uint32_t cap_pairs,
                                cudaStream_t st) {
   k_slab_limits<<<1, 256, 0, st>>>(frame, depth_hist, slabs, cap_pairs);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_pick(const uint32_t* keys, uint32_t cap_nodes, uint32_t* kout, uint32_t* vout, uint32_t* frame,
-                        int slab, uint64_t* status, uint32_t epoch, int sm_count, cudaStream_t st) {
-  const uint64_t tiles = (uint64_t(cap_nodes) * kSlots + kPickTile - 1) / kPickTile;
-  const uint32_t grid = uint32_t(std::min<uint64_t>(tiles, uint64_t(sm_count) * 6u));
-  if (!grid) return cudaSuccess;
-  k_pick<<<grid, kPickThreads, 0, st>>>(keys, cap_nodes, kout, vout, frame, frame + kSlabBase + slab * kSlabWords, status,
-                                        epoch);
   return cudaGetLastError();
 }
 

@@ -582,16 +582,15 @@ v3dg_status enqueue_slab_lists(Pipe* c, int slab, bool filter, const TileLive& l
     CU(launch_pick_slab(P<uint32_t>(c->d_keys0), P<uint2>(c->d_rect), c->cap_nodes, P<uint2>(c->d_list), inst_views, live,
                         filter, depth_range, marks, reinterpret_cast<uint32_t*>(marks + c->cap_nodes),
                         P<uint32_t>(c->d_keys1), P<uint32_t>(c->d_vals1), frame, slab, sm, c->stream));
-    c->ctx->launches += 2;
-  } else {
-    CU(launch_pick(P<uint32_t>(c->d_keys0), c->cap_nodes, P<uint32_t>(c->d_keys1), P<uint32_t>(c->d_vals1), frame, slab,
-                   P<uint64_t>(c->d_status), next_epoch(c), sm, c->stream));
+    c->ctx->launches += 3;
   }
   bool unused = false;
   int nl = 0;
+  const SortSlots slots{P<uint32_t>(c->d_keys0), frame, c->cap_nodes, words};   // (one slab)
   CU(launch_sort(P<uint32_t>(c->d_keys1), P<uint32_t>(c->d_vals1), P<uint32_t>(c->d_keys2), P<uint32_t>(c->d_vals0),
                  words + kSlabCount, c->cap_slots, 0, 32, false, sort_scratch(c, 1 + 2 * slab, true, words + kSlabDepthTiles),
-                 frame + kTimeout, c->epoch, sm, c->stream, &unused, &nl, words + kSlabBits));
+                 frame + kTimeout, c->epoch, sm, c->stream, &unused, &nl, words + kSlabBits,
+                 live.bits ? nullptr : &slots));
   next_epoch(c);
   stage_event(c, 2 + 6 * slab + 1);
   CU(launch_expand(P<uint32_t>(c->d_vals1), P<uint32_t>(c->d_vals0), P<uint2>(c->d_rect), c->cap_slots, c->cap_pairs,
@@ -609,7 +608,7 @@ v3dg_status enqueue_slab_lists(Pipe* c, int slab, bool filter, const TileLive& l
   stage_event(c, 2 + 6 * slab + 3);
   CU(launch_ranges(P<uint32_t>(c->tiles_in1 ? c->d_pk1 : c->d_pk0), c->cap_pairs, frame, slab,
                    P<uint2>(c->d_ranges) + size_t(slab) * size_t(n_tiles), n_tiles, sm, c->stream));
-  c->ctx->launches += uint64_t(nl) + 4;
+  c->ctx->launches += uint64_t(nl) + 3;
   return V3DG_OK;
 }
 

@@ -93,8 +93,7 @@ constexpr int kMaxSlabs = 6, kSlabWords = 24, kFrameWords = kSlabBase + kMaxSlab
 enum SlabWord : int {
   kSlabCount = 0,          // Gaussians picked
   kSlabPairs,              // their pairs
-  kSlabPickTile,           // tile counters of the kernels
-  kSlabDepthTiles,         // 4 words
+  kSlabDepthTiles,         // tile counters of the kernels (4 words)
   kSlabExpandTile = kSlabDepthTiles + 4,
   kSlabPairTiles,          // 4 words
   kSlabBlendItem = kSlabPairTiles + 4,
@@ -198,10 +197,7 @@ cudaError_t launch_frame_init(uint32_t* frame, uint32_t* hist, uint32_t hist_wor
 // After the projection: the frame's pair count and overflow, and the limits of its `slabs` slabs.
 cudaError_t launch_slab_limits(uint32_t* frame, const uint32_t* depth_hist, int slabs, uint32_t cap_pairs,
                                cudaStream_t st);
-// A one-slab frame's visible Gaussians, in slot order: (key - lo, slot).
-cudaError_t launch_pick(const uint32_t* keys, uint32_t cap_nodes, uint32_t* kout, uint32_t* vout, uint32_t* frame,
-                        int slab, uint64_t* status, uint32_t epoch, int sm_count, cudaStream_t st);
-// The same of one of several slabs: keys in [lo, hi) and, with filter, boxes that meet a live tile.
+// The visible Gaussians of one of several slabs, in slot order: (key - lo, slot), keys in [lo, hi) and, with filter, boxes that meet a live tile.
 // depth_range: a conservative depth range per render-list node.  marks, counts: scratch of cap_nodes
 // and ceil(cap_nodes / 256) entries.
 cudaError_t launch_pick_slab(const uint32_t* keys, const uint2* rect, uint32_t cap_nodes, const uint2* list,
@@ -215,6 +211,15 @@ cudaError_t launch_pick_slab(const uint32_t* keys, const uint2* rect, uint32_t c
 // element indices (v0 is not read).  bits_dev (may be NULL): the sort covers key bits
 // [0, *bits_dev) instead, in as few passes as 8-bit digits need (the launches beyond return at
 // once); the result is in (k1, v1) when that number is odd.
+// slots (may be NULL; with bits_dev, no implicit_vals): the first pass reads the slots of a frame's
+// render list instead of (k0, v0): the keys of the visible ones less slab[kSlabLo], their slot numbers
+// as values; slab[kSlabCount] (n_dev) becomes their number.
+struct SortSlots {
+  const uint32_t* keys;    // a key per slot, 0xFFFFFFFF: not visible
+  const uint32_t* frame;
+  uint32_t cap_nodes;
+  uint32_t* slab;
+};
 constexpr int kSortPasses = 4, kSortBins = 256;
 struct SortScratch {
   uint32_t* hist;          // kSortPasses * kSortBins digit counts
@@ -227,7 +232,8 @@ constexpr int kSortThreads = 256, kSortItems = 16, kSortTile = kSortThreads * kS
 cudaError_t launch_sort(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1, const uint32_t* n_dev,
                         uint32_t cap, int begin_bit, int end_bit, bool implicit_vals,
                         const SortScratch& sc, uint32_t* err_flag, uint32_t& epoch, int sm_count,
-                        cudaStream_t st, bool* result_in_1, int* launches, const uint32_t* bits_dev = nullptr);
+                        cudaStream_t st, bool* result_in_1, int* launches, const uint32_t* bits_dev = nullptr,
+                        const SortSlots* slots = nullptr);
 
 // Pair keys: tile id in bits 0..19 (at most 2^20 tiles), then the Gaussian's pixel box clipped
 // to the tile, tile-local and inclusive: rows y0 in bits 20..23 and y1 in 24..27, columns rounded

@@ -1,4 +1,4 @@
-"""Frames taken in depth slabs (2^26 pairs, or 2^24 of large boxes) against the same frames taken in one."""
+"""Frames taken in depth slabs (2^26 pairs, or 2^24 of large boxes) against the same frames taken in one, and the lists of those."""
 import dataclasses
 
 import numpy as np
@@ -103,3 +103,37 @@ def test_most_slabs(tiny_asset):
             imgs.append((rgb.clone(), T.clone()))
         assert _in_slabs(ctx.frame_stats(), 1 << 29), ctx.frame_stats()
     assert bool((imgs[0][0] == imgs[1][0]).all()) and bool((imgs[0][1] == imgs[1][1]).all())
+
+
+@pytest.mark.parametrize("n,distance,away,tau", [
+    (1, 3.0, True, 0.25),     # nothing visible
+    (1, 400.0, False, 64.0),  # one node: a fraction of one sort tile
+    (1, 1.2, False, 1.0),     # part of one asset, many slots outside the image
+    (3, 2.5, False, 0.25),    # several sort tiles
+    (9, 30.0, False, 2.0),
+])
+def test_one_slab_lists(tiny_asset, n, distance, away, tau):
+    """The pair list of a one-slab frame, whose depth sort reads the render list's slots itself, against a stable sort on
+    the host of the projected Gaussians' tiles by (tile, depth), Gaussians in slot order."""
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2505_06523_gb300 import Context
+    target = (0.0, -2.0 * distance, 0.0) if away else (0.0, 0.0, 0.0)
+    with Context(0) as ctx:
+        ctx.load_hierarchy(tiny_asset)
+        ctx.set_instances(_scene(n, 0.5))
+        ctx.select(scenes.look_at((0.0, -distance, 0.3), target, 333, 217, 50.0), tau)
+        ctx.render()
+        proj, pairs, stats = ctx.get_projected(), ctx.get_pairs(), ctx.frame_stats()
+    assert stats["pairs"] < 1 << 24 and (stats["visible"] == 0) == away
+    assert len(proj["local"]) == stats["visible"] and len(pairs["tile"]) == stats["pairs"]
+    tiles_x = (333 + 15) // 16
+    r = proj["rect"].astype(np.int64)   # tiles x0, x1, y0, y1 (inclusive)
+    w, h = r[:, 1] - r[:, 0] + 1, r[:, 3] - r[:, 2] + 1
+    g = np.repeat(np.arange(len(r)), w * h)
+    k = np.arange(len(g)) - np.repeat(np.cumsum(w * h) - w * h, w * h)
+    tile = (r[g, 2] + k // w[g]) * tiles_x + r[g, 0] + k % w[g]
+    order = np.lexsort((g, proj["depth_key"][g], tile))
+    assert (tile[order] == pairs["tile"]).all()
+    for name in ("depth_key", "inst", "local"):
+        assert (proj[name][g[order]] == pairs[name]).all(), name
