@@ -136,11 +136,19 @@ k_hist(const uint32_t* __restrict__ keys, const uint32_t* __restrict__ n_dev, ui
   }
 }
 
+// The words of a standalone sort: n, tile counters and the gave-up flag, and the digit counts.  One
+// launch in place of two memsets and a store (20M pairs, 32 bits: 659 -> 650 us a call; 300k, 13 bits: 72 -> 70).
+__global__ void __launch_bounds__(kBins)
+k_sort_init(uint32_t* __restrict__ words, uint32_t n, uint32_t* __restrict__ hist) {
+  hist[blockIdx.x * kBins + threadIdx.x] = 0;
+  if (blockIdx.x == 0 && threadIdx.x < kSortWords) words[threadIdx.x] = threadIdx.x == 0 ? n : 0u;
+}
+
 // What bounds a pass (20M pairs, ncu): the shared-memory pipe at 72% (38 wavefronts per 32 keys, most of
 // them bank conflicts of the random digits) with 49% of the issue slots, behind it the look-back (9k of
 // a tile's 34k cycles).  Pairs and per-digit words are 8 bytes wide so that ranking takes three shared
 // accesses a key, not five, and reordering one, not two; full tiles test no bounds.  20M pairs, 32 bits:
-// 692 -> 662 us a call, 300k pairs, 13 bits: 84 -> 75 us.  512 threads of 8 keys at 48 warps per SM: 730 us
+// 692 -> 662 us a call, 300k pairs, 13 bits: 84 -> 75 us when they were made.  512 threads of 8 keys at 48 warps per SM: 730 us
 // (more warps wait for the same pipe); 8 status words a look-back round: 686 us.
 // Shared memory of a tile.
 struct SortTile {
@@ -330,6 +338,11 @@ cudaError_t sort_set_attributes() {
   return e;
 }
 
+cudaError_t launch_sort_init(uint32_t* words, uint32_t n, uint32_t* hist, cudaStream_t st) {
+  k_sort_init<<<kSortPasses, kBins, 0, st>>>(words, n, hist);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_sort(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1, const uint32_t* n_dev,
                         uint32_t cap, int begin_bit, int end_bit, bool implicit_vals, const SortScratch& sc,
                         uint32_t* err_flag, uint32_t& epoch, int sm_count, cudaStream_t st, bool* result_in_1,
@@ -343,8 +356,6 @@ cudaError_t launch_sort(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1, 
   // persistent grid: the resident blocks, whatever the capacity (surplus blocks cost launches)
   const uint32_t grid = std::min<uint32_t>(max_tiles, uint32_t(sm_count) * uint32_t(g_sort_blocks_per_sm));
   cudaError_t e = cudaSuccess;
-  if (!sc.hist_zeroed) e = cudaMemsetAsync(sc.hist, 0, sizeof(uint32_t) * kBins * dg.passes, st);
-  if (e != cudaSuccess) return e;
   const SortSlots from = slots ? *slots : SortSlots{};
   if (slots)
     k_hist<true><<<sm_count * 4, 256, 0, st>>>(from.keys, n_dev, cap, dg, bits_dev, sc.hist, from);

@@ -318,12 +318,11 @@ v3dg_status ensure_work(Pipe* c) {
   return V3DG_OK;
 }
 
-// Scratch of the pipe's sort number `which` (each has its own digit counts; zeroed: cleared by the
-// frame's start).
-SortScratch sort_scratch(Pipe* c, int which, bool zeroed, uint32_t* tile_counters) {
+// Scratch of the pipe's sort number `which` (each has its own digit counts, cleared by the frame's
+// start or, for a standalone sort, by launch_sort_init).
+SortScratch sort_scratch(Pipe* c, int which, uint32_t* tile_counters) {
   SortScratch sc;
   sc.hist = P<uint32_t>(c->d_hist) + kSortHist + which * kSortPasses * kSortBins;
-  sc.hist_zeroed = zeroed;
   sc.status = P<uint64_t>(c->d_status);
   sc.max_tiles = c->status_words / 256;
   sc.tile_counters = tile_counters;
@@ -565,8 +564,6 @@ bool use_project_order(const Pipe* c) {
   return c->n_inst_frame >= 2 * uint64_t(std::max<uint32_t>(c->distinct_assets, 1)) && c->n_inst_frame >= 4;
 }
 
-__global__ void k_set_word(uint32_t* p, uint32_t v) { *p = v; }
-
 // One depth slab's Gaussians, depth-sorted, expanded into pairs, tile-sorted, with their tile ranges.
 v3dg_status enqueue_slab_lists(Pipe* c, int slab, bool filter, const TileLive& live) {
   const CamConst& k = c->cc;
@@ -588,7 +585,7 @@ v3dg_status enqueue_slab_lists(Pipe* c, int slab, bool filter, const TileLive& l
   int nl = 0;
   const SortSlots slots{P<uint32_t>(c->d_keys0), frame, c->cap_nodes, words};   // (one slab)
   CU(launch_sort(P<uint32_t>(c->d_keys1), P<uint32_t>(c->d_vals1), P<uint32_t>(c->d_keys2), P<uint32_t>(c->d_vals0),
-                 words + kSlabCount, c->cap_slots, 0, 32, false, sort_scratch(c, 1 + 2 * slab, true, words + kSlabDepthTiles),
+                 words + kSlabCount, c->cap_slots, 0, 32, false, sort_scratch(c, 1 + 2 * slab, words + kSlabDepthTiles),
                  frame + kTimeout, c->epoch, sm, c->stream, &unused, &nl, words + kSlabBits,
                  live.bits ? nullptr : &slots));
   next_epoch(c);
@@ -602,7 +599,7 @@ v3dg_status enqueue_slab_lists(Pipe* c, int slab, bool filter, const TileLive& l
   while ((1 << tile_bits) < n_tiles) ++tile_bits;
   CU(launch_sort(P<uint32_t>(c->d_pk0), P<uint32_t>(c->d_pv0), P<uint32_t>(c->d_pk1), P<uint32_t>(c->d_pv1),
                  words + kSlabPairs, c->cap_pairs, 0, tile_bits, false,
-                 sort_scratch(c, 2 + 2 * slab, true, words + kSlabPairTiles), frame + kTimeout, c->epoch, sm, c->stream,
+                 sort_scratch(c, 2 + 2 * slab, words + kSlabPairTiles), frame + kTimeout, c->epoch, sm, c->stream,
                  &c->tiles_in1, &nl));
   next_epoch(c);
   stage_event(c, 2 + 6 * slab + 3);
@@ -645,7 +642,7 @@ v3dg_status enqueue_render(Pipe* c, float* rgb, float* t_out) {
     bool oin1 = false;
     int nl = 0;
     CU(launch_sort(okeys, okeys + cn, okeys + 2 * cn, okeys + 3 * cn, frame + kRenderNodes, c->cap_nodes, 0,
-                   key_bits - key_shift, true, sort_scratch(c, 0, true, frame + kTileCounters + 11), frame + kTimeout,
+                   key_bits - key_shift, true, sort_scratch(c, 0, frame + kTileCounters + 11), frame + kTimeout,
                    c->epoch, sm, c->stream, &oin1, &nl));
     next_epoch(c);
     c->ctx->launches += nl;
@@ -1893,13 +1890,12 @@ v3dg_status v3dg_sort_pairs(v3dg_ctx* ctx, uint32_t* keys, uint32_t* vals, uint6
   ST(ensure_status(c, ((n + kSortTile - 1) / kSortTile) * 256));
   ST(ensure(c, c->d_hist, sizeof(uint32_t) * kHistWords));
   uint32_t* misc = P<uint32_t>(c->d_misc);  // [0] n, [1..4] tile counters, [5] timeout flag
-  CU(cudaMemsetAsync(misc, 0, sizeof(uint32_t) * 8, c->stream));
-  k_set_word<<<1, 1, 0, c->stream>>>(misc, uint32_t(n));
-  CU(cudaGetLastError());
+  const SortScratch sc = sort_scratch(c, 0, misc + 1);
+  CU(launch_sort_init(misc, uint32_t(n), sc.hist, c->stream));
   bool in1 = false;
   int nl = 0;
   CU(launch_sort(keys, vals, P<uint32_t>(c->d_sort_k), P<uint32_t>(c->d_sort_v), misc, uint32_t(n), begin_bit, end_bit,
-                 false, sort_scratch(c, 0, false, misc + 1), misc + 5, c->epoch, ctx->sm_count, c->stream, &in1, &nl));
+                 false, sc, misc + 5, c->epoch, ctx->sm_count, c->stream, &in1, &nl));
   next_epoch(c);
   ctx->launches += nl + 1;
   if (in1) {

@@ -222,13 +222,15 @@ struct SortSlots {
 };
 constexpr int kSortPasses = 4, kSortBins = 256;
 struct SortScratch {
-  uint32_t* hist;          // kSortPasses * kSortBins digit counts
-  bool hist_zeroed;        // already zero (else launch_sort clears them)
+  uint32_t* hist;          // kSortPasses * kSortBins digit counts (zero)
   uint64_t* status;        // max_tiles * 256
   uint32_t max_tiles;
   uint32_t* tile_counters; // one per pass (zeroed by the caller's frame memset)
 };
 constexpr int kSortThreads = 256, kSortItems = 16, kSortTile = kSortThreads * kSortItems;
+// Before a standalone sort: words = n, its tile counters ([1..4]) and gave-up flag ([5]); the digit counts.
+constexpr int kSortWords = 8;
+cudaError_t launch_sort_init(uint32_t* words, uint32_t n, uint32_t* hist, cudaStream_t st);
 cudaError_t launch_sort(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1, const uint32_t* n_dev,
                         uint32_t cap, int begin_bit, int end_bit, bool implicit_vals,
                         const SortScratch& sc, uint32_t* err_flag, uint32_t& epoch, int sm_count,

@@ -48,8 +48,6 @@ std::atomic<uint64_t> g_calls{0};
 // each call takes 8 consecutive epochs (the sort uses at most 4); the sequence has this period
 constexpr uint64_t kEpochCalls = ((1u << 30) - 16u) / 8u;
 
-__global__ void k_store_n(uint32_t* p, uint32_t v) { *p = v; }
-
 }  // namespace
 
 extern "C" v3dg_status v3dg_sort_pairs_noalloc(uint32_t* keys, uint32_t* vals, uint64_t n, int begin_bit, int end_bit,
@@ -76,14 +74,12 @@ extern "C" v3dg_status v3dg_sort_pairs_noalloc(uint32_t* keys, uint32_t* vals, u
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   unsigned char* b = static_cast<unsigned char*>(base);
   uint32_t* misc = reinterpret_cast<uint32_t*>(b + kOffMisc);
-  if (cudaMemsetAsync(misc, 0, 64, st) != cudaSuccess) return V3DG_ECUDA;
-  k_store_n<<<1, 1, 0, st>>>(misc, uint32_t(n));
   SortScratch sc;
   sc.hist = reinterpret_cast<uint32_t*>(b + kOffHist);
-  sc.hist_zeroed = false;
   sc.status = reinterpret_cast<uint64_t*>(b + kOffStatus);
   sc.max_tiles = kTiles;
   sc.tile_counters = misc + 1;
+  if (launch_sort_init(misc, uint32_t(n), sc.hist, st) != cudaSuccess) return V3DG_ECUDA;
   // fresh epochs for the look-back status words, which keep earlier calls' contents; when the
   // sequence starts over, clear them so that no word left by an earlier call matches an epoch
   const uint64_t call = g_calls.fetch_add(1);
