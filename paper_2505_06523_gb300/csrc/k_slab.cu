@@ -8,9 +8,9 @@
 // more than half of those stages.  The image does not change: a pixel that has stopped takes no
 // further record, and a slab's records come in the same order as in the whole list.
 // Measured on a GB300, one slab -> several: depth sort, binning, tile sort and ranges of the 1080p crowd
-// 5.2 -> 2.7 ms (its blend 1.3 -> 2.0 ms: each slab waits for its longest tile), of the 5000-instance
-// 4K crowd 51 -> 13.5 ms, of 16 crowd views 50 -> 27 ms; one asset filling 1080p (31M pairs of 225k
-// Gaussians, all tiles finished after 3% of them) 2.4 -> 0.65 ms.
+// 5.2 -> 2.6 ms (its blend 1.3 -> 1.8 ms: each slab waits for its longest tile), of the 5000-instance
+// 4K crowd 51 -> 11 ms, of 16 crowd views 50 -> 23.4 ms; one asset filling 1080p (31M pairs of 225k
+// Gaussians, all tiles finished after 3% of them) 2.4 -> 0.5 ms.
 #include <algorithm>
 
 #include "dev_common.cuh"

@@ -104,7 +104,8 @@ struct Pipe {
   // the marked slots, and their counts
   DevBuf d_tlive, d_state, d_marks;
   bool tiles_in1 = false;
-  // pairs and visible Gaussians of the previous frame (of one still running: of the one before)
+  // pairs and visible Gaussians of the previous frame (of one still running: of the one before), within
+  // an eighth
   uint32_t pairs_hint = 0, visible_hint = 0;
   int slabs = 1;             // depth slabs of the last rendered frame
   bool full_lists = false;   // the sorted Gaussians and pairs of the whole frame are on the device
@@ -257,6 +258,15 @@ int slab_count(const Pipe* c) {
   return pairs < 2 * kManyPairs ? 3 : pairs < 8 * kManyPairs ? 4 : kMaxSlabs;
 }
 
+// The counts that slab_count goes by.  Changes of less than an eighth are not followed: either side of a
+// line costs about the same there, and frames that hover at one keep their buffers and captured graph.
+void note_counts(Pipe* c, uint32_t pairs, uint32_t visible) {
+  const auto moved = [](uint64_t now, uint64_t was) { return 8u * (now > was ? now - was : was - now) > was; };
+  if (!moved(pairs, c->pairs_hint) && !moved(visible, c->visible_hint)) return;
+  c->pairs_hint = pairs;
+  c->visible_hint = visible;
+}
+
 TileLive tile_live(Pipe* c, int slabs) {
   TileLive l{};
   l.tiles_x = uint32_t(c->cc.tiles_x);
@@ -378,8 +388,7 @@ v3dg_status setup_views(Pipe* c, const ViewSpec* views, uint32_t n_views) {
   const v3dg_camera* cam = views[0].cam;
   if (c->rendered) {
     const volatile uint32_t* f = c->h_frame;
-    c->pairs_hint = f[kPairs];
-    c->visible_hint = f[kVisible];
+    note_counts(c, f[kPairs], f[kVisible]);
   }
   if (c->ctx->assets.empty()) return fail(c, V3DG_ENOTFOUND, "no hierarchy loaded");
   const uint64_t tiles = uint64_t((cam->width + kTile - 1) / kTile) * uint64_t((cam->height + kTile - 1) / kTile);
@@ -711,8 +720,7 @@ v3dg_status ensure_full_lists(Pipe* c) {
 v3dg_status grow_and_reselect(Pipe* c) {
   const uint32_t* f = c->h_frame;
   bool grew = false;
-  c->pairs_hint = f[kPairs];
-  c->visible_hint = f[kVisible];
+  note_counts(c, f[kPairs], f[kVisible]);
   if (f[kRenderNodes] > c->cap_nodes) {
     if (f[kRenderNodes] > kMaxNodes)
       return fail(c, V3DG_EOVERFLOW, "render list of %u nodes exceeds the limit", f[kRenderNodes]);
