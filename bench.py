@@ -463,7 +463,7 @@ def main():
 
     served, view_samples = None, []
     if args.slots > 0:
-        # the autotuner times the blend of one FP16 walk frame with every batch size and split
+        # the autotuner times the blend of one FP16 walk frame in both variants
         ctx.set_instances(inst16)
         ctx.select(cams[timed_ids[0]], args.tau)
         ctx.render(rgb)
@@ -950,7 +950,8 @@ BLEND_OPS_EVAL, BLEND_OPS_CONTRIB = 8, 10
 
 # DRAM bytes per unit from one ncu capture of the same kernel on the crowd's profiling case (2
 # assets, 300 instances): dram__bytes_read.sum + dram__bytes_write.sum of one launch / the units
-# of its frame.  Scaled to a full launch by the units processed (traffic grows with them).
+# of its frame (one depth slab).  Scaled to a full frame by its units; a frame in several slabs moves
+# less than that for its blend and binning.
 NCU_DRAM_PER_UNIT = {
     "blend": (7.21, "pair", "profiles/k_blend_crowd_small.md"),      # (250.3 + 6.2) MB / 35.6M pairs
     "project": (98.9, "slot", "profiles/k_project_crowd_small.md"),   # (897.0 + 838.8) MB / 17.56M slots
@@ -970,7 +971,8 @@ def roofline_for(stage, stage_ms, fs, peaks, peak_kind):
         "select": 8 * nodes,
         # projection: 236 B of attributes per slot read -- once per distinct cluster (64 slots) when
         # the render list is projected grouped by cluster, the instances after the first reading
-        # them from L2, plus the entry, its FP64 reference and its order (8 + 32 + 4 B per node) --
+        # them from L2, plus the entry, its FP64 reference and its order (8 + 32 + 4 B per node;
+        # the reference stays in shared memory now, so this is 32 B a node, under 1%, too much) --
         # and a 48 B record + 8 B rect + 4 B key written per visible Gaussian
         "project": ((236 * 64 * clusters + 44 * nodes) if clusters else 236 * slots)
                    + (48 + 8 + 4) * vis + 4 * (slots - vis),
@@ -989,6 +991,10 @@ def roofline_for(stage, stage_ms, fs, peaks, peak_kind):
         per_stage["select"]["bound"] = "latency"
         per_stage["select"]["note"] = ("node tables L2/L1-resident; HBM bytes are the render list written; "
                                        "issue and L2 figures in profiles/k_select_crowd_small.md")
+    for k in ("depth_sort", "bin", "tile_sort", "ranges"):
+        if k in per_stage:   # large frames go in depth slabs that leave out what the front hides
+            per_stage[k]["note"] = ("bytes of the whole frame's Gaussians and pairs; a frame in several depth slabs "
+                                    "handles fewer of them, so this is no rate of bytes moved")
     mhz = float(peaks.get("sm_max_mhz", 2070.0))
     alu_peak = FP32_LANES * mhz * 1e6 / 1e12
     if fs.get("blend_evals") and stage_ms.get("blend"):

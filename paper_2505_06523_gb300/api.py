@@ -205,7 +205,7 @@ class Context:
         return out
 
     def autotune_blend(self) -> dict:
-        """Time the last frame's blend with every kernel variant, batch size and split threshold
+        """Time the last frame's blend as variant 0 and as variant 1 with every batch size
         and keep the fastest (v3dg_autotune_blend)."""
         m, b, sp, ms = N.v3dg_autotune_blend(self.ctx)
         return {"mode": m, "batch": b, "split_pairs": sp, "ms": ms}

@@ -19,7 +19,7 @@
 // sub-tile -> and long lists by blocks: 96x80 thumbnail 158 -> 37 -> 29 us, 256x256 viewer 266 -> 62 ->
 // 51 us, 200 instances at 640x360 655 -> 275 -> 174 us, one asset filling 1080p 1671 -> 346 -> 364 us, the
 // same 50 units away 768 -> 230 -> 127 us, crowd at 1080p (four slabs) 2.75 -> 2.03 -> 1.70 ms, 16 crowd
-// views 31.9 -> 11.7 -> 12.0 ms (full frames lose a little: five blocks per SM, not six).  (With three
+// views 31.9 -> 11.7 -> 12.0 ms (full frames lose a little: five blocks per SM, not six).  (With two
 // slabs the near asset takes 353 us, with six the 16 views 12.3 ms; the crowd 1.80 ms on this code.)  The warp kernel
 // with 8x8 pixels a warp (two per lane, four lists): 57 us, 510 us, 293 us and 1.74 ms on the thumbnail,
 // the 200 instances, the near asset and the crowd; 8x4 with one list: 72, 414, 307 us and 1.41 ms

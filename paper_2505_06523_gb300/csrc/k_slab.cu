@@ -10,7 +10,7 @@
 // Measured on a GB300, one slab -> several: depth sort, binning, tile sort and ranges of the 1080p crowd
 // 5.2 -> 2.6 ms (its blend 1.3 -> 1.8 ms: each slab waits for its longest tile), of the 5000-instance
 // 4K crowd 51 -> 11 ms, of 16 crowd views 50 -> 23.4 ms; one asset filling 1080p (31M pairs of 225k
-// Gaussians, all tiles finished after 3% of them) 2.4 -> 0.5 ms.
+// Gaussians, all tiles finished after 3% of them) 2.4 -> 0.43 ms.
 #include <algorithm>
 
 #include "dev_common.cuh"
@@ -46,14 +46,16 @@ k_frame_init(uint32_t* __restrict__ frame, uint32_t* __restrict__ hist, uint32_t
 }
 
 // The slabs' limits: at the depths where these thousandths of the frame's pairs lie in front (the first slab
-// is small, because everything in it is kept; the last takes what the others have not hidden).  A slab
-// more leaves out a few more pairs and costs about 20 launches and a tail of the blend, so larger
-// frames take more of them (see slab_count).  Whole frames by number of slabs, 3 / 4 / 6: one asset filling
-// 1080p (31M pairs) 0.93 / 1.03 / 1.29 ms, crowd at 1080p (157M) 6.46 / 6.06 / 6.84 ms, 5000 instances at
-// 4K (1.9G) 29.8 / 27.1 / 25.5 ms, 16 crowd views (1.3G) 53.6 / 47.8 / 45.2 ms.  Limits tried with four:
-// {20, 80, 250}, {30, 120, 350}, {40, 160, 400}, {60, 200, 400}, {70, 250, 450}, {100, 300, 500}: the crowd 7.32,
+// is kept whole; the last takes what the others have not hidden).  A slab more leaves out a few more pairs
+// and costs about 20 launches and a tail of the blend, so larger frames take more of them (see slab_count).
+// Whole frames by number of slabs, 3 / 4 / 6: crowd at 1080p (157M pairs) 6.46 / 6.06 / 6.84 ms, 5000 instances at
+// 4K (1.9G) 29.8 / 27.1 / 25.5 ms, 16 crowd views (1.3G) 53.6 / 47.8 / 45.2 ms; 2 / 3: crowd of 600 instances (99M)
+// 4.34 / 4.72 ms, one asset filling 1080p (31M) 0.87 / 0.95 ms.  Two slabs' limit at 250, 350 and 450: that crowd
+// 4.34, 4.48, 4.51 ms; the asset 0.88, 0.87, 0.90 ms, from 3 units (44M) 1.85, 1.64, 1.65 ms: frames of
+// large boxes take the later limit.  Limits tried with four: {20, 80, 250}, {30, 120, 350}, {40, 160, 400}, {60, 200, 400}, {70, 250, 450}, {100, 300, 500}: the crowd 7.32,
 // 6.68, 6.87, 6.85, 6.32, 6.15 ms.
-__constant__ const uint32_t kLimits3[2] = {100, 350}, kLimits4[3] = {83, 300, 500}, kLimits6[5] = {50, 140, 280, 430, 600};
+__constant__ const uint32_t kLimits2[1] = {250}, kLimits2Large[1] = {350}, kLimits4[3] = {83, 300, 500},
+                            kLimits6[5] = {50, 140, 280, 430, 600};
 
 __global__ void __launch_bounds__(256)
 k_slab_limits(uint32_t* __restrict__ frame, const uint32_t* __restrict__ depth_hist, int slabs, uint32_t cap_pairs) {
@@ -73,7 +75,7 @@ k_slab_limits(uint32_t* __restrict__ frame, const uint32_t* __restrict__ depth_h
     }
     uint32_t all, excl = block_exclusive_scan<8>(sum, s_scan, &all);
     // thousandths of the pairs
-    const uint32_t* const limits = slabs <= 3 ? kLimits3 : slabs == 4 ? kLimits4 : kLimits6;
+    const uint32_t* const limits = slabs == 2 ? (large_boxes(total, frame[kVisible]) ? kLimits2Large : kLimits2) : slabs == 4 ? kLimits4 : kLimits6;
     uint32_t target[kMaxSlabs - 1];
 #pragma unroll
     for (int k = 0; k < kMaxSlabs - 1; ++k)

@@ -248,14 +248,18 @@ constexpr uint32_t kSortHist = kMaxSlabs * kItemClasses, kDepthHist = kSortHist 
 // previous frame: the frame's own are not known when its launches are made, and consecutive frames of
 // a viewer or a batch are alike.  The image does not depend on it.  One below kManyPairs, and for blend
 // variant 1, which keeps no state between slabs: each slab costs about 20 launches and a tail of the
-// blend (crowds of 30 to 60M pairs, one slab / three: 2.92 / 3.12 and 4.52 / 4.66 ms).  Frames whose
-// Gaussians cover many tiles each (a camera close to an asset) hide theirs early, so they take three
-// from a quarter of that on (one asset at 1.7 and 2 units, 33 and 36M pairs: 1.14 / 1.08 and 1.31 / 1.26 ms).
+// blend (crowds of 120, 250 and 450 instances, 10, 34 and 59M pairs, one slab / two: 1.78 / 1.94, 2.85 / 2.90 and
+// 4.40 / 4.26 ms).  Frames of large boxes hide theirs early, so they take two from a quarter of that on (one
+// asset at 1.7, 2 and 2.5 units, 33, 36 and 47M pairs, one / two: 1.14 / 0.95, 1.31 / 1.11 and 1.73 / 1.55 ms) and stay
+// at two (at 4K, 117 and 131M pairs, four / two: 2.47 / 2.40 and 3.33 / 3.15 ms).  Crowd frames of 69, 91, 95, 98,
+// 123 and 133M pairs, two / four: 4.73 / 5.09, 5.06 / 5.40, 5.46 / 5.73, 5.20 / 5.13, 6.22 / 5.70 and 5.53 / 5.33 ms.
+constexpr uint64_t kFourSlabs = 96'000'000;
 int slab_count(const Pipe* c) {
   const uint64_t pairs = c->pairs_hint;
   if (c->ctx->blend_mode != 0) return 1;
-  if (pairs < kManyPairs) return pairs >= kManyPairs / 4 && pairs >= 16ull * c->visible_hint ? 3 : 1;
-  return pairs < 2 * kManyPairs ? 3 : pairs < 8 * kManyPairs ? 4 : kMaxSlabs;
+  if (large_boxes(pairs, c->visible_hint)) return pairs >= kManyPairs / 4 ? 2 : 1;
+  if (pairs < kManyPairs) return 1;
+  return pairs < kFourSlabs ? 2 : pairs < 8 * kManyPairs ? 4 : kMaxSlabs;
 }
 
 // The counts that slab_count goes by.  Changes of less than an eighth are not followed: either side of a

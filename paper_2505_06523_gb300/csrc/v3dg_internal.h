@@ -90,6 +90,8 @@ enum Counter : int {
 // visible Gaussians with depth keys in [lo, hi).  From the second slab on, Gaussians and pairs that
 // only meet tiles whose pixels have all stopped are left out (they cannot change a pixel).
 constexpr int kMaxSlabs = 6, kSlabWords = 24, kFrameWords = kSlabBase + kMaxSlabs * kSlabWords;
+// A frame whose Gaussians cover many tiles each: a camera close to an asset.
+__host__ __device__ inline bool large_boxes(uint64_t pairs, uint64_t visible) { return pairs >= 16u * visible; }
 enum SlabWord : int {
   kSlabCount = 0,          // Gaussians picked
   kSlabPairs,              // their pairs

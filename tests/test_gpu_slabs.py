@@ -21,9 +21,10 @@ def _in_slabs(stats, at_least):
 
 
 @pytest.mark.parametrize("n,spread,width,height,fov,views,graphs,at_least", [
-    (12, 0.5, 1920, 1080, 70.0, 1, 0, 1 << 24),    # a pile next to the camera: large boxes, early stops: three slabs
+    (12, 0.5, 1920, 1080, 70.0, 1, 0, 1 << 24),    # a pile next to the camera: large boxes, early stops: two slabs
     (12, 0.5, 1001, 563, 40.0, 3, 0, 1 << 24),     # ragged images, several views
     (12, 0.5, 1001, 563, 40.0, 3, 1, 1 << 24),     # the same, captured
+    (40, 3.0, 1601, 901, 50.0, 4, 0, 1 << 26),     # two slabs, small boxes
     (40, 3.0, 1601, 901, 50.0, 8, 0, 1 << 27),     # four slabs
 ])
 def test_slabs_change_nothing(tiny_asset, n, spread, width, height, fov, views, graphs, at_least):
