@@ -948,14 +948,14 @@ FP32_LANES = 152 * 128
 BLEND_OPS_EVAL, BLEND_OPS_CONTRIB = 8, 10
 
 
-# DRAM bytes per unit from one ncu capture of the same kernel on the crowd's profiling case (2
-# assets, 300 instances): dram__bytes_read.sum + dram__bytes_write.sum of one launch / the units
+# DRAM bytes per unit from one ncu capture of the same kernel on the crowd's profiling case (2 or 3
+# assets, 300 instances): dram__bytes.sum.per_second x the duration of one launch / the units
 # of its frame (one depth slab).  Scaled to a full frame by its units; a frame in several slabs moves
 # less than that for its blend and binning.
 NCU_DRAM_PER_UNIT = {
-    "blend": (7.21, "pair", "profiles/k_blend_crowd_small.md"),      # (250.3 + 6.2) MB / 35.6M pairs
-    "project": (98.9, "slot", "profiles/k_project_crowd_small.md"),   # (897.0 + 838.8) MB / 17.56M slots
-    "bin": (11.84, "pair", "profiles/k_expand_crowd_small.md"),       # (175.4 + 245.8) MB / 35.6M pairs
+    "blend": (7.28, "pair", "profiles/k_blend_crowd_small.md"),      # 316.9 MB / 43.5M pairs
+    "project": (85.4, "slot", "profiles/k_project_crowd_small.md"),   # 1748 MB / 20.47M slots
+    "bin": (9.81, "pair", "profiles/k_expand_crowd_small.md"),       # 426.6 MB / 43.5M pairs
 }
 
 
