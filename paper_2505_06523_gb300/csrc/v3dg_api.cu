@@ -1856,7 +1856,8 @@ v3dg_status v3dg_autotune_blend(v3dg_ctx* ctx, uint32_t* mode_out, uint32_t* bat
       if (mode == 0 && b != 512) continue;   // variant 0 has no batch size (512 is the option's default)
       float t_min = INFINITY;
       for (int rep = 0; rep < 4 && e == cudaSuccess; ++rep) {   // the first run warms up
-        e = cudaMemsetAsync(frame + kSlabBase + kSlabBlendItem, 0, sizeof(uint32_t), c->stream);
+        // both of the blend's work counters: kSlabBlendItem, kSlabBlendLong
+        e = cudaMemsetAsync(frame + kSlabBase + kSlabBlendItem, 0, 2 * sizeof(uint32_t), c->stream);
         if (e == cudaSuccess) e = cudaMemsetAsync(c->d_hist.p, 0, sizeof(uint32_t) * kItemClasses, c->stream);
         if (e == cudaSuccess) e = cudaEventRecord(e0, c->stream);
         if (e == cudaSuccess)

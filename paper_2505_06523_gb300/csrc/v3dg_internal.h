@@ -105,6 +105,7 @@ enum SlabWord : int {
   kSlabLarge,              // Gaussians left to the large-box expansion
 };
 static_assert(kSlabLarge < kSlabWords, "slab words");
+static_assert(kSlabBlendLong == kSlabBlendItem + 1, "the blend's work counters are cleared together");
 constexpr int kItemClasses = 16;   // classes of the blend's work items
 
 // Depth histogram of the pairs (weights: tiles covered), for the slabs' limits: 16 bins per octave
@@ -270,7 +271,7 @@ cudaError_t launch_ranges(const uint32_t* tile_keys, uint32_t cap_pairs, const u
 // sticky[0] |= frame[kOverflow], sticky[1] |= frame[kTimeout] (the flags of every frame since the
 // host last cleared them).
 // items, class_count: kItemClasses * n_tiles words of scratch and kItemClasses zeroed words (the tiles
-// by the length of their lists); the slab's word kSlabBlendItem is zero.  live.bits != NULL: one of
+// by the length of their lists); the slab's words kSlabBlendItem and kSlabBlendLong are zero.  live.bits != NULL: one of
 // several slabs, first to last from 0 -- the pixels' state is kept in live.state and the image
 // between them (mode 0 only).
 // batch: records that variant 1 stages per batch, 128, 256 or 512.  n_views
