@@ -114,8 +114,9 @@ enum {
                                larger buffers on overflow; 0: fully asynchronous, the caller
                                checks v3dg_frame_stats */
   V3DG_OPT_STAGE_TIMING = 2, /* 1: record CUDA events around every stage (see v3dg_stage_times) */
-  V3DG_OPT_CAP_NODES = 3,    /* current render-list capacity in clusters (>= 64); grows on demand */
-  V3DG_OPT_CAP_PAIRS = 4,    /* current (tile, Gaussian) pair capacity (>= 4096); grows on demand */
+  V3DG_OPT_CAP_NODES = 3,    /* render-list capacity in clusters (>= 64) from the next selection on
+                                (graph frames: the next render); grows on demand */
+  V3DG_OPT_CAP_PAIRS = 4,    /* likewise the (tile, Gaussian) pair capacity (>= 4096) */
   V3DG_OPT_COUNT_WORK = 5,   /* 1: the blend also counts its evaluations (v3dg_stats.blend_*) */
   V3DG_OPT_SPLIT_PAIRS = 6,  /* 1 .. 2^32 - 1: accepted and without effect (blend variant 0 always
                                 spreads a tile over eight warps, variant 1 never splits one) */

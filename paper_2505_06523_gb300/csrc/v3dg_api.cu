@@ -94,6 +94,7 @@ struct Pipe {
   uint32_t* h_tmp = nullptr;     // pinned scratch: [0, 48) frame words of read-backs, [48, 52) blend work
 
   uint32_t cap_nodes = 0, cap_slots = 0, cap_pairs = 0, status_words = 0, cap_cut = 0;
+  uint32_t set_nodes = 0, set_pairs = 0;   // capacities set by option (0: none), taken over when the buffers are next sized
   // d_keys0: the projection's depth keys per slot; (d_keys1, d_vals1) and (d_keys2, d_vals0): the
   // depth sort's buffers
   DevBuf d_list, d_keys0, d_keys1, d_keys2, d_vals0, d_vals1, d_rec, d_rect;
@@ -307,6 +308,9 @@ v3dg_status ensure_image_work(Pipe* c) {
 
 // Work buffers sized by the current capacities.
 v3dg_status ensure_work(Pipe* c) {
+  if (c->set_nodes) c->cap_nodes = c->set_nodes;
+  if (c->set_pairs) c->cap_pairs = c->set_pairs;
+  c->set_nodes = c->set_pairs = 0;
   if (c->cap_nodes == 0) c->cap_nodes = kInitNodes;
   if (c->cap_pairs == 0) c->cap_pairs = kInitPairs;
   c->cap_slots = c->cap_nodes * uint32_t(kSlots);
@@ -1000,6 +1004,7 @@ void pipe_trim(Pipe* c) {
   DevBuf* const* bs = frame_buffers(c, &n);
   for (size_t i = 0; i < n; ++i) dfree(c, *bs[i]);
   c->cap_nodes = c->cap_pairs = c->cap_slots = c->status_words = c->cap_cut = 0;
+  c->set_nodes = c->set_pairs = 0;
   c->selected = c->rendered = false;
 }
 
@@ -1394,11 +1399,11 @@ v3dg_status v3dg_set_option(v3dg_ctx* ctx, int option, int64_t value) {
       break;
     case V3DG_OPT_CAP_NODES:
       if (value < 64 || value > int64_t(kMaxNodes)) return fail(c, V3DG_EINVAL, "node capacity out of range");
-      c->cap_nodes = uint32_t(value);
+      c->set_nodes = uint32_t(value);
       break;
     case V3DG_OPT_CAP_PAIRS:
       if (value < 4096 || value > int64_t(kMaxPairs)) return fail(c, V3DG_EINVAL, "pair capacity out of range");
-      c->cap_pairs = uint32_t(value);
+      c->set_pairs = uint32_t(value);
       break;
     default: return fail(c, V3DG_EINVAL, "unknown option %d", option);
   }
