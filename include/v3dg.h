@@ -211,14 +211,15 @@ v3dg_status v3dg_select_views(v3dg_ctx* ctx, const v3dg_camera* cams, uint32_t n
  * (V3DG_ENOTFOUND otherwise). */
 v3dg_status v3dg_render(v3dg_ctx* ctx, float* rgb_out, float* T_out);
 
-/* Autotuner of the blend's kernel variant and batch size.  Re-runs the blend stage of the last
- * rendered frame (its sorted pairs and records are still on the device) with variant 0
- * (V3DG_OPT_BLEND_MODE) and with variant 1 at 128, 256 and 512 records per batch, times each with
- * CUDA events (best of 3 after one warm-up run) and keeps the fastest as V3DG_OPT_BLEND_MODE and
+/* Autotuner of the blend's kernel variant and batch size.  Renders the last rendered frame again
+ * (its render list is still on the device) with variant 0 (V3DG_OPT_BLEND_MODE) and with variant 1
+ * at 128, 256 and 512 records per batch, each as the frames that follow would run (variant 0 takes
+ * large frames in depth slabs, variant 1 none), times each with CUDA events from the projection on
+ * (best of 3 after one warm-up run) and keeps the fastest as V3DG_OPT_BLEND_MODE and
  * V3DG_OPT_BLEND_BATCH for the frames that follow; *split_pairs is 2^32 - 1.  None changes the
  * image.  Synchronous; the caller's image is not touched.  V3DG_ENOTFOUND without a rendered
  * frame, V3DG_EOVERFLOW if that frame was not valid.  mode, batch, split_pairs, best_ms: the choice
- * and its time, each may be NULL.  The paper has no counterpart (its rasterizer is fixed). */
+ * and its blend's time, each may be NULL.  The paper has no counterpart (its rasterizer is fixed). */
 v3dg_status v3dg_autotune_blend(v3dg_ctx* ctx, uint32_t* mode, uint32_t* batch, uint32_t* split_pairs, float* best_ms);
 
 /* v3dg_render into HOST buffers (same layouts): the image is produced on the device and copied

@@ -205,8 +205,8 @@ class Context:
         return out
 
     def autotune_blend(self) -> dict:
-        """Time the last frame's blend as variant 0 and as variant 1 with every batch size
-        and keep the fastest (v3dg_autotune_blend)."""
+        """Time the last frame with blend variant 0 and with variant 1 at every batch size and keep the
+        fastest; "ms" is its blend's time (v3dg_autotune_blend)."""
         m, b, sp, ms = N.v3dg_autotune_blend(self.ctx)
         return {"mode": m, "batch": b, "split_pairs": sp, "ms": ms}
 

@@ -632,6 +632,7 @@ v3dg_status enqueue_render(Pipe* c, float* rgb, float* t_out) {
   const int sm = c->ctx->sm_count;
   const int slabs = slab_count(c);
   const int n_tiles = k.tiles_x * k.tiles_y * int(c->n_views);   // (view, tile) ids
+  c->full_lists = false;
   ST(ensure_image_work(c));
   const TileLive live = tile_live(c, slabs);
   uint32_t* depth_hist = slabs > 1 ? P<uint32_t>(c->d_hist) + kDepthHist : nullptr;
@@ -697,8 +698,7 @@ v3dg_status enqueue_render(Pipe* c, float* rgb, float* t_out) {
   return V3DG_OK;
 }
 
-// The whole frame's sorted Gaussians, pairs and tile ranges (the parity read-backs and the blend
-// autotuner read them): a frame rendered in several slabs has only the last one's, so its lists are
+// The whole frame's sorted Gaussians, pairs and tile ranges (the parity read-backs read them): a frame rendered in several slabs has only the last one's, so its lists are
 // made again in one slab without the filter, from the keys, boxes and records that are still there.
 v3dg_status ensure_full_lists(Pipe* c) {
   if (c->full_lists) return V3DG_OK;
@@ -863,6 +863,19 @@ v3dg_status render_frame(Pipe* c, float* rgb, float* t_out, bool sync) {
     c->select_pending = false;
   }
   return run_frame(c, rgb, t_out, sync);
+}
+
+// A stage's device time of the last frame rendered with stage events, over the frame's slabs.
+cudaError_t stage_ms(const Pipe* c, int stage, float* ms) {
+  if (stage <= kStageProject) return cudaEventElapsedTime(ms, c->ev[stage], c->ev[stage + 1]);
+  *ms = 0.f;
+  for (int slab = 0; slab < c->slabs; ++slab) {
+    float t = 0.f;
+    const cudaError_t e = cudaEventElapsedTime(&t, c->ev[6 * slab + stage], c->ev[6 * slab + stage + 1]);
+    if (e != cudaSuccess) return e;
+    *ms += t;
+  }
+  return cudaSuccess;
 }
 
 v3dg_status sync_frame(Pipe* c) {
@@ -1815,18 +1828,7 @@ v3dg_status v3dg_stage_times(v3dg_ctx* ctx, float* ms, int n, uint64_t* launches
   if (ms && n > 0) {
     if (!ctx->stage_timing || !c->rendered) return fail(c, V3DG_ENOTFOUND, "stage timing is off or no frame rendered");
     CU(cudaStreamSynchronize(c->stream));
-    for (int i = 0; i < n && i < kStages; ++i) {
-      ms[i] = 0.f;
-      if (i < 2) {   // selection, projection
-        CU(cudaEventElapsedTime(ms + i, c->ev[i], c->ev[i + 1]));
-        continue;
-      }
-      for (int slab = 0; slab < c->slabs; ++slab) {   // the other stages, over the frame's slabs
-        float t = 0.f;
-        CU(cudaEventElapsedTime(&t, c->ev[6 * slab + i], c->ev[6 * slab + i + 1]));
-        ms[i] += t;
-      }
-    }
+    for (int i = 0; i < n && i < kStages; ++i) CU(stage_ms(c, i, ms + i));
   }
   c->err.clear();
   return V3DG_OK;
@@ -1839,58 +1841,72 @@ v3dg_status v3dg_autotune_blend(v3dg_ctx* ctx, uint32_t* mode_out, uint32_t* bat
   if (!c->rendered) return fail(c, V3DG_ENOTFOUND, "no frame rendered");
   ST(sync_frame(c));
   if (c->h_frame[kOverflow] || c->h_frame[kTimeout]) return fail(c, V3DG_EOVERFLOW, "the last frame was not valid");
-  ST(ensure_full_lists(c));
-  const CamConst& k = c->cc;
-  const size_t px = size_t(k.width) * size_t(k.height) * c->n_views;
+  note_counts(c, c->h_frame[kPairs], c->h_frame[kVisible]);   // the frames that follow take their slabs by this one
+  const size_t px = size_t(c->cc.width) * size_t(c->cc.height) * c->n_views;
   ST(ensure(c, c->d_img, sizeof(float) * 3 * std::max<size_t>(px, 1)));
-  const uint32_t* tk = P<uint32_t>(c->tiles_in1 ? c->d_pk1 : c->d_pk0);
-  const uint32_t* tv = P<uint32_t>(c->tiles_in1 ? c->d_pv1 : c->d_pv0);
-  uint32_t* frame = P<uint32_t>(c->d_frame);
-  cudaEvent_t e0 = nullptr, e1 = nullptr;
-  CU(cudaEventCreate(&e0));
-  if (cudaEventCreate(&e1) != cudaSuccess) {
-    cudaEventDestroy(e0);
-    return fail(c, V3DG_ECUDA, "cudaEventCreate failed");
-  }
-  const int batches[] = {128, 256, 512};
-  float best = INFINITY;
-  int best_b = ctx->blend_batch, best_m = ctx->blend_mode;
-  cudaError_t e = cudaSuccess;
-  for (int mode = 0; mode < 2; ++mode)
-    for (int b : batches) {
-      if (mode == 0 && b != 512) continue;   // variant 0 has no batch size (512 is the option's default)
-      float t_min = INFINITY;
-      for (int rep = 0; rep < 4 && e == cudaSuccess; ++rep) {   // the first run warms up
-        // both of the blend's work counters: kSlabBlendItem, kSlabBlendLong
-        e = cudaMemsetAsync(frame + kSlabBase + kSlabBlendItem, 0, 2 * sizeof(uint32_t), c->stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(c->d_hist.p, 0, sizeof(uint32_t) * kItemClasses, c->stream);
-        if (e == cudaSuccess) e = cudaEventRecord(e0, c->stream);
-        if (e == cudaSuccess)
-          e = launch_blend(P<uint2>(c->d_ranges), P<uint32_t>(c->d_order), P<uint32_t>(c->d_hist), tk, tv,
-                           P<float4>(c->d_rec), c->cap_slots, k, P<float>(c->d_img), nullptr, nullptr, frame, P<uint32_t>(c->d_misc) + 12, 0, TileLive{}, b,
-                           mode, int(c->n_views), ctx->sm_count, c->stream);
-        if (e == cudaSuccess) e = cudaEventRecord(e1, c->stream);
-        if (e == cudaSuccess) e = cudaEventSynchronize(e1);
-        float ms = 0.f;
-        if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
-        if (e == cudaSuccess && rep > 0) t_min = std::min(t_min, ms);
-        ctx->launches += 2;
-      }
-      if (t_min < best) {
-        best = t_min;
-        best_b = b;
-        best_m = mode;
-      }
+  // events of its own, and the caller's options and stage times back in place whatever happens
+  struct Restore {
+    Pipe* c;
+    cudaEvent_t ev[2 + 6 * kMaxSlabs] = {};
+    int mode, batch, slabs;
+    bool timing, count;
+    explicit Restore(Pipe* p)
+        : c(p), mode(p->ctx->blend_mode), batch(p->ctx->blend_batch), slabs(p->slabs), timing(p->ctx->stage_timing),
+          count(p->ctx->count_work) {
+      std::swap(ev, c->ev);
     }
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
-  if (e != cudaSuccess) return fail(c, V3DG_ECUDA, "CUDA error %s", cudaGetErrorString(e));
+    ~Restore() {
+      std::swap(ev, c->ev);
+      for (cudaEvent_t e : ev)
+        if (e) cudaEventDestroy(e);
+      c->ctx->blend_mode = mode;
+      c->ctx->blend_batch = batch;
+      c->ctx->stage_timing = timing;
+      c->ctx->count_work = count;
+      c->slabs = slabs;
+    }
+  };
+  const int batches[] = {128, 256, 512};
+  float best = INFINITY, best_blend = INFINITY;
+  int best_b = ctx->blend_batch, best_m = ctx->blend_mode;
+  {
+    Restore restore(c);
+    for (auto& e : c->ev) CU(cudaEventCreate(&e));
+    ctx->stage_timing = true;
+    ctx->count_work = false;
+    for (int mode = 0; mode < 2; ++mode)
+      for (int b : batches) {
+        if (mode == 0 && b != 512) continue;   // variant 0 has no batch size (512 is the option's default)
+        ctx->blend_mode = mode;
+        ctx->blend_batch = b;
+        float frame_min = INFINITY, blend_min = INFINITY;
+        for (int rep = 0; rep < 4; ++rep) {   // the first run warms up
+          ST(enqueue_render(c, P<float>(c->d_img), nullptr));
+          CU(cudaStreamSynchronize(c->stream));
+          if (c->h_frame[kTimeout]) return fail(c, V3DG_ETIMEOUT, "a bounded device-side wait gave up");
+          float frame = 0.f, blend = 0.f;
+          for (int i = kStageProject; i < kStages; ++i) {
+            CU(stage_ms(c, i, &blend));
+            frame += blend;   // (the blend is the last stage)
+          }
+          if (rep == 0) continue;
+          frame_min = std::min(frame_min, frame);
+          blend_min = std::min(blend_min, blend);
+        }
+        if (frame_min < best) {
+          best = frame_min;
+          best_blend = blend_min;
+          best_b = b;
+          best_m = mode;
+        }
+      }
+  }
   ctx->blend_batch = best_b;
   ctx->blend_mode = best_m;
   if (mode_out) *mode_out = uint32_t(best_m);
   if (batch_out) *batch_out = uint32_t(best_b);
   if (split_out) *split_out = 0xFFFFFFFFu;
-  if (ms_out) *ms_out = best;
+  if (ms_out) *ms_out = best_blend;
   c->err.clear();
   return V3DG_OK;
 }

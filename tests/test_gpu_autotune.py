@@ -52,3 +52,38 @@ def test_times_the_whole_blend():
         best = ctx.autotune_blend()
     assert best["split_pairs"] == 0xFFFFFFFF
     assert 0.5 * frame[best["mode"]] <= best["ms"] <= 2.0 * frame[best["mode"]], (best, frame)
+
+
+def test_candidates_are_whole_frames(tiny_asset):
+    """A candidate is timed as the frame that its choice would bring, with or without depth slabs: four runs (one warms up)
+    of the frame's launches for variant 0, here in two slabs, and four for each batch size of variant 1, in one.  The
+    frame's stage times, image and lists stay."""
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2505_06523_gb300 import Context
+    from paper_2505_06523_gb300._native import V3DG_OPT_BLEND_MODE, V3DG_OPT_STAGE_TIMING
+    n, rng = 12, np.random.Generator(np.random.PCG64(12))
+    inst = scenes.Instances(np.zeros(n, np.uint32), scenes.random_rotations(rng, n), rng.uniform(-0.5, 0.5, (n, 3)),
+                            rng.uniform(0.7, 1.4, n))
+    cam = scenes.look_at((0.0, -2.5, 0.5), (0.0, 0.0, 0.0), 1920, 1080, 70.0)
+    with Context(0) as ctx:
+        ctx.load_hierarchy(tiny_asset)
+        ctx.set_instances(inst)
+        ctx.set_option(V3DG_OPT_STAGE_TIMING, 1)
+        launches = {}
+        for mode in (1, 0):
+            ctx.set_option(V3DG_OPT_BLEND_MODE, mode)
+            for _ in range(2):
+                ctx.select(cam, 0.25)
+                before = ctx.launches()
+                img = ctx.render()[0]
+            launches[mode] = ctx.launches() - before
+        assert launches[0] > launches[1]   # (slabs)
+        times, ranges, proj, kept = ctx.stage_times()[0], ctx.tile_ranges(), ctx.get_projected(), img.clone()
+        before = ctx.launches()
+        best = ctx.autotune_blend()
+        assert ctx.launches() - before == 4 * launches[0] + 12 * launches[1]
+        assert ctx.stage_times()[0] == times and bool((img == kept).all())
+        assert (ctx.tile_ranges() == ranges).all() and all(np.array_equal(v, proj[k]) for k, v in ctx.get_projected().items())
+        ctx.select(cam, 0.25)
+        assert bool((ctx.render()[0] == kept).all()) and best["ms"] > 0
