@@ -53,12 +53,18 @@ constexpr uint32_t kInitNodes = 1u << 14;
 constexpr uint32_t kInitPairs = 1u << 22;
 constexpr uint32_t kMaxNodes = 1u << 25;               // render-list clusters: at most 2^31 slots
 constexpr uint32_t kMaxPairs = 0xFFFFFFFFu - 4096u;    // pair indices are 32-bit (a sort tile of headroom)
-constexpr uint64_t kManyPairs = 1u << 26;              // pairs of the previous frame from which one is taken in slabs
+constexpr uint64_t kManyPairs = 1u << 26;              // expected pairs from which a frame is taken in slabs
 enum { kStageSelect = 0, kStageProject, kStageDepthSort, kStageBin, kStageTileSort, kStageRanges, kStageBlend, kStages };
 
 }  // namespace
 
 struct Server;
+
+// Counts of a frame and what estimate_frame expected of it.
+struct FrameCounts {
+  double expected = 0.0, pairs = 0.0, visible = 0.0;   // expected 0: no frame yet
+};
+constexpr int kCountClasses = 40;
 
 // Per-frame state of one pipeline: the instance table and camera set-up of its frames, its work
 // buffers and their capacities, frame counters and the stream its work goes to.  The context's
@@ -105,9 +111,11 @@ struct Pipe {
   // the marked slots, and their counts
   DevBuf d_tlive, d_state, d_marks;
   bool tiles_in1 = false;
-  // pairs and visible Gaussians of the previous frame (of one still running: of the one before), within
-  // an eighth
-  uint32_t pairs_hint = 0, visible_hint = 0;
+  // pairs and visible Gaussians of the pipe's frames (of one still running: of the one before), by the
+  // octave of the pairs that estimate_frame expects; those expected of the current frame (its estimate's)
+  FrameCounts seen[kCountClasses];
+  double expected = 1.0;
+  uint64_t pairs_hint = 0, visible_hint = 0;
   int slabs = 1;             // depth slabs of the last rendered frame
   bool full_lists = false;   // the sorted Gaussians and pairs of the whole frame are on the device
   uint32_t epoch = 1;
@@ -245,9 +253,30 @@ constexpr int kFrameSorts = 1 + 2 * kMaxSlabs;
 constexpr uint32_t kSortHist = kMaxSlabs * kItemClasses, kDepthHist = kSortHist + kFrameSorts * kSortPasses * kSortBins,
                    kHistWords = kDepthHist + kDepthBins;
 
-// Depth slabs of the next frame (see k_slab.cu), by the pairs and visible Gaussians of the pipe's
-// previous frame: the frame's own are not known when its launches are made, and consecutive frames of
-// a viewer or a batch are alike.  The image does not depend on it.  One below kManyPairs, and for blend
+// Estimated size of a frame, for a request's admission and the buffers of its first frame (so that it
+// rarely overflows and re-runs), and for carrying one frame's counts over to another: about 1,000
+// render-list clusters per instance of a 1M-leaf crowd at tau 1 px (1.0M for the 1000-instance crowd at
+// 1920x1080), growing with sqrt(1 / tau) (a finer cut) and 25% headroom; pairs 2.25 per visible slot at 1920x1080, growing
+// with the square root of the pixel count (Gaussians span more tiles).  Bytes: per slot the depth
+// keys and values, record and box (72 B), per pair keys and values (16 B), per pixel 64 B.
+struct FrameEstimate {
+  uint64_t nodes, pairs, bytes;
+};
+
+FrameEstimate estimate_frame(uint32_t n_inst, const v3dg_camera& cam, float tau_px) {
+  const double px = double(cam.width) * double(cam.height);
+  const double nodes = 1250.0 * double(n_inst) * std::sqrt(1.0 / std::max(double(tau_px), 0.25));
+  const double pairs = nodes * 64.0 * 2.25 * std::sqrt(px / (1920.0 * 1080.0));
+  FrameEstimate e;
+  e.nodes = uint64_t(nodes);
+  e.pairs = uint64_t(pairs);
+  e.bytes = uint64_t(nodes * 64.0 * 72.0 + pairs * 16.0 + px * 64.0);
+  return e;
+}
+
+// Depth slabs of the next frame (see k_slab.cu), by the pairs and visible Gaussians that expect_counts
+// takes from the pipe's earlier frames: the frame's own are not known when its launches are made, and
+// consecutive frames of a viewer or a batch are alike.  The image does not depend on it.  One below kManyPairs, and for blend
 // variant 1, which keeps no state between slabs: each slab costs about 20 launches and a tail of the
 // blend (crowds of 120, 250 and 450 instances, 10, 34 and 59M pairs, one slab / two: 1.78 / 1.94, 2.85 / 2.90 and
 // 4.40 / 4.26 ms).  Frames of large boxes hide theirs early, so they take two from a quarter of that on (one
@@ -263,13 +292,31 @@ int slab_count(const Pipe* c) {
   return pairs < kFourSlabs ? 2 : pairs < 8 * kManyPairs ? 4 : kMaxSlabs;
 }
 
-// The counts that slab_count goes by.  Changes of less than an eighth are not followed: either side of a
-// line costs about the same there, and frames that hover at one keep their buffers and captured graph.
+int count_class(double expected) { return std::min(std::max(std::ilogb(expected), 0), kCountClasses - 1); }
+
+// The counts that slab_count goes by: those of the pipe's last frame of about the same estimated size, by
+// the ratio of the estimates.  A slot's requests have nothing to do with each other: by the last
+// frame alone, small ones between large ones were taken in slabs and the large ones not.
+void expect_counts(Pipe* c) {
+  const int cls = count_class(c->expected);
+  const FrameCounts* f = nullptr;
+  for (int d = 0; d < kCountClasses && !f; ++d)
+    for (int k : {cls - d, cls + d})
+      if (!f && k >= 0 && k < kCountClasses && c->seen[k].expected > 0.0) f = c->seen + k;
+  const double by = f ? c->expected / f->expected : 0.0;
+  c->pairs_hint = f ? uint64_t(f->pairs * by) : 0u;
+  c->visible_hint = f ? uint64_t(f->visible * by) : 0u;
+}
+
+// Notes the counts of the pipe's last frame.  Changes of less than an eighth are not followed: either
+// side of a line of slab_count costs about the same there, and frames that hover at one keep their
+// buffers and captured graph.
 void note_counts(Pipe* c, uint32_t pairs, uint32_t visible) {
-  const auto moved = [](uint64_t now, uint64_t was) { return 8u * (now > was ? now - was : was - now) > was; };
-  if (!moved(pairs, c->pairs_hint) && !moved(visible, c->visible_hint)) return;
-  c->pairs_hint = pairs;
-  c->visible_hint = visible;
+  FrameCounts& f = c->seen[count_class(c->expected)];
+  const double by = f.expected > 0.0 ? c->expected / f.expected : 0.0;
+  const auto moved = [by](double now, double was) { return 8.0 * std::fabs(now - was * by) > was * by; };
+  if (moved(pairs, f.pairs) || moved(visible, f.visible)) f = {c->expected, double(pairs), double(visible)};
+  expect_counts(c);
 }
 
 TileLive tile_live(Pipe* c, int slabs) {
@@ -429,6 +476,9 @@ v3dg_status setup_views(Pipe* c, const ViewSpec* views, uint32_t n_views) {
   c->select_items = select_items(nf, max_nodes, c->ctx->sm_count);
   c->n_inst_frame = nf;
   c->n_views = n_views;
+  c->expected = 1.0;
+  for (uint32_t v = 0; v < n_views; ++v) c->expected += double(estimate_frame(views[v].n, *views[v].cam, views[v].tau_px).pairs);
+  expect_counts(c);
   c->frame_asset.resize(nf);
   // the projection is specialised for the colour formats of the assets this frame draws
   c->color_formats = 0;
@@ -1083,29 +1133,6 @@ struct Server {
 
 namespace {
 
-// Admission estimate of a request's device memory: image and per-pixel buffers plus a share per
-// instance for its cut, records and pairs.
-// Estimated frame size of a request, for admission and for sizing its buffers before the first
-// frame (so that it rarely overflows and re-runs): about 1,000 render-list clusters per instance of
-// a 1M-leaf crowd at tau 1 px (1.0M for the 1000-instance crowd at 1920x1080), growing with
-// sqrt(1 / tau) (a finer cut) and 25% headroom; pairs 2.25 per visible slot at 1920x1080, growing
-// with the square root of the pixel count (Gaussians span more tiles).  Bytes: per slot the depth
-// keys and values, record and box (72 B), per pair keys and values (16 B), per pixel 64 B.
-struct FrameEstimate {
-  uint64_t nodes, pairs, bytes;
-};
-
-FrameEstimate estimate_frame(uint32_t n_inst, const v3dg_camera& cam, float tau_px) {
-  const double px = double(cam.width) * double(cam.height);
-  const double nodes = 1250.0 * double(n_inst) * std::sqrt(1.0 / std::max(double(tau_px), 0.25));
-  const double pairs = nodes * 64.0 * 2.25 * std::sqrt(px / (1920.0 * 1080.0));
-  FrameEstimate e;
-  e.nodes = uint64_t(nodes);
-  e.pairs = uint64_t(pairs);
-  e.bytes = uint64_t(nodes * 64.0 * 72.0 + pairs * 16.0 + px * 64.0);
-  return e;
-}
-
 uint64_t request_bytes(uint32_t n_inst, const v3dg_camera& cam, float tau_px) {
   return estimate_frame(n_inst, cam, tau_px).bytes;
 }
@@ -1177,6 +1204,7 @@ v3dg_status run_requests(Pipe* c, std::vector<Request>& rqs, Finished* f) {
   f->visible = c->h_frame[kVisible];
   f->pairs = c->h_frame[kPairs];
   f->batch_views = nv;
+  note_counts(c, c->h_frame[kPairs], c->h_frame[kVisible]);   // (the slot may give up its frame)
   return V3DG_OK;
 }
 

@@ -1,0 +1,61 @@
+"""How many depth slabs a frame is taken in, seen by its launches."""
+import numpy as np
+import pytest
+
+from synth import scenes
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def api():
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2505_06523_gb300 import Context, _native
+    return Context, _native
+
+
+def _pile(n, spread):
+    """n copies of asset 0, turned and scaled differently, around the origin."""
+    rng = np.random.Generator(np.random.PCG64(n))
+    return scenes.Instances(np.zeros(n, np.uint32), scenes.random_rotations(rng, n), rng.uniform(-spread, spread, (n, 3)),
+                            rng.uniform(0.7, 1.4, n))
+
+
+def _launches(ctx, frame):
+    before = ctx.launches()
+    frame()
+    return ctx.launches() - before
+
+
+NEAR = scenes.look_at((0.0, -2.5, 0.5), (0.0, 0.0, 0.0), 1920, 1080, 70.0)   # at the pile: large boxes, two slabs
+SMALL = scenes.look_at((0.0, -3.0, 0.3), (0.0, 0.0, 0.0), 160, 96, 60.0)
+
+
+def test_requests_of_different_sizes(api, tiny_asset):
+    """A server slot that takes large and small requests in turn runs each as a context that only renders it does: the
+    large one in slabs, the small one in one."""
+    Context, _ = api
+    large, small = (_pile(12, 0.5), NEAR, 0.25), (scenes.single_instance(), SMALL, 1.0)
+    alone = []
+    for inst, cam, tau in (large, small):
+        with Context(0) as ctx:
+            ctx.load_hierarchy(tiny_asset)
+            ctx.set_instances(inst)
+
+            def frame():
+                ctx.select(cam, tau)
+                ctx.render_host()
+            alone.append([_launches(ctx, frame) for _ in range(3)])
+    assert alone[0][1] == alone[0][2] > alone[1][2] == alone[1][1]
+    with Context(0) as ctx:
+        ctx.load_hierarchy(tiny_asset)
+        ctx.server_start(1)
+
+        def serve(inst, cam, tau):
+            t = ctx.submit(inst, cam, tau)
+            while ctx.poll(t, 100_000) is None:
+                pass
+        got = [(_launches(ctx, lambda: serve(*large)), _launches(ctx, lambda: serve(*small))) for _ in range(5)]
+        ctx.server_stop()
+    assert got[1:] == [(alone[0][2], alone[1][2])] * 4, (got, alone)   # (the slot's first large one grows its buffers)
