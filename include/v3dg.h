@@ -157,7 +157,7 @@ enum {
                                 v3dg_render runs the selection and the whole render as one CUDA
                                 graph, captured the first time a configuration (instance and view
                                 count, image size and intrinsics, buffer capacities, options,
-                                output pointers) is seen and replayed after that.  Same images;
+                                output pointers, depth slabs) is seen and replayed after that.  Same images;
                                 the frame counters are valid after v3dg_render.  Not used while
                                 V3DG_OPT_STAGE_TIMING is on.  Default 0. */
 };

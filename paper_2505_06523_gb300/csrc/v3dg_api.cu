@@ -123,12 +123,17 @@ struct Pipe {
   // blend, its end)
   cudaEvent_t ev[2 + 6 * kMaxSlabs] = {};
   // CUDA-graph frames (V3DG_OPT_GRAPHS): the selection is enqueued with the render, and both are
-  // captured once per configuration (gkey) on cap_stream, then replayed on `stream`
+  // captured once per configuration (the graph's key) on cap_stream, then replayed on `stream`.  One
+  // graph for each number of slabs: views of one size that alternate between two of them capture
+  // no frame again.
   bool select_pending = false;
   cudaStream_t cap_stream = nullptr;
-  cudaGraphExec_t gexec = nullptr;
-  std::vector<uint64_t> gkey;
-  uint64_t glaunches = 0;   // kernel launches in the captured graph
+  struct FrameGraph {
+    cudaGraphExec_t exec = nullptr;
+    std::vector<uint64_t> key;
+    uint64_t launches = 0;   // kernel launches in the captured graph
+  };
+  FrameGraph graphs[kMaxSlabs + 1];
 };
 
 struct v3dg_ctx {
@@ -809,10 +814,14 @@ v3dg_status run_frame(Pipe* c, float* rgb, float* t_out, bool sync) {
   return fail(c, V3DG_EOVERFLOW, "frame still overflows after growing the buffers");
 }
 
-void drop_graph(Pipe* c) {
-  if (c->gexec) cudaGraphExecDestroy(c->gexec);
-  c->gexec = nullptr;
-  c->gkey.clear();
+void drop_graph(Pipe::FrameGraph& g) {
+  if (g.exec) cudaGraphExecDestroy(g.exec);
+  g.exec = nullptr;
+  g.key.clear();
+}
+
+void drop_graphs(Pipe* c) {
+  for (Pipe::FrameGraph& g : c->graphs) drop_graph(g);
 }
 
 // What a captured frame depends on besides the contents of the instance frames (uploaded before
@@ -849,8 +858,9 @@ v3dg_status run_graph_frame(Pipe* c, float* rgb, float* t_out, bool sync) {
     ST(topdown_buffers(c, &td));
   }
   std::vector<uint64_t> key = graph_key(c, rgb, t_out);
-  if (!c->gexec || key != c->gkey) {
-    drop_graph(c);
+  Pipe::FrameGraph& graph = c->graphs[slab_count(c)];
+  if (!graph.exec || key != graph.key) {
+    drop_graph(graph);
     if (!c->cap_stream) CU(cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking));
     CU(cudaStreamSynchronize(c->stream));   // the capture stream must not run ahead of earlier work
     cudaStream_t saved = c->stream;
@@ -867,19 +877,19 @@ v3dg_status run_graph_frame(Pipe* c, float* rgb, float* t_out, bool sync) {
       if (e == cudaSuccess) e = e2;
     }
     c->stream = saved;
-    if (e == cudaSuccess && st == V3DG_OK) e = cudaGraphInstantiate(&c->gexec, g, 0);
+    if (e == cudaSuccess && st == V3DG_OK) e = cudaGraphInstantiate(&graph.exec, g, 0);
     if (g) cudaGraphDestroy(g);
     if (st != V3DG_OK) return st;
     if (e != cudaSuccess) {
-      c->gexec = nullptr;
+      graph.exec = nullptr;
       return fail(c, V3DG_ECUDA, "frame capture failed: %s", cudaGetErrorString(e));
     }
-    c->gkey = std::move(key);
-    c->glaunches = c->ctx->launches - launches0;
-    c->ctx->launches -= c->glaunches;   // counted when the graph runs
+    graph.key = std::move(key);
+    graph.launches = c->ctx->launches - launches0;
+    c->ctx->launches -= graph.launches;   // counted when the graph runs
   }
-  CU(cudaGraphLaunch(c->gexec, c->stream));
-  c->ctx->launches += c->glaunches;
+  CU(cudaGraphLaunch(graph.exec, c->stream));
+  c->ctx->launches += graph.launches;
   c->slabs = slab_count(c);
   c->full_lists = c->slabs == 1;
   c->rendered = true;
@@ -1014,7 +1024,7 @@ v3dg_status pipe_init(v3dg_ctx* ctx, Pipe* c, cudaStream_t stream) {
 
 void pipe_free(Pipe* c) {
   if (c->stream) cudaStreamSynchronize(c->stream);
-  drop_graph(c);
+  drop_graphs(c);
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
   c->cap_stream = nullptr;
   DevBuf* bs[] = {&c->d_inst, &c->d_frame, &c->d_cutframe, &c->d_misc, &c->d_list, &c->d_keys0,
@@ -1059,10 +1069,10 @@ uint64_t pipe_bytes(Pipe* c) {
 }
 
 // Releases the frame buffers (after the pipe's stream has finished with them); capacities start
-// over and grow again on demand.  A captured frame graph refers to them, so it is dropped.
+// over and grow again on demand.  The captured frame graphs refer to them, so they are dropped.
 void pipe_trim(Pipe* c) {
   if (c->stream) cudaStreamSynchronize(c->stream);
-  drop_graph(c);
+  drop_graphs(c);
   size_t n = 0;
   DevBuf* const* bs = frame_buffers(c, &n);
   for (size_t i = 0; i < n; ++i) dfree(c, *bs[i]);

@@ -59,3 +59,45 @@ def test_requests_of_different_sizes(api, tiny_asset):
         got = [(_launches(ctx, lambda: serve(*large)), _launches(ctx, lambda: serve(*small))) for _ in range(5)]
         ctx.server_stop()
     assert got[1:] == [(alone[0][2], alone[1][2])] * 4, (got, alone)   # (the slot's first large one grows its buffers)
+
+
+def test_alternating_graph_frames(api, tiny_asset):
+    """Captured frames of one size that alternate between two slab counts are captured once for each: after that a render
+    call, which only replays, takes the host no more than four times as long as when the view stays (a capture of the frame's 40
+    launches takes thirteen times as long).  Every image is the view's own."""
+    import time
+
+    import torch
+    Context, N = api
+    far = scenes.look_at((0.0, -60.0, 0.5), (0.0, 0.0, 0.0), 1920, 1080, 70.0)
+    buf, flush = torch.empty((1080, 1920, 3), device="cuda"), torch.cuda.synchronize
+    with Context(0) as ctx:
+        ctx.set_option(N.V3DG_OPT_GRAPHS, 1)
+        ctx.load_hierarchy(tiny_asset)
+        ctx.set_instances(_pile(12, 0.5))
+
+        def frame(cam):
+            ctx.select(cam, 0.25)
+            flush()
+            t0 = time.perf_counter()
+            ctx.render(buf)
+            t = time.perf_counter() - t0
+            flush()
+            return t
+        steady, images, launches = {}, {}, {}
+        for cam in (NEAR, far, NEAR, far):
+            for _ in range(4):
+                frame(cam)
+            launches[id(cam)] = _launches(ctx, lambda: frame(cam))
+            images[id(cam)] = buf.clone()
+        assert launches[id(NEAR)] > launches[id(far)]
+        ctx.set_option(N.V3DG_OPT_SYNC_CHECK, 0)   # (a render call then only enqueues)
+        for cam in (NEAR, far):
+            steady[id(cam)] = np.median([frame(cam) for _ in range(20)][4:])
+        alternating = {id(NEAR): [], id(far): []}
+        for _ in range(20):
+            for cam in (NEAR, far):
+                alternating[id(cam)].append(frame(cam))
+                assert bool((buf == images[id(cam)]).all())
+    for k, t in alternating.items():
+        assert np.median(t[4:]) <= 4.0 * max(steady.values()), (np.median(t[4:]), steady)
