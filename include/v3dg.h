@@ -316,7 +316,7 @@ v3dg_status v3dg_sort_pairs_noalloc(uint32_t* keys, uint32_t* vals, uint64_t n, 
  * started beside others would otherwise only take turns with them kernel by kernel: every stage
  * runs on a persistent grid).  A request's estimate (also used to size its frame buffers before its
  * first frame) grows with its instances, the square root of 1 / tau_px and, for its pairs, of its
- * pixel count (about 9 MB per instance of a 1M-leaf crowd at 1920x1080, tau 1).  A request
+ * pixel count (about 9.4 MB per instance of a 1M-leaf crowd at 1920x1080, tau 1).  A request
  * estimated above half its slot's share of the budget is heavy: it saturates the GPU on its own,
  * so at most one heavy request is in flight (light ones still overlap it).  A
  * request that starts while no other one is in flight, or whose estimate is at most a quarter of

@@ -262,10 +262,9 @@ constexpr uint32_t kSortHist = kMaxSlabs * kItemClasses, kDepthHist = kSortHist 
 // rarely overflows and re-runs), and for carrying one frame's counts over to another: about 1,000
 // render-list clusters per instance of a 1M-leaf crowd at tau 1 px (1.0M for the 1000-instance crowd at
 // 1920x1080), growing with sqrt(1 / tau) (a finer cut) and 25% headroom; pairs 2.25 per visible slot at 1920x1080, growing
-// with the square root of the pixel count (Gaussians span more tiles).  Bytes: per slot the depth
-// keys and values, record and box (72 B), per pair keys and values (16 B), per pixel 64 B.
+// with the square root of the pixel count (Gaussians span more tiles).
 struct FrameEstimate {
-  uint64_t nodes, pairs, bytes;
+  uint64_t nodes, pairs;
 };
 
 FrameEstimate estimate_frame(uint32_t n_inst, const v3dg_camera& cam, float tau_px) {
@@ -275,7 +274,6 @@ FrameEstimate estimate_frame(uint32_t n_inst, const v3dg_camera& cam, float tau_
   FrameEstimate e;
   e.nodes = uint64_t(nodes);
   e.pairs = uint64_t(pairs);
-  e.bytes = uint64_t(nodes * 64.0 * 72.0 + pairs * 16.0 + px * 64.0);
   return e;
 }
 
@@ -564,6 +562,12 @@ v3dg_status setup_frame(Pipe* c, const v3dg_camera* cams, uint32_t n_views, floa
   return setup_views(c, vs.data(), n_views);
 }
 
+uint64_t max_asset_nodes(const v3dg_ctx* ctx) {
+  uint64_t n = 0;
+  for (const AssetHost& a : ctx->assets) n = std::max<uint64_t>(n, a.n_nodes);
+  return n;
+}
+
 // Buffers of the top-down selection for the current instances: two frontiers that can each hold
 // every node of every instance, the per-level counts and the selection bitmap.
 v3dg_status topdown_buffers(Pipe* c, TopDown* td) {
@@ -592,12 +596,11 @@ v3dg_status topdown_buffers(Pipe* c, TopDown* td) {
 // the flat kernel would test more than kTopDownTests (instance, node) pairs (2, the default; on
 // small scenes the walk's one launch per level costs more than it saves).
 constexpr uint64_t kTopDownTests = 8u << 20;
-bool use_topdown(const Pipe* c) {
-  if (c->ctx->topdown != 2) return c->ctx->topdown == 1;
-  uint64_t max_nodes = 0;
-  for (const AssetHost& a : c->ctx->assets) max_nodes = std::max<uint64_t>(max_nodes, a.n_nodes);
-  return uint64_t(c->n_inst_frame) * max_nodes > kTopDownTests;
+bool use_topdown(const v3dg_ctx* ctx, uint64_t n_inst) {
+  if (ctx->topdown != 2) return ctx->topdown == 1;
+  return n_inst * max_asset_nodes(ctx) > kTopDownTests;
 }
+bool use_topdown(const Pipe* c) { return use_topdown(c->ctx, c->n_inst_frame); }
 
 // Selection into `out` (mode 0: the render list, mode 1: the cut), flat or top-down.
 v3dg_status launch_selection(Pipe* c, int mode, uint2* out, uint32_t cap, uint32_t* frame) {
@@ -1143,8 +1146,22 @@ struct Server {
 
 namespace {
 
-uint64_t request_bytes(uint32_t n_inst, const v3dg_camera& cam, float tau_px) {
-  return estimate_frame(n_inst, cam, tau_px).bytes;
+// A request's device memory, for its admission: the buffers of a frame of the estimated size in the
+// most slabs, as ensure_work, ensure_image_work and topdown_buffers allocate them, and its image.
+uint64_t request_bytes(const v3dg_ctx* ctx, uint32_t n_inst, const v3dg_camera& cam, float tau_px) {
+  const FrameEstimate e = estimate_frame(n_inst, cam, tau_px);
+  constexpr uint64_t kNodeBytes = 2 * sizeof(uint2) + sizeof(float2);                 // list, marks, depth range
+  constexpr uint64_t kSlotBytes = 5 * sizeof(uint32_t) + 3 * sizeof(float4) + sizeof(uint2);   // keys and values, record, box
+  constexpr uint64_t kPairBytes = 4 * sizeof(uint32_t);
+  constexpr uint64_t kTileBytes = sizeof(uint2) * kMaxSlabs + sizeof(uint32_t) * (kItemClasses + 2);   // ranges, items, liveness
+  constexpr uint64_t kPixelBytes = 5 * sizeof(float);                                 // image, transmittance, state
+  const uint64_t slots = e.nodes * kSlots;
+  const uint64_t tiles = uint64_t((cam.width + kTile - 1) / kTile) * uint64_t((cam.height + kTile - 1) / kTile);
+  uint64_t bytes = e.nodes * kNodeBytes + slots * kSlotBytes + e.pairs * kPairBytes + tiles * kTileBytes +
+                   uint64_t(cam.width) * uint64_t(cam.height) * kPixelBytes;
+  bytes += std::max(slots, e.pairs) / kSortTile * 256 * sizeof(uint64_t);             // the chained scans' status words
+  if (use_topdown(ctx, n_inst)) bytes += uint64_t(n_inst) * max_asset_nodes(ctx) * (2 * sizeof(uint2)) + uint64_t(n_inst) * (max_asset_nodes(ctx) / 8);
+  return bytes;
 }
 
 constexpr uint64_t kMergePixels = 3840ull * 2160ull;   // pixels of a merged frame (all its views)
@@ -2115,7 +2132,7 @@ v3dg_status v3dg_submit(v3dg_ctx* ctx, const v3dg_request* req, uint64_t* ticket
   rq.rgb = req->rgb_out;
   rq.t = req->t_out;
   rq.out_device = req->out_on_device != 0;
-  rq.est_bytes = request_bytes(n, cam, req->tau_px);
+  rq.est_bytes = request_bytes(ctx, n, cam, req->tau_px);
   rq.heavy = rq.est_bytes > sv->budget / (2 * uint64_t(sv->slots.size()));
   {
     std::lock_guard<std::mutex> lk(sv->mu);
