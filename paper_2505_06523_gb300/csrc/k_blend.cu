@@ -42,19 +42,21 @@ constexpr int kPxThreads = 256;
 constexpr int kPxWarps = kPxThreads / 32;
 constexpr float kLog2MinAlpha = -7.9943534f;  // log2(1/255)
 
-// log2(alpha) of a staged record at tile-local pixel centre (fx, fy); one definition for both phases
+// log2(alpha) of a staged record at tile-local pixel centre (fx, fy); one definition for both variants
 __device__ __forceinline__ float log2_alpha(const float4 g, const float4 c, float fx, float fy) {
   const float dx = fx - g.x, dy = fy - g.y;
   return fmaf(dx, fmaf(g.z, dx, g.w * dy), fmaf(c.x * dy, dy, c.y));
 }
 
-// One front-to-back step at a pixel (Sec. 2.1): alpha = min(0.999, 2^l2a), skipped below 1/255,
-// the pixel stops before T (1 - alpha) < 1e-4, else C += alpha T c and T *= 1 - alpha.  Both blend
-// kernels composite through this function, so their images are bit-identical.  Returns whether
-// the record contributed.
+// One front-to-back step at a pixel (Sec. 2.1): alpha = min(0.999, 2^l2a), skipped below 1/255 and where
+// l2a is not a number (a covariance that overflows), the pixel stops before T (1 - alpha) < 1e-4, else
+// C += alpha T c and T *= 1 - alpha.  Variant 1 composites through this function, variant 0 through
+// blend_step and blend_alpha: three forms of one rule, with the same roundings in the same order (2^l2a
+// has the same bits from exp2f and ex2.approx for l2a >= log2(1/255)), so the images are bit-identical;
+// a change goes into all three.  Returns whether the record contributed.
 __device__ __forceinline__ bool composite_step(float l2a, float r, float g, float b, float& T, float& cr, float& cg,
                                                float& cb, bool& done) {
-  const float a = l2a < kLog2MinAlpha ? 0.f : fminf(0.999f, exp2f(l2a));
+  const float a = l2a >= kLog2MinAlpha ? fminf(0.999f, exp2f(l2a)) : 0.f;
   if (a < 1.f / 255.f) return false;
   const float tn = T * (1.f - a);
   if (tn < 1e-4f) {

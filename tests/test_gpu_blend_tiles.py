@@ -111,3 +111,29 @@ def test_long_lists(n, aside):
     # the centre pixel's alpha is the opacity (2^(log2 o), a few ulp); it stops before T < 1e-4
     want = (1.0 - float(o)) ** min(stack, int(np.log(1e-4) / np.log(1.0 - float(o))))
     assert abs(float(out[0][1][12, 20]) / want - 1.0) <= 1e-5 + 4 * n * 2.0 ** -24 * (1 + float(o) / (1 - float(o)))
+
+
+def test_records_that_are_not_numbers_in_both_variants(small_asset):
+    """A Gaussian whose covariance overflows (log alpha is not a number) adds nothing in either variant: the images are the
+    same bit for bit, and not hidden behind it."""
+    import dataclasses
+
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2505_06523_gb300 import Context
+    from paper_2505_06523_gb300._native import V3DG_OPT_BLEND_MODE
+    ls = small_asset.log_scales.copy()
+    ls[7] = 46.0
+    huge = dataclasses.replace(small_asset, log_scales=ls)
+    cam = scenes.look_at((0.0, -2.6, 0.4), (0.0, 0.0, 0.0), 40, 24, 60.0)
+    imgs = []
+    with Context(0) as ctx:
+        ctx.load_hierarchy(huge)
+        ctx.set_instances(scenes.single_instance())
+        for mode in (0, 1):
+            ctx.set_option(V3DG_OPT_BLEND_MODE, mode)
+            ctx.select(cam, 0.25)
+            imgs.append([x.cpu().numpy() for x in ctx.render(want_T=True)])
+        proj = ctx.get_projected()
+    assert not np.isfinite(proj["conic"][proj["local"] == 7]).any() and (proj["local"] == 7).sum() == 1
+    assert (imgs[0][0] == imgs[1][0]).all() and (imgs[0][1] == imgs[1][1]).all()
