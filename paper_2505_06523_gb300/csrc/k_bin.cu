@@ -54,7 +54,8 @@ k_expand(const uint32_t* __restrict__ slots0, const uint32_t* __restrict__ slots
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t n = min(slab[kSlabCount], cap);
   const uint32_t ntiles = (n + kExpTile - 1) / kExpTile;
-  if (blockIdx.x >= ntiles || frame[kOverflow]) return;   // (an overflowed frame has no pairs)
+  // an overflowed frame has no pairs; after a wait that gave up the slots may be anything
+  if (blockIdx.x >= ntiles || frame[kOverflow] || frame[kTimeout]) return;
   const uint32_t* __restrict__ slots = (sort_passes(slab[kSlabBits]) & 1u) ? slots1 : slots0;
   for (;;) {   // persistent blocks: tiles in the order of an atomic counter
   if (threadIdx.x == 0) s_tile = atomicAdd(slab + kSlabExpandTile, 1u);

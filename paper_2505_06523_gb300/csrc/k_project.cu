@@ -51,7 +51,7 @@ __global__ void __launch_bounds__(256)
 k_order_keys(const uint2* __restrict__ list, uint32_t cap, const InstFrame* __restrict__ inst,
              const AssetDev* __restrict__ assets, const uint32_t* __restrict__ frame, uint32_t* __restrict__ order_keys,
              int key_shift) {
-  const uint32_t n = min(frame[kRenderNodes], cap);
+  const uint32_t n = frame[kTimeout] ? 0u : min(frame[kRenderNodes], cap);
   for (uint32_t ci = blockIdx.x * blockDim.x + threadIdx.x; ci < n; ci += gridDim.x * blockDim.x) {
     const uint2 e = list[ci];
     order_keys[ci] = (assets[inst[e.x].asset].node_base + e.y) >> key_shift;
@@ -349,7 +349,8 @@ k_project(const uint2* __restrict__ list, uint32_t cap_nodes, const InstFrame* _
   __shared__ uint32_t s_hist[kSlabs ? kDepthBins : 1];
   __shared__ EntryConst s_ent[kProjThreads / 32][kMaxChunk];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint32_t n_nodes = min(frame[kRenderNodes], cap_nodes);
+  // (after a wait of the selection or of the order's sort that gave up, the entries may be anything)
+  const uint32_t n_nodes = frame[kTimeout] ? 0u : min(frame[kRenderNodes], cap_nodes);
   // small frames: chunks just large enough that every warp gets one, then half entries, so that the
   // few entries there are do not queue up in a few warps (96x80 thumbnail, 313 entries in chunks of 16:
   // 59 us; halves: 17 us)

@@ -759,6 +759,7 @@ v3dg_status enqueue_render(Pipe* c, float* rgb, float* t_out) {
 // The whole frame's sorted Gaussians, pairs and tile ranges (the parity read-backs read them): a frame rendered in several slabs has only the last one's, so its lists are
 // made again in one slab without the filter, from the keys, boxes and records that are still there.
 v3dg_status ensure_full_lists(Pipe* c) {
+  if (c->h_frame[kTimeout]) return fail(c, V3DG_ETIMEOUT, "a bounded device-side wait gave up; frame invalid");
   if (c->full_lists) return V3DG_OK;
   const int n_tiles = c->cc.tiles_x * c->cc.tiles_y * int(c->n_views);
   uint32_t* frame = P<uint32_t>(c->d_frame);
