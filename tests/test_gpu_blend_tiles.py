@@ -137,3 +137,34 @@ def test_records_that_are_not_numbers_in_both_variants(small_asset):
         proj = ctx.get_projected()
     assert not np.isfinite(proj["conic"][proj["local"] == 7]).any() and (proj["local"] == 7).sum() == 1
     assert (imgs[0][0] == imgs[1][0]).all() and (imgs[0][1] == imgs[1][1]).all()
+
+
+def test_lists_on_both_sides_of_the_block_threshold(tiny_asset, small_asset):
+    """A crowd with lists that a block blends together beside lists that single warps do, in many tiles: bit for bit the
+    image of the block-per-tile variant."""
+    import torch
+
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2505_06523_gb300 import Context
+    from paper_2505_06523_gb300._native import V3DG_OPT_BLEND_MODE
+    inst = scenes.crowd_instances(200, n_assets=2, half_extent=70.0)
+    cam = scenes.crowd_camera(40, 640, 360)
+    out = []
+    with Context(0) as ctx:
+        for a in (tiny_asset, small_asset):
+            ctx.load_hierarchy(a)
+        ctx.set_instances(inst)
+        for mode in (1, 0):
+            ctx.set_option(V3DG_OPT_BLEND_MODE, mode)
+            ctx.select(cam, 1.0)
+            out.append([x.cpu().numpy() for x in ctx.render(want_T=True)])
+        r = ctx.tile_ranges().astype(np.int64)
+        pairs = ctx.frame_stats()["pairs"]
+    # long: the octaves of at least a warp's share of the pairs, each key read by eight warps, and of at least 256 (five
+    # blocks of four warps per SM)
+    n, warps = r[:, 1] - r[:, 0], 4 * 5 * torch.cuda.get_device_properties(0).multi_processor_count
+    octave = 1 << int(np.ceil(np.log2(max(pairs // (warps // 8), 256))))
+    assert (n >= octave).sum() >= 8 and ((n > 0) & (n < octave)).sum() >= 8, (octave, np.sort(n)[-16:])
+    assert float(np.abs(out[0][0]).sum()) > 0
+    assert (out[0][0] == out[1][0]).all() and (out[0][1] == out[1][1]).all()
