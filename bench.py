@@ -304,6 +304,37 @@ def cpu_baseline_leg(assets_n, inst, tau):
                                              "whole frames (selection, projection, image in 16-row bands on the pool)"}}
 
 
+def _short(v):
+    """The same value with seven significant digits in its floats."""
+    if isinstance(v, dict):
+        return {k: _short(x) for k, x in v.items()}
+    if isinstance(v, (list, tuple)):
+        return [_short(x) for x in v]
+    return float(f"{v:.7g}") if isinstance(v, float) else v
+
+
+def headline(full):
+    """The line that goes to stdout: the run's own figures, and of the extra legs what sums them up, short enough
+    (below 3,000 characters) for whoever keeps only the end of the output.  The full record goes to stderr."""
+    line = {k: v for k, v in full.items() if k not in ("served", "orbit", "v3dg_vs_vanilla", "roofline", "cpu_baseline",
+                                                       "frame_mean", "select_flat_ms", "project_list_order_ms")}
+    if full.get("served"):
+        s = full["served"]
+        line["served"] = {"plain": s["plain"]["closed"], "served": s["served"]["closed"],
+                          "frames_per_s_ratio": s["served_vs_plain"]["frames_per_s"],
+                          "psnr_fp16_vs_fp32_min_db": min(s["psnr_fp16_vs_fp32_db"]), "autotune": s["autotune"]}
+        if "batched" in s:
+            line["served"]["batched_frames_per_s"] = {f"tau{k}": t["value"] for k, t in s["batched"]["taus"].items()}
+    if full.get("v3dg_vs_vanilla"):
+        line["speedup_vs_vanilla"] = full["v3dg_vs_vanilla"]["speedup"]
+    line["roofline"] = {k: full["roofline"][k] for k in ("stage", "bound", "achieved", "peak", "unit", "frac", "traffic")}
+    line["roofline"]["frame_frac"] = full["roofline"]["frame"]["frac"]
+    if full.get("cpu_baseline"):
+        line["cpu_baseline"] = {k: full["cpu_baseline"][k] for k in ("value", "unit", "cores", "kind", "extrapolated")}
+    line["frame_mean"] = {k: full["frame_mean"][k] for k in ("render_nodes", "visible", "pairs")}
+    return _short(line)
+
+
 REF_RUN_S = 150.0   # wall time of the whole reference run (warm-up and timed steps), seconds
 
 
@@ -529,7 +560,8 @@ def main():
             "cpu_baseline": cpu,
             "clocks": clk.summary(),
         }
-        print(json.dumps(line), flush=True)
+        print(json.dumps(line), file=sys.stderr, flush=True)
+        print(json.dumps(headline(line)), flush=True)
     ctx.close()
     if world > 1:
         torch.distributed.destroy_process_group()

@@ -135,3 +135,39 @@ def test_request_mix_scenes():
     assert {k: v.n for k, v in sc.items()} == {100: 100, 1000: 1000, 5000: 5000}
     assert (sc[100].trans == crowd.trans[:100]).all() and (sc[5000].trans[:1000] == crowd.trans).all()
     assert sc[5000].asset.max() < 3
+
+
+def test_line_on_stdout_is_short():
+    """The line on stdout holds the run's own figures and the sums of the extra legs in less than 3,000 characters, whatever
+    the full record's legs hold."""
+    import json
+    x = 123.45678901234567
+    lat = {"value": x, "unit": "frames/s", "p50_ms": x, "p99_ms": x}
+    arm = {"path": "FP16 colour, 4 slots, autotuned blend", "closed": lat, "poisson": [lat, lat]}
+    taus = {"1": {"frames": 48, "value": x, "psnr_fp16_vs_fp32_db": [x] * 16}, "2": {"frames": 48, "value": x}}
+    full = {
+        "metric": bench.METRIC, "value": x, "unit": "frames/s", "n_gpus": 1, "steps": 20, "warmup": 5, "ms_per_step": x,
+        "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f32", "data": "synthetic",
+        "config": {"workload": bench.WORKLOAD, "tau_px": 1.0, "path": "plain FP32, one frame at a time",
+                   "parallelism": "replicas x1", "l2": "inputs larger than L2 (3.1 GB of attributes; per-frame gathers of the "
+                                                      "selected Gaussians exceed the 129 MB L2)"},
+        "p50_ms": x, "p99_ms": x, "e2e": {"value": x, "unit": "frames/s", "h2d_bytes_per_step": 256000, "d2h_bytes_per_step": 24883200},
+        "served": {"plain": arm, "served": arm, "served_vs_plain": {"frames_per_s": x, "p99_at_90pct_load": x},
+                   "psnr_fp16_vs_fp32_db": [x] * 16, "autotune": {"mode": 0, "batch": 512, "split_pairs": 0xFFFFFFFF, "ms": x},
+                   "mix": {"rates": [lat] * 200}, "batched": {"taus": taus}},
+        "v3dg_vs_vanilla": {"speedup": x, "v3dg": {"ms": x}}, "orbit": {"rows": [lat] * 100}, "gpu_launches": 1460,
+        "stages_ms": {k: x for k in STAGE_MS}, "select_flat_ms": x, "project_list_order_ms": x,
+        "frame_mean": {k: 136564308 for k in ("cut_nodes", "cut_gaussians", "render_nodes", "render_clusters", "visible", "pairs",
+                                              "blend_evals", "blend_contribs")},
+        "stages_sum_ms": x, "roofline": bench.roofline_for("project", STAGE_MS, FS, PEAKS, "measured"),
+        "cpu_baseline": {"value": x, "unit": "frames/s", "cores": 16, "kind": "oracle", "extrapolated": True, "sample": "y" * 900},
+        "clocks": {"sm_mhz": 2070.0, "sm_max_mhz": 2070.0, "reasons": ["sw_power_cap"], "samples": 12}}
+    line = bench.headline(full)
+    assert len(json.dumps(line)) < 3000, len(json.dumps(line))
+    for k in ("metric", "unit", "n_gpus", "steps", "warmup", "higher_is_better", "scaling", "vs_baseline", "dtype", "data", "config",
+              "e2e", "gpu_launches", "clocks"):
+        assert line[k] == bench._short(full[k]), k
+    assert line["value"] == pytest.approx(x, rel=1e-6) and line["ms_per_step"] == pytest.approx(x, rel=1e-6)
+    assert line["served"]["served"]["p99_ms"] == pytest.approx(x, rel=1e-6)
+    # without the extra legs
+    assert "served" not in bench.headline({**full, "served": None, "v3dg_vs_vanilla": None, "cpu_baseline": None})
