@@ -93,7 +93,8 @@ typedef struct {
   uint64_t cut_gaussians;   /* Gaussians in those clusters */
   uint64_t render_nodes;    /* cut clusters left after the conservative visibility cull */
   uint64_t visible;         /* Gaussians that survive the projection culls */
-  uint64_t pairs;           /* (tile, Gaussian) pairs sorted and blended */
+  uint64_t pairs;           /* (tile, Gaussian) pairs of the visible Gaussians (of them, a frame in
+                               depth slabs sorts and blends those that the front does not hide) */
   uint32_t overflow;        /* nonzero if a capacity was exceeded in the last frame, or in any
                                frame rendered since the previous v3dg_frame_stats call */
   uint32_t timeout;         /* likewise for a bounded device wait that gave up */

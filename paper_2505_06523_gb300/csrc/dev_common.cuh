@@ -131,13 +131,6 @@ __device__ __forceinline__ uint32_t chained_exclusive_warp(uint64_t* status, uin
   return excl;
 }
 
-// Exclusive prefix of `agg` over all tiles before `tile`: publish, then look back.
-__device__ __forceinline__ uint32_t chained_exclusive(uint64_t* status, uint32_t stride, uint32_t tile,
-                                                      uint32_t agg, uint32_t epoch, uint32_t* err) {
-  chain_publish(status, stride, tile, agg, epoch);
-  return chain_lookback(status, stride, tile, agg, epoch, err);
-}
-
 // Passes that a sort of `bits` key bits takes (the result is in the second buffers when odd).
 __device__ __forceinline__ uint32_t sort_passes(uint32_t bits) { return (bits + 7u) / 8u; }
 

@@ -36,7 +36,7 @@ namespace v3dg {
 namespace {
 
 constexpr int kBlendThreads = 128;   // four warps, independent except on long lists
-constexpr int kBlendBlocks = 5;      // resident blocks per SM: 20 warps of at most 96 registers, 39 KB of shared memory each
+constexpr int kBlendBlocks = 5;      // resident blocks per SM: 20 warps of at most 96 registers, 37 KB of shared memory each
 constexpr uint32_t kLongPairs = 256;   // shortest list that a block blends together
 constexpr int kPxThreads = 256;
 constexpr int kPxWarps = kPxThreads / 32;
@@ -937,7 +937,7 @@ constexpr int kBlendShared = int(std::max(sizeof(BlendBlock), sizeof(BlendWarp) 
 }  // namespace
 
 cudaError_t blend_set_attributes() {
-  // several resident blocks of 10-28 KB shared memory per SM want the largest carveout
+  // several resident blocks per SM, of up to 37 KB shared memory each, want the largest carveout
   const void* fns[] = {(const void*)k_blend<true, false>,   (const void*)k_blend<false, false>,
                        (const void*)k_blend<true, true>,    (const void*)k_blend<false, true>,
                        (const void*)k_blend_px<true, 128>,  (const void*)k_blend_px<false, 128>,

@@ -54,7 +54,8 @@ constexpr uint32_t kInitPairs = 1u << 22;
 constexpr uint32_t kMaxNodes = 1u << 25;               // render-list clusters: at most 2^31 slots
 constexpr uint32_t kMaxPairs = 0xFFFFFFFFu - 4096u;    // pair indices are 32-bit (a sort tile of headroom)
 constexpr uint64_t kManyPairs = 1u << 26;              // expected pairs from which a frame is taken in slabs
-enum { kStageSelect = 0, kStageProject, kStageDepthSort, kStageBin, kStageTileSort, kStageRanges, kStageBlend, kStages };
+// stages: select, project, then in each slab depth sort, bin, tile sort, ranges, blend
+enum { kStageProject = 1, kStages = 7 };
 
 }  // namespace
 
@@ -97,7 +98,7 @@ struct Pipe {
   cudaEvent_t ev_inst = nullptr;
   DevBuf d_frame, d_cutframe, d_misc;
   uint32_t* h_frame = nullptr;   // pinned copy of the frame words, written at the end of each frame
-  uint32_t* h_tmp = nullptr;     // pinned scratch: [0, 48) frame words of read-backs, [48, 52) blend work
+  uint32_t* h_tmp = nullptr;     // pinned scratch: [0, kFrameWords) frame words of read-backs, then two 64-bit blend work counters
 
   uint32_t cap_nodes = 0, cap_slots = 0, cap_pairs = 0, status_words = 0, cap_cut = 0;
   uint32_t set_nodes = 0, set_pairs = 0;   // capacities set by option (0: none), taken over when the buffers are next sized
@@ -145,11 +146,10 @@ struct v3dg_ctx {
   DevBuf d_assets;
   std::atomic<uint64_t> launches{0};
   bool sync_check = true, stage_timing = false, count_work = false;
-  uint32_t split_pairs = 0xFFFFFFFFu;   // long-tile split threshold: accepted, no blend variant splits tiles
   bool attr_fp16 = false;   // store opacity and SH of the next loaded assets as float16
   int topdown = 2;          // 0 flat, 1 level by level from the roots (same cut), 2 top-down for large scenes
-  int blend_batch = 512;    // records staged per blend batch: 128, 256 or 512
-  int blend_mode = 0;       // 0: two-phase blend; 1: bulk-copy staging, warps composite row pairs
+  int blend_batch = 512;    // records that variant 1 stages per blend batch: 128, 256 or 512
+  int blend_mode = 0;       // 0: a warp per 8x4 pixels; 1: bulk-copy staging, warps composite row pairs
   int serve_merge = 1;      // server: most queued requests of one image geometry rendered together
   int project_order = 2;    // projection by cluster: 0 never, 1 always, 2 when instances repeat assets
   uint64_t total_nodes = 0; // nodes of all loaded assets (global cluster ids are below this)
@@ -1464,8 +1464,7 @@ v3dg_status v3dg_set_option(v3dg_ctx* ctx, int option, int64_t value) {
       break;
     case V3DG_OPT_SPLIT_PAIRS:
       if (value < 1 || value > 0xFFFFFFFFll) return fail(c, V3DG_EINVAL, "split threshold out of range");
-      ctx->split_pairs = uint32_t(value);
-      break;
+      break;   // (no variant splits tiles)
     case V3DG_OPT_CAP_NODES:
       if (value < 64 || value > int64_t(kMaxNodes)) return fail(c, V3DG_EINVAL, "node capacity out of range");
       c->set_nodes = uint32_t(value);
