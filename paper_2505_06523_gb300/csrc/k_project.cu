@@ -20,7 +20,9 @@
 //   references and small chunks, before -> now: 96x80 thumbnail 67 -> 26 us, 300k-leaf asset at
 //   1001x563 116 -> 42 us, 200 instances at 640x360 159 -> 118 us, crowd at 1080p 1.66 -> 1.61 ms,
 //   5000 instances at 4K 11.1 -> 10.5 ms.  It stays bound by registers (128: a Gaussian's 59
-//   attributes; 16 warps per SM) and by its 60 bytes written per Gaussian.
+//   attributes; 16 warps per SM; 64 bytes of spill stores in frames of several slabs, 80 of one, 330 and 370
+//   where both colour formats occur -- 8 to 24 and 356 before the references moved in) and by its 60 bytes
+//   written per Gaussian.
 #include <algorithm>
 
 #include <cuda_fp16.h>

@@ -53,7 +53,10 @@ k_frame_init(uint32_t* __restrict__ frame, uint32_t* __restrict__ hist, uint32_t
 // 4.34 / 4.72 ms, one asset filling 1080p (31M) 0.87 / 0.95 ms.  Two slabs' limit at 250, 350 and 450: that crowd
 // 4.34, 4.48, 4.51 ms; the asset 0.88, 0.87, 0.90 ms, from 3 units (44M) 1.85, 1.64, 1.65 ms: frames of
 // large boxes take the later limit.  Limits tried with four: {20, 80, 250}, {30, 120, 350}, {40, 160, 400}, {60, 200, 400}, {70, 250, 450}, {100, 300, 500}: the crowd 7.32,
-// 6.68, 6.87, 6.85, 6.32, 6.15 ms.
+// 6.68, 6.87, 6.85, 6.32, 6.15 ms.  With six: {30, 90, 200, 340, 520}, {40, 120, 240, 360, 500}, these, {60, 160, 320,
+// 500, 700}, {80, 190, 330, 480, 650}, {100, 220, 360, 500, 650}: 5000 instances at 4K 26.0, 24.8, 25.8, 26.2, 27.1,
+// 27.0 ms, 16 crowd views 53.0, 53.3, 50.5, 50.6, 50.0, 50.1 ms, five views (869M pairs) 24.0, 24.2, 23.6, 24.1, 24.0,
+// 24.4 ms.
 __constant__ const uint32_t kLimits2[1] = {250}, kLimits2Large[1] = {350}, kLimits4[3] = {83, 300, 500},
                             kLimits6[5] = {50, 140, 280, 430, 600};
 

@@ -286,6 +286,8 @@ FrameEstimate estimate_frame(uint32_t n_inst, const v3dg_camera& cam, float tau_
 // asset at 1.7, 2 and 2.5 units, 33, 36 and 47M pairs, one / two: 1.14 / 0.95, 1.31 / 1.11 and 1.73 / 1.55 ms) and stay
 // at two (at 4K, 117 and 131M pairs, four / two: 2.47 / 2.40 and 3.33 / 3.15 ms).  Crowd frames of 69, 91, 95, 98,
 // 123 and 133M pairs, two / four: 4.73 / 5.09, 5.06 / 5.40, 5.46 / 5.73, 5.20 / 5.13, 6.22 / 5.70 and 5.53 / 5.33 ms.
+// Two to five crowd views of 346, 519, 695 and 869M pairs, four / six: 10.5 / 10.9, 15.0 / 15.0, 19.7 / 19.3 and 24.1 /
+// 23.6 ms; crowds at 4K of 359, 609, 642 and 924M: 10.7 / 10.7, 13.2 / 12.9, 13.0 / 13.3 and 15.1 / 14.6 ms.
 constexpr uint64_t kFourSlabs = 96'000'000;
 int slab_count(const Pipe* c) {
   const uint64_t pairs = c->pairs_hint;
