@@ -117,7 +117,7 @@ struct Pipe {
   FrameCounts seen[kCountClasses];
   double expected = 1.0;
   uint64_t pairs_hint = 0, visible_hint = 0;
-  int slabs = 1;             // depth slabs of the last rendered frame
+  int timed_slabs = 1;       // depth slabs of the last frame rendered with stage events
   bool full_lists = false;   // the sorted Gaussians and pairs of the whole frame are on the device
   uint32_t epoch = 1;
   // stage events: [0] select, [1] project, then six per slab (depth sort, bin, tile sort, ranges,
@@ -752,7 +752,7 @@ v3dg_status enqueue_render(Pipe* c, float* rgb, float* t_out) {
   if (work)
     CU(cudaMemcpyAsync(c->h_tmp + kFrameWords, work, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, c->stream));
   CU(cudaMemcpyAsync(c->h_frame, c->d_frame.p, sizeof(uint32_t) * kFrameWords, cudaMemcpyDeviceToHost, c->stream));
-  c->slabs = slabs;
+  if (c->ctx->stage_timing) c->timed_slabs = slabs;
   c->full_lists = slabs == 1;
   c->rendered = true;
   return V3DG_OK;
@@ -896,8 +896,7 @@ v3dg_status run_graph_frame(Pipe* c, float* rgb, float* t_out, bool sync) {
   }
   CU(cudaGraphLaunch(graph.exec, c->stream));
   c->ctx->launches += graph.launches;
-  c->slabs = slab_count(c);
-  c->full_lists = c->slabs == 1;
+  c->full_lists = slab_count(c) == 1;
   c->rendered = true;
   if (!sync) return V3DG_OK;
   CU(cudaStreamSynchronize(c->stream));
@@ -935,7 +934,7 @@ v3dg_status render_frame(Pipe* c, float* rgb, float* t_out, bool sync) {
 cudaError_t stage_ms(const Pipe* c, int stage, float* ms) {
   if (stage <= kStageProject) return cudaEventElapsedTime(ms, c->ev[stage], c->ev[stage + 1]);
   *ms = 0.f;
-  for (int slab = 0; slab < c->slabs; ++slab) {
+  for (int slab = 0; slab < c->timed_slabs; ++slab) {
     float t = 0.f;
     const cudaError_t e = cudaEventElapsedTime(&t, c->ev[6 * slab + stage], c->ev[6 * slab + stage + 1]);
     if (e != cudaSuccess) return e;
@@ -1908,7 +1907,7 @@ v3dg_status v3dg_autotune_blend(v3dg_ctx* ctx, uint32_t* mode_out, uint32_t* bat
     int mode, batch, slabs;
     bool timing, count;
     explicit Restore(Pipe* p)
-        : c(p), mode(p->ctx->blend_mode), batch(p->ctx->blend_batch), slabs(p->slabs), timing(p->ctx->stage_timing),
+        : c(p), mode(p->ctx->blend_mode), batch(p->ctx->blend_batch), slabs(p->timed_slabs), timing(p->ctx->stage_timing),
           count(p->ctx->count_work) {
       std::swap(ev, c->ev);
     }
@@ -1920,7 +1919,7 @@ v3dg_status v3dg_autotune_blend(v3dg_ctx* ctx, uint32_t* mode_out, uint32_t* bat
       c->ctx->blend_batch = batch;
       c->ctx->stage_timing = timing;
       c->ctx->count_work = count;
-      c->slabs = slabs;
+      c->timed_slabs = slabs;
     }
   };
   const int batches[] = {128, 256, 512};

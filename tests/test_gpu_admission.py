@@ -33,7 +33,7 @@ def test_admitted_for_their_buffers(tiny_asset):
     with Context(0) as ctx:
         ctx.load_hierarchy(tiny_asset)
         ctx.server_start(2, sum(held) - 1)
-        for _ in range(2):   # (the first round warms the pinned images and the pool up)
+        for _ in range(2):   # (the first time warms the pinned images and the pool up)
             tickets = [ctx.submit(inst, cam, tau) for inst, tau in requests]
             done = {}
             while len(done) < 3:

@@ -158,3 +158,26 @@ def test_frames_run_in_slabs(api, tiny_asset, n, spread, width, height, fov, vie
     assert float(np.abs(out[0][0]).sum()) > 0
     for rgb, T in out[1:]:
         assert (rgb == out[0][0]).all() and (T == out[0][1]).all()
+
+
+def test_stage_times_are_of_the_last_timed_frame(api, tiny_asset):
+    """Frames rendered with stage timing off, whatever their slabs, leave the stage times of the last timed one."""
+    Context, N = api
+    with Context(0) as ctx:
+        ctx.load_hierarchy(tiny_asset)
+        ctx.set_instances(_pile(12, 0.5))
+
+        def frame():
+            ctx.select(NEAR, 0.25)
+            ctx.render()
+        ctx.set_option(N.V3DG_OPT_STAGE_TIMING, 1)
+        ctx.set_option(N.V3DG_OPT_BLEND_MODE, 1)
+        frame()   # (one slab)
+        one = ctx.stage_times()[0]
+        ctx.set_option(N.V3DG_OPT_STAGE_TIMING, 0)
+        ctx.set_option(N.V3DG_OPT_BLEND_MODE, 0)
+        assert _launches(ctx, frame) > 30   # (two slabs)
+        ctx.set_option(N.V3DG_OPT_STAGE_TIMING, 1)
+        assert ctx.stage_times()[0] == one and min(one) > 0
+        frame()
+        assert ctx.stage_times()[0] != one
